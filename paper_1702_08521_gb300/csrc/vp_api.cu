@@ -155,10 +155,11 @@ void free_buffers(vp_ctx *c) {
     cudaFree(c->d_phi);
     cudaFree(c->d_acc);
     cudaFree(c->d_rho_s);
-    cudaFree(c->d_phi_s);
     cudaFree(c->d_fft);
     cudaFree(c->d_green);
     cudaFree(c->d_ghat);
+    cudaFree(c->d_roots);
+    cudaFree(c->d_conv);
     cudaFree(c->d_part);
     cudaFree(c->d_diag);
     cudaFree(c->d_flag);
@@ -222,13 +223,13 @@ int enqueue_step(vp_ctx *c, double dt, int split, double *acc, const float *wts)
             if ((rc = sweep_all(c, 1, d, 0.5 * dt, acc + d * NX))) return rc;
         if ((rc = drifts(dt))) return rc;
         if ((rc = vp_launch_moment(c, c->d_rho_s))) return rc;
-        if ((rc = vp_launch_poisson(c, c->d_rho_s, c->d_phi_s, acc))) return rc;
+        if ((rc = vp_launch_poisson(c, c->d_rho_s, nullptr, acc))) return rc;
         for (int d = 0; d < g.dv; ++d)
             if ((rc = sweep_all(c, 1, d, 0.5 * dt, acc + d * NX))) return rc;
     } else {
         if ((rc = drifts(0.5 * dt))) return rc;
         if ((rc = vp_launch_moment(c, c->d_rho_s))) return rc;
-        if ((rc = vp_launch_poisson(c, c->d_rho_s, c->d_phi_s, acc))) return rc;
+        if ((rc = vp_launch_poisson(c, c->d_rho_s, nullptr, acc))) return rc;
         for (int d = 0; d < g.dv; ++d)
             if ((rc = sweep_all(c, 1, d, dt, acc + d * NX))) return rc;
         if ((rc = drifts(0.5 * dt))) return rc;
@@ -293,7 +294,6 @@ int vp_create(const vp_grid *grid, void *cuda_stream, vp_ctx **out) {
     ALLOC(c->d_phi, sizeof(double) * c->NX);
     ALLOC(c->d_acc, sizeof(double) * c->NX * c->g.dx);
     ALLOC(c->d_rho_s, sizeof(double) * c->NX);
-    ALLOC(c->d_phi_s, sizeof(double) * c->NX);
     ALLOC(c->d_part, sizeof(double) * c->NX * 6);
     ALLOC(c->d_diag, sizeof(double) * VP_NDIAG);
     ALLOC(c->d_flag, sizeof(int));
@@ -403,7 +403,7 @@ int vp_poisson_solve(vp_ctx *c, const double *rho_dev, double *phi_dev, double *
     int rc = check_ctx(c, false);
     if (rc) return rc;
     if (!rho_dev || !accel_dev) return vp_fail(c, VP_EINVAL, "rho_dev and accel_dev are required");
-    return vp_launch_poisson(c, rho_dev, phi_dev ? phi_dev : c->d_phi, accel_dev);
+    return vp_launch_poisson(c, rho_dev, phi_dev, accel_dev);
 }
 
 int vp_set_option(vp_ctx *c, int option, long long value) {

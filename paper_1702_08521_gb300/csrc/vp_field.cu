@@ -77,138 +77,324 @@ __global__ void __launch_bounds__(kBlock) k_moment(const T *__restrict__ f, long
     if (threadIdx.x == 0) rho[blockIdx.x] = s * dV;
 }
 
-// ---- Fourier transform along one axis of a row-major complex array ----------
-// One CTA per line; power-of-two lengths use an in-shared-memory radix-2
-// decimation-in-time transform, other lengths a direct sum.  sign = -1 is the
-// forward transform sum_j q_j exp(-i k j 2 pi / n) (Eq. C4), +1 the inverse
-// without 1/n.
+// ---- Fourier transforms of the field solve ---------------------------------------
+//
+// FP64 is the scarce unit here (two FMA lanes per SM and clock) and a launch
+// costs 2.5-4 us, so the solve is few launches that spread the FP64 work:
+//   * k_fft_lines transforms B lines of one axis in shared memory (Stockham,
+//     radices 4, 2, 3, 5 and direct sums for larger primes) with a table of
+//     the n roots of unity, read from the context or, for callers without
+//     one, computed once per CTA.  The first axis reads rho itself, and the
+//     last forward axis multiplies by the Green function and transforms back
+//     in the same pass.  Before (radix 2 with a double-precision sincospi per
+//     butterfly, direct sums with one per term): 17 us per axis at 64 points
+//     and 500 us per axis at 2024 lines of 40 points.
+//     The field solve of a 22 x 20 x 23 isolated box: 6.0 -> 0.25 ms; of a
+//     64 x 64 periodic box: 84 -> 42 us with its launches.
+//   * k_conv1: in one dimension the solve is a cyclic convolution, n^2 FMAs
+//     spread over the chip in one launch.
 
-__global__ void k_fft_axis(double2 *__restrict__ a, long long inner, int n, int sign) {
-    extern __shared__ double2 sbuf[];
-    double2 *x = sbuf;
-    double2 *y = sbuf + n;
-    const long long line = blockIdx.x;
-    const long long o = line / inner, c = line % inner;
-    double2 *base = a + o * (long long)n * inner + c;
-    const bool pow2 = (n & (n - 1)) == 0;
-    int logn = 0;
-    while ((1 << logn) < n) ++logn;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        int dst = j;
-        if (pow2 && n > 1) dst = (int)(__brev((unsigned)j) >> (32 - logn));
-        x[dst] = base[(long long)j * inner];
-    }
-    __syncthreads();
-    if (pow2) {
-        for (int len = 2; len <= n; len <<= 1) {
-            const int half = len >> 1;
-            for (int t = threadIdx.x; t < n / 2; t += blockDim.x) {
-                const int grp = t / half, k = t - grp * half;
-                const int i0 = grp * len + k, i1 = i0 + half;
-                double sn, cs;
-                sincospi((double)sign * 2.0 * (double)k / (double)len, &sn, &cs);
-                const double2 u = x[i0], v = x[i1];
-                const double2 tw = make_double2(v.x * cs - v.y * sn, v.x * sn + v.y * cs);
-                x[i0] = make_double2(u.x + tw.x, u.y + tw.y);
-                x[i1] = make_double2(u.x - tw.x, u.y - tw.y);
+constexpr int kFftMaxRad = 12;  // factors of an axis length <= 4096
+
+struct FftPlan {
+    int n, nr;
+    int rad[kFftMaxRad];
+};
+
+__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
+    return make_double2(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x));
+}
+
+// sum_j x_j exp(sign 2 pi i j k / n) of B lines (line b at x + b n), ping-pong
+// between x and y; w[j] = exp(-2 pi i j / n).  Returns the buffer that holds
+// the result (natural order); the caller's data must be in place (barrier
+// before), and a barrier follows the last pass.
+__device__ double2 *fft_lines(double2 *x, double2 *y, const double2 *w, const FftPlan &p, int B, int sign) {
+    const int n = p.n;
+    const double sg = sign < 0 ? 1.0 : -1.0;  // the table holds the forward roots
+    int Ns = 1;
+    for (int f = 0; f < p.nr; ++f) {
+        const int r = p.rad[f];
+        const int m = n / r, ts = m / Ns;  // butterflies per line, table stride of exp(-2 pi i / (Ns r))
+        if (r == 4 || r == 2) {
+            for (int t = threadIdx.x; t < B * m; t += blockDim.x) {
+                const int b = t / m, j = t - b * m;
+                const int k = j % Ns;
+                const double2 *xi = x + b * n + j;
+                double2 *yo = y + b * n + (j - k) * r + k;
+                auto tw = [&](int q) {
+                    const double2 v = w[q * k * ts];
+                    return cmul(xi[q * m], make_double2(v.x, sg * v.y));
+                };
+                if (r == 2) {
+                    const double2 a = xi[0], c = tw(1);
+                    yo[0] = cadd(a, c);
+                    yo[Ns] = csub(a, c);
+                } else {
+                    const double2 a = xi[0], c = tw(2), d = tw(1), e = tw(3);
+                    const double2 s0 = cadd(a, c), s1 = csub(a, c), s2 = cadd(d, e), s3 = csub(d, e);
+                    const double2 rot = make_double2(sg * s3.y, -sg * s3.x);  // -i (forward) or +i times s3
+                    yo[0] = cadd(s0, s2);
+                    yo[Ns] = cadd(s1, rot);
+                    yo[2 * Ns] = csub(s0, s2);
+                    yo[3 * Ns] = csub(s1, rot);
+                }
             }
-            __syncthreads();
-        }
-        for (int j = threadIdx.x; j < n; j += blockDim.x) base[(long long)j * inner] = x[j];
-    } else {
-        for (int k = threadIdx.x; k < n; k += blockDim.x) {
-            double sr = 0.0, si = 0.0;
-            for (int j = 0; j < n; ++j) {
-                const long long m = ((long long)j * k) % n;
-                double sn, cs;
-                sincospi((double)sign * 2.0 * (double)m / (double)n, &sn, &cs);
-                const double2 v = x[j];
-                sr += v.x * cs - v.y * sn;
-                si += v.x * sn + v.y * cs;
+        } else {
+            // direct: output o = (block, q, k) sums r inputs with the roots
+            // exp(-2 pi i p (k + q Ns) / (Ns r))
+            for (int t = threadIdx.x; t < B * n; t += blockDim.x) {
+                const int b = t / n, o = t - b * n;
+                const int blk = o / (Ns * r), kq = o - blk * (Ns * r);
+                const double2 *xi = x + b * n + blk * Ns + kq % Ns;
+                const int step = kq * ts;  // < n
+                double2 a0 = xi[0], a1 = make_double2(0.0, 0.0);
+                int idx = 0;
+                for (int q = 1; q < r; ++q) {
+                    idx += step;
+                    idx -= idx >= n ? n : 0;
+                    const double2 v = w[idx], u = xi[q * m];
+                    const double wy = sg * v.y;
+                    a0.x = fma(u.x, v.x, a0.x);
+                    a0.y = fma(u.x, wy, a0.y);
+                    a1.x = fma(-u.y, wy, a1.x);
+                    a1.y = fma(u.y, v.x, a1.y);
+                }
+                y[t] = cadd(a0, a1);
             }
-            y[k] = make_double2(sr, si);
         }
         __syncthreads();
-        for (int j = threadIdx.x; j < n; j += blockDim.x) base[(long long)j * inner] = y[j];
+        double2 *z = x;
+        x = y;
+        y = z;
+        Ns *= r;
+    }
+    return x;
+}
+
+// what a pass of k_fft_lines does with its lines
+enum { FFT_FWD = -1, FFT_INV = 1, FFT_CONV = 2 };
+
+struct FftArgs {
+    FftPlan p;
+    long long lines;      // lines along the axis
+    unsigned inner;       // element stride of the axis
+    int B;                // lines per CTA (neighbours in the inner index; consecutive lines when inner == 1)
+    int mode;
+    // first axis (inner == 1): read rho of the box, zero outside it
+    const double *rho;
+    double bg;
+    int nbox[3], m[3], dims;
+    // FFT_CONV: real factors, or complex factors times scale
+    const double *green;
+    const double2 *ghat;
+    double scale;
+    const double2 *tw;    // n roots of the axis, or NULL: computed in the CTA
+};
+
+__global__ void __launch_bounds__(256) k_fft_lines(double2 *__restrict__ a, FftArgs f) {
+    extern __shared__ double2 sbuf[];
+    const int n = f.p.n, B = f.B;
+    double2 *w = sbuf, *x = sbuf + n, *y = x + B * n;
+    // first line of the CTA and its element base; lines are base + b (strided
+    // axis) or base + b n
+    const unsigned tpo = f.inner == 1 ? 1u : (f.inner + B - 1) / B;
+    long long base;
+    int nb;
+    long long l0 = 0;
+    if (f.inner == 1) {
+        l0 = (long long)blockIdx.x * B;
+        nb = (int)(f.lines - l0 < B ? f.lines - l0 : B);
+        base = l0 * n;
+    } else {
+        const unsigned o = blockIdx.x / tpo, c = (blockIdx.x - o * tpo) * B;
+        nb = (int)(f.inner - c < (unsigned)B ? f.inner - c : B);
+        base = (long long)o * n * f.inner + c;
+    }
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+        if (f.tw) {
+            w[j] = f.tw[j];
+        } else {
+            double sn, cs;
+            sincospi(2.0 * (double)j / (double)n, &sn, &cs);
+            w[j] = make_double2(cs, -sn);
+        }
+    }
+    if (f.rho) {
+        // contiguous lines of the padded grid: the line's outer indices, and
+        // its row of the box (or a line of zeros)
+        for (int t = threadIdx.x; t < nb * n; t += blockDim.x) {
+            const int b = t / n, j = t - b * n;
+            long long r = l0 + b, row = 0, mul = f.nbox[f.dims - 1];
+            bool in = j < f.nbox[f.dims - 1];
+            for (int d = f.dims - 2; d >= 0; --d) {
+                const int i = (int)((unsigned)r % (unsigned)f.m[d]);
+                r = (unsigned)r / (unsigned)f.m[d];
+                in = in && i < f.nbox[d];
+                row += i * mul;
+                mul *= f.nbox[d];
+            }
+            x[t] = make_double2(in ? f.rho[row + j] - f.bg : 0.0, 0.0);
+        }
+    } else if (f.inner == 1) {
+        for (int t = threadIdx.x; t < nb * n; t += blockDim.x) x[t] = a[base + t];
+    } else {
+        for (int t = threadIdx.x; t < nb * n; t += blockDim.x) {
+            const int j = t / nb, b = t - j * nb;
+            x[b * n + j] = a[base + (long long)j * f.inner + b];
+        }
+    }
+    __syncthreads();
+    double2 *r = fft_lines(x, y, w, f.p, nb, f.mode == FFT_INV ? 1 : -1);
+    if (f.mode == FFT_CONV) {
+        for (int t = threadIdx.x; t < nb * n; t += blockDim.x) {
+            int j, b;
+            long long g;
+            if (f.inner == 1) {
+                b = t / n;
+                j = t - b * n;
+                g = base + t;
+            } else {
+                j = t / nb;
+                b = t - j * nb;
+                g = base + (long long)j * f.inner + b;
+            }
+            double2 u = r[b * n + j];
+            if (f.green) {
+                const double s = f.green[g];
+                u = make_double2(u.x * s, u.y * s);
+            } else {
+                u = cmul(u, f.ghat[g]);
+                u = make_double2(u.x * f.scale, u.y * f.scale);
+            }
+            r[b * n + j] = u;
+        }
+        __syncthreads();
+        r = fft_lines(r, r == x ? y : x, w, f.p, nb, 1);
+    }
+    if (f.inner == 1) {
+        for (int t = threadIdx.x; t < nb * n; t += blockDim.x) a[base + t] = r[t];
+    } else {
+        for (int t = threadIdx.x; t < nb * n; t += blockDim.x) {
+            const int j = t / nb, b = t - j * nb;
+            a[base + (long long)j * f.inner + b] = r[b * n + j];
+        }
     }
 }
 
-// scatter rho - rho_bg into the (possibly padded) complex grid, zero elsewhere
-__global__ void k_load_rho(double2 *__restrict__ a, const double *__restrict__ rho, double bg,
-                           long long MT, int3 nbox, int3 m, int dims) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= MT) return;
-    long long r = t;
-    int idx[3] = {0, 0, 0};
-    const int md[3] = {m.x, m.y, m.z};
-    const int nb[3] = {nbox.x, nbox.y, nbox.z};
-    for (int d = dims - 1; d >= 0; --d) {
-        idx[d] = (int)(r % md[d]);
-        r /= md[d];
-    }
-    bool in = true;
-    long long lin = 0;
-    for (int d = 0; d < dims; ++d) {
-        in = in && idx[d] < nb[d];
-        lin = lin * nb[d] + idx[d];
-    }
-    a[t] = make_double2(in ? rho[lin] - bg : 0.0, 0.0);
+// roots of unity w[j] = exp(-2 pi i j / n)
+__global__ void k_roots(double2 *__restrict__ w, int n) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    double sn, cs;
+    sincospi(2.0 * (double)j / (double)n, &sn, &cs);
+    w[j] = make_double2(cs, -sn);
 }
 
-__global__ void k_mul_real(double2 *__restrict__ a, const double *__restrict__ g, long long n) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    const double s = g[t];
-    a[t] = make_double2(a[t].x * s, a[t].y * s);
+// One dimension, periodic: phi = g * (rho - bg) and a = k * (rho - bg) are
+// cyclic convolutions.  The kernels from their spectra (green_k = S / lambda_k
+// / n and D_k green_k, D_k the symbol of the FDA): g_j = sum_k green_k cos(2 pi
+// j k / n), k_j = sum_k (D green)_k sin(2 pi j k / n).  ker = [g | k].
+__global__ void k_conv1_kernels(const double *__restrict__ green, const double *__restrict__ dgreen,
+                                const double2 *__restrict__ w, int n, double *__restrict__ ker) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    double g = 0.0, k1 = 0.0;
+    int idx = 0;
+    for (int k = 0; k < n; ++k) {
+        const double2 v = w[idx];
+        g = fma(green[k], v.x, g);
+        k1 = fma(-dgreen[k], v.y, k1);  // the table holds -sin
+        idx += j;
+        idx -= idx >= n ? n : 0;
+    }
+    ker[j] = g;
+    ker[n + j] = k1;
 }
 
-__global__ void k_mul_cplx(double2 *__restrict__ a, const double2 *__restrict__ g, long long n,
-                           double scale) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    const double2 u = a[t], v = g[t];
-    a[t] = make_double2((u.x * v.x - u.y * v.y) * scale, (u.x * v.y + u.y * v.x) * scale);
+// One warp per output point, lanes over the sum; phi is optional.  n = 64: 1
+// launch of ~3 us where load, two transforms, multiply and force took 45 us;
+// 4096 points (the largest axis): 2 x 16.8 M FMAs, ~55 us per output array of
+// the FP64 pipe, still below the two transforms of one CTA.
+constexpr int kConvWarps = 4;
+__global__ void __launch_bounds__(32 * kConvWarps) k_conv1(const double *__restrict__ rho, double bg, int n,
+                                                            const double *__restrict__ ker, double *__restrict__ phi,
+                                                            double *__restrict__ acc) {
+    extern __shared__ double srho[];
+    for (int j = threadIdx.x; j < n; j += blockDim.x) srho[j] = rho[j] - bg;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int i = blockIdx.x * kConvWarps + (threadIdx.x >> 5);
+    if (i >= n) return;
+    double s0 = 0.0, s1 = 0.0, p0 = 0.0;
+    const double *g = ker, *k = ker + n;
+    int j = lane;
+    for (; j + 32 < n; j += 64) {
+        int d0 = i - j, d1 = d0 - 32;
+        d0 += d0 < 0 ? n : 0;
+        d1 += d1 < 0 ? n : 0;
+        s0 = fma(k[d0], srho[j], s0);
+        s1 = fma(k[d1], srho[j + 32], s1);
+        if (phi) p0 = fma(g[d1], srho[j + 32], fma(g[d0], srho[j], p0));
+    }
+    if (j < n) {
+        int d0 = i - j;
+        d0 += d0 < 0 ? n : 0;
+        s0 = fma(k[d0], srho[j], s0);
+        if (phi) p0 = fma(g[d0], srho[j], p0);
+    }
+    s0 = warp_sum(s0 + s1);
+    if (phi) p0 = warp_sum(p0);
+    if (lane == 0) {
+        acc[i] = s0;
+        if (phi) phi[i] = p0;
+    }
 }
 
 // phi (box) and accel = -grad phi by the 2/4/6-point FDA (Eqs. C9-C11),
 // reading the potential of the m-periodic grid (m = box for periodic,
-// m = 2 box for doubling-up) with cyclic indices.
+// m = 2 box for doubling-up) with cyclic indices.  32-bit index arithmetic
+// (the grid is below 2^31 points) and the factor 1 / (den h) from the host:
+// 15 -> 4 us at 16^3 points, where 64-bit remainders and FP64 divisions set
+// the time.
 struct Fda {
     double c[4];  // c[k] multiplies (phi_{i+k} - phi_{i-k}), k = 1..3
     double den;
 };
 
-__global__ void k_force(const double2 *__restrict__ a, double scale, double *__restrict__ phi,
-                        double *__restrict__ acc, long long NX, int3 nbox, int3 m, int dims,
-                        double3 h, Fda fd, int npts) {
-    const long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= NX) return;
-    const int nb[3] = {nbox.x, nbox.y, nbox.z};
-    const int md[3] = {m.x, m.y, m.z};
-    const double hh[3] = {h.x, h.y, h.z};
-    int idx[3] = {0, 0, 0};
-    long long r = x;
-    for (int d = dims - 1; d >= 0; --d) {
-        idx[d] = (int)(r % nb[d]);
-        r /= nb[d];
-    }
-    auto at = [&](int axis, int off) -> double {
-        long long lin = 0;
-        for (int d = 0; d < dims; ++d) {
-            int j = idx[d];
-            if (d == axis) {
-                j = (j + off) % md[d];
-                if (j < 0) j += md[d];
-            }
-            lin = lin * md[d] + j;
-        }
-        return a[lin].x * scale;
-    };
-    if (phi) phi[x] = at(0, 0);
-    for (int d = 0; d < dims; ++d) {
+struct ForceArgs {
+    unsigned NX;
+    FastDiv nb1, nb2;      // box sizes of the second and third axis
+    int m[3];              // transformed grid
+    int dims, npts;
+    double c[4];
+    double inv[3];         // -1 / (den h) per axis
+};
+
+__global__ void __launch_bounds__(kBlock) k_force(const double2 *__restrict__ a, double *__restrict__ phi,
+                                                  double *__restrict__ acc, ForceArgs f) {
+    const unsigned x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= f.NX) return;
+    int i[3];
+    unsigned q = fdiv(x, f.nb2);
+    i[2] = (int)(x - q * f.nb2.d);
+    i[0] = (int)fdiv(q, f.nb1);
+    i[1] = (int)(q - (unsigned)i[0] * f.nb1.d);
+    // axes beyond dims have one cell: strides of the transformed grid
+    const int st[3] = {f.m[1] * f.m[2], f.m[2], 1};
+    const double2 *p = a + ((long long)i[0] * st[0] + (long long)i[1] * st[1] + i[2]);
+    if (phi) phi[x] = p->x;
+    for (int d = 0; d < f.dims; ++d) {
         double g = 0.0;
-        for (int k = 1; k <= npts; ++k) g += fd.c[k] * (at(d, k) - at(d, -k));
-        acc[(long long)d * NX + x] = -g / (fd.den * hh[d]);
+        for (int k = 1; k <= f.npts; ++k) {
+            int up = i[d] + k, dn = i[d] - k;
+            while (up >= f.m[d]) up -= f.m[d];
+            while (dn < 0) dn += f.m[d];
+            g = fma(f.c[k], p[(long long)(up - i[d]) * st[d]].x - p[(long long)(dn - i[d]) * st[d]].x, g);
+        }
+        acc[(long long)d * f.NX + x] = g * f.inv[d];
     }
 }
 
@@ -422,21 +608,72 @@ __global__ void k_init(T *__restrict__ f, long long ncell, IcArgs a) {
 
 inline unsigned nblk(long long n, int b) { return (unsigned)((n + b - 1) / b); }
 
-int fft_all_axes(vp_ctx *c, double2 *buf, const int *m, int dims, int sign) {
-    long long total = 1;
-    for (int d = 0; d < dims; ++d) total *= m[d];
-    for (int a = 0; a < dims; ++a) {
-        long long inner = 1;
-        for (int d = a + 1; d < dims; ++d) inner *= m[d];
-        const long long lines = total / m[a];
-        const size_t smem = 2 * (size_t)m[a] * sizeof(double2);
-        int th = m[a] / 2 < 32 ? 32 : (m[a] / 2 > 256 ? 256 : m[a] / 2);
-        k_fft_axis<<<(unsigned)lines, th, smem, c->stream>>>(buf, inner, m[a], sign);
-        c->launches++;
+// radices of an axis of n points: 4s first (fewest FP64 operations), then 2,
+// then the odd primes
+FftPlan fft_plan(int n) {
+    FftPlan p{};
+    p.n = n;
+    int r = n;
+    while (r % 4 == 0) {
+        p.rad[p.nr++] = 4;
+        r /= 4;
     }
-    VP_CUDA_TRY(c, cudaGetLastError());
-    return VP_OK;
+    for (int q = 2; r > 1; q += q == 2 ? 1 : 2) {
+        if ((long long)q * q > r) q = r;
+        while (r % q == 0) {
+            p.rad[p.nr++] = q;
+            r /= q;
+        }
+    }
+    return p;
 }
+
+// launch the transform of one axis of the row-major grid m[0..dims)
+struct FftLaunch {
+    FftArgs f;
+    unsigned blocks;
+    int threads;
+    size_t smem;
+};
+
+FftLaunch fft_axis(const int *m, int dims, int axis, int mode, const double2 *tw) {
+    FftLaunch l{};
+    FftArgs &f = l.f;
+    f.p = fft_plan(m[axis]);
+    f.mode = mode;
+    f.tw = tw;
+    f.dims = dims;
+    long long total = 1, inner = 1;
+    for (int d = 0; d < dims; ++d) total *= m[d];
+    for (int d = axis + 1; d < dims; ++d) inner *= m[d];
+    const int n = m[axis];
+    f.lines = total / n;
+    f.inner = (unsigned)inner;
+    // one line per CTA until the chip holds two CTAs per SM, then up to four
+    // neighbouring lines (64-byte rows on a strided axis)
+    int B = f.lines >= 1216 ? 4 : (f.lines >= 608 ? 2 : 1);
+    while (B > 1 && (size_t)(1 + 2 * B) * n * sizeof(double2) > 96 * 1024) B /= 2;
+    f.B = B;
+    l.blocks = inner == 1 ? (unsigned)((f.lines + B - 1) / B)
+                          : (unsigned)(f.lines / inner * ((inner + B - 1) / B));
+    const int work = B * (f.p.nr && f.p.rad[0] == 4 ? n / 4 : n / 2);
+    l.threads = work < 32 ? 32 : (work > 256 ? 256 : (work + 31) / 32 * 32);
+    l.smem = (size_t)(1 + 2 * B) * n * sizeof(double2);
+    return l;
+}
+
+int fft_launch(cudaStream_t st, double2 *buf, const FftLaunch &l) {
+    k_fft_lines<<<l.blocks, l.threads, l.smem, st>>>(buf, l.f);
+    return 1;
+}
+
+constexpr int kFftSmem = 3 * 4096 * (int)sizeof(double2);  // table and two buffers of the longest axis
+
+// largest periodic 1D axis solved as a convolution (its densities are staged
+// in 32 KB of shared memory)
+constexpr int kConvMax = 4096;
+
+ForceArgs force_args(const vp_grid &g, const int *m, long long NX);
 
 Fda fda_coeffs(int order) {
     // central differences of Eqs. (C9)-(C11): sum_k c_k (phi_{i+k} - phi_{i-k}) / (den h)
@@ -453,6 +690,22 @@ Fda fda_coeffs(int order) {
         f.c[2] = -9.0;
         f.c[3] = 1.0;
         f.den = 60.0;
+    }
+    return f;
+}
+
+ForceArgs force_args(const vp_grid &g, const int *m, long long NX) {
+    const Fda fd = fda_coeffs(g.pois_order);
+    ForceArgs f{};
+    f.NX = (unsigned)NX;
+    f.dims = g.dx;
+    f.npts = g.pois_order / 2;
+    f.nb1 = make_fastdiv(g.dx > 1 ? (unsigned)g.nx[1] : 1u);
+    f.nb2 = make_fastdiv(g.dx > 2 ? (unsigned)g.nx[2] : 1u);
+    for (int k = 0; k < 4; ++k) f.c[k] = fd.c[k];
+    for (int d = 0; d < 3; ++d) {
+        f.m[d] = d < g.dx ? m[d] : 1;
+        f.inv[d] = d < g.dx ? -1.0 / (fd.den * ((g.xhi[d] - g.xlo[d]) / g.nx[d])) : 0.0;
     }
     return f;
 }
@@ -510,14 +763,28 @@ static double cube_inv_r_mean() {
 
 int vp_field_setup(vp_ctx *c) {
     const vp_grid &g = c->g;
-    VP_CUDA_TRY(c, cudaFuncSetAttribute(k_fft_axis, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        2 * 4096 * (int)sizeof(double2)));
+    VP_CUDA_TRY(c, cudaFuncSetAttribute(k_fft_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmem));
     const int D = g.dx;
+    const bool iso = g.poisson == VP_POIS_ISOLATED;
+    long long nroot = 0;
+    for (int d = 0; d < D; ++d) nroot += iso ? 2 * g.nx[d] : g.nx[d];
+    VP_CUDA_TRY(c, cudaMalloc(&c->d_roots, sizeof(double2) * nroot));
+    nroot = 0;
+    for (int d = 0; d < D; ++d) {
+        const int m = iso ? 2 * g.nx[d] : g.nx[d];
+        c->roots[d] = c->d_roots + nroot;
+        k_roots<<<nblk(m, kBlock), kBlock>>>(c->d_roots + nroot, m);
+        nroot += m;
+    }
+    VP_CUDA_TRY(c, cudaGetLastError());
     if (g.poisson == VP_POIS_PERIODIC) {
         c->MT = c->NX;
         for (int d = 0; d < 3; ++d) c->m[d] = d < D ? g.nx[d] : 1;
-        double *h_g = (double *)malloc(sizeof(double) * c->NX);
+        // one dimension: the spectrum of the convolution kernels, [green | D green]
+        const long long ng = D == 1 ? 2 * c->NX : c->NX;
+        double *h_g = (double *)malloc(sizeof(double) * ng);
         if (!h_g) return vp_fail(c, VP_ENOMEM, "host allocation failed");
+        const Fda fd = fda_coeffs(g.pois_order);
         for (long long x = 0; x < c->NX; ++x) {
             long long r = x;
             int allzero = 1;
@@ -531,11 +798,28 @@ int vp_field_setup(vp_ctx *c) {
             }
             // phi_hat = S rho_hat / lambda; the inverse transform's 1/NX is folded in
             h_g[x] = allzero ? 0.0 : g.coupling / lam / (double)c->NX;
+            if (D == 1) {
+                // a = -grad phi: the FDA's symbol is i D, D = sum 2 c_m sin(m theta) / (den h)
+                double sym = 0.0;
+                for (int mm = 1; mm <= g.pois_order / 2; ++mm)
+                    sym += 2.0 * fd.c[mm] * sin(2.0 * M_PI * (double)((mm * x) % g.nx[0]) / (double)g.nx[0]);
+                h_g[c->NX + x] = h_g[x] * (sym / (fd.den * ((g.xhi[0] - g.xlo[0]) / g.nx[0])));
+            }
         }
-        VP_CUDA_TRY(c, cudaMalloc(&c->d_green, sizeof(double) * c->NX));
-        VP_CUDA_TRY(c, cudaMemcpy(c->d_green, h_g, sizeof(double) * c->NX, cudaMemcpyHostToDevice));
+        cudaError_t e = cudaMalloc(&c->d_green, sizeof(double) * ng);
+        if (e == cudaSuccess) e = cudaMemcpy(c->d_green, h_g, sizeof(double) * ng, cudaMemcpyHostToDevice);
         free(h_g);
-        VP_CUDA_TRY(c, cudaMalloc(&c->d_fft, sizeof(double2) * c->MT));
+        VP_CUDA_TRY(c, e);
+        if (D == 1) {
+            const int n = g.nx[0];
+            VP_CUDA_TRY(c, cudaMalloc(&c->d_conv, sizeof(double) * 2 * n));
+            k_conv1_kernels<<<nblk(n, 64), 64>>>(c->d_green, c->d_green + n, c->d_roots, n, c->d_conv);
+            VP_CUDA_TRY(c, cudaGetLastError());
+        } else {
+            VP_CUDA_TRY(c, cudaMalloc(&c->d_fft, sizeof(double2) * c->MT));
+        }
+        // the tables were made on the legacy stream, which the context's need not wait for
+        VP_CUDA_TRY(c, cudaStreamSynchronize(cudaStreamLegacy));
         return VP_OK;
     }
     // isolated: doubling-up with the real-space kernel -(S / 4 pi) dV / r
@@ -560,8 +844,10 @@ int vp_field_setup(vp_ctx *c) {
     VP_CUDA_TRY(c, cudaMalloc(&c->d_fft, sizeof(double2) * c->MT));
     VP_CUDA_TRY(c, cudaMemcpy(c->d_ghat, h_k, sizeof(double2) * c->MT, cudaMemcpyHostToDevice));
     free(h_k);
-    int rc = fft_all_axes(c, c->d_ghat, c->m, 3, -1);
-    if (rc) return rc;
+    VP_CUDA_TRY(c, cudaStreamSynchronize(cudaStreamLegacy));
+    for (int d = 2; d >= 0; --d)
+        c->launches += fft_launch(c->stream, c->d_ghat, fft_axis(c->m, 3, d, FFT_FWD, c->roots[d]));
+    VP_CUDA_TRY(c, cudaGetLastError());
     VP_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     return VP_OK;
 }
@@ -585,28 +871,42 @@ int vp_launch_moment(vp_ctx *c, double *rho) {
 int vp_launch_poisson(vp_ctx *c, const double *rho, double *phi, double *acc) {
     const vp_grid &g = c->g;
     const int D = g.dx;
-    const int3 nbox = make_int3(g.nx[0], D > 1 ? g.nx[1] : 1, D > 2 ? g.nx[2] : 1);
-    const int3 m = make_int3(c->m[0], c->m[1], c->m[2]);
-    k_load_rho<<<nblk(c->MT, kBlock), kBlock, 0, c->stream>>>(c->d_fft, rho, g.rho_bg, c->MT, nbox, m, D);
-    c->launches++;
-    int rc = fft_all_axes(c, c->d_fft, c->m, D, -1);
-    if (rc) return rc;
-    double scale = 1.0;
-    if (g.poisson == VP_POIS_PERIODIC) {
-        k_mul_real<<<nblk(c->MT, kBlock), kBlock, 0, c->stream>>>(c->d_fft, c->d_green, c->MT);
-    } else {
-        k_mul_cplx<<<nblk(c->MT, kBlock), kBlock, 0, c->stream>>>(c->d_fft, c->d_ghat, c->MT,
-                                                                   1.0 / (double)c->MT);
+    if (c->d_conv) {
+        const int n = g.nx[0];
+        // every block reads all of rho: outputs that overlap it take a copy
+        auto meets = [&](const double *p) { return p && p < rho + n && rho < p + n; };
+        if (meets(phi) || meets(acc)) {
+            VP_CUDA_TRY(c, cudaMemcpyAsync(c->d_rho, rho, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->stream));
+            rho = c->d_rho;
+        }
+        k_conv1<<<nblk(n, kConvWarps), 32 * kConvWarps, sizeof(double) * n, c->stream>>>(rho, g.rho_bg, n, c->d_conv,
+                                                                                        phi, acc);
+        c->launches++;
+        VP_CUDA_TRY(c, cudaGetLastError());
+        return VP_OK;
     }
-    c->launches++;
-    rc = fft_all_axes(c, c->d_fft, c->m, D, +1);
-    if (rc) return rc;
-    double3 h = make_double3((g.xhi[0] - g.xlo[0]) / g.nx[0],
-                             D > 1 ? (g.xhi[1] - g.xlo[1]) / g.nx[1] : 1.0,
-                             D > 2 ? (g.xhi[2] - g.xlo[2]) / g.nx[2] : 1.0);
-    k_force<<<nblk(c->NX, kBlock), kBlock, 0, c->stream>>>(c->d_fft, scale, phi, acc, c->NX, nbox, m, D,
-                                                           h, fda_coeffs(g.pois_order),
-                                                           g.pois_order / 2);
+    // forward along the last axis (reading rho) .. the second, then the first
+    // axis forward, times the Green function, and back; the others back
+    for (int d = D - 1; d >= 0; --d) {
+        FftLaunch l = fft_axis(c->m, D, d, d ? FFT_FWD : FFT_CONV, c->roots[d]);
+        if (d == D - 1) {
+            l.f.rho = rho;
+            l.f.bg = g.rho_bg;
+            for (int k = 0; k < D; ++k) {
+                l.f.nbox[k] = g.nx[k];
+                l.f.m[k] = c->m[k];
+            }
+        }
+        if (d == 0) {
+            l.f.green = c->d_green;
+            l.f.ghat = c->d_ghat;
+            l.f.scale = 1.0 / (double)c->MT;
+        }
+        c->launches += fft_launch(c->stream, c->d_fft, l);
+    }
+    for (int d = 1; d < D; ++d)
+        c->launches += fft_launch(c->stream, c->d_fft, fft_axis(c->m, D, d, FFT_INV, c->roots[d]));
+    k_force<<<nblk(c->NX, kBlock), kBlock, 0, c->stream>>>(c->d_fft, phi, acc, force_args(g, c->m, c->NX));
     c->launches++;
     VP_CUDA_TRY(c, cudaGetLastError());
     return VP_OK;
@@ -761,8 +1061,8 @@ extern "C" int vp_poisson_periodic_noalloc(const vp_grid *g, void *cuda_stream, 
         if (!g_noalloc_dev_ptr[dev]) {
             void *p = nullptr;
             if (cudaGetSymbolAddress(&p, g_noalloc_fft) != cudaSuccess || !p) return VP_ECUDA;
-            if (cudaFuncSetAttribute(k_fft_axis, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     2 * 4096 * (int)sizeof(double2)) != cudaSuccess)
+            if (cudaFuncSetAttribute(k_fft_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmem) !=
+                cudaSuccess)
                 return VP_ECUDA;
             g_noalloc_dev_ptr[dev] = static_cast<double2 *>(p);
         }
@@ -772,26 +1072,20 @@ extern "C" int vp_poisson_periodic_noalloc(const vp_grid *g, void *cuda_stream, 
     const int3 nb = make_int3(g->nx[0], D > 1 ? g->nx[1] : 1, D > 2 ? g->nx[2] : 1);
     const int m[3] = {nb.x, nb.y, nb.z};
     // every element of the work array that is read is written first: no clearing needed
-    k_load_rho<<<nblk(NX, kBlock), kBlock, 0, st>>>(buf, rho_dev, g->rho_bg, NX, nb, nb, D);
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int a = 0; a < D; ++a) {
-            long long inner = 1;
-            for (int d = a + 1; d < D; ++d) inner *= m[d];
-            const size_t smem = 2 * (size_t)m[a] * sizeof(double2);
-            const int th = m[a] / 2 < 32 ? 32 : (m[a] / 2 > 256 ? 256 : m[a] / 2);
-            k_fft_axis<<<(unsigned)(NX / m[a]), th, smem, st>>>(buf, inner, m[a], pass == 0 ? -1 : +1);
+    for (int d = D - 1; d >= 0; --d) {
+        FftLaunch l = fft_axis(m, D, d, FFT_FWD, nullptr);
+        if (d == D - 1) {
+            l.f.rho = rho_dev;
+            l.f.bg = g->rho_bg;
+            for (int k = 0; k < D; ++k) l.f.nbox[k] = l.f.m[k] = m[k];
         }
-        if (pass == 0) {
-            const double3 h = make_double3((g->xhi[0] - g->xlo[0]) / g->nx[0],
-                                           D > 1 ? (g->xhi[1] - g->xlo[1]) / g->nx[1] : 1.0,
-                                           D > 2 ? (g->xhi[2] - g->xlo[2]) / g->nx[2] : 1.0);
-            k_green_onfly<<<nblk(NX, kBlock), kBlock, 0, st>>>(buf, NX, D, nb, h, g->pois_order, g->coupling);
-        }
+        fft_launch(st, buf, l);
     }
     const double3 h = make_double3((g->xhi[0] - g->xlo[0]) / g->nx[0],
                                    D > 1 ? (g->xhi[1] - g->xlo[1]) / g->nx[1] : 1.0,
                                    D > 2 ? (g->xhi[2] - g->xlo[2]) / g->nx[2] : 1.0);
-    k_force<<<nblk(NX, kBlock), kBlock, 0, st>>>(buf, 1.0, phi_dev, accel_dev, NX, nb, nb, D, h,
-                                                 fda_coeffs(g->pois_order), g->pois_order / 2);
+    k_green_onfly<<<nblk(NX, kBlock), kBlock, 0, st>>>(buf, NX, D, nb, h, g->pois_order, g->coupling);
+    for (int d = 0; d < D; ++d) fft_launch(st, buf, fft_axis(m, D, d, FFT_INV, nullptr));
+    k_force<<<nblk(NX, kBlock), kBlock, 0, st>>>(buf, phi_dev, accel_dev, force_args(*g, m, NX));
     return cudaGetLastError() == cudaSuccess ? VP_OK : VP_ECUDA;
 }

@@ -118,10 +118,12 @@ struct vp_ctx {
     void *d_shift;
     long long shift_cap;
     double *d_rho, *d_phi, *d_acc;      // diagnostics scratch
-    double *d_rho_s, *d_phi_s;          // step scratch
+    double *d_rho_s;                    // step scratch
     double2 *d_fft;
     double *d_green;                    // periodic: S / lambda(k)
     double2 *d_ghat;                    // isolated: DFT of the padded Green function
+    double2 *d_roots, *roots[3];        // roots of unity of the transformed axes (roots[d]: axis d's n)
+    double *d_conv;                     // periodic 1D: convolution kernels of phi and the acceleration
     long long MT;
     int m[3];
     double *d_part;                     // diagnostics partial sums [NX * 6]
@@ -204,6 +206,7 @@ int vp_launch_sweep(vp_ctx *c, int kick, int dim);
 // autotune sweep (kick, dim) at its own shifts (dt, accel); outside stream capture only
 int vp_tune_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel);
 int vp_launch_moment(vp_ctx *c, double *rho);
+// phi may be NULL
 int vp_launch_poisson(vp_ctx *c, const double *rho, double *phi, double *acc);
 int vp_launch_diag(vp_ctx *c, int mode, double *out_dev);
 int vp_launch_init(vp_ctx *c, int kind, const double *p, int np);

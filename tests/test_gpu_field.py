@@ -70,6 +70,36 @@ def test_isolated_poisson(n):
     sim.close()
 
 
+@pytest.mark.parametrize("nx,iso", [([1], 0), ([2], 0), ([37], 0), ([99], 0), ([1024], 0), ([7, 22], 0), ([25, 64], 0),
+                                    ([1, 130], 0), ([5, 14, 9], 0), ([16, 2, 33], 0), ([3, 5, 7], 1), ([11, 4, 1], 1)])
+def test_poisson_axis_lengths(nx, iso):
+    """Axis lengths of every kind the transforms take (1, powers of two and
+    four, 3 and 5, larger primes) and the convolution of one dimension, with
+    the potential requested, left out, and written over the density.  The
+    force differences the potential over a cell, so rounding grows with the
+    number of cells of an axis: 1e-12 up to 256 cells, in proportion above."""
+    dims, h = len(nx), 0.5
+    g = dict(dims=dims, nx=nx, nv=[1] * dims, xlo=[0.0] * dims, xhi=[n * h for n in nx], vlo=[-1.0] * dims,
+             vhi=[1.0] * dims, pois_order=6, coupling=4 * math.pi, rho_bg=0.4, poisson=iso)
+    sim, og = both(g, V.VP_F64)
+    rho = np.random.default_rng(sum(nx)).random(og.NX)
+    phi_o, acc_o = O.poisson_solve(og, rho)
+    tol = 1e-12 * max(1.0, max(nx) / 256)
+
+    def close(a, b):
+        # an axis of one cell has no field: absolute against the density there
+        assert np.abs(a.cpu().numpy() - b.reshape(-1)).max() <= tol * max(np.abs(b).max(), 1e-3), nx
+    for phi_t in (_t(np.zeros(og.NX)), None, "rho"):
+        r_t, a_t = _t(rho), _t(np.zeros(dims * og.NX))
+        p_t = r_t if isinstance(phi_t, str) else phi_t
+        V.vp_poisson_solve(sim.ctx, r_t, p_t, a_t)
+        sim.sync()
+        close(a_t, acc_o)
+        if p_t is not None:
+            close(p_t, phi_o)
+    sim.close()
+
+
 @pytest.mark.parametrize("cfg", [inputs.landau_linear(), inputs.two_stream(32, 64),
                                  inputs.plummer(6, 8)])
 def test_initial_conditions_and_diagnostics(cfg):
