@@ -160,6 +160,8 @@ void free_buffers(vp_ctx *c) {
     cudaFree(c->d_ghat);
     cudaFree(c->d_roots);
     cudaFree(c->d_conv);
+    cudaFree(c->d_vw);
+    cudaFree(c->d_diagblk);
     cudaFree(c->d_part);
     cudaFree(c->d_diag);
     cudaFree(c->d_flag);

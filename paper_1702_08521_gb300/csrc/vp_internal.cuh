@@ -128,6 +128,10 @@ struct vp_ctx {
     int m[3];
     double *d_part;                     // diagnostics partial sums [NX * 6]
     double *d_diag;                     // VP_NDIAG doubles
+    void *d_vw;                         // kinetic-energy weights: velocity rows, then the last axis
+    double vw_unit;                     // the power of two they are divided by
+    double *d_diagblk;                  // diagnostics: per-block results, then the counter of finished blocks
+    unsigned *d_diagctr;
     int *d_flag;                        // non-finite flag
     long long launches;
     int *d_status;                      // device-side error word (bounded waits)

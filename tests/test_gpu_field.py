@@ -136,6 +136,37 @@ def test_fp32_diagnostics_match_oracle_on_evolved_state(cfg):
     sim.close()
 
 
+@pytest.mark.parametrize("precision", [V.VP_F32, V.VP_F64])
+@pytest.mark.parametrize("nx,nv", [([300], [300]), ([5], [1100]), ([3, 4], [7, 5]), ([4, 2], [3, 260]), ([2, 3, 2], [9, 1, 31])])
+def test_diagnostic_sums_over_the_whole_float_range(precision, nx, nv):
+    """Mass, kinetic energy, extrema and norms of cells spread over 1e-44 ..
+    1e25, some negative, on velocity grids below and above a block, against
+    FP64 sums of the same cells.  A thread's pair sum of m cells carries m
+    roundings of its error term, m 2^-48 relative to the sum of the terms'
+    sizes: below 1e-12 for the m <= 256 of these grids.  Also the density,
+    whose cells stay below 1e25 / 1e13 here."""
+    D = len(nx)
+    g = dict(dims=D, nx=nx, nv=nv, xlo=[0.0] * D, xhi=[1.0] * D, vlo=[-2.0] * D, vhi=[3.0] * D)
+    sim, og = both(g, precision)
+    rng = np.random.default_rng(sum(nv))
+    f = rng.random(og.NX * og.NV) * 10.0 ** rng.uniform(-44, 25, size=og.NX * og.NV)
+    f = np.where(rng.random(f.size) < 0.1, -f, f).astype(np.float32).astype(np.float64)
+    to_gpu(sim, f)
+    d = V.vp_diagnostics(sim.ctx, 1)
+    dX, dV = float(np.prod([1.0 / n for n in nx])), float(np.prod([5.0 / n for n in nv]))
+    fx = f.reshape([og.NX] + list(nv))
+    v2 = sum((np.asarray(og.v_centres(k)) ** 2).reshape([-1 if j == k else 1 for j in range(D)]) for k in range(D))
+    terms = dict(mass=fx, ke=0.5 * fx * v2, l1=np.abs(fx), l2=fx ** 2)
+    for k, t in terms.items():
+        assert abs(d[k] - t.sum() * dX * dV) <= 1e-12 * np.abs(t).sum() * dX * dV, k
+    assert d["min_f"] == f.min() and d["max_f"] == f.max()
+    V.vp_density_moment(sim.ctx, sim.rho)
+    sim.sync()
+    rho, size = fx.reshape(og.NX, -1).sum(1) * dV, np.abs(fx).reshape(og.NX, -1).sum(1) * dV
+    assert (np.abs(sim.rho.cpu().numpy() - rho) <= 1e-12 * size).all()
+    sim.close()
+
+
 def test_diagnostics_flags_nonfinite():
     g = dict(dims=1, nx=[8], nv=[8], xlo=[0.0], xhi=[1.0], vlo=[-1.0], vhi=[1.0])
     sim, _ = both(g, V.VP_F32)
