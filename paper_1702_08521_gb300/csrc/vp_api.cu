@@ -4,6 +4,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <type_traits>
 
 #include "vp_internal.cuh"
 
@@ -150,22 +151,9 @@ int validate(const vp_grid *g, char *msg, size_t n) {
 }
 
 void free_buffers(vp_ctx *c) {
-    cudaFree(c->d_shift);
-    cudaFree(c->d_rho);
-    cudaFree(c->d_phi);
-    cudaFree(c->d_acc);
-    cudaFree(c->d_rho_s);
+    cudaFree(c->d_arena);
     cudaFree(c->d_fft);
-    cudaFree(c->d_green);
     cudaFree(c->d_ghat);
-    cudaFree(c->d_roots);
-    cudaFree(c->d_conv);
-    cudaFree(c->d_vw);
-    cudaFree(c->d_diagblk);
-    cudaFree(c->d_part);
-    cudaFree(c->d_diag);
-    cudaFree(c->d_flag);
-    cudaFree(c->d_status);
     cudaFree(c->d_netfrag);
     cudaFree(c->d_learn_out);
     if (c->graph.valid) cudaGraphExecDestroy(c->graph.exec);
@@ -187,9 +175,7 @@ int sweep_all(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
     if (c->g.scheme == VP_SCHEME_RK) return vp_launch_rk_sweep(c, kick, dim, dt, accel);
     if (c->opt_autotune && !c->tune[kick][dim].valid && !capturing(c))
         if ((rc = vp_tune_sweep(c, kick, dim, dt, accel))) return rc;
-    rc = vp_launch_shift_table(c, kick, dim, dt, accel);
-    if (rc) return rc;
-    return vp_launch_sweep(c, kick, dim);
+    return vp_launch_sweep(c, kick, dim, dt, accel);
 }
 
 // one Strang step (Eq. 55) on the context stream
@@ -284,26 +270,44 @@ int vp_create(const vp_grid *grid, void *cuda_stream, vp_ctx **out) {
     ncls = nvsum > ncls ? nvsum : ncls;
     c->shift_cap = ncls;
     const size_t shift_bytes = (size_t)ncls * (c->esize == 4 ? sizeof(LineShift<float>) : sizeof(LineShift<double>));
-#define ALLOC(p, bytes)                                                     \
-    if (cudaMalloc((void **)&(p), (bytes)) != cudaSuccess) {                \
-        free_buffers(c);                                                    \
-        delete c;                                                           \
-        cudaGetLastError();                                                 \
-        return VP_ENOMEM;                                                   \
+    // one allocation for the small buffers: sized on the first pass, handed
+    // out on the second
+    for (int pass = 0; pass < 2; ++pass) {
+        size_t at = 0;
+        auto take = [&](auto &p, size_t bytes) {
+            if (pass) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(static_cast<char *>(c->d_arena) + at);
+            at += (bytes + 255) & ~size_t(255);
+        };
+        take(c->d_shift, shift_bytes);
+        take(c->d_rho, sizeof(double) * c->NX);
+        take(c->d_phi, sizeof(double) * c->NX);
+        take(c->d_acc, sizeof(double) * c->NX * c->g.dx);
+        take(c->d_rho_s, sizeof(double) * c->NX);
+        take(c->d_part, sizeof(double) * c->NX * 6);
+        take(c->d_diag, sizeof(double) * VP_NDIAG);
+        take(c->d_flag, sizeof(int));
+        take(c->d_status, sizeof(int));
+        const FieldSizes fs = vp_field_sizes(c);
+        take(c->d_green, fs.green);
+        take(c->d_roots, fs.roots);
+        take(c->d_conv, fs.conv);
+        take(c->d_vw, fs.weights);
+        take(c->d_diagblk, fs.diagblk);
+        take(c->d_diagctr, sizeof(unsigned));
+        if (!fs.conv) c->d_conv = nullptr;
+        if (!fs.green) c->d_green = nullptr;
+        if (!pass && cudaMalloc(&c->d_arena, at) != cudaSuccess) {
+            c->d_arena = nullptr;
+            free_buffers(c);
+            delete c;
+            cudaGetLastError();
+            return VP_ENOMEM;
+        }
     }
-    ALLOC(c->d_shift, shift_bytes);
-    ALLOC(c->d_rho, sizeof(double) * c->NX);
-    ALLOC(c->d_phi, sizeof(double) * c->NX);
-    ALLOC(c->d_acc, sizeof(double) * c->NX * c->g.dx);
-    ALLOC(c->d_rho_s, sizeof(double) * c->NX);
-    ALLOC(c->d_part, sizeof(double) * c->NX * 6);
-    ALLOC(c->d_diag, sizeof(double) * VP_NDIAG);
-    ALLOC(c->d_flag, sizeof(int));
-    ALLOC(c->d_status, sizeof(int));
-#undef ALLOC
     c->opt_autotune = 1;
     c->opt_wait_limit = 1u << 26;
-    if (cudaMemset(c->d_status, 0, sizeof(int)) != cudaSuccess) {
+    if (cudaMemset(c->d_status, 0, sizeof(int)) != cudaSuccess ||
+        cudaMemset(c->d_diagctr, 0, sizeof(unsigned)) != cudaSuccess) {
         free_buffers(c);
         delete c;
         return VP_ECUDA;

@@ -1005,6 +1005,19 @@ static double cube_inv_r_mean() {
 
 static int diag_weights(vp_ctx *c);
 
+FieldSizes vp_field_sizes(const vp_ctx *c) {
+    const vp_grid &g = c->g;
+    const bool iso = g.poisson == VP_POIS_ISOLATED, conv = !iso && g.dx == 1;
+    FieldSizes s{};
+    for (int d = 0; d < g.dx; ++d) s.roots += sizeof(double2) * (iso ? 2 : 1) * g.nx[d];
+    s.green = iso ? 0 : sizeof(double) * (conv ? 2 : 1) * c->NX;
+    s.conv = conv ? sizeof(double) * 2 * c->NX : 0;
+    const int nlast = g.nv[g.dv - 1];
+    s.weights = sizeof(double) * (c->NV / nlast + nlast);
+    s.diagblk = sizeof(double) * (kDiagSums + 2) * nblk(c->NX, kBlock);
+    return s;
+}
+
 int vp_field_setup(vp_ctx *c) {
     const vp_grid &g = c->g;
     const int rcw = diag_weights(c);
@@ -1013,9 +1026,6 @@ int vp_field_setup(vp_ctx *c) {
     const int D = g.dx;
     const bool iso = g.poisson == VP_POIS_ISOLATED;
     long long nroot = 0;
-    for (int d = 0; d < D; ++d) nroot += iso ? 2 * g.nx[d] : g.nx[d];
-    VP_CUDA_TRY(c, cudaMalloc(&c->d_roots, sizeof(double2) * nroot));
-    nroot = 0;
     for (int d = 0; d < D; ++d) {
         const int m = iso ? 2 * g.nx[d] : g.nx[d];
         c->roots[d] = c->d_roots + nroot;
@@ -1052,13 +1062,11 @@ int vp_field_setup(vp_ctx *c) {
                 h_g[c->NX + x] = h_g[x] * (sym / (fd.den * ((g.xhi[0] - g.xlo[0]) / g.nx[0])));
             }
         }
-        cudaError_t e = cudaMalloc(&c->d_green, sizeof(double) * ng);
-        if (e == cudaSuccess) e = cudaMemcpy(c->d_green, h_g, sizeof(double) * ng, cudaMemcpyHostToDevice);
+        const cudaError_t e = cudaMemcpy(c->d_green, h_g, sizeof(double) * ng, cudaMemcpyHostToDevice);
         free(h_g);
         VP_CUDA_TRY(c, e);
         if (D == 1) {
             const int n = g.nx[0];
-            VP_CUDA_TRY(c, cudaMalloc(&c->d_conv, sizeof(double) * 2 * n));
             k_conv1_kernels<<<nblk(n, 64), 64>>>(c->d_green, c->d_green + n, c->d_roots, n, c->d_conv);
             VP_CUDA_TRY(c, cudaGetLastError());
         } else {
@@ -1201,7 +1209,6 @@ static int diag_weights(vp_ctx *c) {
     w.unit = c->vw_unit = std::isfinite(vmax * vmax) && vmax * vmax > 0.0 ? ldexp(1.0, e) : 1.0;
     const int nlast = g.nv[g.dv - 1];
     const long long rows = c->NV / nlast, most = rows > nlast ? rows : nlast;
-    VP_CUDA_TRY(c, cudaMalloc(&c->d_vw, sizeof(double) * (rows + nlast)));
     if (g.precision == VP_F32)
         k_vweights<WPair><<<nblk(most, kBlock), kBlock>>>(w, rows, static_cast<WPair *>(c->d_vw),
                                                          static_cast<WPair *>(c->d_vw) + rows);
@@ -1209,10 +1216,6 @@ static int diag_weights(vp_ctx *c) {
         k_vweights<double><<<nblk(most, kBlock), kBlock>>>(w, rows, static_cast<double *>(c->d_vw),
                                                           static_cast<double *>(c->d_vw) + rows);
     VP_CUDA_TRY(c, cudaGetLastError());
-    const size_t nb = nblk(c->NX, kBlock);
-    VP_CUDA_TRY(c, cudaMalloc(&c->d_diagblk, sizeof(double) * (kDiagSums + 2) * nb + sizeof(unsigned)));
-    c->d_diagctr = reinterpret_cast<unsigned *>(c->d_diagblk + (kDiagSums + 2) * nb);
-    VP_CUDA_TRY(c, cudaMemset(c->d_diagctr, 0, sizeof(unsigned)));
     return VP_OK;
 }
 

@@ -114,7 +114,8 @@ struct vp_ctx {
     int esize;
     void *f;
     WPoly wp;
-    // library-owned device buffers
+    // library-owned device buffers (the small ones in one allocation, d_arena)
+    void *d_arena;
     void *d_shift;
     long long shift_cap;
     double *d_rho, *d_phi, *d_acc;      // diagnostics scratch
@@ -206,7 +207,8 @@ int vp_learned_drift_io(vp_ctx *c, int dim, double dt, const float *wts, int use
 // RK-MPP5 sweeps: kernel attributes once per process, one sweep (table + fused stages)
 int vp_rk_setup();
 int vp_launch_rk_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel);
-int vp_launch_sweep(vp_ctx *c, int kick, int dim);
+// one SL sweep, its shift table included where it needs one
+int vp_launch_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel);
 // autotune sweep (kick, dim) at its own shifts (dt, accel); outside stream capture only
 int vp_tune_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel);
 int vp_launch_moment(vp_ctx *c, double *rho);
@@ -214,7 +216,12 @@ int vp_launch_moment(vp_ctx *c, double *rho);
 int vp_launch_poisson(vp_ctx *c, const double *rho, double *phi, double *acc);
 int vp_launch_diag(vp_ctx *c, int mode, double *out_dev);
 int vp_launch_init(vp_ctx *c, int kind, const double *p, int np);
-int vp_field_setup(vp_ctx *c);          // Green function tables (at create)
+// bytes of the field solve's and the diagnostics' tables in the arena
+struct FieldSizes {
+    size_t green, roots, conv, weights, diagblk;
+};
+FieldSizes vp_field_sizes(const vp_ctx *c);
+int vp_field_setup(vp_ctx *c);          // fills those tables, the isolated Green function (at create)
 // CSL weight polynomials of the given order (5 or 7), from the definition of the SL flux
 WPoly vp_csl_weight_polys(int order);
 // learned flux correction network: 9 features, 3 hidden layers of 32

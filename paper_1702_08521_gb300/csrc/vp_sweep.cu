@@ -30,6 +30,7 @@
 namespace {
 
 using vp_core::line_class;
+using vp_core::ShiftSrc;
 using vp_core::walk;
 
 // running-pointer store of one line's new values (element stride `step`
@@ -57,9 +58,7 @@ struct PtrStore {
 
 template <typename T, int ORDER, bool PERIODIC, bool FULL, bool PAIR>
 __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_MINB : 1)
-    k_sweep_cols(T *__restrict__ f,
-                                                    const LineShift<T> *__restrict__ tab,
-                                                    SweepGeo geo, LimParams lp) {
+    k_sweep_cols(T *__restrict__ f, const __grid_constant__ ShiftSrc<T> src, SweepGeo geo, LimParams lp) {
     extern __shared__ __align__(16) unsigned char smraw[];
     constexpr int GP = PERIODIC ? 0 : VP_GHOST;
     T *sm = reinterpret_cast<T *>(smraw);
@@ -69,6 +68,20 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
     const int wc = (int)((geo.inner - c0) < W ? (geo.inner - c0) : W);
     T *base = f + (long long)o * L * geo.inner + c0;
     T *data = sm + GP * W;  // row 0 of the line
+    // the tile's shifts: its columns' classes (drift), or its one spatial point (kick)
+    unsigned q0 = 0;
+    int ncl = 1;
+    LineShift<T> *shifts = nullptr;
+    if (!src.tab) {
+        shifts = reinterpret_cast<LineShift<T> *>(smraw + (((size_t)(L + 2 * GP) * W * sizeof(T) + 15) & ~size_t(15)));
+        q0 = geo.cls_from_inner ? fdiv(c0, geo.fd_cdiv) : fdiv(o, geo.fd_cdiv);
+        if (geo.cls_from_inner) ncl = (int)(fdiv(c0 + wc - 1, geo.fd_cdiv) - q0) + 1;
+        vp_core::tile_shifts(shifts, q0, ncl, src, geo);
+    }
+    auto shift_of = [&](unsigned c) -> LineShift<T> {
+        if (src.tab) return src.tab[line_class(geo, o, c)];
+        return shifts[geo.cls_from_inner ? fdiv(c, geo.fd_cdiv) - q0 : 0u];
+    };
     for (int e = threadIdx.x; e < GP * W; e += blockDim.x) {
         sm[e] = T(0);
         data[L * W + e] = T(0);
@@ -105,6 +118,7 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
         }
     }
     __syncthreads();
+    if (!src.tab) vp_core::tile_weights(shifts, ncl, src);
     constexpr int G1 = PERIODIC ? 1 : VP_GHOST;
     if constexpr (PAIR) {
         const unsigned seg = fdiv(threadIdx.x, geo.fd_w2);
@@ -112,9 +126,9 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
         if (cc >= wc || (int)seg >= geo.nseg) return;
         const int r0 = (int)fdiv(seg * (unsigned)L, geo.fd_nseg);
         const int r1 = (int)fdiv((seg + 1) * (unsigned)L, geo.fd_nseg);
-        const LineShift<float> sa = tab[line_class(geo, o, c0 + cc)];
+        const LineShift<float> sa = shift_of(c0 + cc);
         if (cc + 1 < wc) {
-            const LineShift<float> sb = tab[line_class(geo, o, c0 + cc + 1)];
+            const LineShift<float> sb = shift_of(c0 + cc + 1);
             if (sa.n == sb.n && sa.sigma == sb.sigma) {
                 const vp_core::LineShiftP2 sh = vp_core::pair_shift(sa, sb);
                 const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
@@ -136,7 +150,7 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
         const unsigned seg = fdiv(threadIdx.x, geo.fd_w);
         const int cc = (int)(threadIdx.x - seg * (unsigned)W);
         if (cc < wc && (int)seg < geo.nseg) {
-            const LineShift<T> sh = tab[line_class(geo, o, c0 + cc)];
+            const LineShift<T> sh = shift_of(c0 + cc);
             const int r0 = (int)fdiv(seg * (unsigned)L, geo.fd_nseg);
             const int r1 = (int)fdiv((seg + 1) * (unsigned)L, geo.fd_nseg);
             const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
@@ -157,9 +171,7 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
 // conflict-free because P is odd.
 template <typename T, int ORDER, bool PERIODIC, bool FULL, bool PAIR>
 __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_MINB : 1)
-    k_sweep_rows(T *__restrict__ f,
-                                                    const LineShift<T> *__restrict__ tab,
-                                                    SweepGeo geo, LimParams lp) {
+    k_sweep_rows(T *__restrict__ f, const __grid_constant__ ShiftSrc<T> src, SweepGeo geo, LimParams lp) {
     extern __shared__ __align__(16) unsigned char smraw[];
     constexpr int GP = PERIODIC ? 0 : VP_GHOST;
     const int L = geo.L, R = geo.R;
@@ -171,6 +183,21 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
     const int nl = (int)((geo.outer - l0) < R ? (geo.outer - l0) : R);
     T *base = f + l0 * L;
     const int tot = nl * L;
+    // the tile's shifts: a kick's lines belong to consecutive spatial points
+    // (drifts along contiguous lines, one velocity cell, read the table)
+    unsigned q0 = 0;
+    int ncl = 1;
+    LineShift<T> *shifts = nullptr;
+    if (!src.tab) {
+        shifts = reinterpret_cast<LineShift<T> *>(smraw + (((size_t)R * (P + Q) * sizeof(T) + 15) & ~size_t(15)));
+        q0 = fdiv((unsigned)l0, geo.fd_cdiv);
+        ncl = (int)(fdiv((unsigned)(l0 + nl - 1), geo.fd_cdiv) - q0) + 1;
+        vp_core::tile_shifts(shifts, q0, ncl, src, geo);
+    }
+    auto shift_of = [&](int line) -> LineShift<T> {
+        if (src.tab) return src.tab[line_class(geo, (unsigned)(l0 + line), 0u)];
+        return shifts[fdiv((unsigned)(l0 + line), geo.fd_cdiv) - q0];
+    };
     // shared-memory index of cell pos of line r in the input / output tile
     auto iidx = [&](int r, int pos) -> int {
         return PAIR ? (r >> 1) * (2 * P) + 2 * (GP + pos) + (r & 1) : r * P + GP + pos;
@@ -239,6 +266,7 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
         }
     }
     __syncthreads();
+    if (!src.tab) vp_core::tile_weights(shifts, ncl, src);
     constexpr int G1 = PERIODIC ? 1 : VP_GHOST;
     if constexpr (PAIR) {
         const unsigned seg = fdiv(threadIdx.x, geo.fd_w2);
@@ -246,10 +274,10 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
         if (line < nl && (int)seg < geo.nseg) {
             const int r0 = (int)fdiv(seg * (unsigned)L, geo.fd_nseg);
             const int r1 = (int)fdiv((seg + 1) * (unsigned)L, geo.fd_nseg);
-            const LineShift<float> sa = tab[line_class(geo, (unsigned)(l0 + line), 0u)];
+            const LineShift<float> sa = shift_of(line);
             bool paired = false;
             if (line + 1 < nl) {
-                const LineShift<float> sb = tab[line_class(geo, (unsigned)(l0 + line + 1), 0u)];
+                const LineShift<float> sb = shift_of(line + 1);
                 if (sa.n == sb.n && sa.sigma == sb.sigma) {
                     const vp_core::LineShiftP2 sh = vp_core::pair_shift(sa, sb);
                     const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
@@ -276,7 +304,7 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
         const unsigned seg = fdiv(threadIdx.x, geo.fd_w);
         const int line = (int)(threadIdx.x - seg * (unsigned)R);
         if (line < nl && (int)seg < geo.nseg) {
-            const LineShift<T> sh = tab[line_class(geo, (unsigned)(l0 + line), 0u)];
+            const LineShift<T> sh = shift_of(line);
             const int r0 = (int)fdiv(seg * (unsigned)L, geo.fd_nseg);
             const int r1 = (int)fdiv((seg + 1) * (unsigned)L, geo.fd_nseg);
             const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
@@ -424,28 +452,42 @@ __global__ void __launch_bounds__(512) k_sweep_cols_tma(const __grid_constant__ 
 // Shift decomposition of every line class, in double precision so that the
 // integer part is exact: s = c dt / h, n = nearest integer (halves away from
 // zero), zeta = s - n, nu = |zeta|; the weights are the CSL polynomials at nu.
+// Eight lanes per class, one weight each (one thread per class spent 5.5 us in
+// a chain of 49 FP64 FMAs and a division).
 template <typename T>
 __global__ void k_shift_table(LineShift<T> *__restrict__ tab, int nclass, int kick, double lo,
                               double dvel, const double *__restrict__ accel, double dt, double h,
-                              WPoly wp) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+                              const __grid_constant__ WPoly wp) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = t >> 3, k = t & 7;
     if (c >= nclass) return;
     const double speed = kick ? accel[c] : vp_core::cell_centre(lo, dvel, c);
-    tab[c] = vp_core::make_shift<T>(speed, dt, h, wp);
+    LineShift<T> sh;
+    const double nu = vp_core::split_shift(speed, dt, h, sh);
+    if (k < 7) {
+        tab[c].w[k] = (T)vp_core::csl_weight(wp, k, nu);
+    } else {
+        tab[c].nu = sh.nu;
+        tab[c].n = sh.n;
+        tab[c].sigma = sh.sigma;
+    }
 }
+
+// a staged tile of at most 200 KB and up to 128 shifts behind it
+constexpr int kSweepSmem = 216 * 1024;
 
 template <typename T, int ORDER, bool PER, bool FULL>
 void set_attrs_one() {
     cudaFuncSetAttribute(k_sweep_cols<T, ORDER, PER, FULL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         200 * 1024);
+                         kSweepSmem);
     if constexpr (sizeof(T) == 4)
         cudaFuncSetAttribute(k_sweep_cols<T, ORDER, PER, FULL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             200 * 1024);
+                             kSweepSmem);
     cudaFuncSetAttribute(k_sweep_rows<T, ORDER, PER, FULL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         200 * 1024);
+                         kSweepSmem);
     if constexpr (sizeof(T) == 4)
         cudaFuncSetAttribute(k_sweep_rows<T, ORDER, PER, FULL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             200 * 1024);
+                             kSweepSmem);
     cudaFuncSetAttribute(k_sweep_cols_tma<T, ORDER, PER, FULL>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
@@ -499,6 +541,16 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return fn;
 }
 
+// one sweep's speeds: class c of a kick moves at accel[c]; tab_ready: the
+// context's table already holds this sweep's shifts, from class cls0 on
+struct SweepShift {
+    int kick, dim;
+    double dt;
+    const double *accel;
+    bool tab_ready;
+    long long cls0;
+};
+
 // ghost rows staged on each side of a line
 inline int ghost_rows(const SweepGeo &geo) { return geo.periodic ? 0 : VP_GHOST; }
 
@@ -527,10 +579,50 @@ bool pair_eligible(const vp_ctx *c, const SweepGeo &geo, int W) {
 // line classes and tile coordinates are computed in 32-bit arithmetic
 inline bool geo_fits_32(const SweepGeo &geo) { return geo.outer < (1LL << 32) && geo.inner < (1LL << 32); }
 
+// The most classes a tile of w columns (or lines) meets, and whether its CTAs
+// decompose their own shifts (true) or read a table that a launch of its own
+// makes first.  Own shifts pay while the whole sweep is at most four CTAs per
+// SM: the table's launch and the wait for it cost 3-4 us there, the FP64 chain
+// in front of the walk well under 1 us.  With more waves the chain is paid by
+// every wave (kicks of the 32^3 x 64^3 grid, one class per tile: 109 -> 119 ms
+// per step), the table once.
+inline int tile_classes(const SweepGeo &geo, int w) {
+    const bool many = geo.cls_from_inner || geo.inner == 1;
+    const long long n = many ? (w - 1) / geo.cdiv + 2 : 1;
+    return (int)(n > w ? w : n);
+}
+inline bool own_shifts(const vp_ctx *c, const SweepGeo &geo, long long tiles) {
+    return !(geo.cls_from_inner && geo.inner == 1) && tiles <= 4LL * c->sm_count;
+}
+
+// the tile's shift source: own (ncl > 0) or the context's table, made here
 template <typename T>
-int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu) {
+int shift_source(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, int w, long long tiles, bool table,
+                 ShiftSrc<T> &src) {
+    const vp_grid &g = c->g;
+    src = ShiftSrc<T>{};
+    if (!table && own_shifts(c, geo, tiles)) {
+        const int d = sw.dim;
+        src.accel = sw.kick ? sw.accel : nullptr;
+        src.lo = g.vlo[d];
+        src.dvel = (g.vhi[d] - g.vlo[d]) / g.nv[d];
+        src.h = sw.kick ? src.dvel : (g.xhi[d] - g.xlo[d]) / g.nx[d];
+        src.dt = sw.dt;
+        src.ncl = tile_classes(geo, w);
+        src.wp = c->wp;
+        return VP_OK;
+    }
+    src.tab = static_cast<const LineShift<T> *>(c->d_shift);
+    if (sw.tab_ready) {
+        src.tab += sw.cls0;
+        return VP_OK;
+    }
+    return vp_launch_shift_table(c, sw.kick, sw.dim, sw.dt, sw.accel);
+}
+
+template <typename T>
+int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &sw) {
     if (!geo_fits_32(geo)) return vp_fail(c, VP_ENOTSUP, "sweep geometry exceeds 32-bit line indexing");
-    const LineShift<T> *tab = static_cast<const LineShift<T> *>(c->d_shift);
     const LimParams lp{c->g.alpha, c->g.mp, c->g.pp};
     T *f = static_cast<T *>(c->f);
     const int L = geo.L;
@@ -554,7 +646,15 @@ int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu) {
     const int order = c->g.order;
     const bool per = geo.periodic != 0;
     const bool full = c->g.mp && c->g.pp;
-    if (tu.impl == 2 && tma_eligible<T>(c, geo, W)) {
+    const bool tma = tu.impl == 2 && tma_eligible<T>(c, geo, W);
+    const size_t tile = (size_t)(L + 2 * ghost_rows(geo)) * W * sizeof(T);
+    if (!tma && tile > 200 * 1024) return vp_fail(c, VP_ENOTSUP, "line of %d cells too long to stage", L);
+    ShiftSrc<T> src;
+    const int rc = shift_source<T>(c, sw, geo, W, tiles, tma, src);
+    if (rc) return rc;
+    const size_t smem = tile + vp_core::shift_smem<T>(tile, src.ncl);
+    if (tma) {
+        const LineShift<T> *tab = src.tab;
         CUtensorMap map;
         const cuuint64_t dims[3] = {(cuuint64_t)geo.inner, (cuuint64_t)L, (cuuint64_t)geo.outer};
         const cuuint64_t strides[2] = {(cuuint64_t)geo.inner * sizeof(T),
@@ -567,10 +667,10 @@ int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu) {
                                           CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return vp_fail(c, VP_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
-        const size_t smem = tma_smem<T>(L, W, ghost_rows(geo));
+        const size_t tsmem = tma_smem<T>(L, W, ghost_rows(geo));
         int per_sm = tu.ctas_per_sm;
         if (per_sm <= 0) {
-#define VP_OCC(O, P, F) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_cols_tma<T, O, P, F>, threads, smem)
+#define VP_OCC(O, P, F) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_cols_tma<T, O, P, F>, threads, tsmem)
             VP_DISPATCH(order, per, full, VP_OCC);
 #undef VP_OCC
             per_sm = per_sm < 1 ? 1 : per_sm;
@@ -578,24 +678,20 @@ int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu) {
         long long grid = (long long)per_sm * c->sm_count;
         grid = grid > tiles ? tiles : grid;
 #define VP_LAUNCH(O, P, F) \
-    k_sweep_cols_tma<T, O, P, F><<<(unsigned)grid, threads, smem, c->stream>>>(map, tab, geo, lp, c->d_status, \
+    k_sweep_cols_tma<T, O, P, F><<<(unsigned)grid, threads, tsmem, c->stream>>>(map, tab, geo, lp, c->d_status, \
                                                                                 c->opt_wait_limit)
         VP_DISPATCH(order, per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     } else if (pair) {
-        const size_t smem = (size_t)(L + 2 * ghost_rows(geo)) * W * sizeof(T);
-        if (smem > 200 * 1024) return vp_fail(c, VP_ENOTSUP, "line of %d cells too long to stage", L);
         const int pthreads = threads;
         geo.fd_w2 = make_fastdiv((unsigned)(W >> 1));
 #define VP_LAUNCH(O, P, F) \
-    k_sweep_cols<T, O, P, F, sizeof(T) == 4><<<(unsigned)tiles, pthreads, smem, c->stream>>>(f, tab, geo, lp)
+    k_sweep_cols<T, O, P, F, sizeof(T) == 4><<<(unsigned)tiles, pthreads, smem, c->stream>>>(f, src, geo, lp)
         VP_DISPATCH(order, per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     } else {
-        const size_t smem = (size_t)(L + 2 * ghost_rows(geo)) * W * sizeof(T);
-        if (smem > 200 * 1024) return vp_fail(c, VP_ENOTSUP, "line of %d cells too long to stage", L);
 #define VP_LAUNCH(O, P, F) \
-    k_sweep_cols<T, O, P, F, false><<<(unsigned)tiles, threads, smem, c->stream>>>(f, tab, geo, lp)
+    k_sweep_cols<T, O, P, F, false><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp)
         VP_DISPATCH(order, per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     }
@@ -610,9 +706,8 @@ size_t rows_smem(int L, int R, int gp) {
 }
 
 template <typename T>
-int launch_rows(vp_ctx *c, SweepGeo geo, const SweepTune &tu) {
+int launch_rows(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &sw) {
     if (!geo_fits_32(geo)) return vp_fail(c, VP_ENOTSUP, "sweep geometry exceeds 32-bit line indexing");
-    const LineShift<T> *tab = static_cast<const LineShift<T> *>(c->d_shift);
     const LimParams lp{c->g.alpha, c->g.mp, c->g.pp};
     T *f = static_cast<T *>(c->f);
     const int L = geo.L;
@@ -631,8 +726,12 @@ int launch_rows(vp_ctx *c, SweepGeo geo, const SweepTune &tu) {
     geo.fd_l = make_fastdiv((unsigned)L);
     const long long blocks = (geo.outer + R - 1) / R;
     if (blocks >= (1LL << 31)) return vp_fail(c, VP_ENOTSUP, "sweep has too many tiles");
-    const size_t smem = rows_smem<T>(L, R, ghost_rows(geo));
-    if (smem > 200 * 1024) return vp_fail(c, VP_ENOTSUP, "line of %d cells too long to stage", L);
+    const size_t tile = rows_smem<T>(L, R, ghost_rows(geo));
+    if (tile > 200 * 1024) return vp_fail(c, VP_ENOTSUP, "line of %d cells too long to stage", L);
+    ShiftSrc<T> src;
+    const int rc = shift_source<T>(c, sw, geo, R, blocks, false, src);
+    if (rc) return rc;
+    const size_t smem = tile + vp_core::shift_smem<T>(tile, src.ncl);
     const int threads = ((per_row * nseg + 31) / 32) * 32;
     const bool per = geo.periodic != 0;
     const bool full = c->g.mp && c->g.pp;
@@ -640,12 +739,12 @@ int launch_rows(vp_ctx *c, SweepGeo geo, const SweepTune &tu) {
         geo.fd_w2 = make_fastdiv((unsigned)(R >> 1));
         const int pthreads = threads;
 #define VP_LAUNCH(O, P, F) \
-    k_sweep_rows<T, O, P, F, sizeof(T) == 4><<<(unsigned)blocks, pthreads, smem, c->stream>>>(f, tab, geo, lp)
+    k_sweep_rows<T, O, P, F, sizeof(T) == 4><<<(unsigned)blocks, pthreads, smem, c->stream>>>(f, src, geo, lp)
         VP_DISPATCH(c->g.order, per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     } else {
 #define VP_LAUNCH(O, P, F) \
-    k_sweep_rows<T, O, P, F, false><<<(unsigned)blocks, threads, smem, c->stream>>>(f, tab, geo, lp)
+    k_sweep_rows<T, O, P, F, false><<<(unsigned)blocks, threads, smem, c->stream>>>(f, src, geo, lp)
         VP_DISPATCH(c->g.order, per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     }
@@ -690,13 +789,14 @@ SweepTune default_tune(const vp_ctx *c, const SweepGeo &geo) {
 }
 
 template <typename T>
-int launch_sweep_t(vp_ctx *c, int kick, int dim) {
+int launch_sweep_t(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
     const SweepGeo geo = vp_make_geo(c, kick, dim);
+    const SweepShift sw{kick, dim, dt, accel, false, 0};
     SweepTune tu = c->tune[kick][dim];
     if (!tu.valid || (c->opt_impl && tu.impl != c->opt_impl)) tu = default_tune<T>(c, geo);
     if (c->opt_impl == 1) tu.impl = 1;
-    if (geo.inner > 1) return launch_cols<T>(c, geo, tu);
-    return launch_rows<T>(c, geo, tu);
+    if (geo.inner > 1) return launch_cols<T>(c, geo, tu, sw);
+    return launch_rows<T>(c, geo, tu, sw);
 }
 
 // Autotuner: time candidate tile shapes of one sweep geometry with the
@@ -712,7 +812,7 @@ int launch_sweep_t(vp_ctx *c, int kick, int dim) {
 constexpr size_t kTuneBytes = size_t(256) << 20;
 
 template <typename T>
-int tune_on(vp_ctx *c, int kick, int dim, const SweepGeo &geo, const SweepGeo &sub, SweepTune best);
+int tune_on(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, const SweepGeo &sub, SweepTune best);
 
 template <typename T>
 int tune_t(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
@@ -771,12 +871,13 @@ int tune_t(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
                  ? VP_OK : vp_fail(c, VP_ECUDA, "tuning copy failed");
     if (rc == VP_OK) rc = vp_launch_shift_table(c, kick, dim, dt, accel);
     if (rc == VP_OK) {
-        void *f = c->f, *tab = c->d_shift;
+        void *f = c->f;
         c->f = scratch;
-        if (!geo.cls_from_inner) c->d_shift = static_cast<LineShift<T> *>(c->d_shift) + o0 / geo.cdiv;
-        rc = tune_on<T>(c, kick, dim, geo, sub, best);
+        // a kick window starts at spatial point o0 / cdiv
+        const long long cls0 = geo.cls_from_inner ? 0 : o0 / geo.cdiv;
+        const SweepShift sw{kick, dim, dt, kick ? accel + cls0 : accel, true, cls0};
+        rc = tune_on<T>(c, sw, geo, sub, best);
         c->f = f;
-        c->d_shift = tab;
     }
     cudaStreamSynchronize(c->stream);
     cudaFree(scratch);
@@ -785,7 +886,8 @@ int tune_t(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
 
 // time the candidates of geometry geo on sub (the tuning copy bound as f)
 template <typename T>
-int tune_on(vp_ctx *c, int kick, int dim, const SweepGeo &geo, const SweepGeo &sub, SweepTune best) {
+int tune_on(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, const SweepGeo &sub, SweepTune best) {
+    const int kick = sw.kick, dim = sw.dim;
     int rc = VP_OK;
     constexpr int kMaxCand = 48;
     SweepTune cand[kMaxCand];
@@ -838,7 +940,7 @@ int tune_on(vp_ctx *c, int kick, int dim, const SweepGeo &geo, const SweepGeo &s
         float ms = 1e30f;
         for (int rep = 0; rep < 2; ++rep) {
             cudaEventRecord(e0, c->stream);
-            rc = geo.inner > 1 ? launch_cols<T>(c, sub, cand[i]) : launch_rows<T>(c, sub, cand[i]);
+            rc = geo.inner > 1 ? launch_cols<T>(c, sub, cand[i], sw) : launch_rows<T>(c, sub, cand[i], sw);
             cudaEventRecord(e1, c->stream);
             if (rc) break;
             const cudaError_t se = cudaEventSynchronize(e1);
@@ -885,8 +987,8 @@ int vp_launch_shift_table(vp_ctx *c, int kick, int dim, double dt, const double 
     const double h = kick ? (g.vhi[dim] - g.vlo[dim]) / g.nv[dim] : (g.xhi[dim] - g.xlo[dim]) / g.nx[dim];
     const double lo = g.vlo[dim];
     const double dvel = (g.vhi[dim] - g.vlo[dim]) / g.nv[dim];
-    const int th = 128;
-    const int bl = (nclass + th - 1) / th;
+    const int th = 64;
+    const int bl = (8 * nclass + th - 1) / th;
     if (g.precision == VP_F32)
         k_shift_table<float><<<bl, th, 0, c->stream>>>(static_cast<LineShift<float> *>(c->d_shift),
                                                        nclass, kick, lo, dvel, accel, dt, h, c->wp);
@@ -898,9 +1000,9 @@ int vp_launch_shift_table(vp_ctx *c, int kick, int dim, double dt, const double 
     return VP_OK;
 }
 
-int vp_launch_sweep(vp_ctx *c, int kick, int dim) {
-    if (c->g.precision == VP_F32) return launch_sweep_t<float>(c, kick, dim);
-    return launch_sweep_t<double>(c, kick, dim);
+int vp_launch_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+    if (c->g.precision == VP_F32) return launch_sweep_t<float>(c, kick, dim, dt, accel);
+    return launch_sweep_t<double>(c, kick, dim, dt, accel);
 }
 
 int vp_tune_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel) {

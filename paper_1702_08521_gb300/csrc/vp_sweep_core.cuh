@@ -481,24 +481,30 @@ __device__ __forceinline__ void walk(const T *__restrict__ sm0, int ss, int L, c
 // from zero), zeta = s - n, nu = |zeta|, sigma = sign(zeta); the CSL weights
 // are the weight polynomials evaluated at nu.
 template <typename T>
-__device__ __forceinline__ LineShift<T> make_shift(double speed, double dt, double h, const WPoly &wp) {
+__device__ __forceinline__ double split_shift(double speed, double dt, double h, LineShift<T> &sh) {
     const double s = __ddiv_rn(__dmul_rn(speed, dt), h);
     double n = round(s);
     const double z = __dadd_rn(s, -n);
     const double nu = fabs(z);
-    LineShift<T> sh;
-#pragma unroll
-    for (int k = 0; k < 7; ++k) {
-        double acc = 0.0;
-        for (int j = wp.nterm - 1; j >= 0; --j) acc = fma(acc, nu, wp.c[j][k]);
-        sh.w[k] = (T)acc;
-    }
     // shifts beyond a billion cells only happen with absurd inputs; clamp so
     // the integer conversion stays defined (a zero-inflow line is empty anyway)
     n = fmin(fmax(n, -1.0e9), 1.0e9);
     sh.nu = (T)nu;
     sh.n = (int)n;
     sh.sigma = z < 0.0 ? -1 : 1;
+    return nu;
+}
+__device__ __forceinline__ double csl_weight(const WPoly &wp, int k, double nu) {
+    double acc = 0.0;
+    for (int j = wp.nterm - 1; j >= 0; --j) acc = fma(acc, nu, wp.c[j][k]);
+    return acc;
+}
+template <typename T>
+__device__ __forceinline__ LineShift<T> make_shift(double speed, double dt, double h, const WPoly &wp) {
+    LineShift<T> sh;
+    const double nu = split_shift(speed, dt, h, sh);
+#pragma unroll
+    for (int k = 0; k < 7; ++k) sh.w[k] = (T)csl_weight(wp, k, nu);
     return sh;
 }
 
@@ -509,6 +515,73 @@ __device__ __forceinline__ double cell_centre(double lo, double dvel, int j) {
 
 __device__ __forceinline__ unsigned line_class(const SweepGeo &g, unsigned o, unsigned c) {
     return g.cls_from_inner ? fmod_u(fdiv(c, g.fd_cdiv), g.fd_cmod) : fdiv(o, g.fd_cdiv);
+}
+
+// Where a sweep's lines get their shifts: a table with one entry per class,
+// or (tab == NULL) from the speeds themselves, decomposed by every CTA for the
+// `ncl` consecutive classes (at most) that its tile meets.  The same numbers
+// either way.
+template <typename T>
+struct ShiftSrc {
+    const LineShift<T> *tab;
+    const double *accel;  // kick: speed of class c is accel[c]; NULL: drift, cell c of the velocity axis
+    double lo, dvel, dt, h;
+    int ncl;
+    WPoly wp;
+};
+
+// bytes of shared memory behind a tile of `tile` bytes for ncl shifts
+template <typename T>
+__host__ __device__ inline size_t shift_smem(size_t tile, int ncl) {
+    return ncl ? ((tile + 15) & ~size_t(15)) - tile + (size_t)ncl * (sizeof(LineShift<T>) + sizeof(double)) : 0;
+}
+
+// The tile's shifts s[0..ncl), class (q0 + i) mod cmod (no mod for kicks).  Up
+// to four classes: eight lanes each of the first warp, every lane splitting the
+// shift and taking one weight.  More: the split first (tile_shifts, before the
+// tile's barrier), the weights spread over the block after it (tile_weights,
+// followed by a barrier of its own): 32 classes cost 1200 cycles of the FP64
+// pipe, where one thread per class took 1200 by itself and its own launch.
+template <typename T>
+__device__ __forceinline__ double class_speed(const ShiftSrc<T> &src, const SweepGeo &g, unsigned q) {
+    return src.accel ? src.accel[q] : cell_centre(src.lo, src.dvel, (int)fmod_u(q, g.fd_cmod));
+}
+template <typename T>
+__device__ __forceinline__ void tile_shifts(LineShift<T> *s, unsigned q0, int ncl, const ShiftSrc<T> &src,
+                                            const SweepGeo &g) {
+    double *nus = reinterpret_cast<double *>(s + src.ncl);
+    if (src.ncl <= 4) {
+        const int i = threadIdx.x >> 3, k = threadIdx.x & 7;
+        if (i < ncl) {
+            LineShift<T> sh;
+            const double nu = split_shift(class_speed(src, g, q0 + i), src.dt, src.h, sh);
+            if (k < 7) {
+                s[i].w[k] = (T)csl_weight(src.wp, k, nu);
+            } else {
+                s[i].nu = sh.nu;
+                s[i].n = sh.n;
+                s[i].sigma = sh.sigma;
+            }
+        }
+    } else {
+        for (int i = threadIdx.x; i < ncl; i += blockDim.x) {
+            LineShift<T> sh;
+            nus[i] = split_shift(class_speed(src, g, q0 + i), src.dt, src.h, sh);
+            s[i].nu = sh.nu;
+            s[i].n = sh.n;
+            s[i].sigma = sh.sigma;
+        }
+    }
+}
+template <typename T>
+__device__ __forceinline__ void tile_weights(LineShift<T> *s, int ncl, const ShiftSrc<T> &src) {
+    if (src.ncl <= 4) return;
+    const double *nus = reinterpret_cast<const double *>(s + src.ncl);
+    for (int t = threadIdx.x; t < 7 * ncl; t += blockDim.x) {
+        const int i = t / 7, k = t - 7 * i;
+        s[i].w[k] = (T)csl_weight(src.wp, k, nus[i]);
+    }
+    __syncthreads();
 }
 
 }  // namespace vp_core

@@ -250,13 +250,24 @@ struct DriftAxes {
     int nv0, nv1;
 };
 
+// (eight lanes per entry, one weight each)
 template <typename T>
-__global__ void k_drift_tables(LineShift<T> *__restrict__ tab, DriftAxes ax, double dt, WPoly wp) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_drift_tables(LineShift<T> *__restrict__ tab, DriftAxes ax, double dt,
+                               const __grid_constant__ WPoly wp) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int e = t >> 3, w = t & 7;
     if (e >= ax.nv0 + ax.nv1) return;
     const int d = e < ax.nv0 ? 0 : 1;
     const int k = d ? e - ax.nv0 : e;
-    tab[e] = vp_core::make_shift<T>(vp_core::cell_centre(ax.lo[d], ax.dvel[d], k), dt, ax.h[d], wp);
+    LineShift<T> sh;
+    const double nu = vp_core::split_shift(vp_core::cell_centre(ax.lo[d], ax.dvel[d], k), dt, ax.h[d], sh);
+    if (w < 7) {
+        tab[e].w[w] = (T)vp_core::csl_weight(wp, w, nu);
+    } else {
+        tab[e].nu = sh.nu;
+        tab[e].n = sh.n;
+        tab[e].sigma = sh.sigma;
+    }
 }
 
 template <typename T>
@@ -448,7 +459,7 @@ int run_t(vp_ctx *c, double dt, int nsteps, void *scratch, int G) {
     ax.nv1 = g.nv[1];
     LineShift<T> *tab = static_cast<LineShift<T> *>(c->d_shift);
     const int ne = ax.nv0 + ax.nv1;
-    k_drift_tables<T><<<(ne + 127) / 128, 128, 0, c->stream>>>(tab, ax, dt, c->wp);
+    k_drift_tables<T><<<(8 * ne + 63) / 64, 64, 0, c->stream>>>(tab, ax, dt, c->wp);
     c->launches++;
     VP_CUDA_TRY(c, cudaGetLastError());
     T *a = static_cast<T *>(c->f), *b = static_cast<T *>(scratch);
