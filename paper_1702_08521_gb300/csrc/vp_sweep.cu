@@ -892,39 +892,61 @@ int tune_on(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, const SweepGeo
     constexpr int kMaxCand = 48;
     SweepTune cand[kMaxCand];
     int nc = 0;
+    // Small grids (fewer 32-line tiles than two per SM) take narrow tiles of
+    // short segments, so that the walk's serial chain is short and every SM has
+    // work: 64 x 128 in FP64 had 4 and 8 CTAs (drift 50 us, kick 23 us, the FP64
+    // pipe of those SMs busy throughout), 512 x 512 in FP64 16 and 64 (214 and
+    // 60 us).  A segment of l cells computes l + 1 interfaces, hence l >= 4.
+    const bool small = geo.outer * geo.inner < 64LL * c->sm_count;
+    auto add = [&](int impl, int W, int nseg) {
+        if (nc < kMaxCand) cand[nc++] = SweepTune{1, impl, W, nseg, 0};
+    };
     if (geo.inner > 1) {
         const int impls[3] = {3, 2, 1};
         // lines too long for a 32-column tile take 4-16 columns and more segments
         const bool longl = (size_t)(geo.L + 2 * ghost_rows(geo)) * 32 * sizeof(T) > 200 * 1024;
         for (int ii = 0; ii < 3; ++ii) {
-            if (c->opt_impl && impls[ii] != c->opt_impl) continue;
-            for (int W = longl ? 4 : 32; W <= (longl ? 16 : 128); W *= 2)
-                for (int nseg = 1; nseg <= (longl ? 64 : 8); nseg *= 2) {
-                    const int th = (impls[ii] == 3 ? W / 2 : W) * nseg;
-                    if (th < (impls[ii] == 3 ? 32 : 64) || th > (impls[ii] == 3 ? VP_PAIR_THREADS : 512) ||
-                        nseg > geo.L || (longl && nseg * 8 > geo.L))
+            const int impl = impls[ii], per = impl == 3 ? 2 : 1;
+            if (c->opt_impl && impl != c->opt_impl) continue;
+            const int w0 = small ? (int)(16 / sizeof(T)) : (longl ? 4 : 32);
+            for (int W = w0; W <= (small ? 8 * w0 : (longl ? 16 : 128)); W *= 2)
+                for (int nseg = 1; nseg <= (small ? 128 : (longl ? 64 : 8)); nseg *= 2) {
+                    const int th = W / per * nseg;
+                    if (th > (impl == 3 ? VP_PAIR_THREADS : 512) || nseg > geo.L) continue;
+                    if (small) {
+                        // segments of 4 to 32 cells, one warp at least where the line has the cells
+                        if (nseg * 4 > geo.L || (nseg < 128 && nseg * 64 <= geo.L) || (th < 32 && nseg * 8 <= geo.L))
+                            continue;
+                    } else if (th < (impl == 3 ? 32 : 64) || (longl && nseg * 8 > geo.L)) {
                         continue;
+                    }
                     const int Weff = geo.inner < W ? (int)geo.inner : W;
-                    if (impls[ii] == 2 && !tma_eligible<T>(c, geo, Weff)) continue;
-                    if (impls[ii] == 3 && !pair_eligible<T>(c, geo, Weff)) continue;
-                    if (impls[ii] != 2 && (size_t)(geo.L + 2 * ghost_rows(geo)) * W * sizeof(T) > 200 * 1024)
+                    if (impl == 2 && !tma_eligible<T>(c, geo, Weff)) continue;
+                    if (impl == 3 && !pair_eligible<T>(c, geo, Weff)) continue;
+                    if (impl != 2 && (size_t)(geo.L + 2 * ghost_rows(geo)) * W * sizeof(T) > 200 * 1024)
                         continue;
-                    if (nc < kMaxCand) cand[nc++] = SweepTune{1, impls[ii], W, nseg, 0};
+                    add(impl, W, nseg);
                 }
         }
     } else {
         // long lines take fewer lines per CTA (the staged tile must fit) and
-        // more segments per line (segments of at least 8 cells)
+        // more segments per line (segments of at least 8 cells; 4 on small grids)
         for (int impl = 1; impl <= 3; impl += 2) {
+            const int per = impl == 3 ? 2 : 1;
             if ((c->opt_impl == 1 && impl != 1) || (c->opt_impl == 3 && impl != 3) || (impl == 3 && sizeof(T) != 4))
                 continue;
-            for (int R = 8; R <= 128; R *= 2)
-                for (int nseg = 1; nseg <= 64; nseg *= 2) {
-                    const int th = (impl == 3 ? R / 2 : R) * nseg;
-                    if (th < (impl == 3 ? 32 : 64) || th > (impl == 3 ? VP_PAIR_THREADS : 512) || nseg * 8 > geo.L)
+            for (int R = small ? per : 8; R <= (small ? 8 : 128); R *= 2)
+                for (int nseg = 1; nseg <= (small ? 256 : 64); nseg *= 2) {
+                    const int th = R / per * nseg;
+                    if (th > (impl == 3 ? VP_PAIR_THREADS : 512)) continue;
+                    if (small) {
+                        if (nseg * 4 > geo.L || (nseg < 256 && nseg * 64 <= geo.L) || (th < 32 && nseg * 8 <= geo.L))
+                            continue;
+                    } else if (th < (impl == 3 ? 32 : 64) || nseg * 8 > geo.L) {
                         continue;
+                    }
                     if (rows_smem<T>(geo.L, R, ghost_rows(geo)) > 200 * 1024) continue;
-                    if (nc < kMaxCand) cand[nc++] = SweepTune{1, impl, R, nseg, 0};
+                    add(impl, R, nseg);
                 }
         }
     }
