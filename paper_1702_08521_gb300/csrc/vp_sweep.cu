@@ -154,8 +154,12 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
             const int r0 = (int)fdiv(seg * (unsigned)L, geo.fd_nseg);
             const int r1 = (int)fdiv((seg + 1) * (unsigned)L, geo.fd_nseg);
             const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
-            PtrStore<T> st{base + cc + (long long)i0 * geo.inner, (long long)sh.sigma * geo.inner};
-            walk<T, ORDER, PERIODIC, FULL, G1>(data + cc, W, L, sh, r0, r1, (T)lp.alpha, lp.mp, lp.pp, st);
+            vp_core::walk_line<T, ORDER, PERIODIC, FULL, G1>(
+                data + cc, W, L, sh, r0, r1, (T)lp.alpha, lp.mp, lp.pp, [&](auto t) {
+                    using U = decltype(t);
+                    return PtrStore<U>{reinterpret_cast<U *>(base + cc + (long long)i0 * geo.inner),
+                                       (long long)sh.sigma * geo.inner};
+                });
         }
     }
 }
@@ -308,9 +312,11 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
             const int r0 = (int)fdiv(seg * (unsigned)L, geo.fd_nseg);
             const int r1 = (int)fdiv((seg + 1) * (unsigned)L, geo.fd_nseg);
             const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
-            PtrStore<T> st{out + line * Q + i0, (long long)sh.sigma};
-            walk<T, ORDER, PERIODIC, FULL, G1>(in + line * P + GP, 1, L, sh, r0, r1, (T)lp.alpha, lp.mp, lp.pp,
-                                               st);
+            vp_core::walk_line<T, ORDER, PERIODIC, FULL, G1>(
+                in + line * P + GP, 1, L, sh, r0, r1, (T)lp.alpha, lp.mp, lp.pp, [&](auto t) {
+                    using U = decltype(t);
+                    return PtrStore<U>{reinterpret_cast<U *>(out + line * Q + i0), (long long)sh.sigma};
+                });
         }
     }
     __syncthreads();

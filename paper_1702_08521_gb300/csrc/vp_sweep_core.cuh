@@ -3,6 +3,8 @@
 // ensemble).
 #pragma once
 
+#include <type_traits>
+
 #include "vp_internal.cuh"
 
 namespace vp_core {
@@ -48,6 +50,42 @@ __device__ __forceinline__ P2 fmax(P2 a, P2 b) { return P2(make_float2(fmaxf(a.v
 // both lines equal (the flat-stencil test asks it of both lines of a pair)
 __device__ __forceinline__ bool operator==(P2 a, P2 b) { return a.v.x == b.v.x && a.v.y == b.v.y; }
 
+// ---- FP64 with integer comparisons -------------------------------------------
+//
+// A warp's FP64 instruction takes 16 cycles of the SM's two FMA lanes, and
+// min, max and comparisons of doubles run there too: ~28 of the ~50 FP64
+// instructions of a cell-update.  FD orders doubles by their bits on the
+// integer pipe instead (the same minimum or maximum for every pair of finite
+// numbers, up to the sign of zero).  Numbers that are not finite, or so large
+// that the arithmetic between the comparisons could overflow, are ordered
+// differently from fmin / fmax: the walk notes them (FD::kBig) and its caller
+// repeats the segment in plain double.
+struct FD {
+    double v;
+    static constexpr int kBig = (1023 + 1000) << 20;  // high word of 2^1000
+    FD() = default;
+    __device__ __forceinline__ explicit FD(double x) : v(x) {}
+};
+__device__ __forceinline__ FD operator+(FD a, FD b) { return FD(__dadd_rn(a.v, b.v)); }
+__device__ __forceinline__ FD operator-(FD a, FD b) { return FD(__dadd_rn(a.v, -b.v)); }
+__device__ __forceinline__ FD operator-(FD a) {
+    return FD(__hiloint2double(__double2hiint(a.v) ^ (int)0x80000000, __double2loint(a.v)));
+}
+__device__ __forceinline__ FD operator*(FD a, FD b) { return FD(__dmul_rn(a.v, b.v)); }
+__device__ __forceinline__ FD fma(FD a, FD b, FD c) { return FD(__fma_rn(a.v, b.v, c.v)); }
+__device__ __forceinline__ FD mul_rn(FD a, FD b) { return FD(__dmul_rn(a.v, b.v)); }
+// equal bits (0 and -0 differ: the flat-stencil test then computes the flux)
+__device__ __forceinline__ bool operator==(FD a, FD b) {
+    return __double_as_longlong(a.v) == __double_as_longlong(b.v);
+}
+// a < b for a, b of different bits: two's-complement order, reversed where both are negative
+__device__ __forceinline__ bool below(FD a, FD b) {
+    const long long x = __double_as_longlong(a.v), y = __double_as_longlong(b.v);
+    return (x < y) != ((__double2hiint(a.v) & __double2hiint(b.v)) < 0);
+}
+__device__ __forceinline__ FD fmin(FD a, FD b) { return below(a, b) ? a : b; }
+__device__ __forceinline__ FD fmax(FD a, FD b) { return below(a, b) ? b : a; }
+
 // shift decompositions of a pair of lines walked together (equal n and sigma)
 struct LineShiftP2 {
     P2 w[7];
@@ -81,6 +119,8 @@ template <typename T>
 __device__ __forceinline__ T c43() { return T(4) / T(3); }
 template <>
 __device__ __forceinline__ P2 c43<P2>() { return P2(4.0f / 3.0f); }
+template <>
+__device__ __forceinline__ FD c43<FD>() { return FD(4.0 / 3.0); }
 
 // minmod of four: min if all > 0, max if all < 0, else 0 (= max(min,0) + min(max,0))
 template <typename T>
@@ -104,6 +144,8 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 }
 __device__ __forceinline__ double min3(double a, double b, double c) { return fmin(fmin(a, b), c); }
 __device__ __forceinline__ double max3(double a, double b, double c) { return fmax(fmax(a, b), c); }
+__device__ __forceinline__ FD min3(FD a, FD b, FD c) { return fmin(fmin(a, b), c); }
+__device__ __forceinline__ FD max3(FD a, FD b, FD c) { return fmax(fmax(a, b), c); }
 __device__ __forceinline__ P2 min3(P2 a, P2 b, P2 c) {
     return P2(make_float2(min3(a.v.x, b.v.x, c.v.x), min3(a.v.y, b.v.y, c.v.y)));
 }
@@ -201,6 +243,7 @@ __device__ __forceinline__ T mp_limit(T phi, T um2, T um1, T u0, T u1, T u2, T a
 // may take out of a non-negative cell so that two of them leave it >= 0.
 __device__ __forceinline__ float half_rd(float u) { return __fmul_rd(u, 0.5f); }
 __device__ __forceinline__ double half_rd(double u) { return __dmul_rd(u, 0.5); }
+__device__ __forceinline__ FD half_rd(FD u) { return FD(__dmul_rd(u.v, 0.5)); }
 __device__ __forceinline__ P2 half_rd(P2 u) { return P2(__fmul2_rd(u.v, make_float2(0.5f, 0.5f))); }
 __device__ __forceinline__ P2 mul_rn(P2 a, P2 b) { return P2(__fmul2_rn(a.v, b.v)); }
 
@@ -319,9 +362,14 @@ __device__ __forceinline__ T flux_walk(const SH &sh, T um3, T um2, T um1, T u0, 
 
 template <typename T, int ORDER, bool PERIODIC, bool FULL, int GP, bool NEG = false, bool FLAT = true,
           typename Store, typename SH>
-__device__ __forceinline__ void walk(const T *__restrict__ sm0, int ss, int L, const SH &sh,
+__device__ __forceinline__ bool walk(const T *__restrict__ sm0, int ss, int L, const SH &sh,
                                      int r0, int r1, T alpha, int mp, int pp, Store store) {
-    if (r0 >= r1) return;
+    if (r0 >= r1) return false;
+    // FD: the largest |u| of the segment (high words), for the caller's repeat
+    int big = 0;
+    auto note = [&](const T &x) {
+        if constexpr (std::is_same<T, FD>::value) big = max(big, __double2hiint(x.v) & 0x7fffffff);
+    };
     const int sg = sh.sigma;
     const T nu = sh.nu;
     int i = sg > 0 ? r0 : r1 - 1;
@@ -351,7 +399,10 @@ __device__ __forceinline__ void walk(const T *__restrict__ sm0, int ss, int L, c
     int inc = 0;
     T w[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) w[k] = *row(p0 + k * sg);
+    for (int k = 0; k < 8; ++k) {
+        w[k] = *row(p0 + k * sg);
+        note(w[k]);
+    }
     // incoming mass of the first cell: upwind cell i - sg, stencil w[0..6]
     T dc = T(0), m4m = T(0);  // curvature at the next upwind cell, d^{M4} at its upwind face
     T m4p = T(0);
@@ -425,6 +476,7 @@ __device__ __forceinline__ void walk(const T *__restrict__ sm0, int ss, int L, c
         fin = fout;                                                                               \
         i += sg;                                                                                  \
         w[K & 7] = *src;                                                                          \
+        note(w[K & 7]);                                                                           \
         src += inc;                                                                               \
     }
 
@@ -474,6 +526,22 @@ __device__ __forceinline__ void walk(const T *__restrict__ sm0, int ss, int L, c
         }
     }
 #undef VP_WALK_STEP
+    return big >= FD::kBig;
+}
+
+// The walk of one line in the arithmetic of its type: FP64 lines with integer
+// comparisons, repeated in plain double where the data ask for it (the store
+// writes the same cells again).
+template <typename T, int ORDER, bool PERIODIC, bool FULL, int GP, typename MakeStore>
+__device__ __forceinline__ void walk_line(const T *sm0, int ss, int L, const LineShift<T> &sh, int r0, int r1,
+                                          T alpha, int mp, int pp, MakeStore store) {
+    if constexpr (sizeof(T) == 8) {
+        if (!walk<FD, ORDER, PERIODIC, FULL, GP>(reinterpret_cast<const FD *>(sm0), ss, L,
+                                                 reinterpret_cast<const LineShift<FD> &>(sh), r0, r1, FD(alpha), mp,
+                                                 pp, store(FD())))
+            return;
+    }
+    walk<T, ORDER, PERIODIC, FULL, GP>(sm0, ss, L, sh, r0, r1, alpha, mp, pp, store(T()));
 }
 
 // Shift decomposition of one line, in double precision so that the integer

@@ -255,3 +255,53 @@ def test_fp32_positivity_exact_down_to_subnormals(dims, nx, nv):
         assert f_g.min() >= 0.0
     assert rel_l1(f_g, f_o) <= 1e-5
     sim.close()
+
+
+def _with_specials(rng, shape):
+    """Non-negative cells of every size, with zeros of both signs, numbers near
+    both ends of the range, infinities and NaN scattered among them."""
+    f = rng.random(shape) * 10.0 ** rng.uniform(-320, 299, size=shape)
+    f[rng.random(shape) < 0.2] = 0.0
+    for v in (-0.0, 5e-324, 1e299, 1e302, 1.7e308, np.inf, np.nan, -1e303):
+        f[rng.random(shape) < 0.004] = v
+    return f
+
+
+@pytest.mark.parametrize("order", [5, 7])
+@pytest.mark.parametrize("xbc", [0, 1])
+@pytest.mark.parametrize("n,nv", [(40, 16), (64, 48)])
+def test_fp64_integer_comparisons_give_the_plain_result(order, xbc, n, nv):
+    """The staged FP64 kernels order doubles by their bits and repeat a segment
+    in plain double where a cell is not finite or nearly overflows: the same
+    numbers as the TMA kernel, which computes in plain double throughout, on
+    ordinary data and on data full of special values.  Strided lines directly;
+    contiguous lines against strided copies of them on a grid with a second
+    velocity axis."""
+    rng = np.random.default_rng(order + nv)
+    g1 = dict(dims=1, nx=[n], nv=[nv], xlo=[0.0], xhi=[1.0], vlo=[-3.0], vhi=[2.5], order=order, xbc=xbc)
+    g2 = dict(dims=2, nx=[n, 1], nv=[nv, 16], xlo=[0.0, 0.0], xhi=[1.0, 1.0], vlo=[-3.0, 0.0], vhi=[2.5, 1.0],
+              order=order, xbc=xbc)
+    acc = rng.uniform(-2.0, 2.0, size=n)
+
+    def run(g, impl, f0, kick):
+        sim, _ = both(g, V.VP_F64)
+        V.vp_set_option(sim.ctx, V.VP_OPT_SWEEP_IMPL, impl)
+        to_gpu(sim, f0)
+        if kick:
+            V.vp_kick_sweep(sim.ctx, 0, 0.31, accel_tensor(sim, acc))
+        else:
+            V.vp_drift_sweep(sim.ctx, 0, 0.017)
+        out, impl_used = from_gpu(sim), V.vp_get_tuning(sim.ctx, kick, 0)["impl"]
+        sim.close()
+        return out, impl_used
+    for f0 in (inputs.random_f(n * nv, seed=5).reshape(n, nv), _with_specials(rng, (n, nv))):
+        wide = np.repeat(f0[:, :, None], 16, axis=2)
+        ref, used = run(g1, 2, f0, 0)
+        assert used == 2
+        got, used = run(g1, 1, f0, 0)
+        assert used == 1 and np.array_equal(got, ref, equal_nan=True)
+        ref, used = run(g2, 2, wide, 1)
+        assert used == 2
+        ref = ref.reshape(n, nv, 16)[:, :, 0].reshape(-1)
+        got, _ = run(g1, 1, f0, 1)
+        assert np.array_equal(got, ref, equal_nan=True)
