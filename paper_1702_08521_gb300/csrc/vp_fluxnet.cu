@@ -263,179 +263,346 @@ __global__ void k_adam(float *__restrict__ wts, float *__restrict__ m, float *__
 
 // ---- training data -----------------------------------------------------------------
 
-// Mass through interfaces of fine lines, in fine-cell units, for one sweep:
-// G_{i+1/2} = sum of the N whole cells swept through + nu Phi_hat at the
-// shifted interface (the flux form of the SL update: f'_i = f_i + G_{i-1/2}
-// - G_{i+1/2}).  Lines: f viewed as [outer][L][inner]; one thread per line;
-// the line's class (speed) as in the sweeps.  Output: G at interfaces
-// j * every - 1/2 for j = 0 .. L/every (boundary interfaces included).
-__global__ void k_fine_flux(const float *__restrict__ f, long long outer, int L, long long inner,
-                            int periodic, int kick, int from_inner, long long cdiv, long long cmod,
-                            const double *__restrict__ accel, double lo, double dvel, double dt,
-                            double h, WPoly wp, int every, double *__restrict__ G, float alpha) {
-    extern __shared__ double fx[];  // [L][blockDim] prefix sums (FP64)
-    const long long line = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int T = blockDim.x;
-    const bool ok = line < outer * inner;
-    const long long o = ok ? line / inner : 0, c = ok ? line % inner : 0;
-    const float *base = f + o * L * inner + c;
-    const long long cls = from_inner ? (c / cdiv) % cmod : o / cdiv;
-    const double speed = kick ? accel[cls] : vp_core::cell_centre(lo, dvel, (int)cls);
-    const LineShift<float> sh = vp_core::make_shift<float>(speed, dt, h, wp);
-    const int sg = sh.sigma;
-    // value of the line in the upwind frame (reversed when sigma < 0)
-    auto val = [&](long long k) -> float {
-        if (periodic) {
-            k %= L;
-            if (k < 0) k += L;
-        } else if (k < 0 || k >= L) {
-            return 0.f;
-        }
-        const long long kk = sg > 0 ? k : L - 1 - k;
-        return base[kk * inner];
-    };
-    // prefix sums S(k) = sum_{m < k} u_m in the upwind frame
-    double acc = 0.0;
-    if (ok)
-        for (int k = 0; k < L; ++k) {
-            fx[k * T + threadIdx.x] = acc;
-            acc += val(k);
-        }
-    const double total = acc;
-    auto S = [&](long long k) -> double {  // sum_{m < k}, extended beyond the line
-        if (periodic) {
-            long long q = k / L, r = k % L;
-            if (r < 0) {
-                r += L;
-                q -= 1;
-            }
-            return fx[r * T + threadIdx.x] + (double)q * total;
-        }
-        if (k <= 0) return 0.0;
-        if (k >= L) return total;
-        return fx[k * T + threadIdx.x];
-    };
-    if (!ok) return;
-    const int n = sh.n * sg;  // whole cells swept, in the upwind frame (>= 0)
-    const int nout = L / every + 1;
-    for (int j = 0; j < nout; ++j) {
-        // interface between cells (i - 1) and i of the original line, i = j * every
-        const int i = j * every;
-        // in the upwind frame the interface sits between cells ip - 1 and ip
-        const int ip = sg > 0 ? i : L - i;
-        // G' = sum_{m = ip - n}^{ip - 1} u_m + nu Phi(upwind cell ip - 1 - n)
-        const long long up = (long long)ip - 1 - n;
-        float u[7];
-#pragma unroll
-        for (int k = 0; k < 7; ++k) u[k] = val(up - 3 + k);
-        const float M = vp_core::flux<float, 7, true>(sh, u[0], u[1], u[2], u[3], u[4], u[5], u[6], alpha, 1, 1);
-        const double g = (S(ip) - S(ip - n)) + (double)M;
-        G[line * nout + j] = sg > 0 ? g : -g;
+// FP64 instructions take 16 cycles each here, conversions included, and the
+// outputs are tens of millions of doubles: sums of a few floats are kept as a
+// value and its error term (two-sum), and the exact conversion of a normal
+// float to a double is done on its bits.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)  // normal
+        return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+    return m ? (double)x : __hiloint2double((int)b, 0);
+}
+
+struct PairSum {
+    float s, e;
+    __device__ __forceinline__ void add(float x) {
+        const float t = s + x;
+        const float bp = t - s;
+        e += (s - (t - bp)) + (x - bp);
+        s = t;
+    }
+    __device__ __forceinline__ double value() const { return widen(s) + widen(e); }
+};
+
+// geometry of the line kernels below: lines of L cells at stride inner, W (a
+// power of two, at most kTileLines) consecutive lines per CTA
+constexpr int kTileLines = 64;
+
+struct LineTile {
+    long long lines, inner;
+    int L, W, logW, periodic, from_inner;
+    unsigned cdiv, cmod;
+};
+// element of a line's first cell, and its class
+struct LinePos {
+    long long base[kTileLines];
+    unsigned cls[kTileLines];
+};
+__device__ __forceinline__ void place_lines(const LineTile &q, long long l0, int nl, LinePos &p) {
+    for (int i = threadIdx.x; i < nl; i += blockDim.x) {
+        const long long o = (l0 + i) / q.inner, c = (l0 + i) - o * q.inner;
+        p.base[i] = o * q.L * q.inner + c;
+        p.cls[i] = q.from_inner ? (unsigned)c / q.cdiv % q.cmod : (unsigned)o / q.cdiv;
     }
 }
 
+// rows beyond the line that the 7- and 8-cell stencils reach (zero, or the
+// wrapped cells of a periodic line)
+constexpr int kEdge = 8;
+
+__device__ __forceinline__ int wrap_row(int r, int L) {
+    while (r < 0) r += L;
+    while (r >= L) r -= L;
+    return r;
+}
+
+// Stage nl lines (base elements plus `off`; a line with use(i) false is zero):
+// put(line, row, value) for rows -kEdge .. L + kEdge - 1.  Lanes run over the
+// lines where neighbouring lines are neighbours in memory, else along the line.
+template <typename Use, typename Put>
+__device__ __forceinline__ void stage_lines(const float *__restrict__ f, const LineTile &q, const LinePos &p, int nl,
+                                            long long off, Use use, Put put) {
+    const int R = q.L + 2 * kEdge;
+    auto cell = [&](int i, int row) {
+        int r = row;
+        bool in = use(i);
+        if (q.periodic) r = wrap_row(r, q.L);
+        else in = in && r >= 0 && r < q.L;
+        put(i, row, in ? __ldg(f + p.base[i] + off + (long long)r * q.inner) : 0.f);
+    };
+    if (q.inner >= 16) {
+#pragma unroll 4
+        for (int t = threadIdx.x; t < R << q.logW; t += blockDim.x) {
+            const int i = t & (q.W - 1);
+            if (i < nl) cell(i, (t >> q.logW) - kEdge);
+        }
+    } else {
+        for (int i = threadIdx.x >> 5; i < nl; i += blockDim.x >> 5)
+            for (int r = (threadIdx.x & 31); r < R; r += 32) cell(i, r - kEdge);
+    }
+}
+
+// Mass through interfaces of fine lines, in fine-cell units, for one sweep:
+// G_{i+1/2} = sum of the N whole cells swept through + nu Phi_hat at the
+// shifted interface (the flux form of the SL update: f'_i = f_i + G_{i-1/2}
+// - G_{i+1/2}).  Output: G[line][j] at interfaces j * every - 1/2 for j = 0 ..
+// L/every (boundary interfaces included).
+// A CTA stages W lines and the block of results, which it writes as one
+// contiguous run (one thread per line, its results in rows of its own, its
+// stencil from global memory and double-precision prefix sums took 2783 us for
+// 6.7e7 cells; the output alone is 80 us of HBM).  Whole-cell parts of at most
+// kFewCells cells are summed directly; PREFIX: longer ones from double prefix
+// sums of the line.
+constexpr int kFewCells = 8;
+
+template <bool PREFIX>
+__global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, LineTile q,
+                                                   const LineShift<float> *__restrict__ tab, int every,
+                                                   double *__restrict__ G, float alpha) {
+    extern __shared__ __align__(16) unsigned char fsm[];
+    const int L = q.L, W = q.W, nout = L / every + 1, NP = nout | 1, WP = W + 1;
+    double *Gs = reinterpret_cast<double *>(fsm);            // [W][NP]
+    double *S = Gs + W * NP;                                  // PREFIX: [L + 1][W]
+    float *u = reinterpret_cast<float *>(S + (PREFIX ? (L + 1) * W : 0)) + kEdge * WP;  // rows of WP, from row -kEdge
+    __shared__ LinePos pos;
+    const long long l0 = (long long)blockIdx.x * W;
+    const int nl = (int)(q.lines - l0 < W ? q.lines - l0 : W);
+    place_lines(q, l0, nl, pos);
+    __syncthreads();
+    stage_lines(f, q, pos, nl, 0, [](int) { return true; }, [&](int i, int row, float v) { u[row * WP + i] = v; });
+    __syncthreads();
+    if (PREFIX) {
+        for (int i = threadIdx.x; i < nl; i += blockDim.x) {
+            double a = 0.0;
+            for (int k = 0; k < L; ++k) {
+                S[k * W + i] = a;
+                a += widen(u[k * WP + i]);
+            }
+            S[L * W + i] = a;
+        }
+        __syncthreads();
+    }
+    const int i = threadIdx.x & (W - 1);
+    if (i < nl) {
+        const LineShift<float> sh = tab[pos.cls[i]];
+        const int sg = sh.sigma;
+        const int n = sh.n * sg;  // whole cells swept, in the upwind frame
+        // the shift of the stencil: modulo the line, or just off its ends
+        const int ns = q.periodic ? n % L : (n < -2 * L - 8 ? -2 * L - 8 : (n > 2 * L + 8 ? 2 * L + 8 : n));
+        const float *ui = u + i;
+        for (int j = threadIdx.x >> q.logW; j < nout; j += blockDim.x >> q.logW) {
+            // interface between cells c - 1 and c; its stencil in the upwind
+            // frame is centred n cells upwind: rows a .. a + 6 of the line
+            const int c = j * every;
+            int a = sg > 0 ? c - ns - 4 : c + ns - 3;
+            a = q.periodic ? wrap_row(a, L) : (a < -7 ? -7 : (a > L ? L : a));
+            float w[7];
+#pragma unroll
+            for (int k = 0; k < 7; ++k) w[k] = ui[(a + (sg > 0 ? k : 6 - k)) * WP];
+            const float M = vp_core::flux<float, 7, true>(sh, w[0], w[1], w[2], w[3], w[4], w[5], w[6], alpha, 1, 1);
+            double g;
+            if (PREFIX) {
+                // sum of the cells before k, extended beyond the line
+                auto upto = [&](int k) -> double {
+                    if (q.periodic) {
+                        int w0 = k / L, r = k - w0 * L;
+                        if (r < 0) {
+                            r += L;
+                            --w0;
+                        }
+                        return S[r * W + i] + (double)w0 * S[L * W + i];
+                    }
+                    return S[(k < 0 ? 0 : (k > L ? L : k)) * W + i];
+                };
+                // cells c - n .. c - 1 (swept rightwards) or c .. c + n - 1
+                g = (sg > 0 ? upto(c) - upto(c - n) : upto(c + n) - upto(c)) + widen(M);
+            } else {
+                PairSum p{0.f, 0.f};
+                int k = sg > 0 ? (n >= 0 ? c - n : c) : (n >= 0 ? c : c + n);
+                const float one = n >= 0 ? 1.f : -1.f;
+                for (int m = n >= 0 ? n : -n; m > 0; --m, ++k) {
+                    const bool in = q.periodic || (k >= 0 && k < L);
+                    p.add(in ? one * ui[(q.periodic ? wrap_row(k, L) : k) * WP] : 0.f);
+                }
+                p.add(M);
+                g = p.value();
+            }
+            Gs[i * NP + j] = sg > 0 ? g : -g;
+        }
+    }
+    __syncthreads();
+    double *out = G + l0 * nout;
+    for (int k = threadIdx.x >> 5; k < nl; k += blockDim.x >> 5)
+        for (int j = threadIdx.x & 31; j < nout; j += 32) out[(long long)k * nout + j] = Gs[k * NP + j];
+}
+
 // coarse state: mean over the (factor1 x factor2) fine velocity cells of a
-// velocity grid [nf1][nf2] (nf2 = factor2 = 1 for one velocity dimension)
-__global__ void k_restrict_v2(const float *__restrict__ ff, float *__restrict__ fc, long long NX, int nf1,
-                              int nf2, int factor1, int factor2) {
-    const int nc1 = nf1 / factor1, nc2 = nf2 / factor2;
+// velocity grid [nf1][nf2] (nf2 = factor2 = 1 for one velocity dimension).
+// The sum as a float pair (a conversion and an addition in double per fine
+// cell took 328 us for 6.7e7 cells); quad: factor2 = 4 on 16-byte rows.
+__global__ void __launch_bounds__(256) k_restrict_v2(const float *__restrict__ ff, float *__restrict__ fc,
+                                                     long long total, FastDiv nc12, FastDiv nc2, int nf2, long long nf12,
+                                                     int factor1, int factor2, int quad, double inv) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= NX * nc1 * nc2) return;
-    const long long x = t / (nc1 * nc2);
-    const int J = (int)(t % (nc1 * nc2));
-    const int J1 = J / nc2, J2 = J % nc2;
-    double s = 0.0;
-    for (int a = 0; a < factor1; ++a)
-        for (int b = 0; b < factor2; ++b)
-            s += ff[x * nf1 * nf2 + (long long)(J1 * factor1 + a) * nf2 + (J2 * factor2 + b)];
-    fc[t] = (float)(s / (factor1 * factor2));
+    if (t >= total) return;
+    long long x;
+    unsigned J;
+    if (total < (1LL << 32)) {
+        x = fdiv((unsigned)t, nc12);
+        J = (unsigned)t - (unsigned)x * nc12.d;
+    } else {
+        x = t / nc12.d;
+        J = (unsigned)(t - x * nc12.d);
+    }
+    const unsigned J1 = fdiv(J, nc2), J2 = J - J1 * nc2.d;
+    const float *p = ff + x * nf12 + (long long)J1 * factor1 * nf2 + (long long)J2 * factor2;
+    PairSum a{0.f, 0.f};
+    if (quad) {
+#pragma unroll 4
+        for (int k = 0; k < factor1; ++k) {
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(p + (long long)k * nf2));
+            a.add(v.x);
+            a.add(v.y);
+            a.add(v.z);
+            a.add(v.w);
+        }
+    } else {
+        for (int k = 0; k < factor1; ++k)
+            for (int b = 0; b < factor2; ++b) a.add(p[(long long)k * nf2 + b]);
+    }
+    fc[t] = (float)(inv != 0.0 ? a.value() * inv : a.value() / (factor1 * factor2));
 }
 
 // Samples on coarse lines: for every coarse interface with |zeta| >= zmin,
 // features of the coarse stencil and the normalised target
 // y = (Phi_target - Phi_CSL7) / s.  Gc: coarse-unit masses through the
 // coarse interfaces ([coarse line][L + 1]).  Invalid samples get y = NaN.
-__global__ void k_make_samples(const float *__restrict__ fc, long long outer, int L, long long inner,
-                               int periodic, int kick, int from_inner, long long cdiv, long long cmod,
-                               const double *__restrict__ accel, double lo, double dvel, double dt,
-                               double h, WPoly wp, const double *__restrict__ Gc, double zmin,
-                               float *__restrict__ X, float *__restrict__ y, float *__restrict__ sc,
-                               float alpha) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long nlines = outer * inner;
-    if (t >= nlines * (L + 1)) return;
-    const long long line = t / (L + 1);
-    const int i = (int)(t % (L + 1));  // interface between cells i - 1 and i
-    const long long o = line / inner, c = line % inner;
-    const float *base = fc + o * L * inner + c;
-    const long long cls = from_inner ? (c / cdiv) % cmod : o / cdiv;
-    const double speed = kick ? accel[cls] : vp_core::cell_centre(lo, dvel, (int)cls);
-    const LineShift<float> sh = vp_core::make_shift<float>(speed, dt, h, wp);
-    const double s_full = speed * dt / h;
-    const double zeta = s_full - round(s_full);
-    float *xo = X + t * NF;
-    if (fabs(zeta) < zmin || (periodic && i == L)) {
-        for (int k = 0; k < NF; ++k) xo[k] = 0.f;
-        y[t] = __int_as_float(0x7fc00000);
-        if (sc) sc[t] = 0.f;
-        return;
+// A CTA stages W lines and the lines of their velocity neighbours (STAGED; a
+// line too long for shared memory is read in place) and takes their samples in
+// output order, 256 at a time, lanes along a line; the 25 features leave
+// through shared memory as contiguous 16-byte stores.  With a shift
+// decomposition, 64-bit remainders for every stencil cell and rows of 100 bytes
+// written by single threads it took 1205 us for 4.3e6 samples (430 MB).
+constexpr int kSampleThreads = 256;
+
+template <bool STAGED>
+__global__ void __launch_bounds__(kSampleThreads)
+    k_make_samples(const float *__restrict__ fc, LineTile q, const LineShift<float> *__restrict__ tab, int kick,
+                   const double *__restrict__ accel, double lo, double dvel, double dt, double h,
+                   const double *__restrict__ Gc, double zmin, float *__restrict__ X, float *__restrict__ y,
+                   float *__restrict__ sc, float alpha) {
+    extern __shared__ __align__(16) unsigned char ssm[];
+    float *xs = reinterpret_cast<float *>(ssm);  // [256][NF]
+    const int L = q.L, W = q.W, P = (L + 2 * kEdge) | 1;
+    float *tile = xs + kSampleThreads * NF;      // STAGED: [3][W][P]: the lines, +, - neighbours
+    const long long l0 = (long long)blockIdx.x * W;
+    const int nl = (int)(q.lines - l0 < W ? q.lines - l0 : W);
+    __shared__ LinePos pos;
+    // velocity neighbours: 1: class + 1 is the + one (larger |v|), 2: class + 1
+    // is in the box, 4: class - 1 is
+    __shared__ int nbr[kTileLines];
+    place_lines(q, l0, nl, pos);
+    __syncthreads();
+    for (int i = threadIdx.x; i < nl; i += blockDim.x) {
+        const unsigned cls = pos.cls[i];
+        nbr[i] = kick ? 0
+                      : (vp_core::cell_centre(lo, dvel, (int)cls) >= 0.0 ? 1 : 0) | (cls + 1 < q.cmod ? 2 : 0) |
+                            (cls > 0 ? 4 : 0);
     }
-    const int sg = sh.sigma;
-    auto val = [&](long long k) -> float {
-        if (periodic) {
-            k %= L;
-            if (k < 0) k += L;
-        } else if (k < 0 || k >= L) {
-            return 0.f;
+    __syncthreads();
+    if (STAGED) {
+        for (int k = 0; k < 3; ++k) {  // the lines, then class + 1 and class - 1
+            float *d = tile + (size_t)k * W * P + kEdge;
+            stage_lines(fc, q, pos, nl, k == 0 ? 0 : (k == 1 ? 1 : -1) * (long long)q.cdiv,
+                        [&](int i) { return k == 0 || (nbr[i] & (k == 1 ? 2 : 4)); },
+                        [&](int i, int row, float v) { d[i * P + row] = v; });
         }
-        const long long kk = sg > 0 ? k : L - 1 - k;
-        return base[kk * inner];
-    };
-    const int ip = sg > 0 ? i : L - i;
-    const int n = sh.n * sg;
-    const long long up = (long long)ip - 1 - n;
-    float u[8], unp[8], unm[8];
-    for (int k = 0; k < 8; ++k) u[k] = val(up - 3 + k);
-    // velocity-neighbour lines of a spatial sweep (+: larger |v|), zero
-    // outside the velocity box; none for a velocity sweep
-    for (int k = 0; k < 8; ++k) unp[k] = unm[k] = 0.f;
-    if (!kick) {
-        const int sp = speed >= 0.0 ? 1 : -1;
-        const long long J = (c / cdiv) % cmod;
-        auto nval = [&](long long dj, long long k) -> float {
-            const long long Jn = J + dj;
-            if (Jn < 0 || Jn >= cmod) return 0.f;
-            if (periodic) {
-                k %= L;
-                if (k < 0) k += L;
-            } else if (k < 0 || k >= L) {
-                return 0.f;
+        __syncthreads();
+    }
+    const int ns = nl * (L + 1);
+    const long long t0 = l0 * (L + 1);
+    for (int b0 = 0; b0 < ns; b0 += kSampleThreads) {
+        const int t = b0 + threadIdx.x;
+        float x[NF];
+        if (t < ns) {
+            const int i = t / (L + 1), j = t - i * (L + 1);  // line, interface between cells j - 1 and j
+            const long long line = l0 + i;
+            const unsigned cls = pos.cls[i];
+            const LineShift<float> sh = tab[cls];
+            bool none = q.periodic && j == L;
+            if (zmin > 0.0 && !none) {
+                const double speed = kick ? accel[cls] : vp_core::cell_centre(lo, dvel, (int)cls);
+                const double s_full = speed * dt / h;
+                none = fabs(s_full - round(s_full)) < zmin;
             }
-            const long long kk = sg > 0 ? k : L - 1 - k;
-            return base[kk * inner + dj * cdiv];
-        };
-        for (int k = 0; k < 8; ++k) {
-            unp[k] = nval(sp, up - 3 + k);
-            unm[k] = nval(-sp, up - 3 + k);
+            if (none) {
+#pragma unroll
+                for (int k = 0; k < NF; ++k) x[k] = 0.f;
+                y[t0 + t] = __int_as_float(0x7fc00000);
+                if (sc) sc[t0 + t] = 0.f;
+            } else {
+                const int sg = sh.sigma, n = sh.n * sg;
+                // row r of the line, or of the neighbour of class + 1 / - 1
+                const float *own = tile + kEdge + i * P, *base = fc + pos.base[i];
+                auto cell = [&](int nb, int r) -> float {
+                    if (STAGED) return own[(nb == 0 ? 0 : (nb > 0 ? 1 : 2)) * (W * P) + r];
+                    if (nb && !(nbr[i] & (nb > 0 ? 2 : 4))) return 0.f;
+                    if (q.periodic) r = wrap_row(r, L);
+                    else if (r < 0 || r >= L) return 0.f;
+                    return base[(long long)r * q.inner + nb * (long long)q.cdiv];
+                };
+                // stencil cells: rows a .. a + 7, in upwind order by sg
+                const int nsh = q.periodic ? n % L : (n < -2 * L - 8 ? -2 * L - 8 : (n > 2 * L + 8 ? 2 * L + 8 : n));
+                int a = sg > 0 ? j - nsh - 4 : j + nsh - 4;
+                a = q.periodic ? wrap_row(a, L) : (a < -8 ? -8 : (a > L ? L : a));
+                float u[8], unp[8], unm[8];
+                const int sp = (nbr[i] & 1) ? 1 : -1;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int r = a + (sg > 0 ? k : 7 - k);
+                    u[k] = cell(0, r);
+                    unp[k] = cell(sp, r);
+                    unm[k] = cell(-sp, r);
+                }
+                // whole cells swept in the upwind frame, signed (n < 0 when the
+                // integer shift opposes the fractional one)
+                double whole = 0.0;
+                int k = sg > 0 ? (n >= 0 ? j - n : j) : (n >= 0 ? j : j + n);
+                int r = q.periodic ? k % L : k;
+                r = q.periodic && r < 0 ? r + L : r;
+                for (int m = n >= 0 ? n : -n; m > 0; --m) {
+                    if (q.periodic || (r >= 0 && r < L)) whole += widen(cell(0, r));
+                    ++r;
+                    if (q.periodic && r == L) r = 0;
+                }
+                if (n < 0) whole = -whole;
+                const double gc = Gc[line * (L + 1) + j];
+                const double g = sg > 0 ? gc : -gc;
+                // coarse fractional mass as the plain sweep computes it: CSL7, then MP
+                float phi = sh.w[0] * u[0];
+#pragma unroll
+                for (int m = 1; m < 7; ++m) phi = fmaf(sh.w[m], u[m], phi);
+                phi = vp_core::mp_limit(phi, u[1], u[2], u[3], u[4], u[5], alpha);
+                const float s = net_features(u, unp, unm, sh.nu, x);
+                y[t0 + t] = (float)((g - whole - widen(sh.nu) * widen(phi)) / widen(s));
+                if (sc) sc[t0 + t] = s;
+            }
+#pragma unroll
+            for (int k = 0; k < NF; ++k) xs[threadIdx.x * NF + k] = x[k];
         }
+        __syncthreads();
+        const int m = (ns - b0 < kSampleThreads ? ns - b0 : kSampleThreads) * NF;
+        float *out = X + (t0 + b0) * NF;
+        if ((reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+            for (int e = 4 * threadIdx.x; e + 3 < m; e += 4 * kSampleThreads)
+                *reinterpret_cast<float4 *>(out + e) = *reinterpret_cast<const float4 *>(xs + e);
+            for (int e = (m & ~3) + threadIdx.x; e < m; e += kSampleThreads) out[e] = xs[e];
+        } else {
+            for (int e = threadIdx.x; e < m; e += kSampleThreads) out[e] = xs[e];
+        }
+        __syncthreads();
     }
-    // whole cells swept in the upwind frame, signed: sum_{m = ip - n}^{ip - 1} u_m
-    // (n < 0 when the integer shift opposes the fractional one)
-    double whole = 0.0;
-    if (n >= 0)
-        for (long long m = ip - n; m < ip; ++m) whole += val(m);
-    else
-        for (long long m = ip; m < ip - n; ++m) whole -= val(m);
-    const double g = sg > 0 ? Gc[line * (L + 1) + i] : -Gc[line * (L + 1) + i];
-    // coarse fractional mass as the plain sweep computes it: CSL7, then MP
-    float phi = sh.w[0] * u[0];
-    for (int k = 1; k < 7; ++k) phi = fmaf(sh.w[k], u[k], phi);
-    phi = vp_core::mp_limit(phi, u[1], u[2], u[3], u[4], u[5], alpha);
-    float x[NF];
-    const float s = net_features(u, unp, unm, sh.nu, x);
-    for (int k = 0; k < NF; ++k) xo[k] = x[k];
-    y[t] = (float)((g - whole - (double)sh.nu * (double)phi) / (double)s);
-    if (sc) sc[t] = s;
 }
 
 // cell pairs of the training loss: the residual of the cell between
@@ -456,15 +623,19 @@ __global__ void k_pair_coefs(const float *__restrict__ sc, const long long *__re
 
 // coarse-interface masses from fine ones: mean over `group` fine lines of
 // every fine value, scaled by `scale` (fine -> coarse cell units)
-__global__ void k_group_mean(const double *__restrict__ Gf, long long ncl, int nout, const long long *map,
-                             int group, double scale, double *__restrict__ Gc) {
+// (32-bit indices; a division only where 1 / group is not exact)
+__global__ void __launch_bounds__(256) k_group_mean(const double *__restrict__ Gf, long long total, int nout,
+                                                    FastDiv fd_nout, const long long *__restrict__ map, int group,
+                                                    double scale, double inv, double *__restrict__ Gc) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= ncl * nout) return;
-    const long long cl = t / nout;
-    const int j = (int)(t % nout);
+    if (t >= total) return;
+    const long long cl = total < (1LL << 32) ? (long long)fdiv((unsigned)t, fd_nout) : t / nout;
+    const int j = (int)(t - cl * nout);
+    const long long *m = map + cl * group;
     double s = 0.0;
-    for (int g = 0; g < group; ++g) s += Gf[map[cl * group + g] * nout + j];
-    Gc[t] = scale * s / group;
+#pragma unroll 8
+    for (int g = 0; g < group; ++g) s += Gf[m[g] * nout + j];
+    Gc[t] = inv != 0.0 ? scale * s * inv : scale * s / group;
 }
 
 // ---- inference: the learned coarse sweep, network on the tensor cores -------------------
@@ -886,6 +1057,23 @@ LineGeo line_geo(const vp_grid &g, long long NX, long long NV, int kick, int dim
     q.dvel = (g.vhi[dim] - g.vlo[dim]) / g.nv[dim];
     return q;
 }
+
+LineTile line_tile(const LineGeo &q) {
+    LineTile t{};
+    t.lines = q.outer * q.inner;
+    t.inner = q.inner;
+    t.L = q.L;
+    t.periodic = q.periodic;
+    t.from_inner = q.from_inner;
+    t.cdiv = (unsigned)q.cdiv;
+    t.cmod = (unsigned)q.cmod;
+    return t;
+}
+void set_width(LineTile &t, int W) {
+    t.W = W;
+    t.logW = 0;
+    while ((1 << t.logW) < W) ++t.logW;
+}
 }  // namespace
 
 int vp_learned_prepare(vp_ctx *c) {
@@ -989,14 +1177,32 @@ int vp_fine_flux(vp_ctx *c, int kick, int dim, double dt, const double *accel_de
     if (dim < 0 || dim >= c->g.dx || (kick && !accel_dev)) return vp_fail(c, VP_EINVAL, "bad fine-flux arguments");
     const LineGeo q = line_geo(c->g, c->NX, c->NV, kick, dim);
     if (q.L % every) return vp_fail(c, VP_EINVAL, "line length must be a multiple of `every`");
-    const int T = 64;
-    const size_t smem = (size_t)q.L * T * sizeof(double);
-    if (smem > 200 * 1024) return vp_fail(c, VP_ENOTSUP, "line too long");
-    cudaFuncSetAttribute(k_fine_flux, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    const long long nl = q.outer * q.inner;
-    k_fine_flux<<<(unsigned)((nl + T - 1) / T), T, smem, c->stream>>>(
-        static_cast<const float *>(c->f), q.outer, q.L, q.inner, q.periodic, kick, q.from_inner, q.cdiv, q.cmod,
-        accel_dev, q.lo, q.dvel, dt, q.h, c->wp, every, G_dev, (float)c->g.alpha);
+    if ((size_t)q.L * 64 * sizeof(double) > 200 * 1024) return vp_fail(c, VP_ENOTSUP, "line too long");
+    LineTile t = line_tile(q);
+    // whole-cell parts: a drift's longest is known here, a kick's only on the device
+    const double vmax = std::fmax(std::fabs(c->g.vlo[dim]), std::fabs(c->g.vhi[dim]));
+    const bool prefix = kick || !(vmax * std::fabs(dt) / q.h + 1.0 < kFewCells);
+    const int nout = q.L / every + 1;
+    auto bytes = [&](int W) {
+        return (size_t)W * (nout | 1) * sizeof(double) + (prefix ? (size_t)(q.L + 1) * W * sizeof(double) : 0) +
+               (size_t)(q.L + 2 * kEdge) * (W + 1) * sizeof(float);
+    };
+    int W = kTileLines;
+    while (W > 8 && bytes(W) > 72 * 1024) W /= 2;  // three CTAs per SM
+    set_width(t, W);
+    const size_t smem = bytes(W);
+    const int rc = vp_launch_shift_table_f32(c, kick, dim, dt, accel_dev);
+    if (rc) return rc;
+    VP_CUDA_TRY(c, cudaFuncSetAttribute(k_fine_flux<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    VP_CUDA_TRY(c, cudaFuncSetAttribute(k_fine_flux<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    const LineShift<float> *tab = static_cast<const LineShift<float> *>(c->d_shift);
+    const unsigned blocks = (unsigned)((t.lines + t.W - 1) / t.W);
+    if (prefix)
+        k_fine_flux<true><<<blocks, 256, smem, c->stream>>>(static_cast<const float *>(c->f), t, tab, every, G_dev,
+                                                            (float)c->g.alpha);
+    else
+        k_fine_flux<false><<<blocks, 256, smem, c->stream>>>(static_cast<const float *>(c->f), t, tab, every, G_dev,
+                                                             (float)c->g.alpha);
     c->launches++;
     VP_CUDA_TRY(c, cudaGetLastError());
     return VP_OK;
@@ -1005,9 +1211,13 @@ int vp_fine_flux(vp_ctx *c, int kick, int dim, double dt, const double *accel_de
 int vp_restrict_velocity(const float *f_fine, float *f_coarse, long long NX, int nf1, int nf2, int factor1,
                          int factor2, void *stream) {
     if (!f_fine || !f_coarse || factor1 < 1 || factor2 < 1 || nf1 % factor1 || nf2 % factor2) return VP_EINVAL;
-    const long long n = NX * (nf1 / factor1) * (nf2 / factor2);
+    const int nc1 = nf1 / factor1, nc2 = nf2 / factor2;
+    const long long n = NX * nc1 * nc2;
+    const int quad = factor2 == 4 && (reinterpret_cast<uintptr_t>(f_fine) & 15) == 0, ff = factor1 * factor2;
+    const double inv = (ff & (ff - 1)) == 0 ? 1.0 / ff : 0.0;  // exact
     k_restrict_v2<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        f_fine, f_coarse, NX, nf1, nf2, factor1, factor2);
+        f_fine, f_coarse, n, make_fastdiv((unsigned)(nc1 * nc2)), make_fastdiv((unsigned)nc2), nf2,
+        (long long)nf1 * nf2, factor1, factor2, quad, inv);
     return cudaGetLastError() == cudaSuccess ? VP_OK : VP_ECUDA;
 }
 
@@ -1024,8 +1234,9 @@ int vp_group_mean(const double *G_fine, long long n_coarse_lines, int nout, cons
                   int group, double scale, double *G_coarse, void *stream) {
     if (!G_fine || !map_dev || !G_coarse || group < 1 || nout < 1) return VP_EINVAL;
     const long long n = n_coarse_lines * nout;
+    const double inv = (group & (group - 1)) == 0 ? 1.0 / group : 0.0;  // exact
     k_group_mean<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        G_fine, n_coarse_lines, nout, map_dev, group, scale, G_coarse);
+        G_fine, n, nout, make_fastdiv((unsigned)nout), map_dev, group, scale, inv, G_coarse);
     return cudaGetLastError() == cudaSuccess ? VP_OK : VP_ECUDA;
 }
 
@@ -1089,10 +1300,27 @@ int vp_make_samples(vp_ctx *coarse, int kick, int dim, double dt, const double *
     if (!c || !c->f || !Gc_dev || !X_dev || !y_dev) return VP_EINVAL;
     if (dim < 0 || dim >= c->g.dx || (kick && !accel_dev)) return vp_fail(c, VP_EINVAL, "bad sample arguments");
     const LineGeo q = line_geo(c->g, c->NX, c->NV, kick, dim);
-    const long long n = q.outer * q.inner * (q.L + 1);
-    k_make_samples<<<(unsigned)((n + 127) / 128), 128, 0, c->stream>>>(
-        static_cast<const float *>(c->f), q.outer, q.L, q.inner, q.periodic, kick, q.from_inner, q.cdiv, q.cmod,
-        accel_dev, q.lo, q.dvel, dt, q.h, c->wp, Gc_dev, zmin, X_dev, y_dev, scale_dev, (float)c->g.alpha);
+    LineTile t = line_tile(q);
+    int rc;
+    if ((rc = vp_launch_shift_table_f32(c, kick, dim, dt, accel_dev))) return rc;
+    const LineShift<float> *tab = static_cast<const LineShift<float> *>(c->d_shift);
+    const size_t xbytes = (size_t)kSampleThreads * NF * sizeof(float);
+    auto bytes = [&](int W) { return xbytes + (size_t)3 * W * ((q.L + 2 * kEdge) | 1) * sizeof(float); };
+    int W = 32;
+    while (W > 1 && bytes(W) > 72 * 1024) W /= 2;  // three CTAs per SM
+    const bool staged = bytes(W) <= 200 * 1024;
+    set_width(t, staged ? W : 32);
+    const unsigned blocks = (unsigned)((t.lines + t.W - 1) / t.W);
+    const size_t smem = staged ? bytes(t.W) : xbytes;
+    VP_CUDA_TRY(c, cudaFuncSetAttribute(k_make_samples<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    if (staged)
+        k_make_samples<true><<<blocks, kSampleThreads, smem, c->stream>>>(
+            static_cast<const float *>(c->f), t, tab, kick, accel_dev, q.lo, q.dvel, dt, q.h, Gc_dev, zmin, X_dev,
+            y_dev, scale_dev, (float)c->g.alpha);
+    else
+        k_make_samples<false><<<blocks, kSampleThreads, smem, c->stream>>>(
+            static_cast<const float *>(c->f), t, tab, kick, accel_dev, q.lo, q.dvel, dt, q.h, Gc_dev, zmin, X_dev,
+            y_dev, scale_dev, (float)c->g.alpha);
     c->launches++;
     VP_CUDA_TRY(c, cudaGetLastError());
     return VP_OK;

@@ -196,6 +196,8 @@ inline SweepGeo vp_make_geo(const vp_ctx *c, int kick, int dim) {
 
 // launchers implemented in the kernel files; all enqueue on ctx->stream
 int vp_launch_shift_table(vp_ctx *c, int kick, int dim, double dt, const double *accel);
+// the same in FP32 whatever the grid's precision (the learned part's kernels)
+int vp_launch_shift_table_f32(vp_ctx *c, int kick, int dim, double dt, const double *accel);
 // the context stream is being captured into a graph (no synchronising calls)
 bool vp_capturing(const vp_ctx *c);
 // buffers and kernel attributes of the learned sweep (outside any stream capture)

@@ -464,8 +464,8 @@ template <typename T>
 __global__ void k_shift_table(LineShift<T> *__restrict__ tab, int nclass, int kick, double lo,
                               double dvel, const double *__restrict__ accel, double dt, double h,
                               const __grid_constant__ WPoly wp) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int c = t >> 3, k = t & 7;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = (int)(t >> 3), k = (int)t & 7;
     if (c >= nclass) return;
     const double speed = kick ? accel[c] : vp_core::cell_centre(lo, dvel, c);
     LineShift<T> sh;
@@ -1009,23 +1009,28 @@ int vp_sweep_setup(vp_ctx *c) {
     return VP_OK;
 }
 
-int vp_launch_shift_table(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+template <typename T>
+static int table_launch(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
     const vp_grid &g = c->g;
     const int nclass = kick ? (int)c->NX : g.nv[dim];
     const double h = kick ? (g.vhi[dim] - g.vlo[dim]) / g.nv[dim] : (g.xhi[dim] - g.xlo[dim]) / g.nx[dim];
-    const double lo = g.vlo[dim];
     const double dvel = (g.vhi[dim] - g.vlo[dim]) / g.nv[dim];
     const int th = 64;
-    const int bl = (8 * nclass + th - 1) / th;
-    if (g.precision == VP_F32)
-        k_shift_table<float><<<bl, th, 0, c->stream>>>(static_cast<LineShift<float> *>(c->d_shift),
-                                                       nclass, kick, lo, dvel, accel, dt, h, c->wp);
-    else
-        k_shift_table<double><<<bl, th, 0, c->stream>>>(static_cast<LineShift<double> *>(c->d_shift),
-                                                        nclass, kick, lo, dvel, accel, dt, h, c->wp);
+    const long long bl = (8LL * nclass + th - 1) / th;
+    k_shift_table<T><<<(unsigned)bl, th, 0, c->stream>>>(static_cast<LineShift<T> *>(c->d_shift), nclass, kick,
+                                                         g.vlo[dim], dvel, accel, dt, h, c->wp);
     c->launches++;
     VP_CUDA_TRY(c, cudaGetLastError());
     return VP_OK;
+}
+
+int vp_launch_shift_table(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+    return c->g.precision == VP_F32 ? table_launch<float>(c, kick, dim, dt, accel)
+                                    : table_launch<double>(c, kick, dim, dt, accel);
+}
+
+int vp_launch_shift_table_f32(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+    return table_launch<float>(c, kick, dim, dt, accel);
 }
 
 int vp_launch_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel) {

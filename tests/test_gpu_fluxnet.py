@@ -307,3 +307,131 @@ def test_learned_sweep_velocity_axis_limit():
             assert e.value.code == V.VP_ENOTSUP
             assert np.array_equal(from_gpu(sim), f0)
         sim.close()
+
+
+LINE_CASES = [
+    # dims, nx, nv, xbc, kick, dim, dt: strided and contiguous lines, lines shorter than the
+    # stencil, whole-cell shifts below and above the direct sum's limit, both boundaries
+    (1, [40], [12], 0, 0, 0, 0.3),
+    (1, [40], [70], 1, 0, 0, -3.1),
+    (1, [3], [20], 0, 0, 0, 5.0),
+    (1, [5], [7], 1, 0, 0, 2.9),
+    (1, [9], [64], 1, 1, 0, 0.7),
+    (1, [33], [40], 0, 1, 0, -4.0),
+    (2, [6, 10], [8, 12], 0, 0, 0, 0.4),
+    (2, [6, 10], [8, 12], 0, 0, 1, 1.3),
+    (2, [5, 4], [16, 9], 1, 1, 0, 0.6),
+    (2, [5, 4], [9, 16], 0, 1, 1, 0.8),
+]
+
+
+@pytest.mark.parametrize("dims,nx,nv,xbc,kick,dim,dt", LINE_CASES)
+def test_fluxes_and_samples_of_every_line_kind(dims, nx, nv, xbc, kick, dim, dt):
+    """Fine fluxes against the sweep they describe (f' = f + G_left - G_right;
+    two FP32 updates and the FP64 masses: 1e-6 of the cells of order one), and
+    samples made from them on the same grid: with Gc = G the target is the
+    difference of the limited and unlimited masses, zero (to FP32 rounding)
+    where the PP limiter cannot bind (nu <= 0.4 on cells within 10%); scale and
+    features against numpy's of the same cells."""
+    import torch
+    g = dict(dims=dims, nx=nx, nv=nv, xlo=[0.0] * dims, xhi=[2.0 + 0.3 * d for d in range(dims)],
+             vlo=[-3.0 - 0.5 * d for d in range(dims)], vhi=[2.5] * dims, order=7, xbc=xbc)
+    sim = V.Simulation(g, precision=V.VP_F32)
+    rng = np.random.default_rng(dims + nx[0])
+    f = (1.0 + 0.1 * rng.random(nx + nv)).astype(np.float32)
+    acc = rng.uniform(-4.0, 4.0, size=sim.NX)
+    axis = dims * kick + dim
+    L = f.shape[axis]
+    sim.upload(f.reshape(-1))
+    a = torch.as_tensor(acc, device="cuda") if kick else None
+    lines = f.size // L
+    G = torch.empty(lines * (L + 1), dtype=torch.float64, device="cuda")
+    V.vp_fine_flux(sim.ctx, kick, dim, dt, a, 1, G)
+    X = torch.empty(lines * (L + 1), 25, device="cuda")
+    y, sc = torch.empty(lines * (L + 1), device="cuda"), torch.empty(lines * (L + 1), device="cuda")
+    torch.cuda.synchronize()
+    V.vp_make_samples(sim.ctx, kick, dim, dt, a, G, 0.0, X, y, sc)
+    every = 2 if L % 2 == 0 else L
+    Ge = torch.empty(lines * (L // every + 1), dtype=torch.float64, device="cuda")
+    V.vp_fine_flux(sim.ctx, kick, dim, dt, a, every, Ge)
+    if kick:
+        V.vp_kick_sweep(sim.ctx, dim, dt, a)
+    else:
+        V.vp_drift_sweep(sim.ctx, dim, dt)
+    sim.sync()
+    out = np.moveaxis(sim.f.cpu().numpy().reshape(f.shape), axis, -1).reshape(lines, L).astype(np.float64)
+    fl = np.moveaxis(f, axis, -1).reshape(lines, L).astype(np.float64)
+    G = G.cpu().numpy().reshape(lines, L + 1)
+    assert np.abs(fl + G[:, :-1] - G[:, 1:] - out).max() <= 1e-6
+    assert np.array_equal(Ge.cpu().numpy().reshape(lines, -1), G[:, ::every])
+    X, y, sc = X.cpu().numpy().reshape(lines, L + 1, 25), y.cpu().numpy().reshape(lines, -1), sc.cpu().numpy().reshape(lines, -1)
+    end = not kick and xbc == 0  # the duplicate interface of a periodic line
+    if end:
+        assert np.isnan(y[:, L]).all() and (X[:, L] == 0).all() and (sc[:, L] == 0).all()
+    X, y, sc = X[:, :L], y[:, :L], sc[:, :L]
+    ok = X[:, :, 24] <= 0.4
+    assert ok.any() and np.abs(y[ok]).max() <= 2e-6
+    # speeds, shifts and stencils of every line
+    if kick:
+        speed = np.repeat(acc, lines // sim.NX)
+        h = (g["vhi"][dim] - g["vlo"][dim]) / nv[dim]
+    else:
+        vc = g["vlo"][dim] + (np.arange(nv[dim]) + 0.5) * (g["vhi"][dim] - g["vlo"][dim]) / nv[dim]
+        shape = [1] * (2 * dims)
+        shape[dims + dim] = nv[dim]
+        speed = np.moveaxis(np.broadcast_to(vc.reshape(shape), f.shape), axis, -1).reshape(lines, L)[:, 0]
+        h = (g["xhi"][dim] - g["xlo"][dim]) / nx[dim]
+    s = speed * dt / h
+    n = np.sign(s) * np.floor(np.abs(s) + 0.5)
+    sg = np.where(s - n < 0, -1, 1)
+    wrap = not kick and xbc == 0
+
+    def stencil(lines_f):
+        i = np.arange(L)[None, :, None]
+        up = np.where(sg[:, None, None] > 0, i - 1 - n[:, None, None], i - n[:, None, None]).astype(int)
+        r = up + sg[:, None, None] * np.arange(-3, 5)[None, None, :]
+        v = np.take_along_axis(lines_f[:, None, :].repeat(L, 1), np.mod(r, L), axis=2)
+        return v if wrap else np.where((r >= 0) & (r < L), v, 0.0)
+    u = stencil(fl)
+    scale = np.abs(u).max(-1) + 1e-30
+    assert np.allclose(sc, scale, rtol=1e-6)
+    want = np.zeros((lines, L, 25))
+    want[:, :, :8] = (u - u[:, :, 3:4]) / scale[:, :, None]
+    if not kick:
+        z = np.zeros_like(np.take(f, [0], axis=dims + dim))
+        hi = np.concatenate([np.take(f, range(1, nv[dim]), axis=dims + dim), z], axis=dims + dim)
+        lo = np.concatenate([z, np.take(f, range(nv[dim] - 1), axis=dims + dim)], axis=dims + dim)
+        hi, lo = (np.moveaxis(t, axis, -1).reshape(lines, L).astype(np.float64) for t in (hi, lo))
+        pos = speed[:, None] >= 0
+        p, m = stencil(np.where(pos, hi, lo)), stencil(np.where(pos, lo, hi))
+        want[:, :, 8:16] = (p - m) / (2 * scale[:, :, None])
+        want[:, :, 16:24] = (0.5 * (p + m) - u) / scale[:, :, None]
+    else:
+        want[:, :, 16:24] = -u / scale[:, :, None]
+    want[:, :, 24] = np.abs(s - n)[:, None]
+    assert np.abs(X - want).max() <= 2e-6
+    sim.close()
+
+
+@pytest.mark.parametrize("nf,factors", [((8, 12), (4, 4)), ((6, 15), (3, 5)), ((32, 1), (4, 1)), ((4, 6), (2, 3))])
+def test_restriction_and_group_means(nf, factors):
+    """Coarse cells and coarse masses against numpy's means: one FP32 rounding
+    of an exact mean, and FP64 sums of a few terms."""
+    import torch
+    rng = np.random.default_rng(nf[0])
+    NX, (a, b) = 7, factors
+    f = (rng.random((NX, *nf)) * 10.0 ** rng.uniform(-40, 20, size=(NX, *nf))).astype(np.float32)
+    ft = torch.as_tensor(f.reshape(-1), device="cuda")
+    out = torch.empty(NX * nf[0] // a * (nf[1] // b), device="cuda")
+    V.vp_restrict_velocity(ft, out, NX, nf[0], nf[1], a, b)
+    want = f.astype(np.float64).reshape(NX, nf[0] // a, a, nf[1] // b, b).mean((2, 4)).reshape(-1)
+    torch.cuda.synchronize()
+    assert np.allclose(out.cpu().numpy(), want, rtol=2.0 ** -23, atol=1e-44)
+    n, nout, grp = 23, 11, a * b
+    Gf = rng.standard_normal((40, nout))
+    m = rng.integers(0, 40, size=(n, grp))
+    Gc = torch.empty(n * nout, dtype=torch.float64, device="cuda")
+    V.vp_group_mean(torch.as_tensor(Gf.reshape(-1), device="cuda"), n, nout,
+                    torch.as_tensor(m.reshape(-1), dtype=torch.int64, device="cuda"), grp, 0.25, Gc)
+    torch.cuda.synchronize()
+    assert np.abs(Gc.cpu().numpy().reshape(n, nout) - 0.25 * Gf[m].mean(1)).max() <= 1e-15 * grp
