@@ -75,6 +75,7 @@ struct SweepTune {
     int impl;   // 1: staged loads (k_sweep_cols / k_sweep_rows), 2: TMA pipeline,
                 // 3: staged loads with two lines per thread (FP32 strided sweeps)
     int W, nseg, ctas_per_sm;
+    int flat;   // the walkers vote on flat stencils (1) or leave the vote out (0)
 };
 
 // tile of the unsplit step (T1 x1 rows x T2 x2 cells x TV velocity cells,

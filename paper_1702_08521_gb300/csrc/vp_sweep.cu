@@ -56,7 +56,7 @@ struct PtrStore {
 #define VP_PAIR_THREADS 512
 #define VP_PAIR_MINB 1
 
-template <typename T, int ORDER, bool PERIODIC, bool FULL, bool PAIR>
+template <typename T, int ORDER, bool PERIODIC, bool FULL, bool PAIR, bool FLAT>
 __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_MINB : 1)
     k_sweep_cols(T *__restrict__ f, const __grid_constant__ ShiftSrc<T> src, SweepGeo geo, LimParams lp) {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -134,18 +134,18 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
                 const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
                 PtrStore<vp_core::P2> st{reinterpret_cast<vp_core::P2 *>(base + cc + (long long)i0 * geo.inner),
                                          (long long)sh.sigma * (geo.inner >> 1)};
-                walk<vp_core::P2, ORDER, PERIODIC, FULL, G1>(reinterpret_cast<const vp_core::P2 *>(data + cc),
+                walk<vp_core::P2, ORDER, PERIODIC, FULL, G1, false, FLAT>(reinterpret_cast<const vp_core::P2 *>(data + cc),
                                                              W >> 1, L, sh, r0, r1, vp_core::P2((float)lp.alpha),
                                                              lp.mp, lp.pp, st);
                 return;
             }
             const int i1 = sb.sigma > 0 ? r0 : r1 - 1;
             PtrStore<T> st{base + cc + 1 + (long long)i1 * geo.inner, (long long)sb.sigma * geo.inner};
-            walk<T, ORDER, PERIODIC, FULL, G1>(data + cc + 1, W, L, sb, r0, r1, (T)lp.alpha, lp.mp, lp.pp, st);
+            walk<T, ORDER, PERIODIC, FULL, G1, false, FLAT>(data + cc + 1, W, L, sb, r0, r1, (T)lp.alpha, lp.mp, lp.pp, st);
         }
         const int i0 = sa.sigma > 0 ? r0 : r1 - 1;
         PtrStore<T> st{base + cc + (long long)i0 * geo.inner, (long long)sa.sigma * geo.inner};
-        walk<T, ORDER, PERIODIC, FULL, G1>(data + cc, W, L, sa, r0, r1, (T)lp.alpha, lp.mp, lp.pp, st);
+        walk<T, ORDER, PERIODIC, FULL, G1, false, FLAT>(data + cc, W, L, sa, r0, r1, (T)lp.alpha, lp.mp, lp.pp, st);
     } else {
         const unsigned seg = fdiv(threadIdx.x, geo.fd_w);
         const int cc = (int)(threadIdx.x - seg * (unsigned)W);
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
             const int r0 = (int)fdiv(seg * (unsigned)L, geo.fd_nseg);
             const int r1 = (int)fdiv((seg + 1) * (unsigned)L, geo.fd_nseg);
             const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
-            vp_core::walk_line<T, ORDER, PERIODIC, FULL, G1>(
+            vp_core::walk_line<T, ORDER, PERIODIC, FULL, G1, FLAT>(
                 data + cc, W, L, sh, r0, r1, (T)lp.alpha, lp.mp, lp.pp, [&](auto t) {
                     using U = decltype(t);
                     return PtrStore<U>{reinterpret_cast<U *>(base + cc + (long long)i0 * geo.inner),
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
 // direction, and the odd last line of a ragged tile, are walked one line at
 // a time (element stride 2).  The 16-lane phases of 8-byte accesses stay
 // conflict-free because P is odd.
-template <typename T, int ORDER, bool PERIODIC, bool FULL, bool PAIR>
+template <typename T, int ORDER, bool PERIODIC, bool FULL, bool PAIR, bool FLAT>
 __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_MINB : 1)
     k_sweep_rows(T *__restrict__ f, const __grid_constant__ ShiftSrc<T> src, SweepGeo geo, LimParams lp) {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -286,21 +286,21 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
                     const vp_core::LineShiftP2 sh = vp_core::pair_shift(sa, sb);
                     const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
                     PtrStore<vp_core::P2> st{reinterpret_cast<vp_core::P2 *>(out + oidx(line, i0)), sh.sigma};
-                    walk<vp_core::P2, ORDER, PERIODIC, FULL, G1>(
+                    walk<vp_core::P2, ORDER, PERIODIC, FULL, G1, false, FLAT>(
                         reinterpret_cast<const vp_core::P2 *>(in + iidx(line, 0)), 1, L, sh, r0, r1,
                         vp_core::P2((float)lp.alpha), lp.mp, lp.pp, st);
                     paired = true;
                 } else {
                     const int i1 = sb.sigma > 0 ? r0 : r1 - 1;
                     PtrStore<T> st{out + oidx(line + 1, i1), 2LL * sb.sigma};
-                    walk<T, ORDER, PERIODIC, FULL, G1>(in + iidx(line + 1, 0), 2, L, sb, r0, r1, (T)lp.alpha,
+                    walk<T, ORDER, PERIODIC, FULL, G1, false, FLAT>(in + iidx(line + 1, 0), 2, L, sb, r0, r1, (T)lp.alpha,
                                                        lp.mp, lp.pp, st);
                 }
             }
             if (!paired) {
                 const int i0 = sa.sigma > 0 ? r0 : r1 - 1;
                 PtrStore<T> st{out + oidx(line, i0), 2LL * sa.sigma};
-                walk<T, ORDER, PERIODIC, FULL, G1>(in + iidx(line, 0), 2, L, sa, r0, r1, (T)lp.alpha, lp.mp,
+                walk<T, ORDER, PERIODIC, FULL, G1, false, FLAT>(in + iidx(line, 0), 2, L, sa, r0, r1, (T)lp.alpha, lp.mp,
                                                    lp.pp, st);
             }
         }
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
             const int r0 = (int)fdiv(seg * (unsigned)L, geo.fd_nseg);
             const int r1 = (int)fdiv((seg + 1) * (unsigned)L, geo.fd_nseg);
             const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
-            vp_core::walk_line<T, ORDER, PERIODIC, FULL, G1>(
+            vp_core::walk_line<T, ORDER, PERIODIC, FULL, G1, FLAT>(
                 in + line * P + GP, 1, L, sh, r0, r1, (T)lp.alpha, lp.mp, lp.pp, [&](auto t) {
                     using U = decltype(t);
                     return PtrStore<U>{reinterpret_cast<U *>(out + line * Q + i0), (long long)sh.sigma};
@@ -482,18 +482,24 @@ __global__ void k_shift_table(LineShift<T> *__restrict__ tab, int nclass, int ki
 // a staged tile of at most 200 KB and up to 128 shifts behind it
 constexpr int kSweepSmem = 216 * 1024;
 
+template <typename T, int ORDER, bool PER, bool FULL, bool FLAT>
+void set_attrs_flat() {
+    cudaFuncSetAttribute(k_sweep_cols<T, ORDER, PER, FULL, false, FLAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         kSweepSmem);
+    cudaFuncSetAttribute(k_sweep_rows<T, ORDER, PER, FULL, false, FLAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         kSweepSmem);
+    if constexpr (sizeof(T) == 4) {
+        cudaFuncSetAttribute(k_sweep_cols<T, ORDER, PER, FULL, true, FLAT>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
+        cudaFuncSetAttribute(k_sweep_rows<T, ORDER, PER, FULL, true, FLAT>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
+    }
+}
+
 template <typename T, int ORDER, bool PER, bool FULL>
 void set_attrs_one() {
-    cudaFuncSetAttribute(k_sweep_cols<T, ORDER, PER, FULL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         kSweepSmem);
-    if constexpr (sizeof(T) == 4)
-        cudaFuncSetAttribute(k_sweep_cols<T, ORDER, PER, FULL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kSweepSmem);
-    cudaFuncSetAttribute(k_sweep_rows<T, ORDER, PER, FULL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         kSweepSmem);
-    if constexpr (sizeof(T) == 4)
-        cudaFuncSetAttribute(k_sweep_rows<T, ORDER, PER, FULL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kSweepSmem);
+    set_attrs_flat<T, ORDER, PER, FULL, true>();
+    if constexpr (FULL) set_attrs_flat<T, ORDER, PER, FULL, false>();
     cudaFuncSetAttribute(k_sweep_cols_tma<T, ORDER, PER, FULL>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
@@ -652,6 +658,7 @@ int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
     const int order = c->g.order;
     const bool per = geo.periodic != 0;
     const bool full = c->g.mp && c->g.pp;
+    const bool flat = tu.flat;
     const bool tma = tu.impl == 2 && tma_eligible<T>(c, geo, W);
     const size_t tile = (size_t)(L + 2 * ghost_rows(geo)) * W * sizeof(T);
     if (!tma && tile > 200 * 1024) return vp_fail(c, VP_ENOTSUP, "line of %d cells too long to stage", L);
@@ -691,13 +698,19 @@ int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
     } else if (pair) {
         const int pthreads = threads;
         geo.fd_w2 = make_fastdiv((unsigned)(W >> 1));
-#define VP_LAUNCH(O, P, F) \
-    k_sweep_cols<T, O, P, F, sizeof(T) == 4><<<(unsigned)tiles, pthreads, smem, c->stream>>>(f, src, geo, lp)
+#define VP_LAUNCH(O, P, F)                                                                                     \
+    if (flat)                                                                                                  \
+        k_sweep_cols<T, O, P, F, sizeof(T) == 4, true><<<(unsigned)tiles, pthreads, smem, c->stream>>>(f, src, geo, lp); \
+    else                                                                                                       \
+        k_sweep_cols<T, O, P, F, sizeof(T) == 4, !F><<<(unsigned)tiles, pthreads, smem, c->stream>>>(f, src, geo, lp)
         VP_DISPATCH(order, per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     } else {
-#define VP_LAUNCH(O, P, F) \
-    k_sweep_cols<T, O, P, F, false><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp)
+#define VP_LAUNCH(O, P, F)                                                                                   \
+    if (flat)                                                                                                \
+        k_sweep_cols<T, O, P, F, false, true><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp); \
+    else                                                                                                     \
+        k_sweep_cols<T, O, P, F, false, !F><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp)
         VP_DISPATCH(order, per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     }
@@ -741,16 +754,23 @@ int launch_rows(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
     const int threads = ((per_row * nseg + 31) / 32) * 32;
     const bool per = geo.periodic != 0;
     const bool full = c->g.mp && c->g.pp;
+    const bool flat = tu.flat;
     if (pair) {
         geo.fd_w2 = make_fastdiv((unsigned)(R >> 1));
         const int pthreads = threads;
-#define VP_LAUNCH(O, P, F) \
-    k_sweep_rows<T, O, P, F, sizeof(T) == 4><<<(unsigned)blocks, pthreads, smem, c->stream>>>(f, src, geo, lp)
+#define VP_LAUNCH(O, P, F)                                                                                     \
+    if (flat)                                                                                                  \
+        k_sweep_rows<T, O, P, F, sizeof(T) == 4, true><<<(unsigned)blocks, pthreads, smem, c->stream>>>(f, src, geo, lp); \
+    else                                                                                                       \
+        k_sweep_rows<T, O, P, F, sizeof(T) == 4, !F><<<(unsigned)blocks, pthreads, smem, c->stream>>>(f, src, geo, lp)
         VP_DISPATCH(c->g.order, per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     } else {
-#define VP_LAUNCH(O, P, F) \
-    k_sweep_rows<T, O, P, F, false><<<(unsigned)blocks, threads, smem, c->stream>>>(f, src, geo, lp)
+#define VP_LAUNCH(O, P, F)                                                                                     \
+    if (flat)                                                                                                  \
+        k_sweep_rows<T, O, P, F, false, true><<<(unsigned)blocks, threads, smem, c->stream>>>(f, src, geo, lp); \
+    else                                                                                                       \
+        k_sweep_rows<T, O, P, F, false, !F><<<(unsigned)blocks, threads, smem, c->stream>>>(f, src, geo, lp)
         VP_DISPATCH(c->g.order, per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     }
@@ -764,6 +784,7 @@ template <typename T>
 SweepTune default_tune(const vp_ctx *c, const SweepGeo &geo) {
     SweepTune tu{};
     tu.valid = 1;
+    tu.flat = 1;
     const int L = geo.L;
     if (geo.inner > 1) {
         int W = (int)(32768 / sizeof(T) / L);  // ~32 KB staged tile
@@ -905,7 +926,7 @@ int tune_on(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, const SweepGeo
     // 60 us).  A segment of l cells computes l + 1 interfaces, hence l >= 4.
     const bool small = geo.outer * geo.inner < 64LL * c->sm_count;
     auto add = [&](int impl, int W, int nseg) {
-        if (nc < kMaxCand) cand[nc++] = SweepTune{1, impl, W, nseg, 0};
+        if (nc < kMaxCand) cand[nc++] = SweepTune{1, impl, W, nseg, 0, 1};
     };
     if (geo.inner > 1) {
         const int impls[3] = {3, 2, 1};
@@ -964,11 +985,22 @@ int tune_on(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, const SweepGeo
     VP_CUDA_TRY(c, cudaEventCreate(&e0));
     VP_CUDA_TRY(c, cudaEventCreate(&e1));
     float best_ms = 1e30f;
-    for (int i = 0; i < nc; ++i) {
+    // Every candidate, then the fastest without the walkers' vote on flat
+    // stencils (the same results; the vote pays where f has flat, e.g. empty,
+    // regions and costs 7% where it has none: 2D2V Landau drifts 138 -> 128 us).
+    // What is timed is today's state, and the limiters' work grows as a run fills
+    // its empty space: the TMA pipeline, which walks one line per thread, and the
+    // kernels without the vote have to win by 5% and 2%.
+    for (int i = 0; i <= nc; ++i) {
+        SweepTune t = i < nc ? cand[i] : best;
+        if (i == nc) {
+            if (t.impl == 2 || !(c->g.mp && c->g.pp)) break;
+            t.flat = 0;
+        }
         float ms = 1e30f;
         for (int rep = 0; rep < 2; ++rep) {
             cudaEventRecord(e0, c->stream);
-            rc = geo.inner > 1 ? launch_cols<T>(c, sub, cand[i], sw) : launch_rows<T>(c, sub, cand[i], sw);
+            rc = geo.inner > 1 ? launch_cols<T>(c, sub, t, sw) : launch_rows<T>(c, sub, t, sw);
             cudaEventRecord(e1, c->stream);
             if (rc) break;
             const cudaError_t se = cudaEventSynchronize(e1);
@@ -985,9 +1017,10 @@ int tune_on(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, const SweepGeo
             cudaEventDestroy(e1);
             return rc;
         }
+        ms *= t.impl == 2 ? 1.05f : (t.flat ? 1.f : 1.02f);
         if (ms < best_ms) {
             best_ms = ms;
-            best = cand[i];
+            best = t;
         }
     }
     cudaEventDestroy(e0);
@@ -1000,46 +1033,69 @@ int tune_on(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, const SweepGeo
 
 }  // namespace
 
-int vp_sweep_setup(vp_ctx *c) {
-    set_attrs<float, 5>();
-    set_attrs<float, 7>();
-    set_attrs<double, 5>();
-    set_attrs<double, 7>();
-    VP_CUDA_TRY(c, cudaGetLastError());
-    return VP_OK;
+// The entry points of one precision; the FP64 ones compile in a unit of their
+// own (vp_sweep_f64.cu), which halves the build.
+#ifdef VP_SWEEP_UNIT_F64
+typedef double unit_t;
+#define VP_UNIT(name) name##_f64
+#else
+typedef float unit_t;
+#define VP_UNIT(name) name##_f32
+#endif
+
+void VP_UNIT(vp_sweep_attrs)() {
+    set_attrs<unit_t, 5>();
+    set_attrs<unit_t, 7>();
 }
 
-template <typename T>
-static int table_launch(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+int VP_UNIT(vp_launch_shift_table)(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
     const vp_grid &g = c->g;
     const int nclass = kick ? (int)c->NX : g.nv[dim];
     const double h = kick ? (g.vhi[dim] - g.vlo[dim]) / g.nv[dim] : (g.xhi[dim] - g.xlo[dim]) / g.nx[dim];
     const double dvel = (g.vhi[dim] - g.vlo[dim]) / g.nv[dim];
     const int th = 64;
     const long long bl = (8LL * nclass + th - 1) / th;
-    k_shift_table<T><<<(unsigned)bl, th, 0, c->stream>>>(static_cast<LineShift<T> *>(c->d_shift), nclass, kick,
-                                                         g.vlo[dim], dvel, accel, dt, h, c->wp);
+    k_shift_table<unit_t><<<(unsigned)bl, th, 0, c->stream>>>(static_cast<LineShift<unit_t> *>(c->d_shift), nclass,
+                                                              kick, g.vlo[dim], dvel, accel, dt, h, c->wp);
     c->launches++;
     VP_CUDA_TRY(c, cudaGetLastError());
     return VP_OK;
 }
 
-int vp_launch_shift_table(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
-    return c->g.precision == VP_F32 ? table_launch<float>(c, kick, dim, dt, accel)
-                                    : table_launch<double>(c, kick, dim, dt, accel);
+int VP_UNIT(vp_launch_sweep)(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+    return launch_sweep_t<unit_t>(c, kick, dim, dt, accel);
 }
 
-int vp_launch_shift_table_f32(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
-    return table_launch<float>(c, kick, dim, dt, accel);
+int VP_UNIT(vp_tune_sweep)(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+    return tune_t<unit_t>(c, kick, dim, dt, accel);
+}
+
+#ifndef VP_SWEEP_UNIT_F64
+void vp_sweep_attrs_f64();
+int vp_launch_shift_table_f64(vp_ctx *c, int kick, int dim, double dt, const double *accel);
+int vp_launch_sweep_f64(vp_ctx *c, int kick, int dim, double dt, const double *accel);
+int vp_tune_sweep_f64(vp_ctx *c, int kick, int dim, double dt, const double *accel);
+
+int vp_sweep_setup(vp_ctx *c) {
+    vp_sweep_attrs_f32();
+    vp_sweep_attrs_f64();
+    VP_CUDA_TRY(c, cudaGetLastError());
+    return VP_OK;
+}
+
+int vp_launch_shift_table(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+    return c->g.precision == VP_F32 ? vp_launch_shift_table_f32(c, kick, dim, dt, accel)
+                                    : vp_launch_shift_table_f64(c, kick, dim, dt, accel);
 }
 
 int vp_launch_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
-    if (c->g.precision == VP_F32) return launch_sweep_t<float>(c, kick, dim, dt, accel);
-    return launch_sweep_t<double>(c, kick, dim, dt, accel);
+    return c->g.precision == VP_F32 ? vp_launch_sweep_f32(c, kick, dim, dt, accel)
+                                    : vp_launch_sweep_f64(c, kick, dim, dt, accel);
 }
 
 int vp_tune_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
     if (c->tune[kick][dim].valid) return VP_OK;
-    if (c->g.precision == VP_F32) return tune_t<float>(c, kick, dim, dt, accel);
-    return tune_t<double>(c, kick, dim, dt, accel);
+    return c->g.precision == VP_F32 ? vp_tune_sweep_f32(c, kick, dim, dt, accel)
+                                    : vp_tune_sweep_f64(c, kick, dim, dt, accel);
 }
+#endif

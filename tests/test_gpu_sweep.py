@@ -305,3 +305,40 @@ def test_fp64_integer_comparisons_give_the_plain_result(order, xbc, n, nv):
         ref = ref.reshape(n, nv, 16)[:, :, 0].reshape(-1)
         got, _ = run(g1, 1, f0, 1)
         assert np.array_equal(got, ref, equal_nan=True)
+
+
+@pytest.mark.parametrize("precision", [V.VP_F32, V.VP_F64])
+@pytest.mark.parametrize("dims,nx,nv", [(2, [12, 10], [40, 36]), (1, [200], [150])])
+def test_flat_votes_of_blocks_give_the_same_bits(precision, dims, nx, nv):
+    """The walkers vote once per block of steps on flat stencils, and tuned
+    contexts may leave the vote out: data with empty regions, plateaus of every
+    length down to one cell and steps between them give the same bits with the
+    default kernels and with tuned ones, for every sweep (tuned on smooth data
+    first, where leaving the vote out wins, then run on the plateaus)."""
+    rng = np.random.default_rng(9)
+    n = int(np.prod(nx)) * int(np.prod(nv))
+    runs = np.repeat(rng.random(n), rng.integers(1, 30, size=n))[:n]
+    runs[rng.random(n) < 0.02] = 0.0
+    f0 = (runs * (rng.random(n) < 0.97) * np.repeat(rng.random(n // 50 + 1) < 0.6, 50)[:n]).astype(np.float32)
+    f0 = f0.reshape(list(nx) + list(nv))
+    smooth = np.ones(f0.shape)
+    for k, m in enumerate(f0.shape):
+        smooth = smooth * (1.5 + np.cos(2 * np.pi * (np.arange(m) + 0.5) / m)).reshape([-1 if j == k else 1 for j in range(f0.ndim)])
+    g = grid(dims, nx, nv, order=7)
+    acc = inputs.random_accel(int(np.prod(nx)), dims, seed=3, amax=3.0)
+    for axis in range(2 * dims):
+        kick, d = axis // dims, axis % dims
+        f = np.ascontiguousarray(np.moveaxis(np.sort(np.moveaxis(f0, axis, -1), axis=-1)[..., ::-1], -1, axis)) if d else f0
+        out = []
+        for tune in (0, 1):
+            sim, _ = both(g, precision)
+            V.vp_set_option(sim.ctx, V.VP_OPT_AUTOTUNE, tune)
+            for data in (smooth, f):
+                to_gpu(sim, data)
+                if kick:
+                    V.vp_kick_sweep(sim.ctx, d, 0.21, accel_tensor(sim, acc[d]))
+                else:
+                    V.vp_drift_sweep(sim.ctx, d, 0.047)
+            out.append(from_gpu(sim))
+            sim.close()
+        assert np.array_equal(out[0], out[1]), (kick, d)
