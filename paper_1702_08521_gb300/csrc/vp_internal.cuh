@@ -59,9 +59,11 @@ struct SweepGeo {
     long long cdiv, cmod;
     // column-kernel tile (W columns x full line), row-kernel lines per CTA
     int W, nseg, R;
+    int kblk;  // column kernel: whole outer blocks per tile (W = kblk inner), or 1
+    int vec;   // column kernel: elements per staged piece
     // divisors of the launch: cdiv, cmod, tiles per outer index, W (or R),
     // nseg, L, 16-byte pieces per tile row
-    FastDiv fd_cdiv, fd_cmod, fd_tpo, fd_w, fd_nseg, fd_l, fd_wv, fd_w2;
+    FastDiv fd_cdiv, fd_cmod, fd_tpo, fd_w, fd_nseg, fd_l, fd_wv, fd_w2, fd_inner;
     unsigned tpo;
 };
 

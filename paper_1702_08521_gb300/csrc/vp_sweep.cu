@@ -27,7 +27,20 @@
 #include "vp_sweep_core.cuh"
 #include "vp_tma.cuh"
 
+// A translation unit holds the sweeps of one precision and order (the four
+// compile in parallel): this file itself FP32 of order 7 and the dispatch, the
+// files vp_sweep_*.cu that include it the others.
+#ifndef VP_SWEEP_ORDER
+#define VP_SWEEP_MAIN
+#define VP_SWEEP_ORDER 7
+#define VP_SWEEP_REAL float
+#define VP_UNIT(name) name##_f32_o7
+#endif
+typedef VP_SWEEP_REAL unit_t;
+
 namespace {
+
+constexpr int kOrder = VP_SWEEP_ORDER;
 
 using vp_core::line_class;
 using vp_core::ShiftSrc;
@@ -56,111 +69,143 @@ struct PtrStore {
 #define VP_PAIR_THREADS 512
 #define VP_PAIR_MINB 1
 
-template <typename T, int ORDER, bool PERIODIC, bool FULL, bool PAIR, bool FLAT>
+// GEN: any tile -- ragged last tiles, rows that are no multiple of 16 bytes,
+// several narrow outer blocks side by side.  Not GEN: whole tiles of one block in
+// 16-byte rows, a thread's rows at one column (the general tile's address
+// arithmetic costs 3-6% there: Plummer 16^3 x 64^3 drift x1 1.86 against 1.97 ms).
+template <typename T, int ORDER, bool PERIODIC, bool FULL, bool PAIR, bool FLAT, bool GEN>
 __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_MINB : 1)
     k_sweep_cols(T *__restrict__ f, const __grid_constant__ ShiftSrc<T> src, SweepGeo geo, LimParams lp) {
     extern __shared__ __align__(16) unsigned char smraw[];
     constexpr int GP = PERIODIC ? 0 : VP_GHOST;
     T *sm = reinterpret_cast<T *>(smraw);
     const int W = geo.W, L = geo.L;
-    const unsigned o = fdiv(blockIdx.x, geo.fd_tpo);
-    const unsigned c0 = (blockIdx.x - o * geo.tpo) * (unsigned)W;
-    const int wc = (int)((geo.inner - c0) < W ? (geo.inner - c0) : W);
-    T *base = f + (long long)o * L * geo.inner + c0;
+    // W columns of one outer block, or (kblk > 1) kblk whole blocks side by side
+    const bool packed = GEN && geo.kblk > 1;
+    const unsigned o = packed ? blockIdx.x * (unsigned)geo.kblk : fdiv(blockIdx.x, geo.fd_tpo);
+    const unsigned c0 = packed ? 0u : (blockIdx.x - o * geo.tpo) * (unsigned)W;
+    const int nblk = packed ? (int)(geo.outer - o < geo.kblk ? geo.outer - o : geo.kblk) : 1;
+    const int wc = !GEN ? W : (packed ? nblk * (int)geo.inner : (int)((geo.inner - c0) < W ? (geo.inner - c0) : W));
+    T *const base0 = f + (long long)o * L * geo.inner + c0;
+    // first cell of column cc, its outer block and inner index
+    auto column = [&](int cc, unsigned &ob, unsigned &c) -> T * {
+        const unsigned k = packed ? fdiv((unsigned)cc, geo.fd_inner) : 0u;
+        ob = o + k;
+        c = packed ? cc - k * (unsigned)geo.inner : c0 + cc;
+        return packed ? base0 + (long long)k * L * geo.inner + c : base0 + cc;
+    };
     T *data = sm + GP * W;  // row 0 of the line
-    // the tile's shifts: its columns' classes (drift), or its one spatial point (kick)
+    // the tile's shifts: its columns' classes (drift), or its spatial points (kick)
     unsigned q0 = 0;
     int ncl = 1;
     LineShift<T> *shifts = nullptr;
     if (!src.tab) {
         shifts = reinterpret_cast<LineShift<T> *>(smraw + (((size_t)(L + 2 * GP) * W * sizeof(T) + 15) & ~size_t(15)));
         q0 = geo.cls_from_inner ? fdiv(c0, geo.fd_cdiv) : fdiv(o, geo.fd_cdiv);
-        if (geo.cls_from_inner) ncl = (int)(fdiv(c0 + wc - 1, geo.fd_cdiv) - q0) + 1;
+        const unsigned q1 = geo.cls_from_inner ? fdiv(packed ? (unsigned)geo.inner - 1 : c0 + wc - 1, geo.fd_cdiv)
+                                               : fdiv(o + nblk - 1, geo.fd_cdiv);
+        ncl = (int)(q1 - q0) + 1;
         vp_core::tile_shifts(shifts, q0, ncl, src, geo);
     }
-    auto shift_of = [&](unsigned c) -> LineShift<T> {
-        if (src.tab) return src.tab[line_class(geo, o, c)];
-        return shifts[geo.cls_from_inner ? fdiv(c, geo.fd_cdiv) - q0 : 0u];
-    };
+    // Every piece of the tile in flight at once (cp.async), so the staging is not
+    // limited by one outstanding load per thread: pieces of 16, 8 or 4 bytes, the
+    // widest that the row stride and the tile width are multiples of.  A 22 x 20 x
+    // 23 x 31 x 33 x 30 grid (rows of 8-byte pieces) staged by single loads took
+    // 1.12-1.18 ms per sweep against 0.37 ms of HBM.
+    if constexpr (!GEN) {
+        constexpr int VEC = 16 / sizeof(T);
+        const int wv = W / VEC;
+        const int r = (int)fdiv(threadIdx.x, geo.fd_wv);
+        const int cv = threadIdx.x - r * wv;
+        const int rstep = (int)fdiv(blockDim.x, geo.fd_wv);
+        const T *from = base0 + (long long)r * geo.inner + cv * VEC;
+        T *dst = data + r * W + cv * VEC;
+        const long long sstep = (long long)rstep * geo.inner;
+        for (int rr = r; rr < L; rr += rstep) {
+            vp_tma::cp_async16(dst, from);
+            from += sstep;
+            dst += rstep * W;
+        }
+    } else {
+        const int wv = W / geo.vec;
+        const int r = (int)fdiv(threadIdx.x, geo.fd_wv);
+        const int cv = (threadIdx.x - r * wv) * geo.vec;
+        const int rstep = (int)fdiv(blockDim.x, geo.fd_wv);
+        if (r < rstep && cv < wc) {
+            unsigned ob, c;
+            const T *from = column(cv, ob, c) + (long long)r * geo.inner;
+            T *dst = data + r * W + cv;
+            const long long sstep = (long long)rstep * geo.inner;
+            auto copy = [&](auto bytes) {
+                for (int rr = r; rr < L; rr += rstep) {
+                    vp_tma::cp_async<decltype(bytes)::value>(dst, from);
+                    from += sstep;
+                    dst += rstep * W;
+                }
+            };
+            const int bytes = geo.vec * (int)sizeof(T);
+            if (bytes == 16) copy(std::integral_constant<int, 16>());
+            else if (bytes == 8) copy(std::integral_constant<int, 8>());
+            else copy(std::integral_constant<int, 4>());
+        }
+    }
+    // while the copies are under way: the zero rows, and the thread's column,
+    // segment and shift
     for (int e = threadIdx.x; e < GP * W; e += blockDim.x) {
         sm[e] = T(0);
         data[L * W + e] = T(0);
     }
-    constexpr int VEC = 16 / sizeof(T);
-    const int wv = W / VEC;
-    if (wc == W && geo.inner % VEC == 0 && W % VEC == 0 && fmod_u(blockDim.x, geo.fd_wv) == 0) {
-        // every 16-byte piece of the tile in flight at once (cp.async), so the
-        // staging is not limited by one outstanding load per thread
-        const int r = (int)fdiv(threadIdx.x, geo.fd_wv);
-        const int cv = threadIdx.x - r * wv;
-        const int rstep = (int)fdiv(blockDim.x, geo.fd_wv);
-        const T *src = base + (long long)r * geo.inner + cv * VEC;
-        T *dst = data + r * W + cv * VEC;
-        const long long sstep = (long long)rstep * geo.inner;
-        for (int rr = r; rr < L; rr += rstep) {
-            vp_tma::cp_async16(dst, src);
-            src += sstep;
-            dst += rstep * W;
-        }
-        vp_tma::cp_async_wait_all();
-    } else {
-        // row / column of element e advanced incrementally (no division per element)
-        const int dr = (int)fdiv(blockDim.x, geo.fd_w), dc = blockDim.x - dr * W;
-        int r = (int)fdiv(threadIdx.x, geo.fd_w), cc = threadIdx.x - r * W;
-        for (int e = threadIdx.x; e < L * W; e += blockDim.x) {
-            data[e] = cc < wc ? base[(long long)r * geo.inner + cc] : T(0);
-            r += dr;
-            cc += dc;
-            if (cc >= W) {
-                cc -= W;
-                ++r;
-            }
+    const unsigned seg = fdiv(threadIdx.x, PAIR ? geo.fd_w2 : geo.fd_w);
+    const int cc = PAIR ? 2 * (int)(threadIdx.x - seg * (unsigned)(W >> 1)) : (int)(threadIdx.x - seg * (unsigned)W);
+    const bool act = cc < wc && (int)seg < geo.nseg;
+    unsigned ob = 0, c = 0;
+    T *const base = column(act ? cc : 0, ob, c);  // a pair's columns lie in one block (its width is even)
+    LineShift<T> sa, sb;
+    if (src.tab && act) {
+        sa = src.tab[line_class(geo, ob, c)];
+        if (PAIR) sb = src.tab[line_class(geo, ob, c + (cc + 1 < wc ? 1 : 0))];
+    }
+    vp_tma::cp_async_wait_all();
+    __syncthreads();
+    if (!src.tab) {
+        vp_core::tile_weights(shifts, ncl, src);
+        if (act) {
+            sa = shifts[fdiv(geo.cls_from_inner ? c : ob, geo.fd_cdiv) - q0];
+            if (PAIR) sb = shifts[fdiv(geo.cls_from_inner ? c + (cc + 1 < wc ? 1 : 0) : ob, geo.fd_cdiv) - q0];
         }
     }
-    __syncthreads();
-    if (!src.tab) vp_core::tile_weights(shifts, ncl, src);
+    if (!act) return;
     constexpr int G1 = PERIODIC ? 1 : VP_GHOST;
+    const int r0 = (int)fdiv(seg * (unsigned)L, geo.fd_nseg);
+    const int r1 = (int)fdiv((seg + 1) * (unsigned)L, geo.fd_nseg);
     if constexpr (PAIR) {
-        const unsigned seg = fdiv(threadIdx.x, geo.fd_w2);
-        const int cc = 2 * (int)(threadIdx.x - seg * (unsigned)(W >> 1));
-        if (cc >= wc || (int)seg >= geo.nseg) return;
-        const int r0 = (int)fdiv(seg * (unsigned)L, geo.fd_nseg);
-        const int r1 = (int)fdiv((seg + 1) * (unsigned)L, geo.fd_nseg);
-        const LineShift<float> sa = shift_of(c0 + cc);
         if (cc + 1 < wc) {
-            const LineShift<float> sb = shift_of(c0 + cc + 1);
             if (sa.n == sb.n && sa.sigma == sb.sigma) {
                 const vp_core::LineShiftP2 sh = vp_core::pair_shift(sa, sb);
                 const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
-                PtrStore<vp_core::P2> st{reinterpret_cast<vp_core::P2 *>(base + cc + (long long)i0 * geo.inner),
+                PtrStore<vp_core::P2> st{reinterpret_cast<vp_core::P2 *>(base + (long long)i0 * geo.inner),
                                          (long long)sh.sigma * (geo.inner >> 1)};
-                walk<vp_core::P2, ORDER, PERIODIC, FULL, G1, false, FLAT>(reinterpret_cast<const vp_core::P2 *>(data + cc),
-                                                             W >> 1, L, sh, r0, r1, vp_core::P2((float)lp.alpha),
-                                                             lp.mp, lp.pp, st);
+                walk<vp_core::P2, ORDER, PERIODIC, FULL, G1, false, FLAT>(
+                    reinterpret_cast<const vp_core::P2 *>(data + cc), W >> 1, L, sh, r0, r1,
+                    vp_core::P2((float)lp.alpha), lp.mp, lp.pp, st);
                 return;
             }
             const int i1 = sb.sigma > 0 ? r0 : r1 - 1;
-            PtrStore<T> st{base + cc + 1 + (long long)i1 * geo.inner, (long long)sb.sigma * geo.inner};
-            walk<T, ORDER, PERIODIC, FULL, G1, false, FLAT>(data + cc + 1, W, L, sb, r0, r1, (T)lp.alpha, lp.mp, lp.pp, st);
+            PtrStore<T> st{base + 1 + (long long)i1 * geo.inner, (long long)sb.sigma * geo.inner};
+            walk<T, ORDER, PERIODIC, FULL, G1, false, FLAT>(data + cc + 1, W, L, sb, r0, r1, (T)lp.alpha, lp.mp,
+                                                            lp.pp, st);
         }
         const int i0 = sa.sigma > 0 ? r0 : r1 - 1;
-        PtrStore<T> st{base + cc + (long long)i0 * geo.inner, (long long)sa.sigma * geo.inner};
+        PtrStore<T> st{base + (long long)i0 * geo.inner, (long long)sa.sigma * geo.inner};
         walk<T, ORDER, PERIODIC, FULL, G1, false, FLAT>(data + cc, W, L, sa, r0, r1, (T)lp.alpha, lp.mp, lp.pp, st);
     } else {
-        const unsigned seg = fdiv(threadIdx.x, geo.fd_w);
-        const int cc = (int)(threadIdx.x - seg * (unsigned)W);
-        if (cc < wc && (int)seg < geo.nseg) {
-            const LineShift<T> sh = shift_of(c0 + cc);
-            const int r0 = (int)fdiv(seg * (unsigned)L, geo.fd_nseg);
-            const int r1 = (int)fdiv((seg + 1) * (unsigned)L, geo.fd_nseg);
-            const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
-            vp_core::walk_line<T, ORDER, PERIODIC, FULL, G1, FLAT>(
-                data + cc, W, L, sh, r0, r1, (T)lp.alpha, lp.mp, lp.pp, [&](auto t) {
-                    using U = decltype(t);
-                    return PtrStore<U>{reinterpret_cast<U *>(base + cc + (long long)i0 * geo.inner),
-                                       (long long)sh.sigma * geo.inner};
-                });
-        }
+        const int i0 = sa.sigma > 0 ? r0 : r1 - 1;
+        vp_core::walk_line<T, ORDER, PERIODIC, FULL, G1, FLAT>(
+            data + cc, W, L, sa, r0, r1, (T)lp.alpha, lp.mp, lp.pp, [&](auto t) {
+                using U = decltype(t);
+                return PtrStore<U>{reinterpret_cast<U *>(base + (long long)i0 * geo.inner),
+                                   (long long)sa.sigma * geo.inner};
+            });
     }
 }
 
@@ -217,6 +262,10 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
     }
     constexpr int VEC = 16 / sizeof(T);
     const bool vec = (L % VEC) == 0;
+    // lines whose length is no multiple of a 16-byte piece: the tile is still one
+    // run of memory, and a piece's elements fall into at most two lines
+    const bool ragged = !vec && L >= VEC && (reinterpret_cast<uintptr_t>(base) & 15) == 0;
+    constexpr int ES = PAIR ? 2 : 1;  // shared-memory stride between a line's cells
     // Element e = r L + pos of the tile: a thread starts at e = VEC t (or t)
     // and advances by a fixed (rows, positions) step, so no division per element.
     if (vec) {
@@ -256,6 +305,33 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
                 ++r;
             }
         }
+    } else if (ragged) {
+        constexpr int U = 4;  // 16-byte loads in flight per thread
+        const int st = blockDim.x * VEC;
+        const int dr = (int)fdiv(st, geo.fd_l), dp = st - dr * L;
+        int r = (int)fdiv(threadIdx.x * VEC, geo.fd_l), pos = threadIdx.x * VEC - r * L;
+        const int whole = tot - tot % VEC;
+        for (int e = threadIdx.x * VEC; e < whole; e += U * st) {
+            float4 x[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (e + u * st < whole) x[u] = *reinterpret_cast<const float4 *>(base + e + u * st);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (e + u * st >= whole) break;
+                const T *xv = reinterpret_cast<const T *>(&x[u]);
+                const int i0 = iidx(r, pos), i1 = iidx(r + 1, pos - L);
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) in[(pos + k < L ? i0 : i1) + ES * k] = xv[k];
+                r += dr;
+                pos += dp;
+                if (pos >= L) {
+                    pos -= L;
+                    ++r;
+                }
+            }
+        }
+        for (int e = whole + threadIdx.x; e < tot; e += blockDim.x) in[iidx(nl - 1, e - (nl - 1) * L)] = base[e];
     } else {
         const int dr = (int)fdiv(blockDim.x, geo.fd_l), dp = blockDim.x - dr * L;
         int r = (int)fdiv(threadIdx.x, geo.fd_l), pos = threadIdx.x - r * L;
@@ -338,6 +414,26 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
                 ++r;
             }
         }
+    } else if (ragged) {
+        const int st = blockDim.x * VEC;
+        const int dr = (int)fdiv(st, geo.fd_l), dp = st - dr * L;
+        int r = (int)fdiv(threadIdx.x * VEC, geo.fd_l), pos = threadIdx.x * VEC - r * L;
+        const int whole = tot - tot % VEC;
+        for (int e = threadIdx.x * VEC; e < whole; e += st) {
+            float4 x;
+            T *xv = reinterpret_cast<T *>(&x);
+            const int o0 = oidx(r, pos), o1 = oidx(r + 1, pos - L);
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) xv[k] = out[(pos + k < L ? o0 : o1) + ES * k];
+            *reinterpret_cast<float4 *>(base + e) = x;
+            r += dr;
+            pos += dp;
+            if (pos >= L) {
+                pos -= L;
+                ++r;
+            }
+        }
+        for (int e = whole + threadIdx.x; e < tot; e += blockDim.x) base[e] = out[oidx(nl - 1, e - (nl - 1) * L)];
     } else {
         const int dr = (int)fdiv(blockDim.x, geo.fd_l), dp = blockDim.x - dr * L;
         int r = (int)fdiv(threadIdx.x, geo.fd_l), pos = threadIdx.x - r * L;
@@ -482,57 +578,43 @@ __global__ void k_shift_table(LineShift<T> *__restrict__ tab, int nclass, int ki
 // a staged tile of at most 200 KB and up to 128 shifts behind it
 constexpr int kSweepSmem = 216 * 1024;
 
-template <typename T, int ORDER, bool PER, bool FULL, bool FLAT>
-void set_attrs_flat() {
-    cudaFuncSetAttribute(k_sweep_cols<T, ORDER, PER, FULL, false, FLAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         kSweepSmem);
-    cudaFuncSetAttribute(k_sweep_rows<T, ORDER, PER, FULL, false, FLAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         kSweepSmem);
-    if constexpr (sizeof(T) == 4) {
-        cudaFuncSetAttribute(k_sweep_cols<T, ORDER, PER, FULL, true, FLAT>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
-        cudaFuncSetAttribute(k_sweep_rows<T, ORDER, PER, FULL, true, FLAT>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
-    }
+template <typename T, int ORDER, bool PER, bool FULL, bool PAIR>
+void set_attrs_pair() {
+    constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaFuncSetAttribute(k_sweep_cols<T, ORDER, PER, FULL, PAIR, true, false>, attr, kSweepSmem);
+    cudaFuncSetAttribute(k_sweep_cols<T, ORDER, PER, FULL, PAIR, !FULL, false>, attr, kSweepSmem);
+    cudaFuncSetAttribute(k_sweep_cols<T, ORDER, PER, FULL, PAIR, true, true>, attr, kSweepSmem);
+    cudaFuncSetAttribute(k_sweep_rows<T, ORDER, PER, FULL, PAIR, true>, attr, kSweepSmem);
+    cudaFuncSetAttribute(k_sweep_rows<T, ORDER, PER, FULL, PAIR, !FULL>, attr, kSweepSmem);
 }
 
 template <typename T, int ORDER, bool PER, bool FULL>
 void set_attrs_one() {
-    set_attrs_flat<T, ORDER, PER, FULL, true>();
-    if constexpr (FULL) set_attrs_flat<T, ORDER, PER, FULL, false>();
+    set_attrs_pair<T, ORDER, PER, FULL, false>();
+    if constexpr (sizeof(T) == 4) set_attrs_pair<T, ORDER, PER, FULL, true>();
     cudaFuncSetAttribute(k_sweep_cols_tma<T, ORDER, PER, FULL>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
-template <typename T, int ORDER>
+template <typename T>
 void set_attrs() {
-    set_attrs_one<T, ORDER, true, true>();
-    set_attrs_one<T, ORDER, false, true>();
-    set_attrs_one<T, ORDER, true, false>();
-    set_attrs_one<T, ORDER, false, false>();
+    set_attrs_one<T, kOrder, true, true>();
+    set_attrs_one<T, kOrder, false, true>();
+    set_attrs_one<T, kOrder, true, false>();
+    set_attrs_one<T, kOrder, false, false>();
 }
 
-// compile-time dispatch on the scheme order, the line's periodicity and
-// whether both limiters are on
-#define VP_DISPATCH(ORDER_, PER_, FULL_, CALL)                         \
-    do {                                                               \
-        if ((ORDER_) == 7) {                                           \
-            if (PER_) {                                                \
-                if (FULL_) { CALL(7, true, true); }                    \
-                else { CALL(7, true, false); }                         \
-            } else {                                                   \
-                if (FULL_) { CALL(7, false, true); }                   \
-                else { CALL(7, false, false); }                        \
-            }                                                          \
-        } else {                                                       \
-            if (PER_) {                                                \
-                if (FULL_) { CALL(5, true, true); }                    \
-                else { CALL(5, true, false); }                         \
-            } else {                                                   \
-                if (FULL_) { CALL(5, false, true); }                   \
-                else { CALL(5, false, false); }                        \
-            }                                                          \
-        }                                                              \
+// compile-time dispatch on the line's periodicity and whether both limiters
+// are on (the scheme's order is the unit's)
+#define VP_DISPATCH(PER_, FULL_, CALL)                 \
+    do {                                               \
+        if (PER_) {                                    \
+            if (FULL_) { CALL(kOrder, true, true); }   \
+            else { CALL(kOrder, true, false); }        \
+        } else {                                       \
+            if (FULL_) { CALL(kOrder, false, true); }  \
+            else { CALL(kOrder, false, false); }       \
+        }                                              \
     } while (0)
 
 // geometry of the sweep along axis `dim` (kick: velocity axis, else spatial)
@@ -600,7 +682,7 @@ inline bool geo_fits_32(const SweepGeo &geo) { return geo.outer < (1LL << 32) &&
 // per step), the table once.
 inline int tile_classes(const SweepGeo &geo, int w) {
     const bool many = geo.cls_from_inner || geo.inner == 1;
-    const long long n = many ? (w - 1) / geo.cdiv + 2 : 1;
+    const long long n = many ? (w - 1) / geo.cdiv + 2 : (geo.kblk > 1 ? (geo.kblk - 1) / geo.cdiv + 2 : 1);
     return (int)(n > w ? w : n);
 }
 inline bool own_shifts(const vp_ctx *c, const SweepGeo &geo, long long tiles) {
@@ -639,7 +721,17 @@ int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
     T *f = static_cast<T *>(c->f);
     const int L = geo.L;
     int W = tu.W;
-    if (geo.inner < W) W = (int)geo.inner;
+    geo.kblk = 1;
+    if (geo.inner < W) {
+        // narrow blocks: as many whole ones side by side as the tile holds (30
+        // columns of 33 cells, one block per CTA: 1.18 ms, a warp of them idle)
+        const int wt = (int)geo.inner;
+        const bool tma = tu.impl == 2 && tma_eligible<T>(c, geo, wt);
+        long long k = tma ? 1 : W / wt;
+        k = k > geo.outer ? geo.outer : k;
+        geo.kblk = (int)k;
+        W = wt * geo.kblk;
+    }
     const bool pair = tu.impl == 3 && pair_eligible<T>(c, geo, W);
     // walkers per segment row: W lines, or W / 2 line pairs; at most 512 threads
     const int per_row = pair ? W >> 1 : W;
@@ -647,15 +739,21 @@ int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
     while (nseg > 1 && per_row * nseg > (pair ? VP_PAIR_THREADS : 512)) nseg >>= 1;
     geo.W = W;
     geo.nseg = nseg;
-    const int threads = ((per_row * nseg + 31) / 32) * 32;
-    const long long tiles = geo.outer * ((geo.inner + W - 1) / W);
+    // the widest pieces the rows are made of
+    geo.vec = 16 / (int)sizeof(T);
+    while (geo.inner % geo.vec || W % geo.vec) geo.vec /= 2;
+    const int wv = W / geo.vec;
+    int threads = ((per_row * nseg + 31) / 32) * 32;
+    if (threads < wv) threads = (wv + 31) / 32 * 32;  // one row of pieces at least
+    const long long tiles = geo.kblk > 1 ? (geo.outer + geo.kblk - 1) / geo.kblk
+                                         : geo.outer * ((geo.inner + W - 1) / W);
     if (tiles >= (1LL << 31)) return vp_fail(c, VP_ENOTSUP, "sweep has too many tiles");
     geo.tpo = (unsigned)((geo.inner + W - 1) / W);
     geo.fd_tpo = make_fastdiv(geo.tpo);
     geo.fd_w = make_fastdiv((unsigned)W);
     geo.fd_nseg = make_fastdiv((unsigned)nseg);
-    geo.fd_wv = make_fastdiv((unsigned)(W / (16 / sizeof(T)) > 0 ? W / (16 / sizeof(T)) : 1));
-    const int order = c->g.order;
+    geo.fd_wv = make_fastdiv((unsigned)wv);
+    geo.fd_inner = make_fastdiv((unsigned)geo.inner);
     const bool per = geo.periodic != 0;
     const bool full = c->g.mp && c->g.pp;
     const bool flat = tu.flat;
@@ -684,7 +782,7 @@ int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
         int per_sm = tu.ctas_per_sm;
         if (per_sm <= 0) {
 #define VP_OCC(O, P, F) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep_cols_tma<T, O, P, F>, threads, tsmem)
-            VP_DISPATCH(order, per, full, VP_OCC);
+            VP_DISPATCH(per, full, VP_OCC);
 #undef VP_OCC
             per_sm = per_sm < 1 ? 1 : per_sm;
         }
@@ -693,26 +791,27 @@ int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
 #define VP_LAUNCH(O, P, F) \
     k_sweep_cols_tma<T, O, P, F><<<(unsigned)grid, threads, tsmem, c->stream>>>(map, tab, geo, lp, c->d_status, \
                                                                                 c->opt_wait_limit)
-        VP_DISPATCH(order, per, full, VP_LAUNCH);
-#undef VP_LAUNCH
-    } else if (pair) {
-        const int pthreads = threads;
-        geo.fd_w2 = make_fastdiv((unsigned)(W >> 1));
-#define VP_LAUNCH(O, P, F)                                                                                     \
-    if (flat)                                                                                                  \
-        k_sweep_cols<T, O, P, F, sizeof(T) == 4, true><<<(unsigned)tiles, pthreads, smem, c->stream>>>(f, src, geo, lp); \
-    else                                                                                                       \
-        k_sweep_cols<T, O, P, F, sizeof(T) == 4, !F><<<(unsigned)tiles, pthreads, smem, c->stream>>>(f, src, geo, lp)
-        VP_DISPATCH(order, per, full, VP_LAUNCH);
+        VP_DISPATCH(per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     } else {
-#define VP_LAUNCH(O, P, F)                                                                                   \
-    if (flat)                                                                                                \
-        k_sweep_cols<T, O, P, F, false, true><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp); \
-    else                                                                                                     \
-        k_sweep_cols<T, O, P, F, false, !F><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp)
-        VP_DISPATCH(order, per, full, VP_LAUNCH);
+        geo.fd_w2 = make_fastdiv((unsigned)(W >> 1 > 0 ? W >> 1 : 1));
+        const bool gen = geo.kblk > 1 || geo.vec * sizeof(T) != 16 || geo.inner % W || threads % wv;
+#define VP_LAUNCH_COLS(O, P, F, PAIR)                                                                              \
+    if (gen)                                                                                                       \
+        k_sweep_cols<T, O, P, F, PAIR, true, true><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp); \
+    else if (flat)                                                                                                 \
+        k_sweep_cols<T, O, P, F, PAIR, true, false><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp); \
+    else                                                                                                           \
+        k_sweep_cols<T, O, P, F, PAIR, !F, false><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp)
+#define VP_LAUNCH(O, P, F)                          \
+    if (pair) {                                     \
+        VP_LAUNCH_COLS(O, P, F, sizeof(T) == 4);    \
+    } else {                                        \
+        VP_LAUNCH_COLS(O, P, F, false);             \
+    }
+        VP_DISPATCH(per, full, VP_LAUNCH);
 #undef VP_LAUNCH
+#undef VP_LAUNCH_COLS
     }
     c->launches++;
     VP_CUDA_TRY(c, cudaGetLastError());
@@ -763,7 +862,7 @@ int launch_rows(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
         k_sweep_rows<T, O, P, F, sizeof(T) == 4, true><<<(unsigned)blocks, pthreads, smem, c->stream>>>(f, src, geo, lp); \
     else                                                                                                       \
         k_sweep_rows<T, O, P, F, sizeof(T) == 4, !F><<<(unsigned)blocks, pthreads, smem, c->stream>>>(f, src, geo, lp)
-        VP_DISPATCH(c->g.order, per, full, VP_LAUNCH);
+        VP_DISPATCH(per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     } else {
 #define VP_LAUNCH(O, P, F)                                                                                     \
@@ -771,7 +870,7 @@ int launch_rows(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
         k_sweep_rows<T, O, P, F, false, true><<<(unsigned)blocks, threads, smem, c->stream>>>(f, src, geo, lp); \
     else                                                                                                       \
         k_sweep_rows<T, O, P, F, false, !F><<<(unsigned)blocks, threads, smem, c->stream>>>(f, src, geo, lp)
-        VP_DISPATCH(c->g.order, per, full, VP_LAUNCH);
+        VP_DISPATCH(per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     }
     c->launches++;
@@ -1033,21 +1132,10 @@ int tune_on(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, const SweepGeo
 
 }  // namespace
 
-// The entry points of one precision; the FP64 ones compile in a unit of their
-// own (vp_sweep_f64.cu), which halves the build.
-#ifdef VP_SWEEP_UNIT_F64
-typedef double unit_t;
-#define VP_UNIT(name) name##_f64
-#else
-typedef float unit_t;
-#define VP_UNIT(name) name##_f32
-#endif
+// The entry points of this unit's precision and order.
+void VP_UNIT(vp_sweep_attrs)() { set_attrs<unit_t>(); }
 
-void VP_UNIT(vp_sweep_attrs)() {
-    set_attrs<unit_t, 5>();
-    set_attrs<unit_t, 7>();
-}
-
+#if VP_SWEEP_ORDER == 7
 int VP_UNIT(vp_launch_shift_table)(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
     const vp_grid &g = c->g;
     const int nclass = kick ? (int)c->NX : g.nv[dim];
@@ -1062,6 +1150,8 @@ int VP_UNIT(vp_launch_shift_table)(vp_ctx *c, int kick, int dim, double dt, cons
     return VP_OK;
 }
 
+#endif
+
 int VP_UNIT(vp_launch_sweep)(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
     return launch_sweep_t<unit_t>(c, kick, dim, dt, accel);
 }
@@ -1070,32 +1160,48 @@ int VP_UNIT(vp_tune_sweep)(vp_ctx *c, int kick, int dim, double dt, const double
     return tune_t<unit_t>(c, kick, dim, dt, accel);
 }
 
-#ifndef VP_SWEEP_UNIT_F64
-void vp_sweep_attrs_f64();
-int vp_launch_shift_table_f64(vp_ctx *c, int kick, int dim, double dt, const double *accel);
-int vp_launch_sweep_f64(vp_ctx *c, int kick, int dim, double dt, const double *accel);
-int vp_tune_sweep_f64(vp_ctx *c, int kick, int dim, double dt, const double *accel);
+#ifdef VP_SWEEP_MAIN
+#define VP_DECLARE(U)                                                                      \
+    void vp_sweep_attrs_##U();                                                             \
+    int vp_launch_sweep_##U(vp_ctx *c, int kick, int dim, double dt, const double *accel); \
+    int vp_tune_sweep_##U(vp_ctx *c, int kick, int dim, double dt, const double *accel)
+VP_DECLARE(f32_o5);
+VP_DECLARE(f64_o5);
+VP_DECLARE(f64_o7);
+int vp_launch_shift_table_f64_o7(vp_ctx *c, int kick, int dim, double dt, const double *accel);
 
 int vp_sweep_setup(vp_ctx *c) {
-    vp_sweep_attrs_f32();
-    vp_sweep_attrs_f64();
+    vp_sweep_attrs_f32_o5();
+    vp_sweep_attrs_f32_o7();
+    vp_sweep_attrs_f64_o5();
+    vp_sweep_attrs_f64_o7();
     VP_CUDA_TRY(c, cudaGetLastError());
     return VP_OK;
 }
 
 int vp_launch_shift_table(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
-    return c->g.precision == VP_F32 ? vp_launch_shift_table_f32(c, kick, dim, dt, accel)
-                                    : vp_launch_shift_table_f64(c, kick, dim, dt, accel);
+    return c->g.precision == VP_F32 ? vp_launch_shift_table_f32_o7(c, kick, dim, dt, accel)
+                                    : vp_launch_shift_table_f64_o7(c, kick, dim, dt, accel);
+}
+
+int vp_launch_shift_table_f32(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+    return vp_launch_shift_table_f32_o7(c, kick, dim, dt, accel);
 }
 
 int vp_launch_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
-    return c->g.precision == VP_F32 ? vp_launch_sweep_f32(c, kick, dim, dt, accel)
-                                    : vp_launch_sweep_f64(c, kick, dim, dt, accel);
+    if (c->g.precision == VP_F32)
+        return c->g.order == 7 ? vp_launch_sweep_f32_o7(c, kick, dim, dt, accel)
+                               : vp_launch_sweep_f32_o5(c, kick, dim, dt, accel);
+    return c->g.order == 7 ? vp_launch_sweep_f64_o7(c, kick, dim, dt, accel)
+                           : vp_launch_sweep_f64_o5(c, kick, dim, dt, accel);
 }
 
 int vp_tune_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
     if (c->tune[kick][dim].valid) return VP_OK;
-    return c->g.precision == VP_F32 ? vp_tune_sweep_f32(c, kick, dim, dt, accel)
-                                    : vp_tune_sweep_f64(c, kick, dim, dt, accel);
+    if (c->g.precision == VP_F32)
+        return c->g.order == 7 ? vp_tune_sweep_f32_o7(c, kick, dim, dt, accel)
+                               : vp_tune_sweep_f32_o5(c, kick, dim, dt, accel);
+    return c->g.order == 7 ? vp_tune_sweep_f64_o7(c, kick, dim, dt, accel)
+                           : vp_tune_sweep_f64_o5(c, kick, dim, dt, accel);
 }
 #endif

@@ -17,6 +17,16 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr(smem)), "l"(gmem) : "memory");
 }
 
+// the same for pieces of 4, 8 or 16 bytes (addresses aligned to the piece)
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
+    if constexpr (BYTES == 16)
+        cp_async16(smem, gmem);
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(saddr(smem)), "l"(gmem), "n"(BYTES)
+                     : "memory");
+}
+
 // wait for every cp.async this thread issued
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 

@@ -342,3 +342,37 @@ def test_flat_votes_of_blocks_give_the_same_bits(precision, dims, nx, nv):
             out.append(from_gpu(sim))
             sim.close()
         assert np.array_equal(out[0], out[1]), (kick, d)
+
+
+@pytest.mark.parametrize("precision", [V.VP_F32, V.VP_F64])
+@pytest.mark.parametrize("nx,nv", [([3, 5], [9, 6]), ([7, 1], [21, 2]), ([2, 3], [33, 30]), ([5, 3], [12, 7])])
+def test_blocks_side_by_side_and_rows_of_every_width(precision, nx, nv):
+    """Narrow outer blocks packed side by side in one tile (a last tile with
+    fewer), rows of 16-, 8- and 4-byte pieces, contiguous lines whose 16-byte
+    pieces straddle two lines: default and tuned kernels, one and two lines per
+    thread, give the same bits, and those of FP64 match the oracle."""
+    g = grid(2, nx, nv, order=7, xbc=1)
+    og = O.grid(**g)
+    f0 = inputs.random_f(og.NX * og.NV, seed=nv[0]).astype(np.float32).astype(np.float64)
+    acc = inputs.random_accel(og.NX, 2, seed=2, amax=6.0)
+    for kick in (0, 1):
+        for d in range(2):
+            out = []
+            for impl, tune in ((0, 0), (1, 0), (0, 1), (1, 1)):
+                sim, _ = both(g, precision)
+                V.vp_set_option(sim.ctx, V.VP_OPT_SWEEP_IMPL, impl)
+                V.vp_set_option(sim.ctx, V.VP_OPT_AUTOTUNE, tune)
+                to_gpu(sim, f0)
+                if kick:
+                    V.vp_kick_sweep(sim.ctx, d, 0.43, accel_tensor(sim, acc[d]))
+                else:
+                    V.vp_drift_sweep(sim.ctx, d, 0.29)
+                out.append(from_gpu(sim))
+                sim.close()
+            assert all(np.array_equal(a, out[0]) for a in out[1:]), (kick, d)
+            f_o = f0.copy()
+            if kick:
+                O.kick_sweep(og, f_o, d, 0.43, acc[d])
+            else:
+                O.drift_sweep(og, f_o, d, 0.29)
+            assert rel_l1(out[0], f_o) <= (2e-6 if precision == V.VP_F32 else 1e-12)
