@@ -509,9 +509,8 @@ struct DiagSum<float> {
     // Fallen tails of a distribution are full of such cells; sending them
     // through FP64 instead took 5.9 ms for 3.1e8 cells.
     CSum m0{0.f, 0.f}, m2{0.f, 0.f}, l2{0.f, 0.f}, m2t{0.f, 0.f}, l2t{0.f, 0.f}, neg{0.f, 0.f};
-    double d0 = 0.0, d2 = 0.0, dl2 = 0.0, dneg = 0.0;  // cells above 2^60
     float mn = INFINITY, mx = -INFINITY;
-    bool huge = false, bad = false;
+    bool huge = false, bad = false;  // a cell above 2^60: the point is summed again in double
     static constexpr float kTiny = 8.8817842e-16f, kHuge = 1.1529215e18f, kUp = 1.2676506e30f;
     static __device__ __forceinline__ void weigh(CSum &c, float x, const W &w) {
         c.add_product(x, w.hi);
@@ -521,17 +520,7 @@ struct DiagSum<float> {
         mn = fminf(mn, x);
         mx = fmaxf(mx, x);
         const float ax = fabsf(x);
-        if (!(ax <= kHuge)) {
-            const double v = (double)x;
-            if (!isfinite(x)) bad = true;
-            d0 += v;
-            d2 = fma(v, (double)w.hi + (double)w.lo, d2);
-            if (w2) d2 = fma(v, (double)w2->hi + (double)w2->lo, d2);
-            dl2 = fma(v, v, dl2);
-            if (x < 0.f) dneg += v;
-            huge = true;
-            return;
-        }
+        if (!(ax <= kHuge)) huge = true;
         m0.add(x);
         if (x < 0.f) neg.add(x);
         if (ax < kTiny) {
@@ -553,7 +542,6 @@ struct DiagSum<float> {
         CSum &c = tiny ? m2t : m2;
         weigh(c, y, w);
         c.e = fmaf(m0.e * u, w.hi, c.e);
-        if (huge) d2 = fma(d0, (double)w.hi + (double)w.lo, d2);
     }
     // {sum, weighted sum, sum of negatives, sum of squares} of the warp
     __device__ __forceinline__ void totals(double (&v)[4]) {
@@ -562,14 +550,28 @@ struct DiagSum<float> {
         v[1] = fma(warp_total(m2t), kDown, warp_total(m2));
         v[2] = __any_sync(0xffffffffu, mn < 0.f) ? warp_total(neg) : 0.0;
         v[3] = fma(warp_total(l2t), kDown * kDown, warp_total(l2));
-        if (__any_sync(0xffffffffu, huge)) {
-            v[0] += warp_sum(d0);
-            v[1] += warp_sum(d2);
-            v[2] += warp_sum(dneg);
-            v[3] += warp_sum(dl2);
-        }
     }
 };
+
+// the sums of a point with cells that the float pairs cannot hold, in double
+// (out of line: its arithmetic would otherwise be predicated into every cell)
+__device__ __noinline__ void diag_in_double(const float *p, long long NV, int nlast, const WPair *wrow,
+                                            const WPair *wlast, double (&v)[4], bool &bad) {
+    for (int k = 0; k < 4; ++k) v[k] = 0.0;
+    for (long long i = threadIdx.x; i < NV; i += blockDim.x) {
+        const double x = (double)p[i];
+        const long long r = i / nlast;
+        const WPair a = wrow[r], b = wlast[i - r * nlast];
+        if (!isfinite(x)) bad = true;
+        v[0] += x;
+        v[1] = fma(x, ((double)a.hi + (double)a.lo) + ((double)b.hi + (double)b.lo), v[1]);
+        if (x < 0.0) v[2] += x;
+        v[3] = fma(x, x, v[3]);
+    }
+    for (int k = 0; k < 4; ++k) v[k] = warp_sum(v[k]);
+}
+__device__ __forceinline__ void diag_in_double(const double *, long long, int, const double *, const double *,
+                                               double (&)[4], bool &) {}
 
 template <>
 struct DiagSum<double> {
@@ -577,6 +579,7 @@ struct DiagSum<double> {
     double m0 = 0.0, m2 = 0.0, l2 = 0.0, neg = 0.0;
     double mn = INFINITY, mx = -INFINITY;
     bool bad = false;
+    static constexpr bool huge = false;
     __device__ __forceinline__ void cell(double x, const W &w, const W *w2) {
         mn = fmin(mn, x);
         mx = fmax(mx, x);
@@ -621,8 +624,21 @@ __global__ void __launch_bounds__(kBlock) k_diag_part(const T *__restrict__ f, l
             const long long rows = NV / nlast;
             const T *c = p + threadIdx.x;
             const int step = nr * nlast;
-#pragma unroll 4
-            for (long long r = r0; r < rows; r += nr) {
+            // four cells and weights in flight
+            long long r = r0;
+            for (; r + 3 * nr < rows; r += 4 * nr) {
+                T x[4];
+                typename DiagSum<T>::W w[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    x[k] = *c;
+                    w[k] = wrow[r + k * nr];
+                    c += step;
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) q.cell(x[k], w[k], nullptr);
+            }
+            for (; r < rows; r += nr) {
                 q.cell(*c, wrow[r], nullptr);
                 c += step;
             }
@@ -634,9 +650,10 @@ __global__ void __launch_bounds__(kBlock) k_diag_part(const T *__restrict__ f, l
             q.cell(p[v], wrow[r], wlast + (v - r * nlast));
         }
     }
-    if (q.bad) atomicExch(bad, 1);
     double v[4];
     q.totals(v);
+    if (sizeof(T) == 4 && __syncthreads_or(q.huge)) diag_in_double(p, NV, nlast, wrow, wlast, v, q.bad);
+    if (q.bad) atomicExch(bad, 1);
     T mn = q.mn, mx = q.mx;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {

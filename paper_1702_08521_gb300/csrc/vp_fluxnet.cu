@@ -265,13 +265,16 @@ __global__ void k_adam(float *__restrict__ wts, float *__restrict__ m, float *__
 
 // FP64 instructions take 16 cycles each here, conversions included, and the
 // outputs are tens of millions of doubles: sums of a few floats are kept as a
-// value and its error term (two-sum), and the exact conversion of a normal
-// float to a double is done on its bits.
+// value and its error term (two-sum), and a normal float becomes a double on
+// its bits; other numbers take the conversion, out of line (as a
+// predicated instruction it occupies the FP64 pipe for every number).
+__device__ __noinline__ double widen_rare(float x) { return (double)x; }
 __device__ __forceinline__ double widen(float x) {
     const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-    if (m - 0x00800000u < 0x7f000000u)  // normal
-        return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
-    return m ? (double)x : __hiloint2double((int)b, 0);
+    const unsigned hi = (b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
+    double d = __hiloint2double((int)hi, (int)(b << 29));
+    if (m != 0u && m - 0x00800000u >= 0x7f000000u) d = widen_rare(x);
+    return d;
 }
 
 struct PairSum {
@@ -332,10 +335,17 @@ __device__ __forceinline__ void stage_lines(const float *__restrict__ f, const L
         put(i, row, in ? __ldg(f + p.base[i] + off + (long long)r * q.inner) : 0.f);
     };
     if (q.inner >= 16) {
+        const int i = threadIdx.x & (q.W - 1);
+        const bool in = i < nl && use(i);
+        const float *p0 = f + p.base[i < nl ? i : 0] + off;
+        const int step = blockDim.x >> q.logW;
 #pragma unroll 4
-        for (int t = threadIdx.x; t < R << q.logW; t += blockDim.x) {
-            const int i = t & (q.W - 1);
-            if (i < nl) cell(i, (t >> q.logW) - kEdge);
+        for (int row = (int)(threadIdx.x >> q.logW) - kEdge; row < q.L + kEdge; row += step) {
+            int r = row;
+            bool ok = in;
+            if (q.periodic) r = wrap_row(r, q.L);
+            else ok = ok && r >= 0 && r < q.L;
+            if (i < nl) put(i, row, ok ? __ldg(p0 + (long long)r * q.inner) : 0.f);
         }
     } else {
         for (int i = threadIdx.x >> 5; i < nl; i += blockDim.x >> 5)
@@ -391,16 +401,36 @@ __global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, 
         // the shift of the stencil: modulo the line, or just off its ends
         const int ns = q.periodic ? n % L : (n < -2 * L - 8 ? -2 * L - 8 : (n > 2 * L + 8 ? 2 * L + 8 : n));
         const float *ui = u + i;
-        for (int j = threadIdx.x >> q.logW; j < nout; j += blockDim.x >> q.logW) {
+        // a run of interfaces per thread; the stencil (rows a .. a + 6) slides
+        // along it
+        const int nseg = blockDim.x >> q.logW, seg = threadIdx.x >> q.logW;
+        const int j0 = seg * nout / nseg, j1 = (seg + 1) * nout / nseg;
+        float w[7];
+        int at = 0x40000000;  // row of w[0]
+        for (int j = j0; j < j1; ++j) {
             // interface between cells c - 1 and c; its stencil in the upwind
-            // frame is centred n cells upwind: rows a .. a + 6 of the line
+            // frame is centred n cells upwind (rows down to -kEdge and up to
+            // L + kEdge - 1 are staged)
             const int c = j * every;
             int a = sg > 0 ? c - ns - 4 : c + ns - 3;
-            a = q.periodic ? wrap_row(a, L) : (a < -7 ? -7 : (a > L ? L : a));
-            float w[7];
+            if (q.periodic) {
+                while (a < -kEdge) a += L;
+                while (a > L + 1) a -= L;
+            } else {
+                a = a < -7 ? -7 : (a > L ? L : a);
+            }
+            if (a == at + 1) {
 #pragma unroll
-            for (int k = 0; k < 7; ++k) w[k] = ui[(a + (sg > 0 ? k : 6 - k)) * WP];
-            const float M = vp_core::flux<float, 7, true>(sh, w[0], w[1], w[2], w[3], w[4], w[5], w[6], alpha, 1, 1);
+                for (int k = 0; k < 6; ++k) w[k] = w[k + 1];
+                w[6] = ui[(a + 6) * WP];
+            } else if (a != at) {
+#pragma unroll
+                for (int k = 0; k < 7; ++k) w[k] = ui[(a + k) * WP];
+            }
+            at = a;
+            const float M =
+                sg > 0 ? vp_core::flux<float, 7, true>(sh, w[0], w[1], w[2], w[3], w[4], w[5], w[6], alpha, 1, 1)
+                       : vp_core::flux<float, 7, true>(sh, w[6], w[5], w[4], w[3], w[2], w[1], w[0], alpha, 1, 1);
             double g;
             if (PREFIX) {
                 // sum of the cells before k, extended beyond the line
@@ -417,18 +447,19 @@ __global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, 
                 };
                 // cells c - n .. c - 1 (swept rightwards) or c .. c + n - 1
                 g = (sg > 0 ? upto(c) - upto(c - n) : upto(c + n) - upto(c)) + widen(M);
+                g = sg > 0 ? g : -g;
             } else {
+                // |n| < kFewCells: the cells lie within the staged rows
                 PairSum p{0.f, 0.f};
-                int k = sg > 0 ? (n >= 0 ? c - n : c) : (n >= 0 ? c : c + n);
+                const float *v = ui + (sg > 0 ? (n >= 0 ? c - n : c) : (n >= 0 ? c : c + n)) * WP;
                 const float one = n >= 0 ? 1.f : -1.f;
-                for (int m = n >= 0 ? n : -n; m > 0; --m, ++k) {
-                    const bool in = q.periodic || (k >= 0 && k < L);
-                    p.add(in ? one * ui[(q.periodic ? wrap_row(k, L) : k) * WP] : 0.f);
-                }
+                for (int m = n >= 0 ? n : -n; m > 0; --m, v += WP) p.add(one * *v);
                 p.add(M);
+                p.s = sg > 0 ? p.s : -p.s;
+                p.e = sg > 0 ? p.e : -p.e;
                 g = p.value();
             }
-            Gs[i * NP + j] = sg > 0 ? g : -g;
+            Gs[i * NP + j] = g;
         }
     }
     __syncthreads();
