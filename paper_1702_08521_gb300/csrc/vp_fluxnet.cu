@@ -296,6 +296,7 @@ struct LineTile {
     long long lines, inner;
     int L, W, logW, periodic, from_inner;
     unsigned cdiv, cmod;
+    FastDiv fd_inner, fd_cdiv, fd_cmod;
 };
 // element of a line's first cell, and its class
 struct LinePos {
@@ -304,9 +305,11 @@ struct LinePos {
 };
 __device__ __forceinline__ void place_lines(const LineTile &q, long long l0, int nl, LinePos &p) {
     for (int i = threadIdx.x; i < nl; i += blockDim.x) {
-        const long long o = (l0 + i) / q.inner, c = (l0 + i) - o * q.inner;
+        const long long line = l0 + i;
+        const long long o = q.lines < (1LL << 32) ? (long long)fdiv((unsigned)line, q.fd_inner) : line / q.inner;
+        const long long c = line - o * q.inner;
         p.base[i] = o * q.L * q.inner + c;
-        p.cls[i] = q.from_inner ? (unsigned)c / q.cdiv % q.cmod : (unsigned)o / q.cdiv;
+        p.cls[i] = q.from_inner ? fmod_u(fdiv((unsigned)c, q.fd_cdiv), q.fd_cmod) : fdiv((unsigned)o, q.fd_cdiv);
     }
 }
 
@@ -321,35 +324,33 @@ __device__ __forceinline__ int wrap_row(int r, int L) {
 }
 
 // Stage nl lines (base elements plus `off`; a line with use(i) false is zero):
-// put(line, row, value) for rows -kEdge .. L + kEdge - 1.  Lanes run over the
-// lines where neighbouring lines are neighbours in memory, else along the line.
-template <typename Use, typename Put>
+// at(line, row) is the place of rows -kEdge .. L + kEdge - 1.  Lanes run over
+// the lines where neighbouring lines are neighbours in memory, else along the
+// line; every cell's copy is in flight at once (vp_tma::cp_async_wait_all and a
+// barrier complete them).
+template <typename Use, typename At>
 __device__ __forceinline__ void stage_lines(const float *__restrict__ f, const LineTile &q, const LinePos &p, int nl,
-                                            long long off, Use use, Put put) {
+                                            long long off, Use use, At at) {
     const int R = q.L + 2 * kEdge;
-    auto cell = [&](int i, int row) {
+    auto cell = [&](const float *line, bool in, float *to, int row) {
         int r = row;
-        bool in = use(i);
         if (q.periodic) r = wrap_row(r, q.L);
         else in = in && r >= 0 && r < q.L;
-        put(i, row, in ? __ldg(f + p.base[i] + off + (long long)r * q.inner) : 0.f);
+        if (in) vp_tma::cp_async<4>(to, line + (long long)r * q.inner);
+        else *to = 0.f;
     };
     if (q.inner >= 16) {
         const int i = threadIdx.x & (q.W - 1);
-        const bool in = i < nl && use(i);
-        const float *p0 = f + p.base[i < nl ? i : 0] + off;
-        const int step = blockDim.x >> q.logW;
-#pragma unroll 4
-        for (int row = (int)(threadIdx.x >> q.logW) - kEdge; row < q.L + kEdge; row += step) {
-            int r = row;
-            bool ok = in;
-            if (q.periodic) r = wrap_row(r, q.L);
-            else ok = ok && r >= 0 && r < q.L;
-            if (i < nl) put(i, row, ok ? __ldg(p0 + (long long)r * q.inner) : 0.f);
-        }
+        if (i >= nl) return;
+        const bool in = use(i);
+        const float *line = f + p.base[i] + off;
+        for (int row = (int)(threadIdx.x >> q.logW) - kEdge; row < q.L + kEdge; row += blockDim.x >> q.logW)
+            cell(line, in, at(i, row), row);
     } else {
-        for (int i = threadIdx.x >> 5; i < nl; i += blockDim.x >> 5)
-            for (int r = (threadIdx.x & 31); r < R; r += 32) cell(i, r - kEdge);
+        for (int i = threadIdx.x >> 5; i < nl; i += blockDim.x >> 5) {
+            const bool in = use(i);
+            for (int r = (threadIdx.x & 31); r < R; r += 32) cell(f + p.base[i] + off, in, at(i, r - kEdge), r - kEdge);
+        }
     }
 }
 
@@ -380,7 +381,8 @@ __global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, 
     const int nl = (int)(q.lines - l0 < W ? q.lines - l0 : W);
     place_lines(q, l0, nl, pos);
     __syncthreads();
-    stage_lines(f, q, pos, nl, 0, [](int) { return true; }, [&](int i, int row, float v) { u[row * WP + i] = v; });
+    stage_lines(f, q, pos, nl, 0, [](int) { return true; }, [&](int i, int row) { return u + row * WP + i; });
+    vp_tma::cp_async_wait_all();
     __syncthreads();
     if (PREFIX) {
         for (int i = threadIdx.x; i < nl; i += blockDim.x) {
@@ -547,8 +549,9 @@ __global__ void __launch_bounds__(kSampleThreads)
             float *d = tile + (size_t)k * W * P + kEdge;
             stage_lines(fc, q, pos, nl, k == 0 ? 0 : (k == 1 ? 1 : -1) * (long long)q.cdiv,
                         [&](int i) { return k == 0 || (nbr[i] & (k == 1 ? 2 : 4)); },
-                        [&](int i, int row, float v) { d[i * P + row] = v; });
+                        [&](int i, int row) { return d + i * P + row; });
         }
+        vp_tma::cp_async_wait_all();
         __syncthreads();
     }
     const int ns = nl * (L + 1);
@@ -1098,6 +1101,9 @@ LineTile line_tile(const LineGeo &q) {
     t.from_inner = q.from_inner;
     t.cdiv = (unsigned)q.cdiv;
     t.cmod = (unsigned)q.cmod;
+    t.fd_inner = make_fastdiv((unsigned)q.inner);
+    t.fd_cdiv = make_fastdiv(t.cdiv);
+    t.fd_cmod = make_fastdiv(t.cmod);
     return t;
 }
 void set_width(LineTile &t, int W) {
