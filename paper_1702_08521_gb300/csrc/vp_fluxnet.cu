@@ -25,6 +25,7 @@
 // reductions, Adam.
 #include <cuda_bf16.h>
 
+#include <atomic>
 #include <cmath>
 
 #include "vp_internal.cuh"
@@ -50,45 +51,6 @@ static_assert(NPARAM == VP_NET_NPARAM, "parameter count");
 
 __device__ __forceinline__ float bfr(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
-// ---- network on one sample (SIMT, weights in shared memory, rounded) -------------
-
-struct NetAct {
-    float x[NF], h1[H], h2[H], h3[H];
-    float z1[H], z2[H], z3[H];
-};
-
-__device__ __forceinline__ float net_forward(const float *__restrict__ w, const float *xin, float *h1,
-                                             float *h2, float *h3) {
-    float x[NF];
-#pragma unroll
-    for (int k = 0; k < NF; ++k) x[k] = bfr(xin[k]);
-#pragma unroll 4
-    for (int j = 0; j < H; ++j) {
-        float a = w[OFF_B1 + j];
-#pragma unroll
-        for (int k = 0; k < NF; ++k) a = fmaf(w[OFF_W1 + j * NF + k], x[k], a);
-        h1[j] = bfr(fmaxf(a, 0.f));
-    }
-#pragma unroll 4
-    for (int j = 0; j < H; ++j) {
-        float a = w[OFF_B2 + j];
-#pragma unroll
-        for (int k = 0; k < H; ++k) a = fmaf(w[OFF_W2 + j * H + k], h1[k], a);
-        h2[j] = bfr(fmaxf(a, 0.f));
-    }
-    float g = w[OFF_B4];
-#pragma unroll 4
-    for (int j = 0; j < H; ++j) {
-        float a = w[OFF_B3 + j];
-#pragma unroll
-        for (int k = 0; k < H; ++k) a = fmaf(w[OFF_W3 + j * H + k], h2[k], a);
-        const float v = bfr(fmaxf(a, 0.f));
-        if (h3) h3[j] = v;
-        g = fmaf(w[OFF_W4 + j], v, g);
-    }
-    return g;
-}
-
 // features of the upwind-ordered stencil u[0..7] = u_{-3..4} and of the same
 // cells up / um of the velocity-neighbour lines (+: larger |v|): velocity
 // difference and curvature
@@ -111,139 +73,316 @@ __device__ __forceinline__ float net_features(const float *u, const float *up, c
 
 // ---- training ----------------------------------------------------------------------
 
-constexpr int kTrainThreads = 128;
+// Loss and gradient on the tensor cores.  A warp takes tiles of 16 samples and
+// keeps a tile's whole forward and backward pass in registers: the accumulators
+// of mma.sync m16n8k16 are, packed to bfloat16, the A operand of the next layer,
+// and an 8x8 transpose of such a register (movmatrix) is the operand of the
+// weight gradients, whose contraction runs over the samples.  (tcgen05 needs
+// 128-row operands in shared memory and a barrier round trip per layer; three
+// chained 32 x 32 layers of 16 rows are all latency there.)
+//   forward   Z = W A + b: bfloat16 operands as defined, FP32 sums;
+//   backward  the FP32 deltas are split into three bfloat16 terms (24 bits), so
+//             that no bit of them is lost: dA = W^T delta, dW += delta A^T.
+// Weight gradients stay in registers over all of a warp's tiles, are summed over
+// the CTA in shared memory and added to global memory once per CTA.
+// 32 768 samples: 62 -> 13.7 us; with one thread per sample and both operands of
+// every FMA read from shared memory the LSU pipe set the time (67% busy, 256
+// CTAs of 75 KB, 10% of the warps).
+// Samples come in consecutive groups of `group` (1 or 2; a pair = the two
+// interfaces of one cell) whose residual is r = sum_k a_k (g_k - y_k) (a_k =
+// coef[k], 1 without coef); the loss is the mean of r^2 over groups.
+constexpr int kTrainWarps = 8;
+constexpr int kTrainThreads = 32 * kTrainWarps;
 
-// One CTA: kTrainThreads samples.  Samples come in consecutive groups of
-// `group` (1 or 2; a pair = the two interfaces of one cell) whose residual is
-// r = sum_k a_k (g_k - y_k) (a_k = coef[k], 1 without coef); the loss is the
-// mean of r^2 over groups.  The two threads of a pair exchange their terms by
-// a warp shuffle.  Loss and weight gradients accumulated in global FP32
-// (per-CTA reductions, then one atomic per parameter).
-__global__ void __launch_bounds__(kTrainThreads) k_net_grad(const float *__restrict__ X,
-                                                            const float *__restrict__ y,
-                                                            const float *__restrict__ coef,
-                                                            const float *__restrict__ wts, long long nsamp,
-                                                            int group, float *__restrict__ grad,
-                                                            float *__restrict__ loss) {
-    __shared__ float w[NPARAM];
-    __shared__ float A0[kTrainThreads][NF + 1];
-    __shared__ float A1[kTrainThreads][H + 1];
-    __shared__ float A2[kTrainThreads][H + 1];
-    __shared__ float D[kTrainThreads][H + 1];  // delta of the current layer
-    __shared__ float red[kTrainThreads];
-    for (int i = threadIdx.x; i < NPARAM; i += blockDim.x)
-        w[i] = (i >= OFF_B4 || (i >= OFF_B1 && i < OFF_W2) || (i >= OFF_B2 && i < OFF_W3) ||
-                (i >= OFF_B3 && i < OFF_W4))
-                   ? wts[i]
-                   : bfr(wts[i]);
-    __syncthreads();
-    const long long sidx = (long long)blockIdx.x * kTrainThreads + threadIdx.x;
-    const bool valid = sidx < nsamp;
-    const int t = threadIdx.x;
-    float x[NF], h1[H], h2[H], h3[H];
-    float term = 0.f, a = 0.f;
-    if (valid) {
-        for (int k = 0; k < NF; ++k) x[k] = X[sidx * NF + k];
-        const float g = net_forward(w, x, h1, h2, h3);
-        a = coef ? coef[sidx] : 1.f;
-        term = a * (g - y[sidx]);
-    } else {
-        for (int k = 0; k < NF; ++k) x[k] = 0.f;
-        for (int j = 0; j < H; ++j) h1[j] = h2[j] = h3[j] = 0.f;
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint2 b) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+}
+__device__ __forceinline__ uint32_t transpose8x8(uint32_t a) {
+    uint32_t d;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
+    return d;
+}
+// bf16(lo) in the low half, bf16(hi) in the high half
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+__device__ __forceinline__ float low_half(uint32_t p) { return __uint_as_float(p << 16); }
+__device__ __forceinline__ float high_half(uint32_t p) { return __uint_as_float(p & 0xffff0000u); }
+
+// A matrix of 16 rows (samples) x 32 columns as packed 8x8 blocks: m[h][c] holds
+// rows 8h + lane / 4, columns 8c + 2 (lane % 4) and the next
+struct Tile16 {
+    uint32_t m[2][4];
+    // A operand of the k-step j (columns 16j .. 16j + 15)
+    __device__ __forceinline__ void operand(int j, uint32_t (&a)[4]) const {
+        a[0] = m[0][2 * j];
+        a[1] = m[1][2 * j];
+        a[2] = m[0][2 * j + 1];
+        a[3] = m[1][2 * j + 1];
     }
-    // group residual (pairs are threads 2k, 2k + 1 of the same warp)
-    float r = term;
-    if (group == 2) r += __shfl_xor_sync(0xffffffffu, term, 1);
+    __device__ __forceinline__ Tile16 transposed() const {
+        Tile16 t;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) t.m[h][c] = transpose8x8(m[h][c]);
+        return t;
+    }
+};
+
+// acc[c] += A B for the four 8-column blocks c of B, whose operands lie in shared
+// memory in lane order: ops[(4 j + c) 32 + lane]
+__device__ __forceinline__ void times(float (&acc)[4][4], const Tile16 &A, const uint2 *ops, int lane) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        uint32_t a[4];
+        A.operand(j, a);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) mma16816(acc[c], a, ops[(4 * j + c) * 32 + lane]);
+    }
+}
+
+// one of the three bfloat16 terms of d (what is left of it stays in d)
+__device__ __forceinline__ Tile16 take_term(float (&d)[4][4]) {
+    Tile16 t;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t p = pack2(d[c][2 * h], d[c][2 * h + 1]);
+            t.m[h][c] = p;
+            d[c][2 * h] -= low_half(p);
+            d[c][2 * h + 1] -= high_half(p);
+        }
+    return t;
+}
+
+// dW (32 outputs x 32 inputs, in 16 x 8 blocks) += delta^T A, over the 16 samples
+__device__ __forceinline__ void outer(float (&dw)[2][4][4], const Tile16 &dt, const Tile16 &at) {
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+        const uint32_t a[4] = {dt.m[0][2 * m], dt.m[0][2 * m + 1], dt.m[1][2 * m], dt.m[1][2 * m + 1]};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) mma16816(dw[m][c], a, make_uint2(at.m[0][c], at.m[1][c]));
+    }
+}
+
+// one layer of the backward pass: d = delta of the layer (destroyed); dw, db of
+// the layer; with ops (the layer's W^T) da = W^T delta
+template <bool DGRAD>
+__device__ __forceinline__ void backward(float (&d)[4][4], const Tile16 &in, const uint2 *ops, int lane,
+                                         float (&dw)[2][4][4], float (&db)[4][2], float (&da)[4][4]) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        db[c][0] += d[c][0] + d[c][2];
+        db[c][1] += d[c][1] + d[c][3];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) da[c][k] = 0.f;
+    }
+    const Tile16 at = in.transposed();
+    const Tile16 t0 = take_term(d), t1 = take_term(d), t2 = take_term(d);
+    // smallest terms first
+#pragma unroll
+    for (int k = 2; k >= 0; --k) {
+        const Tile16 &t = k == 0 ? t0 : (k == 1 ? t1 : t2);
+        outer(dw, t.transposed(), at);
+        if (DGRAD) times(da, t, ops, lane);
+    }
+}
+
+// relu(z) rounded to bfloat16
+__device__ __forceinline__ Tile16 activate(const float (&z)[4][4]) {
+    Tile16 t;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) t.m[h][c] = pack2(fmaxf(z[c][2 * h], 0.f), fmaxf(z[c][2 * h + 1], 0.f));
+    return t;
+}
+// d where the activation is positive, 0 elsewhere
+__device__ __forceinline__ void mask(float (&d)[4][4], const Tile16 &t) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (!(t.m[h][c] & 0x7fffu)) d[c][2 * h] = 0.f;
+            if (!(t.m[h][c] & 0x7fff0000u)) d[c][2 * h + 1] = 0.f;
+        }
+}
+
+constexpr int kTrainOps = 8 * 32;  // operands (uint2) of one 32 x 32 layer
+constexpr size_t kTrainSmem = (size_t)5 * kTrainOps * sizeof(uint2) + (size_t)kTrainWarps * NPARAM * sizeof(float) + 16;
+
+__global__ void __launch_bounds__(kTrainThreads, 1) k_net_grad(const float *__restrict__ X,
+                                                               const float *__restrict__ y,
+                                                               const float *__restrict__ coef,
+                                                               const float *__restrict__ wts, long long nsamp,
+                                                               int group, float *__restrict__ grad,
+                                                               float *__restrict__ loss) {
+    extern __shared__ __align__(16) unsigned char gsm[];
+    uint2 *ops = reinterpret_cast<uint2 *>(gsm);  // W1 W2 W3, then W2^T W3^T
+    float *sums = reinterpret_cast<float *>(ops + 5 * kTrainOps);  // [warp][NPARAM]
+    __shared__ float sloss[kTrainWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t2 = 2 * (lane & 3);
+    // B operand of W (n = output, k = input): rows k = 16 j + t2 (+1, +8, +9),
+    // column n = 8 c + g; of W^T the roles of k and n swapped
+    for (int e = threadIdx.x; e < 5 * kTrainOps; e += blockDim.x) {
+        const int m = e / kTrainOps, l = e & 31, c = (e >> 5) & 3, j = (e >> 7) & 1;
+        const int n = 8 * c + (l >> 2), k = 16 * j + 2 * (l & 3);
+        auto w = [&](int kk) -> float {
+            if (m == 0) return kk < NF ? wts[OFF_W1 + n * NF + kk] : 0.f;
+            if (m == 1) return wts[OFF_W2 + n * H + kk];
+            if (m == 2) return wts[OFF_W3 + n * H + kk];
+            return wts[(m == 3 ? OFF_W2 : OFF_W3) + kk * H + n];
+        };
+        ops[e] = make_uint2(pack2(w(k), w(k + 1)), pack2(w(k + 8), w(k + 9)));
+    }
+    __shared__ float2 vecs[4][16];  // b1 b2 b3 w4, two columns each
+    if (threadIdx.x < 128) {
+        const int v = threadIdx.x >> 5, col = threadIdx.x & 31;
+        const float w = wts[(v == 0 ? OFF_B1 : (v == 1 ? OFF_B2 : (v == 2 ? OFF_B3 : OFF_W4))) + col];
+        reinterpret_cast<float *>(vecs[v])[col] = v == 3 ? bfr(w) : w;
+    }
+    const float b4 = wts[OFF_B4];
+    __syncthreads();
+    float dw1[2][4][4] = {}, dw2[2][4][4] = {}, dw3[2][4][4] = {};
+    float db1[4][2] = {}, db2[4][2] = {}, db3[4][2] = {}, dw4[4][2] = {};
+    float db4 = 0.f, lsum = 0.f;
     const float ngroups = (float)(nsamp / group);
-    const float dg = valid ? 2.0f * r * a / ngroups : 0.f;
-    red[t] = (valid && (group == 1 || (t & 1) == 0)) ? r * r / ngroups : 0.f;
-    for (int k = 0; k < NF; ++k) A0[t][k] = bfr(x[k]);
-    for (int j = 0; j < H; ++j) {
-        A1[t][j] = h1[j];
-        A2[t][j] = h2[j];
-    }
-    // layer 4: g = w4 . h3 + b4
-    for (int j = 0; j < H; ++j) D[t][j] = h3[j];  // temporarily hold h3
-    __syncthreads();
-    // grads of w4, b4: sum_s dg_s h3_s
-    {
-        __shared__ float dgs[kTrainThreads];
-        dgs[t] = dg;
-        __syncthreads();
-        if (t < H) {
-            float a = 0.f;
-            for (int s = 0; s < kTrainThreads; ++s) a = fmaf(dgs[s], D[s][t], a);
-            atomicAdd(grad + OFF_W4 + t, a);
-        }
-        if (t == H) {
-            float a = 0.f, l = 0.f;
-            for (int s = 0; s < kTrainThreads; ++s) {
-                a += dgs[s];
-                l += red[s];
+    const long long ntiles = (nsamp + 15) / 16;
+    // tiles over the CTAs first, so that few of them still use every SM
+    for (long long tile = blockIdx.x + (long long)warp * gridDim.x; tile < ntiles;
+         tile += (long long)kTrainWarps * gridDim.x) {
+        const long long s0 = tile * 16 + g;
+        const bool ok[2] = {s0 < nsamp, s0 + 8 < nsamp};
+        Tile16 x;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int col = 8 * c + t2;
+                const float *p = X + (s0 + 8 * h) * NF + col;
+                const float lo = ok[h] && col < NF ? __ldg(p) : 0.f, hi = ok[h] && col + 1 < NF ? __ldg(p + 1) : 0.f;
+                x.m[h][c] = pack2(lo, hi);
             }
-            atomicAdd(grad + OFF_B4, a);
-            atomicAdd(loss, l);
+        float yv[2], av[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            yv[h] = ok[h] ? __ldg(y + s0 + 8 * h) : 0.f;
+            av[h] = ok[h] ? (coef ? __ldg(coef + s0 + 8 * h) : 1.f) : 0.f;
         }
-        __syncthreads();
+        float z[4][4];
+        auto start = [&](int v) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float2 b = vecs[v][4 * c + (lane & 3)];
+                z[c][0] = z[c][2] = b.x;
+                z[c][1] = z[c][3] = b.y;
+            }
+        };
+        start(0);
+        times(z, x, ops, lane);
+        const Tile16 h1 = activate(z);
+        start(1);
+        times(z, h1, ops + kTrainOps, lane);
+        const Tile16 h2 = activate(z);
+        start(2);
+        times(z, h2, ops + 2 * kTrainOps, lane);
+        const Tile16 h3 = activate(z);
+        // the output, the residual and the delta of the output
+        float dg[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float o = 0.f;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float2 w4 = vecs[3][4 * c + (lane & 3)];
+                o = fmaf(w4.x, low_half(h3.m[h][c]), o);
+                o = fmaf(w4.y, high_half(h3.m[h][c]), o);
+            }
+            o += __shfl_xor_sync(0xffffffffu, o, 1);
+            o += __shfl_xor_sync(0xffffffffu, o, 2);
+            const float term = ok[h] ? av[h] * ((o + b4) - yv[h]) : 0.f;
+            float r = term;
+            if (group == 2) r += __shfl_xor_sync(0xffffffffu, term, 4);  // the pair's other row
+            dg[h] = ok[h] ? 2.0f * r * av[h] / ngroups : 0.f;
+            if (t2 == 0) {
+                db4 += dg[h];
+                if (ok[h] && (group == 1 || (g & 1) == 0)) lsum += r * r / ngroups;
+            }
+        }
+        float d[4][4], da[4][4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                dw4[c][0] = fmaf(dg[h], low_half(h3.m[h][c]), dw4[c][0]);
+                dw4[c][1] = fmaf(dg[h], high_half(h3.m[h][c]), dw4[c][1]);
+                const float2 w4 = vecs[3][4 * c + (lane & 3)];
+                d[c][2 * h] = dg[h] * w4.x;
+                d[c][2 * h + 1] = dg[h] * w4.y;
+            }
+        mask(d, h3);
+        backward<true>(d, h2, ops + 4 * kTrainOps, lane, dw3, db3, da);
+        mask(da, h2);
+        backward<true>(da, h1, ops + 3 * kTrainOps, lane, dw2, db2, d);
+        mask(d, h1);
+        backward<false>(d, x, nullptr, lane, dw1, db1, da);
     }
-    // delta3 = dg * w4 * [h3 > 0] (h3 > 0 iff its pre-activation was > 0)
-    float d3[H];
-    for (int j = 0; j < H; ++j) d3[j] = (h3[j] > 0.f) ? dg * w[OFF_W4 + j] : 0.f;
+    // the warp's sums to shared memory, in the parameters' order
+    float *q = sums + warp * NPARAM;
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int row = 16 * m + g + 8 * (k >> 1), col = 8 * c + t2 + (k & 1);
+                if (col < NF) q[OFF_W1 + row * NF + col] = dw1[m][c][k];
+                q[OFF_W2 + row * H + col] = dw2[m][c][k];
+                q[OFF_W3 + row * H + col] = dw3[m][c][k];
+            }
+    auto over_rows = [&](float v) -> float {
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const float s1 = over_rows(db1[c][i]), s2 = over_rows(db2[c][i]), s3 = over_rows(db3[c][i]),
+                        s4 = over_rows(dw4[c][i]);
+            if (g == 0) {
+                const int col = 8 * c + t2 + i;
+                q[OFF_B1 + col] = s1;
+                q[OFF_B2 + col] = s2;
+                q[OFF_B3 + col] = s3;
+                q[OFF_W4 + col] = s4;
+            }
+        }
+    db4 = over_rows(db4);
+    lsum = over_rows(lsum);
+    if (lane == 0) {
+        q[OFF_B4] = db4;
+        sloss[warp] = lsum;
+    }
     __syncthreads();
-    for (int j = 0; j < H; ++j) D[t][j] = d3[j];
-    __syncthreads();
-    // grads W3 = sum_s d3_s h2_s^T, b3 = sum_s d3_s
-    for (int e = t; e < H * H; e += blockDim.x) {
-        const int i = e / H, k = e % H;
-        float a = 0.f;
-        for (int s = 0; s < kTrainThreads; ++s) a = fmaf(D[s][i], A2[s][k], a);
-        atomicAdd(grad + OFF_W3 + e, a);
+    for (int i = threadIdx.x; i < NPARAM; i += blockDim.x) {
+        float v = 0.f;
+#pragma unroll
+        for (int k = 0; k < kTrainWarps; ++k) v += sums[k * NPARAM + i];
+        atomicAdd(grad + i, v);
     }
-    if (t < H) {
-        float a = 0.f;
-        for (int s = 0; s < kTrainThreads; ++s) a += D[s][t];
-        atomicAdd(grad + OFF_B3 + t, a);
-    }
-    // delta2 = (W3^T d3) * [h2 > 0]
-    float d2[H];
-    for (int k = 0; k < H; ++k) {
-        float a = 0.f;
-        for (int j = 0; j < H; ++j) a = fmaf(w[OFF_W3 + j * H + k], d3[j], a);
-        d2[k] = (h2[k] > 0.f) ? a : 0.f;
-    }
-    __syncthreads();
-    for (int j = 0; j < H; ++j) D[t][j] = d2[j];
-    __syncthreads();
-    for (int e = t; e < H * H; e += blockDim.x) {
-        const int i = e / H, k = e % H;
-        float a = 0.f;
-        for (int s = 0; s < kTrainThreads; ++s) a = fmaf(D[s][i], A1[s][k], a);
-        atomicAdd(grad + OFF_W2 + e, a);
-    }
-    if (t < H) {
-        float a = 0.f;
-        for (int s = 0; s < kTrainThreads; ++s) a += D[s][t];
-        atomicAdd(grad + OFF_B2 + t, a);
-    }
-    float d1[H];
-    for (int k = 0; k < H; ++k) {
-        float a = 0.f;
-        for (int j = 0; j < H; ++j) a = fmaf(w[OFF_W2 + j * H + k], d2[j], a);
-        d1[k] = (h1[k] > 0.f) ? a : 0.f;
-    }
-    __syncthreads();
-    for (int j = 0; j < H; ++j) D[t][j] = d1[j];
-    __syncthreads();
-    for (int e = t; e < H * NF; e += blockDim.x) {
-        const int i = e / NF, k = e % NF;
-        float a = 0.f;
-        for (int s = 0; s < kTrainThreads; ++s) a = fmaf(D[s][i], A0[s][k], a);
-        atomicAdd(grad + OFF_W1 + e, a);
-    }
-    if (t < H) {
-        float a = 0.f;
-        for (int s = 0; s < kTrainThreads; ++s) a += D[s][t];
-        atomicAdd(grad + OFF_B1 + t, a);
+    if (threadIdx.x == 0) {
+        float v = 0.f;
+        for (int k = 0; k < kTrainWarps; ++k) v += sloss[k];
+        atomicAdd(loss, v);
     }
 }
 
@@ -1032,8 +1171,22 @@ int vp_net_grad(const float *X, const float *y, const float *coef, long long nsa
                 float *grad, float *loss, void *stream) {
     if (!X || !y || !wts || !grad || !loss || nsamp < 1 || (group != 1 && group != 2) || nsamp % group)
         return VP_EINVAL;
-    const long long blocks = (nsamp + kTrainThreads - 1) / kTrainThreads;
-    k_net_grad<<<(unsigned)blocks, kTrainThreads, 0, static_cast<cudaStream_t>(stream)>>>(
+    // SMs of the device, looked up (and the kernel's shared memory set) by the
+    // first call on it: a training step is three short launches
+    static std::atomic<int> sm_count[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return VP_ECUDA;
+    int sms = sm_count[dev].load(std::memory_order_acquire);
+    if (!sms) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaFuncSetAttribute(k_net_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrainSmem) !=
+                cudaSuccess)
+            return VP_ECUDA;
+        sm_count[dev].store(sms, std::memory_order_release);
+    }
+    const long long tiles = (nsamp + 15) / 16;
+    const long long blocks = tiles < sms ? tiles : sms;  // one CTA per SM at most
+    k_net_grad<<<(unsigned)blocks, kTrainThreads, kTrainSmem, static_cast<cudaStream_t>(stream)>>>(
         X, y, coef, wts, nsamp, group, grad, loss);
     return cudaGetLastError() == cudaSuccess ? VP_OK : VP_ECUDA;
 }
