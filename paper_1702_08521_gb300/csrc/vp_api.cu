@@ -485,7 +485,8 @@ static int run_steps(vp_ctx *c, double dt, int split, int nsteps, double *accel_
     // graph path needs a capturable (non-legacy) stream
     const bool use_graph = c->stream != nullptr && c->stream != cudaStreamLegacy;
     vp_graph_cache &gc = c->graph;
-    if (c->opt_autotune && !capturing(c)) {
+    // (RK-MPP5 sweeps have tile rules of their own)
+    if (c->opt_autotune && c->g.scheme == VP_SCHEME_SL && !capturing(c)) {
         // each sweep tuned at the step it appears in: KDK kicks by dt/2 and
         // drifts by dt, DKD the other way round
         const double hd = split == VP_SPLIT_KDK ? dt : 0.5 * dt, hk = split == VP_SPLIT_KDK ? 0.5 * dt : dt;

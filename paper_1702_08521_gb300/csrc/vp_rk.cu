@@ -193,6 +193,129 @@ __global__ void __launch_bounds__(512) k_rk_cols(T *__restrict__ f, const LineSh
     }
 }
 
+// FP32 strided lines of grids with enough of them to fill the chip: a thread
+// owns whole lines (PAIR: two adjacent ones), so the three stages follow one
+// another without a barrier and in place -- the walk keeps the old values it
+// still needs in registers, and kRkEdge rows on each side hold zeros or, on a
+// periodic line, copies of its ends that the thread renews after each stage.  One
+// shared-memory tile in place of three; f^n itself comes through L2 again where a
+// stage needs it, one cell ahead of its use.  With three tiles the 16^3 x 32^3
+// sweeps held 8-12 warps per SM at 51-60% issue: drifts 930 us (880 with the vote
+// per block), now 690; kicks 780 -> 635.
+constexpr int kRkEdge = 4;
+
+template <typename T>
+struct InPlaceStore {
+    T *p;        // the stage's row (shared memory) or f^{n+1} (global)
+    const T *a;  // f^n of the next cell
+    long long step, astep;
+    T ca, cv, next;
+    int left;    // cells after the next one
+    __device__ __forceinline__ void operator()(int, T v) {
+        const T old = next;
+        if (left > 0) next = *a;
+        --left;
+        a += astep;
+        *p = fma(cv, v, mul_rn(ca, old));
+        p += step;
+    }
+};
+
+template <bool FULL, bool PAIR>
+__global__ void __launch_bounds__(64) k_rk_lines(float *__restrict__ f, const LineShift<float> *__restrict__ tab,
+                                                  SweepGeo geo, LimParams lp) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    using vp_core::P2;
+    constexpr int E = kRkEdge;
+    const int W = geo.W, L = geo.L;
+    float *A = reinterpret_cast<float *>(smraw) + E * W;  // row 0
+    // W columns of one outer block, or kblk whole blocks side by side
+    const bool packed = geo.kblk > 1;
+    const unsigned o0 = packed ? blockIdx.x * (unsigned)geo.kblk : fdiv(blockIdx.x, geo.fd_tpo);
+    const unsigned c0 = packed ? 0u : (blockIdx.x - o0 * geo.tpo) * (unsigned)W;
+    const int nblk = packed ? (int)(geo.outer - o0 < geo.kblk ? geo.outer - o0 : geo.kblk) : 1;
+    const int wc = packed ? nblk * (int)geo.inner : (int)((geo.inner - c0) < W ? (geo.inner - c0) : W);
+    auto column = [&](int cc, unsigned &o, unsigned &c) -> float * {
+        const unsigned k = packed ? fdiv((unsigned)cc, geo.fd_inner) : 0u;
+        o = o0 + k;
+        c = packed ? cc - k * (unsigned)geo.inner : c0 + cc;
+        return f + (long long)o * L * geo.inner + c;
+    };
+    unsigned o, c;
+    {
+        const int wv = W / geo.vec, r = (int)fdiv(threadIdx.x, geo.fd_wv), rstep = (int)fdiv(blockDim.x, geo.fd_wv);
+        const int cv = (threadIdx.x - r * wv) * geo.vec;
+        if (r < rstep && cv < wc) {
+            const float *from = column(cv, o, c) + (long long)r * geo.inner;
+            float *dst = A + r * W + cv;
+            const long long sstep = (long long)rstep * geo.inner;
+            for (int rr = r; rr < L; rr += rstep) {
+                if (geo.vec == 4) vp_tma::cp_async16(dst, from);
+                else if (geo.vec == 2) vp_tma::cp_async<8>(dst, from);
+                else vp_tma::cp_async<4>(dst, from);
+                from += sstep;
+                dst += rstep * W;
+            }
+        }
+    }
+    constexpr int N = PAIR ? 2 : 1;  // lines of the thread
+    const int cc = N * (int)threadIdx.x;
+    const bool act = cc < wc;
+    LineShift<float> sa{}, sb{};
+    float *const base = column(act ? cc : 0, o, c);  // of the thread's (first) line
+    if (act) {
+        sa = tab[vp_core::line_class(geo, o, c)];
+        sb = PAIR && cc + 1 < wc ? tab[vp_core::line_class(geo, o, c + 1)] : sa;
+    }
+    vp_tma::cp_async_wait_all();
+    __syncthreads();
+    if (!act) return;
+    // the edge rows of the thread's lines (row r of a periodic line: r mod L)
+    auto edges = [&]() {
+        for (int k = 0; k < E; ++k) {
+            const int lo = ((-1 - k) % L + L) % L, hi = k % L;
+            for (int i = 0; i < N; ++i) {
+                A[(-1 - k) * W + cc + i] = geo.periodic ? A[lo * W + cc + i] : 0.f;
+                A[(L + k) * W + cc + i] = geo.periodic ? A[hi * W + cc + i] : 0.f;
+            }
+        }
+    };
+    const bool both = PAIR && cc + 1 < wc && sa.sigma == sb.sigma;
+    edges();
+#pragma unroll 1
+    for (int stage = 0; stage < 3; ++stage) {
+        // the walk reads its line as restricted, and a stage reads what the one
+        // before it wrote: no access moves across this point
+        asm volatile("" ::: "memory");
+        const float ca = stage == 0 ? 0.f : (stage == 1 ? 0.75f : 1.f / 3.f);
+        const float cv = stage == 0 ? 1.f : (stage == 1 ? 0.25f : 2.f / 3.f);
+        // cells in walk order from row i0 on; the last stage writes f
+        auto store = [&](auto t, int col, int sigma) {
+            using U = decltype(t);
+            constexpr int M = sizeof(U) / 4;
+            const int i0 = sigma > 0 ? 0 : L - 1;
+            U *g = reinterpret_cast<U *>(base + (col - cc) + (long long)i0 * geo.inner);
+            U *d = stage == 2 ? g : reinterpret_cast<U *>(A + col + i0 * W);
+            const long long gs = (long long)sigma * (geo.inner / M);
+            return InPlaceStore<U>{d, g + (L > 1 ? gs : 0), stage == 2 ? gs : (long long)sigma * (W / M), gs,
+                                   U(ca), U(cv), *g, L - 1};
+        };
+        if (both) {
+            const vp_core::LineShiftP2 sh = vp_core::pair_shift(sa, sb);
+            vp_core::walk<P2, 5, false, FULL, E>(reinterpret_cast<const P2 *>(A + cc), W >> 1, L, sh, 0, L,
+                                                 P2((float)lp.alpha), lp.mp, lp.pp, store(P2(), cc, sh.sigma));
+        } else {
+            for (int k = (PAIR && cc + 1 < wc ? 1 : 0); k >= 0; --k) {
+                const LineShift<float> &sl = k ? sb : sa;
+                vp_core::walk<float, 5, false, FULL, E>(A + cc + k, W, L, sl, 0, L, (float)lp.alpha, lp.mp, lp.pp,
+                                                        store(0.f, cc + k, sl.sigma));
+            }
+        }
+        asm volatile("" ::: "memory");
+        if (geo.periodic && stage < 2) edges();
+    }
+}
+
 // Contiguous lines: R lines per CTA, each a row at odd pitch P (ghosts on
 // both sides); the result goes to a fourth tile at pitch Q and out in rows.
 template <typename T, bool FULL>
@@ -287,7 +410,39 @@ int launch_rk(vp_ctx *c, int kick, int dim) {
     const LimParams lp{c->g.alpha, c->g.mp, c->g.pp};
     T *f = static_cast<T *>(c->f);
     const int L = geo.L;
-    if (geo.inner > 1) {
+    // whole lines per thread where that gives every SM eight warps of them
+    // (smaller grids need the segments' parallelism)
+    const bool even = geo.inner % 2 == 0 && (reinterpret_cast<uintptr_t>(c->f) & 7) == 0 && c->opt_impl != 1;
+    if (sizeof(T) == 4 && geo.inner > 1 && geo.outer * geo.inner >= 8LL * 64 * c->sm_count &&
+        (size_t)(L + 2 * kRkEdge) * 64 * sizeof(float) <= 100 * 1024) {
+        int W = 64;
+        geo.kblk = 1;
+        if (geo.inner < W) {
+            geo.kblk = W / (int)geo.inner;
+            W = geo.kblk * (int)geo.inner;
+        }
+        geo.W = W;
+        geo.fd_inner = make_fastdiv((unsigned)geo.inner);
+        geo.vec = 4;
+        while (geo.inner % geo.vec || W % geo.vec) geo.vec /= 2;
+        geo.tpo = (unsigned)((geo.inner + W - 1) / W);
+        geo.fd_tpo = make_fastdiv(geo.tpo);
+        geo.fd_wv = make_fastdiv((unsigned)(W / geo.vec));
+        const long long tiles = geo.kblk > 1 ? (geo.outer + geo.kblk - 1) / geo.kblk : geo.outer * geo.tpo;
+        if (tiles >= (1LL << 31)) return vp_fail(c, VP_ENOTSUP, "sweep has too many tiles");
+        const bool pair = even && W % 2 == 0;
+        int threads = ((pair ? W / 2 : W) + 31) / 32 * 32;
+        if (threads < W / geo.vec) threads = (W / geo.vec + 31) / 32 * 32;
+        const size_t smem = (size_t)(L + 2 * kRkEdge) * W * sizeof(float);
+        const bool full = c->g.mp && c->g.pp;
+        float *ff = static_cast<float *>(c->f);
+        const LineShift<float> *ft = static_cast<const LineShift<float> *>(c->d_shift);
+        const unsigned nb = (unsigned)tiles;
+        if (pair && full) k_rk_lines<true, true><<<nb, threads, smem, c->stream>>>(ff, ft, geo, lp);
+        else if (pair) k_rk_lines<false, true><<<nb, threads, smem, c->stream>>>(ff, ft, geo, lp);
+        else if (full) k_rk_lines<true, false><<<nb, threads, smem, c->stream>>>(ff, ft, geo, lp);
+        else k_rk_lines<false, false><<<nb, threads, smem, c->stream>>>(ff, ft, geo, lp);
+    } else if (geo.inner > 1) {
         const int gp = geo.periodic ? 0 : VP_GHOST;
         // up to 128 lines per tile within 100 KB, narrower for long lines;
         // segments of at least 16 cells (each stage restarts the walk at every
@@ -385,6 +540,11 @@ void rk_attrs() {
 int vp_rk_setup() {
     rk_attrs<float>();
     rk_attrs<double>();
+    constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaFuncSetAttribute(k_rk_lines<true, true>, attr, 100 * 1024);
+    cudaFuncSetAttribute(k_rk_lines<true, false>, attr, 100 * 1024);
+    cudaFuncSetAttribute(k_rk_lines<false, true>, attr, 100 * 1024);
+    cudaFuncSetAttribute(k_rk_lines<false, false>, attr, 100 * 1024);
     return cudaGetLastError() == cudaSuccess ? VP_OK : VP_ECUDA;
 }
 

@@ -145,3 +145,36 @@ def test_rk_two_line_kernel_gives_the_same_bits(dims, nx, nv):
         sim.close()
     for a, b in zip(out[0], out[1]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("xbc", [0, 1])
+@pytest.mark.parametrize("n1,nv", [(12, [40, 36]), (3, [21, 33]), (7, [64, 18])])
+def test_whole_lines_in_place_give_the_same_bits(xbc, n1, nv):
+    """Grids with many lines run the three stages of whole lines in place, small
+    grids through three tiles: every line of a large grid's strided sweeps (even
+    and odd rows, lines shorter than the stencil, both boundaries and directions,
+    one and two lines per thread) gives the bits it gives in a grid of one x2 row."""
+    n2 = 100_000 // (n1 * min(nv)) + 1
+    rng = np.random.default_rng(n1)
+    f = (rng.random((n1, n2, *nv)) ** 2 * (rng.random((n1, n2, *nv)) < 0.8)).astype(np.float32)
+    acc = rng.uniform(-4.0, 4.0, size=(n1, n2))
+    rows = [0, n2 // 2, n2 - 1]
+
+    def run(n, data, a, kick, d, impl):
+        g = dict(rk_grid(2, [n1, n], nv, xbc=xbc), xlo=[0.0, 0.0], xhi=[1.0, 0.01 * n])
+        sim = V.Simulation(g, precision=V.VP_F32)
+        V.vp_set_option(sim.ctx, V.VP_OPT_SWEEP_IMPL, impl)
+        to_gpu(sim, data)
+        if kick:
+            V.vp_kick_sweep(sim.ctx, d, 0.008, accel_tensor(sim, a))  # |nu| < 0.38
+        else:
+            V.vp_drift_sweep(sim.ctx, d, 0.012)
+        out = from_gpu(sim).reshape(n1, n, *nv)
+        sim.close()
+        return out
+    for kick, d in ((0, 0), (1, 0)):
+        big = [run(n2, f, acc, kick, d, impl) for impl in (0, 1)]
+        assert np.array_equal(big[0], big[1])
+        for r in rows:
+            one = run(1, np.ascontiguousarray(f[:, r:r + 1]), np.ascontiguousarray(acc[:, r]), kick, d, 0)
+            assert np.array_equal(big[0][:, r], one[:, 0]), (kick, d, r)
