@@ -175,28 +175,46 @@ int sweep_all(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
     if (c->g.scheme == VP_SCHEME_RK) return vp_launch_rk_sweep(c, kick, dim, dt, accel);
     if (c->opt_autotune && !c->tune[kick][dim].valid && !capturing(c))
         if ((rc = vp_tune_sweep(c, kick, dim, dt, accel))) return rc;
-    return vp_launch_sweep(c, kick, dim, dt, accel);
+    return vp_launch_sweep(c, kick, dim, dt, accel, false);
+}
+
+// the sweeps of one stage of a step (kicks v_1 .. v_D, drifts x_D .. x_1): the
+// tables of those that read one made by one launch (a launch per sweep cost
+// 3.5-4.6 us each)
+int stage_sweeps(vp_ctx *c, int kick, double dt, const double *accel) {
+    const int D = c->g.dx;
+    int rc;
+    unsigned dims = 0;
+    if (c->g.scheme == VP_SCHEME_SL) {
+        for (int d = 0; d < D; ++d)
+            if (vp_sweep_reads_table(c, kick, d)) dims |= 1u << d;
+        if ((dims & (dims - 1)) == 0) dims = 0;  // one table: its sweep makes it
+        if (dims && (rc = vp_launch_shift_tables(c, kick, dims, dt, accel))) return rc;
+    }
+    for (int i = 0; i < D; ++i) {
+        const int d = kick ? i : D - 1 - i;
+        const double *a = kick ? accel + d * c->NX : nullptr;
+        rc = dims & (1u << d) ? vp_launch_sweep(c, kick, d, dt, a, true) : sweep_all(c, kick, d, dt, a);
+        if (rc) return rc;
+    }
+    return VP_OK;
 }
 
 // one Strang step (Eq. 55) on the context stream
 // one Strang step; with wts the drifts are learned sweeps of that network
 int enqueue_step(vp_ctx *c, double dt, int split, double *acc, const float *wts) {
     const vp_grid &g = c->g;
-    const long long NX = c->NX;
     int rc;
     // the drifts x_D ... x_1 of a stage; learned drifts alternate between f
     // and the library's second array (each reads f^n whole and writes the
     // new lines apart), with the network operands made once per stage and
     // one copy back into f only after an odd number of drifts
     auto drifts = [&](double h) {
-        if (!wts) {
-            for (int d = g.dx - 1; d >= 0; --d)
-                if ((rc = sweep_all(c, 0, d, h, nullptr))) return rc;
-            return VP_OK;
-        }
+        if (!wts) return stage_sweeps(c, 0, h, nullptr);
+        if ((rc = vp_launch_shift_tables(c, 0, (1u << g.dx) - 1, h, nullptr))) return rc;
         float *src = static_cast<float *>(c->f), *dst = static_cast<float *>(c->d_learn_out);
         for (int d = g.dx - 1; d >= 0; --d) {
-            if ((rc = vp_learned_drift_io(c, d, h, wts, 1, src, dst, d == g.dx - 1))) return rc;
+            if ((rc = vp_learned_drift_io(c, d, h, wts, 1, src, dst, d == g.dx - 1, true))) return rc;
             float *t = src;
             src = dst;
             dst = t;
@@ -207,19 +225,16 @@ int enqueue_step(vp_ctx *c, double dt, int split, double *acc, const float *wts)
         return VP_OK;
     };
     if (split == VP_SPLIT_KDK) {
-        for (int d = 0; d < g.dv; ++d)
-            if ((rc = sweep_all(c, 1, d, 0.5 * dt, acc + d * NX))) return rc;
+        if ((rc = stage_sweeps(c, 1, 0.5 * dt, acc))) return rc;
         if ((rc = drifts(dt))) return rc;
         if ((rc = vp_launch_moment(c, c->d_rho_s))) return rc;
         if ((rc = vp_launch_poisson(c, c->d_rho_s, nullptr, acc))) return rc;
-        for (int d = 0; d < g.dv; ++d)
-            if ((rc = sweep_all(c, 1, d, 0.5 * dt, acc + d * NX))) return rc;
+        if ((rc = stage_sweeps(c, 1, 0.5 * dt, acc))) return rc;
     } else {
         if ((rc = drifts(0.5 * dt))) return rc;
         if ((rc = vp_launch_moment(c, c->d_rho_s))) return rc;
         if ((rc = vp_launch_poisson(c, c->d_rho_s, nullptr, acc))) return rc;
-        for (int d = 0; d < g.dv; ++d)
-            if ((rc = sweep_all(c, 1, d, dt, acc + d * NX))) return rc;
+        if ((rc = stage_sweeps(c, 1, dt, acc))) return rc;
         if ((rc = drifts(0.5 * dt))) return rc;
     }
     return VP_OK;
@@ -278,7 +293,7 @@ int vp_create(const vp_grid *grid, void *cuda_stream, vp_ctx **out) {
             if (pass) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(static_cast<char *>(c->d_arena) + at);
             at += (bytes + 255) & ~size_t(255);
         };
-        take(c->d_shift, shift_bytes);
+        take(c->d_shift, shift_bytes * c->g.dx);
         take(c->d_rho, sizeof(double) * c->NX);
         take(c->d_phi, sizeof(double) * c->NX);
         take(c->d_acc, sizeof(double) * c->NX * c->g.dx);

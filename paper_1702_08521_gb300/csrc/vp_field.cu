@@ -155,6 +155,10 @@ constexpr int kFftMaxRad = 12;  // factors of an axis length <= 4096
 struct FftPlan {
     int n, nr;
     int rad[kFftMaxRad];
+    // divisors of the index arithmetic: butterflies per line and distance of a
+    // pass, the line length (an integer division is ~150 cycles of latency, and
+    // a 64-point line is one warp with nothing to hide it)
+    FastDiv fd_m[kFftMaxRad], fd_ns[kFftMaxRad], fd_n;
 };
 
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
@@ -176,8 +180,8 @@ __device__ double2 *fft_lines(double2 *x, double2 *y, const double2 *w, const Ff
         const int m = n / r, ts = m / Ns;  // butterflies per line, table stride of exp(-2 pi i / (Ns r))
         if (r == 4 || r == 2) {
             for (int t = threadIdx.x; t < B * m; t += blockDim.x) {
-                const int b = t / m, j = t - b * m;
-                const int k = j % Ns;
+                const int b = B == 1 ? 0 : (int)fdiv((unsigned)t, p.fd_m[f]), j = t - b * m;
+                const int k = (int)fmod_u((unsigned)j, p.fd_ns[f]);
                 const double2 *xi = x + b * n + j;
                 double2 *yo = y + b * n + (j - k) * r + k;
                 auto tw = [&](int q) {
@@ -202,9 +206,9 @@ __device__ double2 *fft_lines(double2 *x, double2 *y, const double2 *w, const Ff
             // direct: output o = (block, q, k) sums r inputs with the roots
             // exp(-2 pi i p (k + q Ns) / (Ns r))
             for (int t = threadIdx.x; t < B * n; t += blockDim.x) {
-                const int b = t / n, o = t - b * n;
+                const int b = B == 1 ? 0 : (int)fdiv((unsigned)t, p.fd_n), o = t - b * n;
                 const int blk = o / (Ns * r), kq = o - blk * (Ns * r);
-                const double2 *xi = x + b * n + blk * Ns + kq % Ns;
+                const double2 *xi = x + b * n + blk * Ns + (int)fmod_u((unsigned)kq, p.fd_ns[f]);
                 const int step = kq * ts;  // < n
                 double2 a0 = xi[0], a1 = make_double2(0.0, 0.0);
                 int idx = 0;
@@ -282,7 +286,7 @@ __global__ void __launch_bounds__(256) k_fft_lines(double2 *__restrict__ a, FftA
         // contiguous lines of the padded grid: the line's outer indices, and
         // its row of the box (or a line of zeros)
         for (int t = threadIdx.x; t < nb * n; t += blockDim.x) {
-            const int b = t / n, j = t - b * n;
+            const int b = B == 1 ? 0 : (int)fdiv((unsigned)t, f.p.fd_n), j = t - b * n;
             long long r = l0 + b, row = 0, mul = f.nbox[f.dims - 1];
             bool in = j < f.nbox[f.dims - 1];
             for (int d = f.dims - 2; d >= 0; --d) {
@@ -298,7 +302,7 @@ __global__ void __launch_bounds__(256) k_fft_lines(double2 *__restrict__ a, FftA
         for (int t = threadIdx.x; t < nb * n; t += blockDim.x) x[t] = a[base + t];
     } else {
         for (int t = threadIdx.x; t < nb * n; t += blockDim.x) {
-            const int j = t / nb, b = t - j * nb;
+            const int j = nb == 1 ? t : t / nb, b = t - j * nb;
             x[b * n + j] = a[base + (long long)j * f.inner + b];
         }
     }
@@ -309,11 +313,11 @@ __global__ void __launch_bounds__(256) k_fft_lines(double2 *__restrict__ a, FftA
             int j, b;
             long long g;
             if (f.inner == 1) {
-                b = t / n;
+                b = B == 1 ? 0 : (int)fdiv((unsigned)t, f.p.fd_n);
                 j = t - b * n;
                 g = base + t;
             } else {
-                j = t / nb;
+                j = nb == 1 ? t : t / nb;
                 b = t - j * nb;
                 g = base + (long long)j * f.inner + b;
             }
@@ -334,7 +338,7 @@ __global__ void __launch_bounds__(256) k_fft_lines(double2 *__restrict__ a, FftA
         for (int t = threadIdx.x; t < nb * n; t += blockDim.x) a[base + t] = r[t];
     } else {
         for (int t = threadIdx.x; t < nb * n; t += blockDim.x) {
-            const int j = t / nb, b = t - j * nb;
+            const int j = nb == 1 ? t : t / nb, b = t - j * nb;
             a[base + (long long)j * f.inner + b] = r[b * n + j];
         }
     }
@@ -889,6 +893,13 @@ FftPlan fft_plan(int n) {
             r /= q;
         }
     }
+    int Ns = 1;
+    for (int f = 0; f < p.nr; ++f) {
+        p.fd_m[f] = make_fastdiv((unsigned)(n / p.rad[f]));
+        p.fd_ns[f] = make_fastdiv((unsigned)Ns);
+        Ns *= p.rad[f];
+    }
+    p.fd_n = make_fastdiv((unsigned)n);
     return p;
 }
 

@@ -865,7 +865,7 @@ constexpr int kOpAlloc = (kOpBytes + 127) / 128 * 128;
 
 __global__ void k_net_umma(const float *__restrict__ wts, unsigned char *__restrict__ out) {
     constexpr int K = vp_umma::kK;
-    for (int e = threadIdx.x; e < 3 * 32 * K + 16 * K; e += blockDim.x) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < 3 * 32 * K + 16 * K; e += gridDim.x * blockDim.x) {
         int layer, n, k;
         if (e < 3 * 32 * K) {
             layer = e / (32 * K);
@@ -1283,7 +1283,7 @@ int vp_learned_prepare(vp_ctx *c) {
 // net = true the network operands are made from wts first (a stage of
 // several drifts with one network makes them once)
 int vp_learned_drift_io(vp_ctx *c, int dim, double dt, const float *wts, int use_net, const float *fin,
-                        float *fout, bool net) {
+                        float *fout, bool net, bool tab_ready) {
     const LineGeo q = line_geo(c->g, c->NX, c->NV, 0, dim);
     // tile: every class j of its lines times a block of the other indices,
     // about 128 lines (columns)
@@ -1317,13 +1317,14 @@ int vp_learned_drift_io(vp_ctx *c, int dim, double dt, const float *wts, int use
     const size_t smem = (size_t)kLC * kABytes + kOpAlloc;
     const long long blocks = q.outer * tl.tpo;
     if (blocks >= (1LL << 31)) return vp_fail(c, VP_ENOTSUP, "learned sweep has too many tiles");
-    int rc = vp_launch_shift_table(c, 0, dim, dt, nullptr);
+    // the drifts' shifts: with the network's operands, once for a stage
+    int rc = tab_ready ? VP_OK : vp_launch_shift_tables(c, 0, 1u << dim, dt, nullptr);
     if (rc != VP_OK) return rc;
     if (net) {
-        k_net_umma<<<1, 256, 0, c->stream>>>(wts, static_cast<unsigned char *>(c->d_netfrag));
+        k_net_umma<<<(4 * 32 * vp_umma::kK + 255) / 256, 256, 0, c->stream>>>(wts, static_cast<unsigned char *>(c->d_netfrag));
         c->launches++;
     }
-    const LineShift<float> *tab = static_cast<const LineShift<float> *>(c->d_shift);
+    const LineShift<float> *tab = static_cast<const LineShift<float> *>(c->d_shift) + dim * c->shift_cap;
     const uint4 *ops = static_cast<const uint4 *>(c->d_netfrag);
     if (q.periodic)
         k_learned_walk<true, kLC><<<(unsigned)blocks, threads, smem, c->stream>>>(
@@ -1352,7 +1353,8 @@ int vp_learned_sweep(vp_ctx *c, int kick, int dim, double dt, const double *acce
     int rc = vp_learned_prepare(c);
     if (rc != VP_OK) return rc;
     float *fout = static_cast<float *>(c->d_learn_out);
-    if ((rc = vp_learned_drift_io(c, dim, dt, wts, use_net, static_cast<const float *>(c->f), fout, true)))
+    if ((rc = vp_learned_drift_io(c, dim, dt, wts, use_net, static_cast<const float *>(c->f), fout, true,
+                                  false)))
         return rc;
     VP_CUDA_TRY(c, cudaMemcpyAsync(c->f, fout, (size_t)c->ncell * sizeof(float), cudaMemcpyDeviceToDevice,
                                    c->stream));
@@ -1381,11 +1383,11 @@ int vp_fine_flux(vp_ctx *c, int kick, int dim, double dt, const double *accel_de
     while (W > 8 && bytes(W) > 72 * 1024) W /= 2;  // three CTAs per SM
     set_width(t, W);
     const size_t smem = bytes(W);
-    const int rc = vp_launch_shift_table_f32(c, kick, dim, dt, accel_dev);
+    const int rc = vp_launch_shift_tables_f32(c, kick, 1u << dim, dt, accel_dev);
     if (rc) return rc;
     VP_CUDA_TRY(c, cudaFuncSetAttribute(k_fine_flux<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
     VP_CUDA_TRY(c, cudaFuncSetAttribute(k_fine_flux<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    const LineShift<float> *tab = static_cast<const LineShift<float> *>(c->d_shift);
+    const LineShift<float> *tab = static_cast<const LineShift<float> *>(c->d_shift) + dim * c->shift_cap;
     const unsigned blocks = (unsigned)((t.lines + t.W - 1) / t.W);
     if (prefix)
         k_fine_flux<true><<<blocks, 256, smem, c->stream>>>(static_cast<const float *>(c->f), t, tab, every, G_dev,
@@ -1492,8 +1494,8 @@ int vp_make_samples(vp_ctx *coarse, int kick, int dim, double dt, const double *
     const LineGeo q = line_geo(c->g, c->NX, c->NV, kick, dim);
     LineTile t = line_tile(q);
     int rc;
-    if ((rc = vp_launch_shift_table_f32(c, kick, dim, dt, accel_dev))) return rc;
-    const LineShift<float> *tab = static_cast<const LineShift<float> *>(c->d_shift);
+    if ((rc = vp_launch_shift_tables_f32(c, kick, 1u << dim, dt, accel_dev))) return rc;
+    const LineShift<float> *tab = static_cast<const LineShift<float> *>(c->d_shift) + dim * c->shift_cap;
     const size_t xbytes = (size_t)kSampleThreads * NF * sizeof(float);
     auto bytes = [&](int W) { return xbytes + (size_t)3 * W * ((q.L + 2 * kEdge) | 1) * sizeof(float); };
     int W = 32;

@@ -198,22 +198,26 @@ inline SweepGeo vp_make_geo(const vp_ctx *c, int kick, int dim) {
     } while (0)
 
 // launchers implemented in the kernel files; all enqueue on ctx->stream
-int vp_launch_shift_table(vp_ctx *c, int kick, int dim, double dt, const double *accel);
+// the shift tables of the sweeps along the axes of the bit set `dims`, at d_shift
+// + dim * shift_cap; accel: of one axis its array, of several the whole field
+int vp_launch_shift_tables(vp_ctx *c, int kick, unsigned dims, double dt, const double *accel);
 // the same in FP32 whatever the grid's precision (the learned part's kernels)
-int vp_launch_shift_table_f32(vp_ctx *c, int kick, int dim, double dt, const double *accel);
+int vp_launch_shift_tables_f32(vp_ctx *c, int kick, unsigned dims, double dt, const double *accel);
+bool vp_sweep_reads_table(vp_ctx *c, int kick, int dim);
 // the context stream is being captured into a graph (no synchronising calls)
 bool vp_capturing(const vp_ctx *c);
 // buffers and kernel attributes of the learned sweep (outside any stream capture)
 int vp_learned_prepare(vp_ctx *c);
 // one learned drift along dim from fin to fout (distinct arrays of f's size);
-// net: make the network operands from wts first
+// net: make the network operands from wts first; tab_ready: the drift's shift table is made already
 int vp_learned_drift_io(vp_ctx *c, int dim, double dt, const float *wts, int use_net, const float *fin,
-                        float *fout, bool net);
+                        float *fout, bool net, bool tab_ready);
 // RK-MPP5 sweeps: kernel attributes once per process, one sweep (table + fused stages)
 int vp_rk_setup();
 int vp_launch_rk_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel);
-// one SL sweep, its shift table included where it needs one
-int vp_launch_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel);
+// one SL sweep; tab_ready: its shift table is made already, else it makes it
+// where it needs one
+int vp_launch_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel, bool tab_ready);
 // autotune sweep (kick, dim) at its own shifts (dt, accel); outside stream capture only
 int vp_tune_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel);
 int vp_launch_moment(vp_ctx *c, double *rho);

@@ -551,27 +551,36 @@ __global__ void __launch_bounds__(512) k_sweep_cols_tma(const __grid_constant__ 
     if (threadIdx.x == 0) vp_tma::wait_all<0>();
 }
 
-// Shift decomposition of every line class, in double precision so that the
-// integer part is exact: s = c dt / h, n = nearest integer (halves away from
+// Shift decomposition of every line class of the sweeps along the axes
+// `dims` (one table per axis, `cap` entries apart), in double precision so that
+// the integer part is exact: s = c dt / h, n = nearest integer (halves away from
 // zero), zeta = s - n, nu = |zeta|; the weights are the CSL polynomials at nu.
-// Eight lanes per class, one weight each (one thread per class spent 5.5 us in
-// a chain of 49 FP64 FMAs and a division).
+// Eight lanes per class, one weight each (one thread per class spent 5.5 us in a
+// chain of 49 FP64 FMAs and a division), and the axes of a stage in one launch.
+struct TableAxes {
+    int n;
+    int dim[3], nclass[3];
+    double lo[3], dvel[3], h[3];
+    const double *accel[3];
+};
+
 template <typename T>
-__global__ void k_shift_table(LineShift<T> *__restrict__ tab, int nclass, int kick, double lo,
-                              double dvel, const double *__restrict__ accel, double dt, double h,
-                              const __grid_constant__ WPoly wp) {
+__global__ void k_shift_table(LineShift<T> *__restrict__ tab, long long cap, int kick, const __grid_constant__ TableAxes ax,
+                              double dt, const __grid_constant__ WPoly wp) {
+    const int a = blockIdx.y;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int c = (int)(t >> 3), k = (int)t & 7;
-    if (c >= nclass) return;
-    const double speed = kick ? accel[c] : vp_core::cell_centre(lo, dvel, c);
+    if ((t >> 3) >= ax.nclass[a]) return;
+    LineShift<T> *e = tab + ax.dim[a] * cap + c;
+    const double speed = kick ? ax.accel[a][c] : vp_core::cell_centre(ax.lo[a], ax.dvel[a], c);
     LineShift<T> sh;
-    const double nu = vp_core::split_shift(speed, dt, h, sh);
+    const double nu = vp_core::split_shift(speed, dt, ax.h[a], sh);
     if (k < 7) {
-        tab[c].w[k] = (T)vp_core::csl_weight(wp, k, nu);
+        e->w[k] = (T)vp_core::csl_weight(wp, k, nu);
     } else {
-        tab[c].nu = sh.nu;
-        tab[c].n = sh.n;
-        tab[c].sigma = sh.sigma;
+        e->nu = sh.nu;
+        e->n = sh.n;
+        e->sigma = sh.sigma;
     }
 }
 
@@ -695,7 +704,7 @@ int shift_source(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, int w, lo
                  ShiftSrc<T> &src) {
     const vp_grid &g = c->g;
     src = ShiftSrc<T>{};
-    if (!table && own_shifts(c, geo, tiles)) {
+    if (!table && !sw.tab_ready && own_shifts(c, geo, tiles)) {
         const int d = sw.dim;
         src.accel = sw.kick ? sw.accel : nullptr;
         src.lo = g.vlo[d];
@@ -706,12 +715,12 @@ int shift_source(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, int w, lo
         src.wp = c->wp;
         return VP_OK;
     }
-    src.tab = static_cast<const LineShift<T> *>(c->d_shift);
+    src.tab = static_cast<const LineShift<T> *>(c->d_shift) + sw.dim * c->shift_cap;
     if (sw.tab_ready) {
         src.tab += sw.cls0;
         return VP_OK;
     }
-    return vp_launch_shift_table(c, sw.kick, sw.dim, sw.dt, sw.accel);
+    return vp_launch_shift_tables(c, sw.kick, 1u << sw.dim, sw.dt, sw.accel);
 }
 
 template <typename T>
@@ -915,9 +924,9 @@ SweepTune default_tune(const vp_ctx *c, const SweepGeo &geo) {
 }
 
 template <typename T>
-int launch_sweep_t(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+int launch_sweep_t(vp_ctx *c, int kick, int dim, double dt, const double *accel, bool tab_ready) {
     const SweepGeo geo = vp_make_geo(c, kick, dim);
-    const SweepShift sw{kick, dim, dt, accel, false, 0};
+    const SweepShift sw{kick, dim, dt, accel, tab_ready, 0};
     SweepTune tu = c->tune[kick][dim];
     if (!tu.valid || (c->opt_impl && tu.impl != c->opt_impl)) tu = default_tune<T>(c, geo);
     if (c->opt_impl == 1) tu.impl = 1;
@@ -995,7 +1004,7 @@ int tune_t(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
     else
         rc = cudaMemcpyAsync(scratch, src, bytes, cudaMemcpyDeviceToDevice, c->stream) == cudaSuccess
                  ? VP_OK : vp_fail(c, VP_ECUDA, "tuning copy failed");
-    if (rc == VP_OK) rc = vp_launch_shift_table(c, kick, dim, dt, accel);
+    if (rc == VP_OK) rc = vp_launch_shift_tables(c, kick, 1u << dim, dt, accel);
     if (rc == VP_OK) {
         void *f = c->f;
         c->f = scratch;
@@ -1136,24 +1145,47 @@ int tune_on(vp_ctx *c, const SweepShift &sw, const SweepGeo &geo, const SweepGeo
 void VP_UNIT(vp_sweep_attrs)() { set_attrs<unit_t>(); }
 
 #if VP_SWEEP_ORDER == 7
-int VP_UNIT(vp_launch_shift_table)(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+int VP_UNIT(vp_launch_shift_tables)(vp_ctx *c, int kick, unsigned dims, double dt, const double *accel) {
     const vp_grid &g = c->g;
-    const int nclass = kick ? (int)c->NX : g.nv[dim];
-    const double h = kick ? (g.vhi[dim] - g.vlo[dim]) / g.nv[dim] : (g.xhi[dim] - g.xlo[dim]) / g.nx[dim];
-    const double dvel = (g.vhi[dim] - g.vlo[dim]) / g.nv[dim];
+    TableAxes ax{};
+    int most = 0;
+    for (int d = 0; d < g.dx; ++d) {
+        if (!(dims & (1u << d))) continue;
+        const int i = ax.n++;
+        const double dvel = (g.vhi[d] - g.vlo[d]) / g.nv[d];
+        ax.dim[i] = d;
+        ax.nclass[i] = kick ? (int)c->NX : g.nv[d];
+        ax.lo[i] = g.vlo[d];
+        ax.dvel[i] = dvel;
+        ax.h[i] = kick ? dvel : (g.xhi[d] - g.xlo[d]) / g.nx[d];
+        // one axis: its own array; several: the components of a field
+        ax.accel[i] = kick ? accel + ((dims & (dims - 1)) ? d * c->NX : 0) : nullptr;
+        most = ax.nclass[i] > most ? ax.nclass[i] : most;
+    }
     const int th = 64;
-    const long long bl = (8LL * nclass + th - 1) / th;
-    k_shift_table<unit_t><<<(unsigned)bl, th, 0, c->stream>>>(static_cast<LineShift<unit_t> *>(c->d_shift), nclass,
-                                                              kick, g.vlo[dim], dvel, accel, dt, h, c->wp);
+    const dim3 grid((unsigned)((8LL * most + th - 1) / th), (unsigned)ax.n);
+    k_shift_table<unit_t><<<grid, th, 0, c->stream>>>(static_cast<LineShift<unit_t> *>(c->d_shift), c->shift_cap, kick,
+                                                      ax, dt, c->wp);
     c->launches++;
     VP_CUDA_TRY(c, cudaGetLastError());
     return VP_OK;
 }
 
+// whether the sweep along dim reads the context's table (false: its CTAs make
+// their own shifts)
+bool VP_UNIT(vp_sweep_reads_table)(vp_ctx *c, int kick, int dim) {
+    SweepGeo geo = vp_make_geo(c, kick, dim);
+    SweepTune tu = c->tune[kick][dim];
+    if (!tu.valid || (c->opt_impl && tu.impl != c->opt_impl)) tu = default_tune<unit_t>(c, geo);
+    const long long w = geo.inner > 1 ? (geo.inner < tu.W ? geo.inner : tu.W) : (geo.outer < tu.W ? geo.outer : tu.W);
+    const long long per = geo.inner > 1 && geo.inner < tu.W ? tu.W / geo.inner : 1;  // blocks per tile
+    const long long tiles = geo.inner > 1 ? (geo.outer + per - 1) / per * ((geo.inner + w - 1) / w) : (geo.outer + w - 1) / w;
+    return tu.impl == 2 || !own_shifts(c, geo, tiles);
+}
 #endif
 
-int VP_UNIT(vp_launch_sweep)(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
-    return launch_sweep_t<unit_t>(c, kick, dim, dt, accel);
+int VP_UNIT(vp_launch_sweep)(vp_ctx *c, int kick, int dim, double dt, const double *accel, bool tab_ready) {
+    return launch_sweep_t<unit_t>(c, kick, dim, dt, accel, tab_ready);
 }
 
 int VP_UNIT(vp_tune_sweep)(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
@@ -1161,14 +1193,15 @@ int VP_UNIT(vp_tune_sweep)(vp_ctx *c, int kick, int dim, double dt, const double
 }
 
 #ifdef VP_SWEEP_MAIN
-#define VP_DECLARE(U)                                                                      \
-    void vp_sweep_attrs_##U();                                                             \
-    int vp_launch_sweep_##U(vp_ctx *c, int kick, int dim, double dt, const double *accel); \
+#define VP_DECLARE(U)                                                                                      \
+    void vp_sweep_attrs_##U();                                                                             \
+    int vp_launch_sweep_##U(vp_ctx *c, int kick, int dim, double dt, const double *accel, bool tab_ready); \
     int vp_tune_sweep_##U(vp_ctx *c, int kick, int dim, double dt, const double *accel)
 VP_DECLARE(f32_o5);
 VP_DECLARE(f64_o5);
 VP_DECLARE(f64_o7);
-int vp_launch_shift_table_f64_o7(vp_ctx *c, int kick, int dim, double dt, const double *accel);
+int vp_launch_shift_tables_f64_o7(vp_ctx *c, int kick, unsigned dims, double dt, const double *accel);
+bool vp_sweep_reads_table_f64_o7(vp_ctx *c, int kick, int dim);
 
 int vp_sweep_setup(vp_ctx *c) {
     vp_sweep_attrs_f32_o5();
@@ -1179,21 +1212,26 @@ int vp_sweep_setup(vp_ctx *c) {
     return VP_OK;
 }
 
-int vp_launch_shift_table(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
-    return c->g.precision == VP_F32 ? vp_launch_shift_table_f32_o7(c, kick, dim, dt, accel)
-                                    : vp_launch_shift_table_f64_o7(c, kick, dim, dt, accel);
+int vp_launch_shift_tables(vp_ctx *c, int kick, unsigned dims, double dt, const double *accel) {
+    return c->g.precision == VP_F32 ? vp_launch_shift_tables_f32_o7(c, kick, dims, dt, accel)
+                                    : vp_launch_shift_tables_f64_o7(c, kick, dims, dt, accel);
 }
 
-int vp_launch_shift_table_f32(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
-    return vp_launch_shift_table_f32_o7(c, kick, dim, dt, accel);
+int vp_launch_shift_tables_f32(vp_ctx *c, int kick, unsigned dims, double dt, const double *accel) {
+    return vp_launch_shift_tables_f32_o7(c, kick, dims, dt, accel);
 }
 
-int vp_launch_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
+bool vp_sweep_reads_table(vp_ctx *c, int kick, int dim) {
+    return c->g.precision == VP_F32 ? vp_sweep_reads_table_f32_o7(c, kick, dim)
+                                    : vp_sweep_reads_table_f64_o7(c, kick, dim);
+}
+
+int vp_launch_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel, bool tab_ready) {
     if (c->g.precision == VP_F32)
-        return c->g.order == 7 ? vp_launch_sweep_f32_o7(c, kick, dim, dt, accel)
-                               : vp_launch_sweep_f32_o5(c, kick, dim, dt, accel);
-    return c->g.order == 7 ? vp_launch_sweep_f64_o7(c, kick, dim, dt, accel)
-                           : vp_launch_sweep_f64_o5(c, kick, dim, dt, accel);
+        return c->g.order == 7 ? vp_launch_sweep_f32_o7(c, kick, dim, dt, accel, tab_ready)
+                               : vp_launch_sweep_f32_o5(c, kick, dim, dt, accel, tab_ready);
+    return c->g.order == 7 ? vp_launch_sweep_f64_o7(c, kick, dim, dt, accel, tab_ready)
+                           : vp_launch_sweep_f64_o5(c, kick, dim, dt, accel, tab_ready);
 }
 
 int vp_tune_sweep(vp_ctx *c, int kick, int dim, double dt, const double *accel) {
