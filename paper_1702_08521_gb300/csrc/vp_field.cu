@@ -118,8 +118,10 @@ __device__ __forceinline__ double part_sum(const double *p, long long n, int t, 
 constexpr long long kWarpCells = 2048;
 
 template <typename T, bool WARP>
-__global__ void __launch_bounds__(kBlock) k_moment(const T *__restrict__ f, long long NX, long long NV, double dV,
-                                                   double *__restrict__ rho) {
+__global__ void __launch_bounds__(kBlock) k_moment(const T *f, long long NX, long long NV, double dV,
+                                                   double *rho) {
+    dep_wait();
+    dep_launch();
     if (WARP) {
         const long long x = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
         if (x >= NX) return;
@@ -254,7 +256,7 @@ struct FftArgs {
     const double2 *tw;    // n roots of the axis, or NULL: computed in the CTA
 };
 
-__global__ void __launch_bounds__(256) k_fft_lines(double2 *__restrict__ a, FftArgs f) {
+__global__ void __launch_bounds__(256) k_fft_lines(double2 *a, FftArgs f) {
     extern __shared__ double2 sbuf[];
     const int n = f.p.n, B = f.B;
     double2 *w = sbuf, *x = sbuf + n, *y = x + B * n;
@@ -273,6 +275,7 @@ __global__ void __launch_bounds__(256) k_fft_lines(double2 *__restrict__ a, FftA
         nb = (int)(f.inner - c < (unsigned)B ? f.inner - c : B);
         base = (long long)o * n * f.inner + c;
     }
+    if (f.tw) dep_wait();
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
         if (f.tw) {
             w[j] = f.tw[j];
@@ -282,6 +285,8 @@ __global__ void __launch_bounds__(256) k_fft_lines(double2 *__restrict__ a, FftA
             w[j] = make_double2(cs, -sn);
         }
     }
+    dep_wait();
+    dep_launch();
     if (f.rho) {
         // contiguous lines of the padded grid: the line's outer indices, and
         // its row of the box (or a line of zeros)
@@ -379,10 +384,12 @@ __global__ void k_conv1_kernels(const double *__restrict__ green, const double *
 // 4096 points (the largest axis): 2 x 16.8 M FMAs, ~55 us per output array of
 // the FP64 pipe, still below the two transforms of one CTA.
 constexpr int kConvWarps = 4;
-__global__ void __launch_bounds__(32 * kConvWarps) k_conv1(const double *__restrict__ rho, double bg, int n,
-                                                            const double *__restrict__ ker, double *__restrict__ phi,
-                                                            double *__restrict__ acc) {
+__global__ void __launch_bounds__(32 * kConvWarps) k_conv1(const double *rho, double bg, int n,
+                                                            const double *ker, double *phi,
+                                                            double *acc) {
     extern __shared__ double srho[];
+    dep_wait();
+    dep_launch();
     for (int j = threadIdx.x; j < n; j += blockDim.x) srho[j] = rho[j] - bg;
     __syncthreads();
     const int lane = threadIdx.x & 31;
@@ -434,8 +441,10 @@ struct ForceArgs {
     double inv[3];         // -1 / (den h) per axis
 };
 
-__global__ void __launch_bounds__(kBlock) k_force(const double2 *__restrict__ a, double *__restrict__ phi,
-                                                  double *__restrict__ acc, ForceArgs f) {
+__global__ void __launch_bounds__(kBlock) k_force(const double2 *a, double *phi,
+                                                  double *acc, ForceArgs f) {
+    dep_wait();
+    dep_launch();
     const unsigned x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= f.NX) return;
     int i[3];
@@ -612,13 +621,15 @@ __device__ __forceinline__ double vmax(double a, double b) { return fmax(a, b); 
 // once, to the thread's sum) and walks the rows; longer last axes are walked
 // cell by cell with both weights.
 template <typename T>
-__global__ void __launch_bounds__(kBlock) k_diag_part(const T *__restrict__ f, long long NV, int nlast, FastDiv fd_last,
-                                                      const typename DiagSum<T>::W *__restrict__ wrow,
-                                                      const typename DiagSum<T>::W *__restrict__ wlast, double unit,
-                                                      double dV, double *__restrict__ part,
-                                                      double *__restrict__ rho, int *__restrict__ bad) {
+__global__ void __launch_bounds__(kBlock) k_diag_part(const T *f, long long NV, int nlast, FastDiv fd_last,
+                                                      const typename DiagSum<T>::W *wrow,
+                                                      const typename DiagSum<T>::W *wlast, double unit,
+                                                      double dV, double *part,
+                                                      double *rho, int *bad) {
     __shared__ double sh[4][32];
     __shared__ T smin[32], smax[32];
+    dep_wait();
+    dep_launch();
     const T *p = f + (long long)blockIdx.x * NV;
     DiagSum<T> q;
     if (nlast <= (int)blockDim.x) {
@@ -693,14 +704,14 @@ __global__ void __launch_bounds__(kBlock) k_diag_part(const T *__restrict__ f, l
 // points took 189 us at 10120 points, with a double-precision sincospi each.
 constexpr int kDiagSums = 8;
 
-__global__ void __launch_bounds__(kBlock) k_diag_final(const double *__restrict__ part,
-                                                       const double *__restrict__ rho,
-                                                       const double *__restrict__ phi,
-                                                       const double *__restrict__ acc, long long NX, int dims, int n1,
-                                                       long long rest, int mode, const double2 *__restrict__ roots,
+__global__ void __launch_bounds__(kBlock) k_diag_final(const double *part,
+                                                       const double *rho,
+                                                       const double *phi,
+                                                       const double *acc, long long NX, int dims, int n1,
+                                                       long long rest, int mode, const double2 *roots,
                                                        int root_step, double bg, double dX, double dV,
-                                                       double *__restrict__ blk, unsigned *__restrict__ counter,
-                                                       double *__restrict__ out) {
+                                                       double *blk, unsigned *counter,
+                                                       double *out) {
     // eight sums and the extrema over the block's 256 points: one warp per sum
     // reads its column of the shared copy (a shuffle tree per sum and warp
     // keeps the FP64 pipe busy 3x longer: 10.3 us for 256 points)
@@ -737,6 +748,8 @@ __global__ void __launch_bounds__(kBlock) k_diag_final(const double *__restrict_
         __syncthreads();
     };
     static_assert(kDiagSums == kBlock / 32, "one warp per sum");
+    dep_wait();
+    dep_launch();
     const long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (x < NX) {
         const double *q = part + x * 6;
@@ -938,7 +951,7 @@ FftLaunch fft_axis(const int *m, int dims, int axis, int mode, const double2 *tw
 }
 
 int fft_launch(cudaStream_t st, double2 *buf, const FftLaunch &l) {
-    k_fft_lines<<<l.blocks, l.threads, l.smem, st>>>(buf, l.f);
+    vp_launch_dep(k_fft_lines, l.blocks, l.threads, l.smem, st, buf, l.f);
     return 1;
 }
 
@@ -1154,9 +1167,9 @@ static void moment_launch(vp_ctx *c, double *rho) {
     if (c->NV <= kWarpCells) {
         // fewer points per block while the grid would leave SMs idle
         const int wpb = c->NX >= 8LL * 2 * c->sm_count ? 8 : 2;
-        k_moment<T, true><<<nblk(c->NX, wpb), 32 * wpb, 0, c->stream>>>(f, c->NX, c->NV, dV, rho);
+        vp_launch_dep(k_moment<T, true>, nblk(c->NX, wpb), 32 * wpb, 0, c->stream, f, c->NX, c->NV, dV, rho);
     } else {
-        k_moment<T, false><<<(unsigned)c->NX, kBlock, 0, c->stream>>>(f, c->NX, c->NV, dV, rho);
+        vp_launch_dep(k_moment<T, false>, (unsigned)c->NX, kBlock, 0, c->stream, f, c->NX, c->NV, dV, rho);
     }
 }
 
@@ -1179,8 +1192,8 @@ int vp_launch_poisson(vp_ctx *c, const double *rho, double *phi, double *acc) {
             VP_CUDA_TRY(c, cudaMemcpyAsync(c->d_rho, rho, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->stream));
             rho = c->d_rho;
         }
-        k_conv1<<<nblk(n, kConvWarps), 32 * kConvWarps, sizeof(double) * n, c->stream>>>(rho, g.rho_bg, n, c->d_conv,
-                                                                                        phi, acc);
+        vp_launch_dep(k_conv1, nblk(n, kConvWarps), 32 * kConvWarps, sizeof(double) * n, c->stream, rho,
+                      g.rho_bg, n, c->d_conv, phi, acc);
         c->launches++;
         VP_CUDA_TRY(c, cudaGetLastError());
         return VP_OK;
@@ -1206,7 +1219,8 @@ int vp_launch_poisson(vp_ctx *c, const double *rho, double *phi, double *acc) {
     }
     for (int d = 1; d < D; ++d)
         c->launches += fft_launch(c->stream, c->d_fft, fft_axis(c->m, D, d, FFT_INV, c->roots[d]));
-    k_force<<<nblk(c->NX, kBlock), kBlock, 0, c->stream>>>(c->d_fft, phi, acc, force_args(g, c->m, c->NX));
+    vp_launch_dep(k_force, nblk(c->NX, kBlock), kBlock, 0, c->stream, c->d_fft, phi, acc, force_args(g, c->m,
+                  c->NX));
     c->launches++;
     VP_CUDA_TRY(c, cudaGetLastError());
     return VP_OK;
@@ -1220,9 +1234,9 @@ static void diag_part_launch(vp_ctx *c) {
     const long long rows = c->NV / nlast;
     const W *wrow = static_cast<const W *>(c->d_vw);
     const int th = c->NV >= 4096 || nlast > 128 ? 256 : 128;
-    k_diag_part<T><<<(unsigned)c->NX, th, 0, c->stream>>>(static_cast<const T *>(c->f), c->NV, nlast,
-                                                         make_fastdiv((unsigned)nlast), wrow, wrow + rows, c->vw_unit,
-                                                         cell_volume_v(g), c->d_part, c->d_rho, c->d_flag);
+    vp_launch_dep(k_diag_part<T>, (unsigned)c->NX, th, 0, c->stream, static_cast<const T *>(c->f), c->NV, nlast,
+                  make_fastdiv((unsigned)nlast), wrow, wrow + rows, c->vw_unit, cell_volume_v(g), c->d_part,
+                  c->d_rho, c->d_flag);
 }
 
 // the weights of the kinetic energy, once per context
@@ -1265,9 +1279,9 @@ int vp_launch_diag(vp_ctx *c, int mode, double *out_dev) {
     const long long rest = c->NX / g.nx[0];
     mode %= g.nx[0];
     mode = mode < 0 ? mode + g.nx[0] : mode;
-    k_diag_final<<<nblk(c->NX, kBlock), kBlock, 0, c->stream>>>(
-        c->d_part, c->d_rho, c->d_phi, c->d_acc, c->NX, g.dx, g.nx[0], rest, mode, c->roots[0], c->m[0] / g.nx[0],
-        g.rho_bg, dX, cell_volume_v(g), c->d_diagblk, c->d_diagctr, out_dev);
+    vp_launch_dep(k_diag_final, nblk(c->NX, kBlock), kBlock, 0, c->stream, c->d_part, c->d_rho, c->d_phi,
+                  c->d_acc, c->NX, g.dx, g.nx[0], rest, mode, c->roots[0], c->m[0] / g.nx[0], g.rho_bg, dX,
+                  cell_volume_v(g), c->d_diagblk, c->d_diagctr, out_dev);
     c->launches++;
     VP_CUDA_TRY(c, cudaGetLastError());
     return VP_OK;
@@ -1416,6 +1430,6 @@ extern "C" int vp_poisson_periodic_noalloc(const vp_grid *g, void *cuda_stream, 
                                    D > 2 ? (g->xhi[2] - g->xlo[2]) / g->nx[2] : 1.0);
     k_green_onfly<<<nblk(NX, kBlock), kBlock, 0, st>>>(buf, NX, D, nb, h, g->pois_order, g->coupling);
     for (int d = 0; d < D; ++d) fft_launch(st, buf, fft_axis(m, D, d, FFT_INV, nullptr));
-    k_force<<<nblk(NX, kBlock), kBlock, 0, st>>>(buf, phi_dev, accel_dev, force_args(*g, m, NX));
+    vp_launch_dep(k_force, nblk(NX, kBlock), kBlock, 0, st, buf, phi_dev, accel_dev, force_args(*g, m, NX));
     return cudaGetLastError() == cudaSuccess ? VP_OK : VP_ECUDA;
 }

@@ -50,6 +50,42 @@ __device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv &f) {
 __device__ __forceinline__ unsigned fmod_u(unsigned n, const FastDiv &f) { return n - fdiv(n, f) * f.d; }
 #endif
 
+// Programmatic dependent launch: a kernel launched by vp_launch_dep may start
+// while the kernel before it on the stream is still finishing.  It calls
+// dep_wait() before its first access to memory that another launch wrote or still
+// reads (the grids before it are then complete and visible) and dep_launch() to
+// let the next one start.  Its pointers carry no __restrict__, which would let
+// the compiler move their loads above the wait.  A step on a small grid is a chain of kernels of
+// 2-20 us, each of which waited ~1 us for the launch of the next: 1D1V Landau
+// 64 x 128 FP64 36.4 -> 33.8 us a step, two-stream 256 x 1024 499 -> 454,
+// 512 x 512 FP64 sweeps 78.5 -> 73.2.  Only grids of at most one CTA per SM let
+// the next one in early; from larger ones it would take the slots of CTAs that
+// still have work (two-stream 564, a learned 2D2V step 346 -> 361), so there the
+// launch alone overlaps.
+#ifdef __CUDACC__
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_launch() {
+    unsigned sms;
+    asm("mov.u32 %0, %%nsmid;" : "=r"(sms));
+    if (gridDim.x * gridDim.y <= sms) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... KA, typename... A>
+inline void vp_launch_dep(void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = st != nullptr && st != cudaStreamLegacy ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, KA(args)...);
+}
+#endif
+
 struct SweepGeo {
     long long outer, inner;
     int L;

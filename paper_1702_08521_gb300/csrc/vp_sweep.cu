@@ -75,7 +75,7 @@ struct PtrStore {
 // arithmetic costs 3-6% there: Plummer 16^3 x 64^3 drift x1 1.86 against 1.97 ms).
 template <typename T, int ORDER, bool PERIODIC, bool FULL, bool PAIR, bool FLAT, bool GEN>
 __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_MINB : 1)
-    k_sweep_cols(T *__restrict__ f, const __grid_constant__ ShiftSrc<T> src, SweepGeo geo, LimParams lp) {
+    k_sweep_cols(T *f, const __grid_constant__ ShiftSrc<T> src, SweepGeo geo, LimParams lp) {
     extern __shared__ __align__(16) unsigned char smraw[];
     constexpr int GP = PERIODIC ? 0 : VP_GHOST;
     T *sm = reinterpret_cast<T *>(smraw);
@@ -99,6 +99,8 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
     unsigned q0 = 0;
     int ncl = 1;
     LineShift<T> *shifts = nullptr;
+    const bool own_drift = !src.tab && !src.accel;  // shifts of the grid alone: nothing to wait for
+    if (!own_drift) dep_wait();
     if (!src.tab) {
         shifts = reinterpret_cast<LineShift<T> *>(smraw + (((size_t)(L + 2 * GP) * W * sizeof(T) + 15) & ~size_t(15)));
         q0 = geo.cls_from_inner ? fdiv(c0, geo.fd_cdiv) : fdiv(o, geo.fd_cdiv);
@@ -107,6 +109,8 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
         ncl = (int)(q1 - q0) + 1;
         vp_core::tile_shifts(shifts, q0, ncl, src, geo);
     }
+    if (own_drift) dep_wait();
+    dep_launch();
     // Every piece of the tile in flight at once (cp.async), so the staging is not
     // limited by one outstanding load per thread: pieces of 16, 8 or 4 bytes, the
     // widest that the row stride and the tile width are multiples of.  A 22 x 20 x
@@ -220,7 +224,7 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
 // conflict-free because P is odd.
 template <typename T, int ORDER, bool PERIODIC, bool FULL, bool PAIR, bool FLAT>
 __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_MINB : 1)
-    k_sweep_rows(T *__restrict__ f, const __grid_constant__ ShiftSrc<T> src, SweepGeo geo, LimParams lp) {
+    k_sweep_rows(T *f, const __grid_constant__ ShiftSrc<T> src, SweepGeo geo, LimParams lp) {
     extern __shared__ __align__(16) unsigned char smraw[];
     constexpr int GP = PERIODIC ? 0 : VP_GHOST;
     const int L = geo.L, R = geo.R;
@@ -237,6 +241,8 @@ __global__ void __launch_bounds__(PAIR ? VP_PAIR_THREADS : 512, PAIR ? VP_PAIR_M
     unsigned q0 = 0;
     int ncl = 1;
     LineShift<T> *shifts = nullptr;
+    dep_wait();
+    dep_launch();
     if (!src.tab) {
         shifts = reinterpret_cast<LineShift<T> *>(smraw + (((size_t)R * (P + Q) * sizeof(T) + 15) & ~size_t(15)));
         q0 = fdiv((unsigned)l0, geo.fd_cdiv);
@@ -565,8 +571,10 @@ struct TableAxes {
 };
 
 template <typename T>
-__global__ void k_shift_table(LineShift<T> *__restrict__ tab, long long cap, int kick, const __grid_constant__ TableAxes ax,
+__global__ void k_shift_table(LineShift<T> *tab, long long cap, int kick, const __grid_constant__ TableAxes ax,
                               double dt, const __grid_constant__ WPoly wp) {
+    dep_wait();
+    dep_launch();
     const int a = blockIdx.y;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int c = (int)(t >> 3), k = (int)t & 7;
@@ -807,11 +815,14 @@ int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
         const bool gen = geo.kblk > 1 || geo.vec * sizeof(T) != 16 || geo.inner % W || threads % wv;
 #define VP_LAUNCH_COLS(O, P, F, PAIR)                                                                              \
     if (gen)                                                                                                       \
-        k_sweep_cols<T, O, P, F, PAIR, true, true><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp); \
+        vp_launch_dep(k_sweep_cols<T, O, P, F, PAIR, true, true>, (unsigned)tiles, threads, smem, c->stream, f, \
+                      src, geo, lp); \
     else if (flat)                                                                                                 \
-        k_sweep_cols<T, O, P, F, PAIR, true, false><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp); \
+        vp_launch_dep(k_sweep_cols<T, O, P, F, PAIR, true, false>, (unsigned)tiles, threads, smem, c->stream, f, \
+                      src, geo, lp); \
     else                                                                                                           \
-        k_sweep_cols<T, O, P, F, PAIR, !F, false><<<(unsigned)tiles, threads, smem, c->stream>>>(f, src, geo, lp)
+        vp_launch_dep(k_sweep_cols<T, O, P, F, PAIR, !F, false>, (unsigned)tiles, threads, smem, c->stream, f, \
+                      src, geo, lp)
 #define VP_LAUNCH(O, P, F)                          \
     if (pair) {                                     \
         VP_LAUNCH_COLS(O, P, F, sizeof(T) == 4);    \
@@ -868,17 +879,21 @@ int launch_rows(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
         const int pthreads = threads;
 #define VP_LAUNCH(O, P, F)                                                                                     \
     if (flat)                                                                                                  \
-        k_sweep_rows<T, O, P, F, sizeof(T) == 4, true><<<(unsigned)blocks, pthreads, smem, c->stream>>>(f, src, geo, lp); \
+        vp_launch_dep(k_sweep_rows<T, O, P, F, sizeof(T) == 4, true>, (unsigned)blocks, pthreads, smem, \
+                      c->stream, f, src, geo, lp); \
     else                                                                                                       \
-        k_sweep_rows<T, O, P, F, sizeof(T) == 4, !F><<<(unsigned)blocks, pthreads, smem, c->stream>>>(f, src, geo, lp)
+        vp_launch_dep(k_sweep_rows<T, O, P, F, sizeof(T) == 4, !F>, (unsigned)blocks, pthreads, smem, c->stream, \
+                      f, src, geo, lp)
         VP_DISPATCH(per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     } else {
 #define VP_LAUNCH(O, P, F)                                                                                     \
     if (flat)                                                                                                  \
-        k_sweep_rows<T, O, P, F, false, true><<<(unsigned)blocks, threads, smem, c->stream>>>(f, src, geo, lp); \
+        vp_launch_dep(k_sweep_rows<T, O, P, F, false, true>, (unsigned)blocks, threads, smem, c->stream, f, src, \
+                      geo, lp); \
     else                                                                                                       \
-        k_sweep_rows<T, O, P, F, false, !F><<<(unsigned)blocks, threads, smem, c->stream>>>(f, src, geo, lp)
+        vp_launch_dep(k_sweep_rows<T, O, P, F, false, !F>, (unsigned)blocks, threads, smem, c->stream, f, src, \
+                      geo, lp)
         VP_DISPATCH(per, full, VP_LAUNCH);
 #undef VP_LAUNCH
     }
@@ -1164,8 +1179,8 @@ int VP_UNIT(vp_launch_shift_tables)(vp_ctx *c, int kick, unsigned dims, double d
     }
     const int th = 64;
     const dim3 grid((unsigned)((8LL * most + th - 1) / th), (unsigned)ax.n);
-    k_shift_table<unit_t><<<grid, th, 0, c->stream>>>(static_cast<LineShift<unit_t> *>(c->d_shift), c->shift_cap, kick,
-                                                      ax, dt, c->wp);
+    vp_launch_dep(k_shift_table<unit_t>, grid, th, 0, c->stream, static_cast<LineShift<unit_t> *>(c->d_shift),
+                  c->shift_cap, kick, ax, dt, c->wp);
     c->launches++;
     VP_CUDA_TRY(c, cudaGetLastError());
     return VP_OK;
