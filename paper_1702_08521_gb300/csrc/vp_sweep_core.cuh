@@ -377,30 +377,36 @@ __device__ __forceinline__ bool walk(const T *__restrict__ sm0, int ss, int L, c
     // Source row of load k (k = 0, 1, ...) is p0 + k sg; load k feeds step
     // k - 8 of the walk.
     int p0;
+    // Zero-inflow lines read rows outside the staged extent [-GP, L + GP) as
+    // the zero row at its edge; periodic lines wrap.  A wrapped row is a line
+    // length or two away at most (n is reduced first): additions, where eleven
+    // remainders by L cost a short segment as much as its cells.
+    auto wrap = [&](int q) {
+        while (q < 0) q += L;
+        while (q >= L) q -= L;
+        return q;
+    };
+    auto row = [&](int q) -> const T * { return sm0 + min(max(q, -GP), L + GP - 1) * ss; };
     if (PERIODIC) {
-        const int n = sh.n % L;
-        p0 = (i - n - 4 * sg) % L;
-        if (p0 < 0) p0 += L;
+        int n = sh.n;
+        if (n >= L || n <= -L) n %= L;
+        p0 = wrap(i - n - 4 * sg);
     } else {
         p0 = i - sh.n - 4 * sg;
     }
-    // Zero-inflow lines read rows outside the staged extent [-GP, L + GP) as
-    // the zero row at its edge; periodic lines wrap.
-    auto row = [&](int q) -> const T * {
-        if (PERIODIC) {
-            q %= L;
-            if (q < 0) q += L;
-        } else {
-            q = min(max(q, -GP), L + GP - 1);
-        }
-        return sm0 + q * ss;
-    };
     const T *src = sm0;
     int inc = 0;
     T w[8];
+    int pk = p0;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-        w[k] = *row(p0 + k * sg);
+        if (PERIODIC) {
+            w[k] = sm0[pk * ss];
+            pk += sg;
+            pk = pk < 0 ? L - 1 : (pk == L ? 0 : pk);
+        } else {
+            w[k] = *row(p0 + k * sg);
+        }
         note(w[k]);
     }
     // incoming mass of the first cell: upwind cell i - sg, stencil w[0..6]
@@ -523,7 +529,7 @@ __device__ __forceinline__ bool walk(const T *__restrict__ sm0, int ss, int L, c
         const int q = p0 + (t + 8) * sg;  // row of the next load
         int end;
         if (PERIODIC) {
-            const int qq = ((q % L) + L) % L;
+            const int qq = wrap(q);
             src = sm0 + qq * ss;
             inc = sg * ss;
             end = t + (sg > 0 ? L - qq : qq + 1);  // loads before the wrap
