@@ -4,24 +4,33 @@
 //
 // Work queue: one step of every run is a list of items (run, stage, tile)
 // sorted by stage.  Each CTA of a persistent grid pops items with an atomic
-// counter (the next one while it works on the current one), waits (bounded)
-// until the previous stage of that run has finished all its tiles, processes
-// the tile and counts it done.  Items are popped in queue order by running
-// CTAs only, and a CTA takes up its popped item right after its current one,
-// which comes earlier in the queue; every item's dependencies come earlier
-// still, so the earliest unfinished item is always being worked on: no
-// deadlock, whatever the residency.
+// counter (up to two ahead of the one it works on), waits (bounded) until the
+// previous stage of that run has finished all its tiles, processes the tile and
+// counts it done, at the latest before it waits for anything else.  Items are
+// popped in queue order by running CTAs only, and a CTA works its items off in
+// that order; every item's dependencies come earlier in the queue, so the
+// earliest unfinished item is always being worked on: no deadlock, whatever the
+// residency.
 //
 // Stages of a KDK step (Eq. 55), per run:
 //   1D1V: kick v (dt/2) | drift x (dt) | density + Poisson | kick v (dt/2)
 //   2D2V: kick v1, kick v2 (dt/2) | drift x2, drift x1 (dt) | density |
-//         Poisson | kick v1, kick v2 (dt/2)
+//         Poisson (one stage or four) | kick v1, kick v2 (dt/2)
 // Sweeps reuse the line walker of the single-run kernels.  A kick tile's
-// lines share one spatial point, so thread 0 decomposes its shift in FP64
+// lines share one spatial point, so one thread decomposes its shift in FP64
 // once per tile; drift shifts depend only on dt and come from a table made
 // once per dt (k_ens_drift_table).  Data written by other CTAs inside
 // the launch (f of the previous stage, density, field) is read with L1-bypass
 // loads (ld.global.cg).
+//
+// What bounds it: six CTAs of 128 threads share an SM and each item is a chain
+// (descriptor, loads, walk, stores), so what a chain waits for beside its walk
+// counts.  512 1D + 8 2D2V (64^4) runs, 3.03 -> 2.24 ms a step (7.4 GB of sweeps:
+// 3.3 TB/s): the Poisson solve of a 2D run in tiles (it was 500 us of one CTA);
+// the item after the next popped, the next one's descriptor read and the last
+// one's stores drained under a tile's loads; shifts made under them too, with no
+// FP64 division; index arithmetic by multiplications instead of 64-bit divisions;
+// 16-byte loads, four in flight, for contiguous tiles and the density.
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -39,11 +48,18 @@ namespace {
 // against 3.07 ms per step); launch bounds for 6 CTAs per SM, which the
 // staged tiles' shared memory allows anyway, leave 80 registers (no spills)
 constexpr int kThreads = 128;
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 11;
 // shared-memory budget of one staged sweep tile (wider tiles are halved)
 constexpr size_t kTileBytes = 56 * 1024;
 
-enum StageKind { ST_COLS = 0, ST_ROWS = 1, ST_MOMENT = 2, ST_POISSON = 3 };
+enum StageKind {
+    ST_COLS = 0,
+    ST_ROWS,
+    ST_MOMENT,
+    ST_POISSON,                                       // the whole solve in one tile
+    ST_FFT_ROWS, ST_FFT_COLS, ST_FFT_BACK, ST_FORCE   // its four stages
+};
+inline bool field_stage(int kind) { return kind >= ST_MOMENT; }
 
 struct StageDesc {
     int kind;
@@ -53,11 +69,12 @@ struct StageDesc {
     long long outer, inner;
     int L;
     int periodic;
-    int cls_from_inner;
-    long long cdiv, cmod;
     int tiles;
     int tw;          // tile width: columns (strided sweep) or lines (contiguous sweep)
+    int nseg;        // segments a line is walked in (threads of a CTA / tw)
     int done_slot;   // index of this stage's completion counter
+    FastDiv fd_tpo;  // tiles across `inner` (strided)
+    FastDiv fd_tw, fd_L, fd_nseg, fd_cdiv, fd_cmod;
 };
 
 struct RunDesc {
@@ -68,6 +85,7 @@ struct RunDesc {
     double xlo[2], hx[2], vlo[2], hv[2];
     long long acc_off, rho_off;
     long long dsh_off;  // drift shifts: axis 0 at [dsh_off, dsh_off + nv[0]), axis 1 after
+    int kdt_off;        // (dt / 2) / hv of the kicks: axis k at kdt_off + k
     double coupling, rho_bg;
     int pois_order;
     int nstage;
@@ -135,8 +153,9 @@ __device__ __forceinline__ LineShift<float> ens_shift(double speed, double dth, 
 // its lines), computed once per dt outside the step: drift tiles read them
 // instead of spending the narrow FP64 pipe on every line of every tile.
 __global__ void k_ens_drift_table(const RunDesc *__restrict__ runs, LineShift<float> *__restrict__ tab,
-                                  EnsParams P) {
+                                  double *__restrict__ kdt, EnsParams P) {
     const RunDesc &r = runs[blockIdx.x];
+    if ((int)threadIdx.x < r.dims) kdt[r.kdt_off + threadIdx.x] = 0.5 * P.dt / r.hv[threadIdx.x];
     for (int axis = 0; axis < r.dims; ++axis) {
         const double dth = P.dt / r.hx[axis];  // drifts move by the full dt
         const long long base = r.dsh_off + (axis ? r.nv[0] : 0);
@@ -145,27 +164,30 @@ __global__ void k_ens_drift_table(const RunDesc *__restrict__ runs, LineShift<fl
     }
 }
 
-template <int ORDER, bool PER, bool FLAT>
-__device__ void tile_cols(float *pool, const RunDesc &r, const StageDesc &s, int tile,
-                          const double *acc_pool, const LineShift<float> *dsh, const EnsParams &P, float *sm) {
+// what a tile reads besides the pool: accelerations, drift shifts, kick factors
+struct SweepSrc {
+    const double *acc, *kdt;
+    const LineShift<float> *dsh;
+};
+
+// `staged` is the barrier after which the whole tile is in shared memory (it
+// also announces the item before this one, see k_ensemble).  What the walk
+// needs besides the tile is made under the staging's copies.
+template <int ORDER, bool PER, bool FLAT, typename Staged>
+__device__ __forceinline__ void tile_cols(float *pool, const RunDesc &r, const StageDesc &s, int tile, const SweepSrc &src,
+                          const EnsParams &P, float *sm, Staged staged) {
     // zero-inflow lines get VP_GHOST zero rows on each side (direct walks)
     constexpr int GP = PER ? 0 : VP_GHOST;
     const int L = s.L;
     const int W = s.tw;
-    const long long tpo = (s.inner + W - 1) / W;
-    const long long o = tile / tpo;
-    const long long c0 = (tile % tpo) * W;
+    const unsigned o = fdiv((unsigned)tile, s.fd_tpo);
+    const unsigned c0 = ((unsigned)tile - o * s.fd_tpo.d) * (unsigned)W;
     const int wc = (int)((s.inner - c0) < W ? (s.inner - c0) : W);
-    float *base = pool + r.f_off + o * L * s.inner + c0;
+    float *base = pool + r.f_off + (long long)o * L * s.inner + c0;
     float *data = sm + GP * W;  // row 0
     // a kick tile holds one spatial point: its shift, made once (thread 0,
     // while the tile is staged) and shared; drift tiles read the table
     __shared__ LineShift<float> s_sh;
-    if (threadIdx.x == 0 && s.kick) {
-        const double dt = s.half ? 0.5 * P.dt : P.dt;
-        const unsigned cls = (unsigned)(o / s.cdiv);
-        s_sh = ens_shift(ldcg(acc_pool + r.acc_off + (long long)s.axis * r.NX + cls), dt / r.hv[s.axis], P);
-    }
     for (int c = threadIdx.x; c < GP * W; c += blockDim.x) {
         sm[c] = 0.f;
         data[L * W + c] = 0.f;
@@ -174,10 +196,13 @@ __device__ void tile_cols(float *pool, const RunDesc &r, const StageDesc &s, int
     // of it in flight at once as 16-byte cp.async.cg copies (L2, as the
     // L1-bypass loads: earlier stages of this launch wrote it); otherwise
     // four rows per thread in flight, (row, column) advanced incrementally
-    if (wc == W && W % 4 == 0 && s.inner % 4 == 0 && (reinterpret_cast<uintptr_t>(base) & 15) == 0) {
+    const int t_row = (int)fdiv(threadIdx.x, s.fd_tw), t_col = (int)threadIdx.x - t_row * W;
+    const bool whole =
+        wc == W && W % 4 == 0 && s.inner % 4 == 0 && (reinterpret_cast<uintptr_t>(base) & 15) == 0;
+    if (whole) {
         const int wv = W >> 2;
-        const int dr = blockDim.x / wv, dc = blockDim.x - dr * wv;
-        int row = threadIdx.x / wv, cv = threadIdx.x - row * wv;
+        const int dr = (int)fdiv(4 * blockDim.x, s.fd_tw), dc = blockDim.x - dr * wv;
+        int row = (int)fdiv(4 * threadIdx.x, s.fd_tw), cv = threadIdx.x - row * wv;
         while (row < L) {
             vp_tma::cp_async16(data + row * W + 4 * cv, base + (long long)row * s.inner + 4 * cv);
             row += dr;
@@ -187,10 +212,9 @@ __device__ void tile_cols(float *pool, const RunDesc &r, const StageDesc &s, int
                 ++row;
             }
         }
-        vp_tma::cp_async_wait_all();
     } else {
-        const int dr = blockDim.x / W, dc = blockDim.x - dr * W;
-        int row = threadIdx.x / W, cc = threadIdx.x - row * W;
+        const int dr = (int)fdiv(blockDim.x, s.fd_tw), dc = blockDim.x - dr * W;
+        int row = t_row, cc = t_col;
         for (int e = threadIdx.x; e < L * W; e += 4 * blockDim.x) {
             float v[4];
             int rr[4], cq[4];
@@ -211,13 +235,15 @@ __device__ void tile_cols(float *pool, const RunDesc &r, const StageDesc &s, int
                 if (e + u * (int)blockDim.x < L * W) data[rr[u] * W + cq[u]] = v[u];
         }
     }
-    __syncthreads();
-    const int nseg = blockDim.x / W;
-    const int cc = threadIdx.x % W, seg = threadIdx.x / W;
-    if (cc < wc && seg < nseg) {
-        const unsigned cls = s.cls_from_inner ? (unsigned)(((c0 + cc) / s.cdiv) % s.cmod) : (unsigned)(o / s.cdiv);
-        const LineShift<float> sh = s.kick ? s_sh : dsh[r.dsh_off + (s.axis ? r.nv[0] : 0) + cls];
-        const int r0 = seg * L / nseg, r1 = (seg + 1) * L / nseg;
+    if (threadIdx.x == 0 && s.kick)
+        s_sh = ens_shift(ldcg(src.acc + r.acc_off + (long long)s.axis * r.NX + o), src.kdt[r.kdt_off + s.axis], P);
+    if (whole) vp_tma::cp_async_wait_all();
+    staged();
+    const int cc = t_col, seg = t_row;
+    if (cc < wc && seg < s.nseg) {
+        const unsigned cls = fmod_u(fdiv(c0 + cc, s.fd_cdiv), s.fd_cmod);  // drifts: velocity cell
+        const LineShift<float> sh = s.kick ? s_sh : src.dsh[r.dsh_off + (s.axis ? r.nv[0] : 0) + cls];
+        const int r0 = (int)fdiv(seg * L, s.fd_nseg), r1 = (int)fdiv((seg + 1) * L, s.fd_nseg);
         const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
         struct St {
             float *p;
@@ -233,84 +259,93 @@ __device__ void tile_cols(float *pool, const RunDesc &r, const StageDesc &s, int
     }
 }
 
-template <int ORDER, bool FLAT>
-__device__ void tile_rows(float *pool, const RunDesc &r, const StageDesc &s, int tile,
-                          const double *acc_pool, const EnsParams &P, float *sm) {
+template <int ORDER, bool FLAT, typename Staged>
+__device__ __forceinline__ void tile_rows(float *pool, const RunDesc &r, const StageDesc &s, int tile, const SweepSrc &src,
+                          const EnsParams &P, float *sm, Staged staged) {
     constexpr int GP = VP_GHOST;  // velocity lines: zero inflow
     const int L = s.L;
     const int R = s.tw;
     const int Pp = (L + 2 * GP) | 1, Q = L | 1;
     float *in = sm, *out = sm + R * Pp;
-    const long long l0 = (long long)tile * R;
+    const unsigned l0 = (unsigned)tile * (unsigned)R;
     const int nl = (int)((s.outer - l0) < R ? (s.outer - l0) : R);
-    float *base = pool + r.f_off + l0 * L;
-    // lines of one spatial point (a 2D run's v2 kick): one shift, made once by
-    // thread 0 while the tile is staged; otherwise one per line
-    const long long cfirst = l0 / s.cdiv;
-    const bool uniform = cfirst == (l0 + nl - 1) / s.cdiv;
-    __shared__ double s_dth;
-    __shared__ LineShift<float> s_sh;
-    if (threadIdx.x == 0) {
-        s_dth = (s.half ? 0.5 * P.dt : P.dt) / r.hv[s.axis];
-        if (uniform) s_sh = ens_shift(ldcg(acc_pool + r.acc_off + (long long)s.axis * r.NX + cfirst), s_dth, P);
-    }
+    float *base = pool + r.f_off + (long long)l0 * L;
+    // Lines of a few spatial points (a 2D run's v2 kick): their shifts, made
+    // once by the last threads while the tile is staged.  One point per line
+    // (1D): each thread makes its own, since room for a tile's shifts would cost
+    // the sixth CTA per SM.
+    constexpr int kShared = 4;
+    __shared__ LineShift<float> s_sh[kShared];
+    const unsigned cfirst = fdiv(l0, s.fd_cdiv);
+    const int ncl = (int)(fdiv(l0 + nl - 1, s.fd_cdiv) - cfirst) + 1;
+    const double *acc = src.acc + r.acc_off + (long long)s.axis * r.NX + cfirst;
+    const int mine = (int)(blockDim.x - 1 - threadIdx.x);
+    const double speed = ncl <= kShared && mine < ncl ? ldcg(acc + mine) : 0.0;
     for (int k = threadIdx.x; k < nl * GP; k += blockDim.x) {
         const int ln = k / GP, g = k - ln * GP;
         in[ln * Pp + g] = 0.f;
         in[ln * Pp + GP + L + g] = 0.f;
     }
     const int tot = nl * L;
-    const int dr = blockDim.x / L, dp = blockDim.x - dr * L;
     // whole rows of 16-byte pieces (f_off is 128-byte aligned): 16-byte loads and stores
     const bool vec = (L & 3) == 0 && (reinterpret_cast<uintptr_t>(base) & 15) == 0;
+    // four pieces per thread in flight; the position advances incrementally
+    const int piece = vec ? 4 : 1;
+    const int stride = piece * (int)blockDim.x;
+    const int vr = (int)fdiv(stride, s.fd_L), vp = stride - vr * L;
+    const int row0 = (int)fdiv(piece * threadIdx.x, s.fd_L), pos0 = piece * (int)threadIdx.x - row0 * L;
+    auto next = [&](int &row, int &pos) {
+        row += vr;
+        pos += vp;
+        if (pos >= L) {
+            pos -= L;
+            ++row;
+        }
+    };
     if (vec) {
-        const int st4 = 4 * (int)blockDim.x;
-        const int vr = st4 / L, vp = st4 - vr * L;
-        int row = (4 * (int)threadIdx.x) / L, pos = 4 * (int)threadIdx.x - row * L;
-        for (int e = 4 * (int)threadIdx.x; e < tot; e += st4) {
-            const float4 v = __ldcg(reinterpret_cast<const float4 *>(base + e));
-            float *d = in + row * Pp + GP + pos;
-            d[0] = v.x;
-            d[1] = v.y;
-            d[2] = v.z;
-            d[3] = v.w;
-            row += vr;
-            pos += vp;
-            if (pos >= L) {
-                pos -= L;
-                ++row;
+        int row = row0, pos = pos0;
+        for (int e = 4 * (int)threadIdx.x; e < tot; e += 4 * stride) {
+            float4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (e + u * stride < tot) v[u] = __ldcg(reinterpret_cast<const float4 *>(base + e + u * stride));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (e + u * stride < tot) {
+                    float *d = in + row * Pp + GP + pos;
+                    d[0] = v[u].x;
+                    d[1] = v[u].y;
+                    d[2] = v[u].z;
+                    d[3] = v[u].w;
+                }
+                next(row, pos);
             }
         }
     } else {
-        int row = threadIdx.x / L, pos = threadIdx.x - row * L;
-        for (int e = threadIdx.x; e < tot; e += 4 * blockDim.x) {
+        int row = row0, pos = pos0;
+        for (int e = threadIdx.x; e < tot; e += 4 * stride) {
             float v[4];
             int at[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int eu = e + u * (int)blockDim.x;
+                const int eu = e + u * stride;
                 at[u] = row * Pp + GP + pos;
                 v[u] = eu < tot ? ldcg(base + eu) : 0.f;
-                row += dr;
-                pos += dp;
-                if (pos >= L) {
-                    pos -= L;
-                    ++row;
-                }
+                next(row, pos);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                if (e + u * (int)blockDim.x < tot) in[at[u]] = v[u];
+                if (e + u * stride < tot) in[at[u]] = v[u];
         }
     }
-    __syncthreads();
-    const int nseg = blockDim.x / R;
-    const int line = threadIdx.x % R, seg = threadIdx.x / R;
-    if (line < nl && seg < nseg) {
-        const unsigned cls = (unsigned)((l0 + line) / s.cdiv);
-        const LineShift<float> sh =
-            uniform ? s_sh : ens_shift(ldcg(acc_pool + r.acc_off + (long long)s.axis * r.NX + cls), s_dth, P);
-        const int r0 = seg * L / nseg, r1 = (seg + 1) * L / nseg;
+    const double dth = src.kdt[r.kdt_off + s.axis];
+    if (ncl <= kShared && mine < ncl) s_sh[mine] = ens_shift(speed, dth, P);
+    staged();
+    const int seg = (int)fdiv(threadIdx.x, s.fd_tw), line = (int)threadIdx.x - seg * R;
+    if (line < nl && seg < s.nseg) {
+        const unsigned c = fdiv(l0 + line, s.fd_cdiv) - cfirst;
+        const LineShift<float> sh = ncl <= kShared ? s_sh[c] : ens_shift(ldcg(acc + c), dth, P);
+        const int r0 = (int)fdiv(seg * L, s.fd_nseg), r1 = (int)fdiv((seg + 1) * L, s.fd_nseg);
         const int i0 = sh.sigma > 0 ? r0 : r1 - 1;
         struct St {
             float *p;
@@ -325,30 +360,17 @@ __device__ void tile_rows(float *pool, const RunDesc &r, const StageDesc &s, int
                                                      P.pp, st);
     }
     __syncthreads();
+    int row = row0, pos = pos0;
     if (vec) {
-        const int st4 = 4 * (int)blockDim.x;
-        const int vr = st4 / L, vp = st4 - vr * L;
-        int row = (4 * (int)threadIdx.x) / L, pos = 4 * (int)threadIdx.x - row * L;
-        for (int e = 4 * (int)threadIdx.x; e < tot; e += st4) {
-            const float *src = out + row * Q + pos;
-            *reinterpret_cast<float4 *>(base + e) = make_float4(src[0], src[1], src[2], src[3]);
-            row += vr;
-            pos += vp;
-            if (pos >= L) {
-                pos -= L;
-                ++row;
-            }
+        for (int e = 4 * (int)threadIdx.x; e < tot; e += stride) {
+            const float *q = out + row * Q + pos;
+            *reinterpret_cast<float4 *>(base + e) = make_float4(q[0], q[1], q[2], q[3]);
+            next(row, pos);
         }
     } else {
-        int row = threadIdx.x / L, pos = threadIdx.x - row * L;
-        for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+        for (int e = threadIdx.x; e < tot; e += stride) {
             base[e] = out[row * Q + pos];
-            row += dr;
-            pos += dp;
-            if (pos >= L) {
-                pos -= L;
-                ++row;
-            }
+            next(row, pos);
         }
     }
 }
@@ -360,22 +382,47 @@ __device__ double warp_sum_d(double v) {
 }
 
 // density of spatial points [x0, x1): one warp per point, compensated float
-// sums per lane combined in double
+// sums per lane (two, of alternate 16-byte pieces) combined in double
+struct PairSum {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float y) {
+        const float t = s + y, bp = t - s;
+        e += (s - (t - bp)) + (y - bp);
+        s = t;
+    }
+};
 __device__ void density_points(const float *pool, const RunDesc &r, long long x0, long long x1,
                                double *rho_pool) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const double dV = r.dims == 1 ? r.hv[0] : r.hv[0] * r.hv[1];
+    const int NV = (int)r.NV;
+    const int nq = NV % 4 == 0 ? NV / 4 : 0;  // 16-byte pieces (f_off is 128-byte aligned)
     for (long long x = x0 + warp; x < x1; x += nw) {
         const float *p = pool + r.f_off + x * r.NV;
-        float s = 0.f, e = 0.f;
-        for (long long v = lane; v < r.NV; v += 32) {
-            const float y = ldcg(p + v);
-            const float t = s + y;
-            const float bp = t - s;
-            e += (s - (t - bp)) + (y - bp);
-            s = t;
+        const float4 *q = reinterpret_cast<const float4 *>(p);
+        PairSum a, b;
+        int i = lane;
+        for (; i + 96 < nq; i += 128) {
+            float4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = __ldcg(q + i + 32 * u);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                a.add(v[u].x);
+                b.add(v[u].y);
+                a.add(v[u].z);
+                b.add(v[u].w);
+            }
         }
-        const double tot = warp_sum_d((double)s + (double)e);
+        for (; i < nq; i += 32) {
+            const float4 v = __ldcg(q + i);
+            a.add(v.x);
+            b.add(v.y);
+            a.add(v.z);
+            b.add(v.w);
+        }
+        for (int v = 4 * nq + lane; v < NV; v += 32) a.add(ldcg(p + v));
+        const double tot = warp_sum_d(((double)a.s + (double)a.e) + ((double)b.s + (double)b.e));
         if (lane == 0) rho_pool[r.rho_off + x] = tot * dV;
     }
 }
@@ -386,25 +433,13 @@ __device__ void density_points(const float *pool, const RunDesc &r, long long x0
 // length up to 256 (length len uses every (256 / len)-th entry)
 constexpr int kTwN = 256;
 
-// runs with at most this many spatial points transform in shared memory;
-// larger ones in their slice of a global scratch array (L2-resident), so the
-// kernel's shared memory is sized by the sweep tiles alone
-constexpr long long kSmemFftMax = 1024;
+// Runs of at most this many spatial points (every 1D run) solve in one CTA.
+// Larger 2D runs solve in four stages of tiles of about this many points: rows
+// forward, columns forward + Green factors + columns inverse, rows inverse, force.
+// In one CTA the 64 x 64 points of a run took 400-500 us, in which the other
+// CTAs had nothing left to do.
+constexpr int kFftTile = 256;
 
-// element access of the transform array: shared memory, or the global scratch
-// through L2 (other SMs used it in earlier launches)
-template <bool GLOBAL>
-__device__ __forceinline__ double2 ld2(const double2 *p) {
-    if constexpr (GLOBAL) return __ldcg(p);
-    else return *p;
-}
-template <bool GLOBAL>
-__device__ __forceinline__ void st2(double2 *p, double2 v) {
-    if constexpr (GLOBAL) __stcg(p, v);
-    else *p = v;
-}
-
-template <bool GLOBAL>
 __device__ void smem_fft(double2 *a, int dims, int n0, int n1, int axis, int sign, const double2 *__restrict__ tw) {
     const int n = axis == 0 ? n0 : n1;
     const int lines = dims == 1 ? 1 : (axis == 0 ? n1 : n0);
@@ -418,9 +453,9 @@ __device__ void smem_fft(double2 *a, int dims, int n0, int n1, int axis, int sig
         const int rj = logn ? (int)(__brev((unsigned)j) >> (32 - logn)) : 0;
         if (j < rj) {
             double2 *pa = a + l * lstride + j * stride, *pb = a + l * lstride + rj * stride;
-            const double2 tmp = ld2<GLOBAL>(pa);
-            st2<GLOBAL>(pa, ld2<GLOBAL>(pb));
-            st2<GLOBAL>(pb, tmp);
+            const double2 tmp = *pa;
+            *pa = *pb;
+            *pb = tmp;
         }
     }
     __syncthreads();
@@ -433,36 +468,20 @@ __device__ void smem_fft(double2 *a, int dims, int n0, int n1, int axis, int sig
             const double2 twk = tw[k * (kTwN / len)];
             const double cs = twk.x, sn = sign < 0 ? -twk.y : twk.y;
             double2 *pu = a + l * lstride + i0 * stride, *pv = a + l * lstride + i1 * stride;
-            const double2 u = ld2<GLOBAL>(pu), v = ld2<GLOBAL>(pv);
+            const double2 u = *pu, v = *pv;
             const double2 tw = make_double2(v.x * cs - v.y * sn, v.x * sn + v.y * cs);
-            st2<GLOBAL>(pu, make_double2(u.x + tw.x, u.y + tw.y));
-            st2<GLOBAL>(pv, make_double2(u.x - tw.x, u.y - tw.y));
+            *pu = make_double2(u.x + tw.x, u.y + tw.y);
+            *pv = make_double2(u.x - tw.x, u.y - tw.y);
         }
         __syncthreads();
     }
 }
 
-// periodic Poisson + FDA force of one run, all in one CTA (NX <= 4096); the
-// transform array a in shared memory or (GLOBAL) the run's global scratch
-template <bool GLOBAL>
-__device__ void poisson_run(const RunDesc &r, const double *rho_pool, double *acc_pool, double2 *a,
-                            const double2 *__restrict__ tw, const double *__restrict__ green) {
-    const int D = r.dims;
-    const int n0 = r.nx[0], n1 = D == 2 ? r.nx[1] : 1;
-    const long long NX = r.NX;
-    for (long long x = threadIdx.x; x < NX; x += blockDim.x)
-        st2<GLOBAL>(a + x, make_double2(ldcg(rho_pool + r.rho_off + x) - r.rho_bg, 0.0));
-    __syncthreads();
-    for (int ax = 0; ax < D; ++ax) smem_fft<GLOBAL>(a, D, n0, n1, ax, -1, tw);
-    // S / lambda(k) / NX of the run, tabulated at creation (0 at k = 0)
-    for (long long x = threadIdx.x; x < NX; x += blockDim.x) {
-        const double sc = green[r.rho_off + x];
-        const double2 ax = ld2<GLOBAL>(a + x);
-        st2<GLOBAL>(a + x, make_double2(ax.x * sc, ax.y * sc));
-    }
-    __syncthreads();
-    for (int ax = 0; ax < D; ++ax) smem_fft<GLOBAL>(a, D, n0, n1, ax, +1, tw);
-    // a = -grad phi by the 2/4/6-point FDA (Eqs. C9-C11)
+// a = -grad phi by the 2/4/6-point FDA (Eqs. C9-C11) at the points [x0, x1) of a
+// run; at(j) is the potential of point j
+template <typename At>
+__device__ void force_points(const RunDesc &r, int x0, int x1, double *acc_pool, At at) {
+    const int D = r.dims, n0 = r.nx[0], n1 = D == 2 ? r.nx[1] : 1;
     double c1 = 1.0, c2 = 0.0, c3 = 0.0, den = 2.0;
     if (r.pois_order == 4) {
         c1 = 8.0;
@@ -475,20 +494,73 @@ __device__ void poisson_run(const RunDesc &r, const double *rho_pool, double *ac
         den = 60.0;
     }
     const double sc0 = -1.0 / (den * r.hx[0]), sc1 = D == 2 ? -1.0 / (den * r.hx[1]) : 0.0;
-    for (long long x = threadIdx.x; x < NX; x += blockDim.x) {
-        const int i0 = (int)(D == 2 ? x / n1 : x);
-        const int i1 = (int)(D == 2 ? x % n1 : 0);
+    for (int x = x0 + threadIdx.x; x < x1; x += blockDim.x) {
+        const int i0 = D == 2 ? x / n1 : x;
+        const int i1 = D == 2 ? x - i0 * n1 : 0;
         for (int d = 0; d < D; ++d) {
             // power-of-two axes: periodic neighbours by masking
-            auto at = [&](int off) -> double {
+            auto ph = [&](int off) -> double {
                 int j0 = i0, j1 = i1;
                 if (d == 0) j0 = (i0 + off) & (n0 - 1);
                 else j1 = (i1 + off) & (n1 - 1);
-                return ld2<GLOBAL>(a + j0 * n1 + j1).x;
+                return at(j0 * n1 + j1);
             };
-            const double g = c1 * (at(1) - at(-1)) + c2 * (at(2) - at(-2)) + c3 * (at(3) - at(-3));
-            acc_pool[r.acc_off + (long long)d * NX + x] = g * (d == 0 ? sc0 : sc1);
+            const double g = c1 * (ph(1) - ph(-1)) + c2 * (ph(2) - ph(-2)) + c3 * (ph(3) - ph(-3));
+            acc_pool[r.acc_off + (long long)d * r.NX + x] = g * (d == 0 ? sc0 : sc1);
         }
+    }
+}
+
+// periodic Poisson + force of one run, all in one CTA (NX <= kFftTile), the
+// transform array a in shared memory; green: S / lambda(k) / NX of the run,
+// tabulated at creation (0 at k = 0)
+__device__ void poisson_run(const RunDesc &r, const double *rho_pool, double *acc_pool, double2 *a,
+                            const double2 *__restrict__ tw, const double *__restrict__ green) {
+    const int D = r.dims, NX = (int)r.NX;
+    const int n0 = r.nx[0], n1 = D == 2 ? r.nx[1] : 1;
+    for (int x = threadIdx.x; x < NX; x += blockDim.x)
+        a[x] = make_double2(ldcg(rho_pool + r.rho_off + x) - r.rho_bg, 0.0);
+    __syncthreads();
+    for (int ax = 0; ax < D; ++ax) smem_fft(a, D, n0, n1, ax, -1, tw);
+    for (int x = threadIdx.x; x < NX; x += blockDim.x) {
+        const double sc = green[r.rho_off + x];
+        a[x] = make_double2(a[x].x * sc, a[x].y * sc);
+    }
+    __syncthreads();
+    for (int ax = 0; ax < D; ++ax) smem_fft(a, D, n0, n1, ax, +1, tw);
+    force_points(r, 0, NX, acc_pool, [&](int j) { return a[j].x; });
+}
+
+// one tile of a 2D run's solve; buf: the run's transform array in global memory,
+// between stages through L2
+__device__ void poisson_tile(const RunDesc &r, const StageDesc &s, int tile, const double *rho_pool,
+                             double *acc_pool, double2 *buf, double2 *a, const double2 *__restrict__ tw,
+                             const double *__restrict__ green) {
+    const int n0 = r.nx[0], n1 = r.nx[1], w = s.tw;
+    if (s.kind == ST_FORCE) {
+        force_points(r, tile * w, (tile + 1) * w < r.NX ? (tile + 1) * w : (int)r.NX, acc_pool,
+                     [&](int j) { return __ldcg(&buf[j].x); });
+    } else if (s.kind == ST_FFT_COLS) {  // w columns
+        const int c0 = tile * w;
+        for (int t = threadIdx.x; t < n0 * w; t += blockDim.x)
+            a[t] = __ldcg(buf + (t / w) * n1 + c0 + t % w);
+        __syncthreads();
+        smem_fft(a, 2, n0, w, 0, -1, tw);
+        for (int t = threadIdx.x; t < n0 * w; t += blockDim.x) {
+            const double sc = green[r.rho_off + (t / w) * n1 + c0 + t % w];
+            a[t] = make_double2(a[t].x * sc, a[t].y * sc);
+        }
+        __syncthreads();
+        smem_fft(a, 2, n0, w, 0, +1, tw);
+        for (int t = threadIdx.x; t < n0 * w; t += blockDim.x) buf[(t / w) * n1 + c0 + t % w] = a[t];
+    } else {  // w rows, from the density or to the potential
+        const bool fwd = s.kind == ST_FFT_ROWS;
+        const int x0 = tile * w * n1;
+        for (int t = threadIdx.x; t < n1 * w; t += blockDim.x)
+            a[t] = fwd ? make_double2(ldcg(rho_pool + r.rho_off + x0 + t) - r.rho_bg, 0.0) : __ldcg(buf + x0 + t);
+        __syncthreads();
+        smem_fft(a, 2, w, n1, 1, fwd ? -1 : +1, tw);
+        for (int t = threadIdx.x; t < n1 * w; t += blockDim.x) buf[x0 + t] = a[t];
     }
 }
 
@@ -500,68 +572,109 @@ __global__ void __launch_bounds__(kThreads, 6) k_ensemble(float *__restrict__ po
                                                        double *rho_pool, EnsParams P,
                                                        int *__restrict__ status, const double2 *__restrict__ tw,
                                                        const double *__restrict__ green, double2 *fftbuf,
-                                                       const LineShift<float> *__restrict__ dsh) {
+                                                       const LineShift<float> *__restrict__ dsh,
+                                                       const double *__restrict__ kdt) {
     extern __shared__ __align__(16) unsigned char ens_smem[];
-    __shared__ int s_item;
+    __shared__ EnsItem s_item;  // the next item (run < 0: none)
     __shared__ int s_ok;
+    // one thread's state, kept out of everyone's registers: thread 32's last
+    // popped index; thread 0's last dependency seen met (counters only grow)
+    __shared__ int s_popped, s_met_run, s_met_stage;
     unsigned *head = ctr;
     unsigned *done = ctr + 1;
-    if (threadIdx.x == 0) s_item = (int)atomicAdd(head, 1u);
+    const EnsItem none = {-1, 0, 0, 0};
+    const SweepSrc src = {acc_pool, kdt, dsh};
+    // Thread 32 fetches ahead: while an item is worked on, the next one's
+    // descriptor is read and the one after it popped.
+    if (threadIdx.x == 32) {
+        const int first = (int)atomicAdd(head, 1u);
+        s_popped = (int)atomicAdd(head, 1u);
+        s_item = first < nitems ? items[first] : none;
+        s_met_run = s_met_stage = -1;
+    }
     __syncthreads();
-    int met_run = -1, met_stage = -1;  // thread 0: the last dependency seen met (counters only grow)
+    // The item before this one, finished but not announced yet (its counter, or
+    // -1): its stores drain while this item's tile is read, and the barrier after
+    // the staging announces it.  An item whose dependency is not met yet
+    // announces first and waits then, so no CTA waits with work unannounced.
+    int pend = -1;
     while (true) {
-        const int it = s_item;
-        if (it >= nitems) break;
-        const EnsItem e = items[it];
+        const EnsItem e = s_item;
+        if (e.run < 0) break;
         const RunDesc &r = runs[e.run];
         const StageDesc &s = r.st[e.stage];
         if (threadIdx.x == 0) {
-            s_ok = 1;
-            if (e.stage > 0 && (e.run != met_run || e.stage != met_stage)) {
+            int ok = 1;
+            if (e.stage > 0 && (e.run != s_met_run || e.stage != s_met_stage)) {
                 const StageDesc &prev = r.st[e.stage - 1];
-                if (!wait_count(done + prev.done_slot, (unsigned)prev.tiles, P.wait_limit)) {
-                    atomicExch(status, VP_ETIMEOUT);
-                    s_ok = 0;
-                } else {
-                    met_run = e.run;
-                    met_stage = e.stage;
-                }
+                ok = wait_count(done + prev.done_slot, (unsigned)prev.tiles, P.wait_limit ? 1u : 0u);
+                s_met_run = e.run;
+                s_met_stage = e.stage;
             }
+            s_ok = ok;
         }
-        __syncthreads();
-        if (!s_ok) return;
-        // every thread has read s_item: the next item is popped now (by a thread
-        // of the second warp), its latency hidden behind this item's work; the
-        // barrier that ends this item publishes it
-        if (threadIdx.x == 32) s_item = (int)atomicAdd(head, 1u);
+        __syncthreads();  // all threads are done with the item before (and its shared memory)
+        if (!s_ok) {
+            __threadfence();
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                if (pend >= 0) atomicAdd(done + pend, 1u);
+                const StageDesc &prev = r.st[e.stage - 1];
+                s_ok = wait_count(done + prev.done_slot, (unsigned)prev.tiles,
+                                  P.wait_limit ? P.wait_limit - 1u : 0u);
+                if (!s_ok) atomicExch(status, VP_ETIMEOUT);
+            }
+            pend = -1;
+            __syncthreads();
+            if (!s_ok) return;
+        }
+        EnsItem ahead = none;
+        int popped = 0;
+        if (threadIdx.x == 32) {
+            if (s_popped < nitems) ahead = items[s_popped];
+            popped = (int)atomicAdd(head, 1u);
+        }
+        auto staged = [&]() {
+            if (pend >= 0) __threadfence();
+            if (threadIdx.x == 32) {
+                s_item = ahead;
+                s_popped = popped;
+            }
+            __syncthreads();
+            if (threadIdx.x == 0 && pend >= 0) atomicAdd(done + pend, 1u);
+        };
         if (s.kind == ST_COLS) {
             if (s.periodic)
-                tile_cols<ORDER, true, FLAT>(pool, r, s, e.tile, acc_pool, dsh, P,
-                                             reinterpret_cast<float *>(ens_smem));
+                tile_cols<ORDER, true, FLAT>(pool, r, s, e.tile, src, P, reinterpret_cast<float *>(ens_smem),
+                                             staged);
             else
-                tile_cols<ORDER, false, FLAT>(pool, r, s, e.tile, acc_pool, dsh, P,
-                                              reinterpret_cast<float *>(ens_smem));
+                tile_cols<ORDER, false, FLAT>(pool, r, s, e.tile, src, P, reinterpret_cast<float *>(ens_smem),
+                                              staged);
         } else if (s.kind == ST_ROWS) {
-            tile_rows<ORDER, FLAT>(pool, r, s, e.tile, acc_pool, P, reinterpret_cast<float *>(ens_smem));
+            tile_rows<ORDER, FLAT>(pool, r, s, e.tile, src, P, reinterpret_cast<float *>(ens_smem), staged);
         } else if (s.kind == ST_MOMENT) {
+            staged();
             const long long x0 = (long long)e.tile * P.xpt;
             const long long x1 = x0 + P.xpt < r.NX ? x0 + P.xpt : r.NX;
             density_points(pool, r, x0, x1, rho_pool);
+        } else if (s.kind != ST_POISSON) {
+            staged();
+            poisson_tile(r, s, e.tile, rho_pool, acc_pool, fftbuf + r.rho_off,
+                         reinterpret_cast<double2 *>(ens_smem), tw, green);
         } else {
+            staged();
             if (r.dims == 1) {  // the 1D density is small enough to fuse here
                 density_points(pool, r, 0, r.NX, rho_pool);
                 __threadfence_block();
                 __syncthreads();
             }
-            if (r.NX <= kSmemFftMax)
-                poisson_run<false>(r, rho_pool, acc_pool, reinterpret_cast<double2 *>(ens_smem), tw, green);
-            else
-                poisson_run<true>(r, rho_pool, acc_pool, fftbuf + r.rho_off, tw, green);
+            poisson_run(r, rho_pool, acc_pool, reinterpret_cast<double2 *>(ens_smem), tw, green);
         }
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) atomicAdd(done + s.done_slot, 1u);
+        pend = s.done_slot;
     }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && pend >= 0) atomicAdd(done + pend, 1u);
 }
 
 size_t smem_need(const std::vector<RunDesc> &runs) {
@@ -575,7 +688,9 @@ size_t smem_need(const std::vector<RunDesc> &runs) {
             } else if (s.kind == ST_ROWS) {
                 b = (size_t)s.tw * (((s.L + 2 * VP_GHOST) | 1) + (s.L | 1)) * sizeof(float);
             } else if (s.kind == ST_POISSON) {
-                b = r.NX <= kSmemFftMax ? (size_t)r.NX * sizeof(double2) : 0;
+                b = (size_t)r.NX * sizeof(double2);
+            } else if (s.kind == ST_FFT_ROWS || s.kind == ST_FFT_COLS || s.kind == ST_FFT_BACK) {
+                b = kFftTile * sizeof(double2);
             }
             need = b > need ? b : need;
         }
@@ -605,6 +720,7 @@ struct vp_ens {
     long long acc_total, rho_total;
     RunDesc *d_runs;
     EnsItem *d_items_step, *d_items_field;
+    double *d_kdt;     // (dt / 2) / hv of every run's kicks for dsh_dt
     unsigned *d_ctr;
     int nslots;
     int *d_status;
@@ -629,7 +745,7 @@ static int ens_fail(vp_ens *e, int code, const char *msg) {
 static int build_stages(RunDesc &r, int W, int R, int xpt, int &slot) {
     const int D = r.dims;
     auto cols = [&](int kick, int axis, int half, long long outer, int L, long long inner, int per,
-                    int from_inner, long long cdiv, long long cmod) {
+                    long long cdiv, long long cmod) {
         StageDesc s{};
         s.kind = ST_COLS;
         s.kick = kick;
@@ -639,15 +755,18 @@ static int build_stages(RunDesc &r, int W, int R, int xpt, int &slot) {
         s.L = L;
         s.inner = inner;
         s.periodic = per;
-        s.cls_from_inner = from_inner;
-        s.cdiv = cdiv;
-        s.cmod = cmod;
         // tile width: the requested W, halved until the staged tile fits kTileBytes
         int w = W;
         while (w > 8 && (size_t)(L + (per ? 0 : 2 * VP_GHOST)) * w * sizeof(float) > kTileBytes) w /= 2;
         if (inner < w) w = (int)inner;
         s.tw = w;
+        s.nseg = kThreads / w;
         s.tiles = (int)(outer * ((inner + w - 1) / w));
+        s.fd_tpo = make_fastdiv((unsigned)((inner + w - 1) / w));
+        s.fd_tw = make_fastdiv((unsigned)w);
+        s.fd_nseg = make_fastdiv((unsigned)s.nseg);
+        s.fd_cdiv = make_fastdiv((unsigned)cdiv);
+        s.fd_cmod = make_fastdiv((unsigned)cmod);
         return s;
     };
     auto rows = [&](int axis, long long outer, int L, long long cdiv) {
@@ -659,18 +778,21 @@ static int build_stages(RunDesc &r, int W, int R, int xpt, int &slot) {
         s.outer = outer;
         s.L = L;
         s.inner = 1;
-        s.cdiv = cdiv;
-        s.cmod = 1;
         int rr = R;
         while (rr > 8 && (size_t)rr * (((L + 2 * VP_GHOST) | 1) + (L | 1)) * sizeof(float) > kTileBytes) rr /= 2;
         s.tw = rr;
+        s.nseg = kThreads / rr;
         s.tiles = (int)((outer + rr - 1) / rr);
+        s.fd_tw = make_fastdiv((unsigned)rr);
+        s.fd_L = make_fastdiv((unsigned)L);
+        s.fd_nseg = make_fastdiv((unsigned)s.nseg);
+        s.fd_cdiv = make_fastdiv((unsigned)cdiv);
         return s;
     };
     int k = 0;
     if (D == 1) {
         r.st[k++] = rows(0, r.NX, r.nv[0], 1);
-        r.st[k++] = cols(0, 0, 0, 1, r.nx[0], r.NV, 1, 1, 1, r.nv[0]);
+        r.st[k++] = cols(0, 0, 0, 1, r.nx[0], r.NV, 1, 1, r.nv[0]);
         StageDesc p{};
         p.kind = ST_POISSON;
         p.tiles = 1;
@@ -678,20 +800,33 @@ static int build_stages(RunDesc &r, int W, int R, int xpt, int &slot) {
         r.st[k++] = rows(0, r.NX, r.nv[0], 1);
     } else {
         // kick v1 (strided over v2), kick v2 (contiguous)
-        r.st[k++] = cols(1, 0, 1, r.NX, r.nv[0], r.nv[1], 0, 0, 1, 1);
+        r.st[k++] = cols(1, 0, 1, r.NX, r.nv[0], r.nv[1], 0, 1, 1);
         r.st[k++] = rows(1, r.NX * r.nv[0], r.nv[1], r.nv[0]);
         // drift x2 then x1 (Eq. 55 order)
-        r.st[k++] = cols(0, 1, 0, r.nx[0], r.nx[1], r.NV, 1, 1, 1, r.nv[1]);
-        r.st[k++] = cols(0, 0, 0, 1, r.nx[0], (long long)r.nx[1] * r.NV, 1, 1, r.nv[1], r.nv[0]);
+        r.st[k++] = cols(0, 1, 0, r.nx[0], r.nx[1], r.NV, 1, 1, r.nv[1]);
+        r.st[k++] = cols(0, 0, 0, 1, r.nx[0], (long long)r.nx[1] * r.NV, 1, r.nv[1], r.nv[0]);
         StageDesc m{};
         m.kind = ST_MOMENT;
         m.tiles = (int)((r.NX + xpt - 1) / xpt);
         r.st[k++] = m;
-        StageDesc p{};
-        p.kind = ST_POISSON;
-        p.tiles = 1;
-        r.st[k++] = p;
-        r.st[k++] = cols(1, 0, 1, r.NX, r.nv[0], r.nv[1], 0, 0, 1, 1);
+        auto solve = [&](int kind, int w, int tiles) {
+            StageDesc p{};
+            p.kind = kind;
+            p.tw = w;
+            p.tiles = tiles;
+            r.st[k++] = p;
+        };
+        if (r.NX <= kFftTile) {
+            solve(ST_POISSON, 0, 1);
+        } else {  // axes are powers of two: tiles divide them
+            const int n0 = r.nx[0], n1 = r.nx[1];
+            const int wr = kFftTile / n1, wc = kFftTile / n0;
+            solve(ST_FFT_ROWS, wr, n0 / wr);
+            solve(ST_FFT_COLS, wc, n1 / wc);
+            solve(ST_FFT_BACK, wr, n0 / wr);
+            solve(ST_FORCE, kFftTile, (int)(r.NX / kFftTile));
+        }
+        r.st[k++] = cols(1, 0, 1, r.NX, r.nv[0], r.nv[1], 0, 1, 1);
         r.st[k++] = rows(1, r.NX * r.nv[0], r.nv[1], r.nv[0]);
     }
     r.nstage = k;
@@ -710,14 +845,9 @@ static void build_items(vp_ens *e) {
             if (st >= r.nstage) continue;
             for (int t = 0; t < r.st[st].tiles; ++t) e->items_step.push_back(EnsItem{ri, st, t, 0});
         }
-    // field-only list: the density (2D) and Poisson stages, as stages 0/1 of a
-    // separate pass (their waits refer to the previous stage of the same list)
-    for (int ri = 0; ri < (int)e->runs.size(); ++ri) {
-        const RunDesc &r = e->runs[ri];
-        for (int st = 0; st < r.nstage; ++st)
-            if (r.st[st].kind == ST_MOMENT || r.st[st].kind == ST_POISSON)
-                for (int t = 0; t < r.st[st].tiles; ++t) e->items_field.push_back(EnsItem{ri, st, t, 0});
-    }
+    // the field-only list: the same stages without the sweeps
+    for (const EnsItem &it : e->items_step)
+        if (field_stage(e->runs[it.run].st[it.stage].kind)) e->items_field.push_back(it);
 }
 
 static int upload_plan(vp_ens *e) {
@@ -728,7 +858,7 @@ static int upload_plan(vp_ens *e) {
     e->d_items_step = e->d_items_field = nullptr;
     if (cudaMalloc(&e->d_runs, sizeof(RunDesc) * e->runs.size()) != cudaSuccess ||
         cudaMalloc(&e->d_items_step, sizeof(EnsItem) * e->items_step.size()) != cudaSuccess ||
-        cudaMalloc(&e->d_items_field, sizeof(EnsItem) * (e->items_field.size() + 1)) != cudaSuccess)
+        cudaMalloc(&e->d_items_field, sizeof(EnsItem) * e->items_field.size()) != cudaSuccess)
         return ens_fail(e, VP_ENOMEM, "plan allocation failed");
     if (cudaMemcpy(e->d_runs, e->runs.data(), sizeof(RunDesc) * e->runs.size(), cudaMemcpyHostToDevice) !=
             cudaSuccess ||
@@ -740,14 +870,12 @@ static int upload_plan(vp_ens *e) {
     return VP_OK;
 }
 
-// the field pass waits on stage - 1 of the full list; give it its own view in
-// which the density stage (2D) precedes Poisson and nothing precedes density
 // the drift shift table for dt (before a step graph is captured; never inside one)
 static int ensure_drift_table(vp_ens *e, double dt) {
     if (e->dsh_valid && e->dsh_dt == dt) return VP_OK;
     EnsParams P = e->P;
     P.dt = dt;
-    k_ens_drift_table<<<(unsigned)e->runs.size(), 128, 0, e->stream>>>(e->d_runs, e->d_dsh, P);
+    k_ens_drift_table<<<(unsigned)e->runs.size(), 128, 0, e->stream>>>(e->d_runs, e->d_dsh, e->d_kdt, P);
     e->launches++;
     const cudaError_t er = cudaGetLastError();
     if (er != cudaSuccess) return ens_fail(e, VP_ECUDA, cudaGetErrorString(er));
@@ -767,7 +895,7 @@ static void launch_k(vp_ens *e, const EnsItem *items, int nitems, const EnsParam
 #define VP_ENS_LAUNCH(O, F)                                                                                 \
     k_ensemble<O, F><<<grid, kThreads, e->smem, e->stream>>>(e->pool, e->d_runs, items, nitems, e->d_ctr,   \
                                                              e->d_acc, e->d_rho, P, e->d_status, e->d_tw,   \
-                                                             e->d_green, e->d_fft, e->d_dsh)
+                                                             e->d_green, e->d_fft, e->d_dsh, e->d_kdt)
     if (e->P.order == 7) {
         if (e->flat) VP_ENS_LAUNCH(7, true);
         else VP_ENS_LAUNCH(7, false);
@@ -846,6 +974,7 @@ int vp_ensemble_create(const vp_run_desc *runs, int nruns, int order, void *cuda
         r.acc_off = aoff;
         r.rho_off = roff;
         r.dsh_off = soff;
+        r.kdt_off = 2 * i;
         r.coupling = d.coupling;
         r.rho_bg = d.rho_bg;
         r.pois_order = d.pois_order == 2 || d.pois_order == 4 ? d.pois_order : 6;
@@ -866,6 +995,7 @@ int vp_ensemble_create(const vp_run_desc *runs, int nruns, int order, void *cuda
         cudaMalloc(&e->d_rho, sizeof(double) * roff) != cudaSuccess ||
         cudaMalloc(&e->d_fft, sizeof(double2) * roff) != cudaSuccess ||
         cudaMalloc(&e->d_dsh, sizeof(LineShift<float>) * soff) != cudaSuccess ||
+        cudaMalloc(&e->d_kdt, sizeof(double) * 2 * nruns) != cudaSuccess ||
         cudaMalloc(&e->d_ctr, sizeof(unsigned) * (slot + 1)) != cudaSuccess ||
         cudaMalloc(&e->d_status, sizeof(int)) != cudaSuccess) {
         vp_ensemble_destroy(e);
@@ -937,6 +1067,7 @@ void vp_ensemble_destroy(vp_ens *e) {
     cudaFree(e->d_rho);
     cudaFree(e->d_fft);
     cudaFree(e->d_dsh);
+    cudaFree(e->d_kdt);
     cudaFree(e->d_tw);
     cudaFree(e->d_green);
     cudaFree(e->d_ctr);
@@ -977,34 +1108,19 @@ int vp_ensemble_accel(const vp_ens *e, const double **accel_dev) {
 
 int vp_ensemble_field(vp_ens *e) {
     if (!e || !e->pool) return VP_EINVAL;
-    // the field list holds, per run, (density, Poisson) for 2D and (Poisson) for
-    // 1D; the wait of each item refers to stage - 1 of its run in the full
-    // plan, which the field pass has not run: run it stage by stage instead
-    std::vector<EnsItem> pass;
-    for (int phase = 0; phase < 2; ++phase) {
-        pass.clear();
-        for (const EnsItem &it : e->items_field) {
-            const StageDesc &s = e->runs[it.run].st[it.stage];
-            if ((phase == 0) == (s.kind == ST_MOMENT)) pass.push_back(it);
-        }
-        if (pass.empty()) continue;
-        if (cudaMemcpy(e->d_items_field, pass.data(), sizeof(EnsItem) * pass.size(), cudaMemcpyHostToDevice) !=
-            cudaSuccess)
-            return ens_fail(e, VP_ECUDA, "field plan upload failed");
-        // mark every previous stage complete so the waits pass immediately
-        std::vector<unsigned> ctr(e->nslots + 1, 0u);
-        for (const RunDesc &r : e->runs)
-            for (int k = 0; k < r.nstage; ++k) ctr[1 + r.st[k].done_slot] = (unsigned)r.st[k].tiles;
-        for (const EnsItem &it : pass) ctr[1 + e->runs[it.run].st[it.stage].done_slot] = 0;
-        if (cudaMemcpyAsync(e->d_ctr, ctr.data(), sizeof(unsigned) * ctr.size(), cudaMemcpyHostToDevice,
-                            e->stream) != cudaSuccess)
-            return ens_fail(e, VP_ECUDA, "counter upload failed");
-        EnsParams P = e->P;
-        P.dt = 0.0;
-        launch_k(e, e->d_items_field, (int)pass.size(), P);
-        e->launches++;
-        if (cudaStreamSynchronize(e->stream) != cudaSuccess) return ens_fail(e, VP_ECUDA, "field pass failed");
-    }
+    // the waits refer to the full plan's stages: the sweeps count as done
+    std::vector<unsigned> ctr(e->nslots + 1, 0u);
+    for (const RunDesc &r : e->runs)
+        for (int k = 0; k < r.nstage; ++k)
+            if (!field_stage(r.st[k].kind)) ctr[1 + r.st[k].done_slot] = (unsigned)r.st[k].tiles;
+    if (cudaMemcpyAsync(e->d_ctr, ctr.data(), sizeof(unsigned) * ctr.size(), cudaMemcpyHostToDevice, e->stream) !=
+        cudaSuccess)
+        return ens_fail(e, VP_ECUDA, "counter upload failed");
+    EnsParams P = e->P;
+    P.dt = 0.0;
+    launch_k(e, e->d_items_field, (int)e->items_field.size(), P);
+    e->launches++;
+    if (cudaStreamSynchronize(e->stream) != cudaSuccess) return ens_fail(e, VP_ECUDA, "field pass failed");
     return VP_OK;
 }
 

@@ -184,3 +184,32 @@ def test_flat_vote_does_not_change_the_bits():
             assert V.vp_ensemble_get_flat_vote(ens) in (0, 1)
         V.vp_ensemble_destroy(ens)
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("W,R", [(64, 32), (8, 128)])
+@pytest.mark.parametrize("nx,nv", [([16, 16], [5, 7]), ([2, 256], [12, 20]), ([256, 2], [3, 33]), ([16, 32], [40, 12]),
+                                   ([64, 64], [6, 8])])
+def test_solves_of_one_and_of_four_stages(nx, nv, W, R):
+    """2D runs at and above the points that one tile solves, with narrow and
+    wide axes and odd velocity grids, beside 1D runs whose stages they meet in
+    the queue: kicks of tiles that span one, few and many spatial points,
+    against the single-run path.  f of the two differs by the roundings of the
+    shifts' weights (FP32 here), as in the comparison above: 1e-6."""
+    import torch
+    specs = _runs()[:2]
+    for alpha in (0.3, 0.1):
+        specs.append(dict(kind="landau", dims=2, nx=nx, nv=nv, k=[0.5, 1.0], alpha=alpha, xlo=[0.0, 0.0],
+                          xhi=[4 * math.pi, 2 * math.pi], vlo=[-5.0, -6.0], vhi=[6.0, 5.0]))
+    ens, pool = _ensemble(specs, torch.cuda.Stream())
+    V.vp_ensemble_set_tiles(ens, W, R, 0)
+    V.vp_ensemble_step(ens, 0.05, 4)
+    V.vp_ensemble_sync(ens)
+    for i, s in enumerate(specs):
+        sim = V.Simulation(_grid(s), precision=V.VP_F32)
+        V.vp_init_f(sim.ctx, *_ic(s))
+        sim.field()
+        sim.step(0.05, 4, split=V.VP_SPLIT_KDK)
+        sim.sync()
+        assert rel_l1(_run_slice(ens, pool, i, s), sim.f.double().cpu().numpy()) <= 1e-6, i
+        sim.close()
+    V.vp_ensemble_destroy(ens)
