@@ -322,6 +322,10 @@ LINE_CASES = [
     (2, [6, 10], [8, 12], 0, 0, 1, 1.3),
     (2, [5, 4], [16, 9], 1, 1, 0, 0.6),
     (2, [5, 4], [9, 16], 0, 1, 1, 0.8),
+    # lines in fours on 16-byte boundaries: open and kicked ones, a ragged last tile
+    (2, [6, 10], [8, 12], 1, 0, 0, 0.4),
+    (2, [5, 4], [9, 16], 1, 1, 0, 0.6),
+    (1, [33], [140], 0, 0, 0, 0.2),
 ]
 
 
