@@ -151,7 +151,7 @@ def test_rk_two_line_kernel_gives_the_same_bits(dims, nx, nv):
 @pytest.mark.parametrize("n1,nv", [(12, [40, 36]), (3, [21, 33]), (7, [64, 18])])
 def test_whole_lines_in_place_give_the_same_bits(xbc, n1, nv):
     """Grids with many lines run the three stages of whole lines in place, small
-    grids through three tiles: every line of a large grid's strided sweeps (even
+    grids through three tiles: every line of a large grid's sweeps (even
     and odd rows, lines shorter than the stencil, both boundaries and directions,
     one and two lines per thread) gives the bits it gives in a grid of one x2 row."""
     n2 = 100_000 // (n1 * min(nv)) + 1
@@ -172,7 +172,7 @@ def test_whole_lines_in_place_give_the_same_bits(xbc, n1, nv):
         out = from_gpu(sim).reshape(n1, n, *nv)
         sim.close()
         return out
-    for kick, d in ((0, 0), (1, 0)):
+    for kick, d in ((0, 0), (1, 0), (1, 1)):  # strided, strided, contiguous
         big = [run(n2, f, acc, kick, d, impl) for impl in (0, 1)]
         assert np.array_equal(big[0], big[1])
         for r in rows:
