@@ -314,7 +314,7 @@ int vp_ensemble_field(vp_ens *ens);
 /* device pointer to the field array (sum over runs of dims * NX doubles) */
 int vp_ensemble_accel(const vp_ens *ens, const double **accel_dev);
 /* tile shapes: W columns per strided tile, R lines per contiguous tile (both
- * dividing 256), CTAs per SM of the persistent grid (0 = occupancy maximum) */
+ * dividing 128), CTAs per SM of the persistent grid (0 = occupancy maximum) */
 int vp_ensemble_set_tiles(vp_ens *ens, int W, int R, int ctas_per_sm);
 int vp_ensemble_get_tiles(const vp_ens *ens, int *out3);
 /* Whether the line walkers of the ensemble vote, warp by warp, on flat
