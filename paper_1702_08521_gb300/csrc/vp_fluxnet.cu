@@ -565,36 +565,9 @@ __global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, 
         // the shift of the stencil: modulo the line, or just off its ends
         const int ns = q.periodic ? n % L : (n < -2 * L - 8 ? -2 * L - 8 : (n > 2 * L + 8 ? 2 * L + 8 : n));
         const float *ui = u + i;
-        // a run of interfaces per thread; the stencil (rows a .. a + 6) slides
-        // along it
-        const int nseg = blockDim.x >> q.logW, seg = threadIdx.x >> q.logW;
-        const int j0 = seg * nout / nseg, j1 = (seg + 1) * nout / nseg;
-        float w[7];
-        int at = 0x40000000;  // row of w[0]
-        for (int j = j0; j < j1; ++j) {
-            // interface between cells c - 1 and c; its stencil in the upwind
-            // frame is centred n cells upwind (rows down to -kEdge and up to
-            // L + kEdge - 1 are staged)
+        // the mass through interface j, M the fractional one in the upwind frame
+        auto emit = [&](int j, float M) {
             const int c = j * every;
-            int a = sg > 0 ? c - ns - 4 : c + ns - 3;
-            if (q.periodic) {
-                while (a < -kEdge) a += L;
-                while (a > L + 1) a -= L;
-            } else {
-                a = a < -7 ? -7 : (a > L ? L : a);
-            }
-            if (a == at + 1) {
-#pragma unroll
-                for (int k = 0; k < 6; ++k) w[k] = w[k + 1];
-                w[6] = ui[(a + 6) * WP];
-            } else if (a != at) {
-#pragma unroll
-                for (int k = 0; k < 7; ++k) w[k] = ui[(a + k) * WP];
-            }
-            at = a;
-            const float M =
-                sg > 0 ? vp_core::flux<float, 7, true>(sh, w[0], w[1], w[2], w[3], w[4], w[5], w[6], alpha, 1, 1)
-                       : vp_core::flux<float, 7, true>(sh, w[6], w[5], w[4], w[3], w[2], w[1], w[0], alpha, 1, 1);
             double g;
             if (PREFIX) {
                 // sum of the cells before k, extended beyond the line
@@ -614,6 +587,11 @@ __global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, 
                 g = sg > 0 ? g : -g;
             } else {
                 // |n| < kFewCells: the cells lie within the staged rows
+                if (n == 0) {
+                    M = __fadd_rn(M, 0.f);  // (the sum of no cells and M: no -0)
+                    Gs[i * NP + j] = widen(sg > 0 ? M : -M);
+                    return;
+                }
                 PairSum p{0.f, 0.f};
                 const float *v = ui + (sg > 0 ? (n >= 0 ? c - n : c) : (n >= 0 ? c : c + n)) * WP;
                 const float one = n >= 0 ? 1.f : -1.f;
@@ -624,6 +602,55 @@ __global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, 
                 g = p.value();
             }
             Gs[i * NP + j] = g;
+        };
+        // A run of interfaces per thread, upwind to downwind; the stencil (rows a ..
+        // a + 6, w in upwind order from row b) slides along it, in blocks of seven
+        // steps without a move while it meets neither a wrap nor an end
+        const int nseg = blockDim.x >> q.logW, seg = threadIdx.x >> q.logW;
+        const int j0 = seg * nout / nseg, j1 = (seg + 1) * nout / nseg;
+        float w[7];
+        int at = 0x40000000;  // row of w[0]
+        for (int k = 0; k < j1 - j0;) {
+            // interface between cells c - 1 and c; its stencil in the upwind
+            // frame is centred n cells upwind (rows down to -kEdge and up to
+            // L + kEdge - 1 are staged)
+            const int j = sg > 0 ? j0 + k : j1 - 1 - k, c = j * every;
+            int a = sg > 0 ? c - ns - 4 : c + ns - 3;
+            bool inside = true;
+            if (q.periodic) {
+                while (a < -kEdge) a += L;
+                while (a > L + 1) a -= L;
+            } else {
+                inside = a >= -7 && a <= L;
+                a = a < -7 ? -7 : (a > L ? L : a);
+            }
+            const int b = sg > 0 ? a : a + 6;
+            if (b == at + sg) {
+#pragma unroll
+                for (int m = 0; m < 6; ++m) w[m] = w[m + 1];
+                w[6] = ui[(b + 6 * sg) * WP];
+            } else if (b != at) {
+#pragma unroll
+                for (int m = 0; m < 7; ++m) w[m] = ui[(b + m * sg) * WP];
+            }
+            at = b;
+            // (the last row read is a + 13 <= L + kEdge - 1 or a - 7 >= -kEdge)
+            if (every == 1 && inside && k + 7 <= j1 - j0 && (sg > 0 ? a + 6 <= L : a - 6 >= -7)) {
+                const float *v = ui + (b + 7 * sg) * WP;
+#pragma unroll
+                for (int m = 0; m < 7; ++m) {
+                    emit(j + m * sg, vp_core::flux<float, 7, true>(sh, w[m], w[(m + 1) % 7], w[(m + 2) % 7],
+                                                                   w[(m + 3) % 7], w[(m + 4) % 7], w[(m + 5) % 7],
+                                                                   w[(m + 6) % 7], alpha, 1, 1));
+                    w[m] = *v;
+                    v += sg * WP;
+                }
+                at = b + 7 * sg;
+                k += 7;
+            } else {
+                emit(j, vp_core::flux<float, 7, true>(sh, w[0], w[1], w[2], w[3], w[4], w[5], w[6], alpha, 1, 1));
+                ++k;
+            }
         }
     }
     __syncthreads();
