@@ -521,7 +521,7 @@ __device__ __forceinline__ void stage_quads(const float *__restrict__ f, const L
 // A CTA stages W lines and the block of results, which it writes as one
 // contiguous run (one thread per line, its results in rows of its own, its
 // stencil from global memory and double-precision prefix sums took 2783 us for
-// 6.7e7 cells; the output alone is 80 us of HBM).  Whole-cell parts of at most
+// 6.7e7 cells; the output alone is 80 us of HBM; now ~400 us, bound by issue).  Whole-cell parts of at most
 // kFewCells cells are summed directly; PREFIX: longer ones from double prefix
 // sums of the line.
 constexpr int kFewCells = 8;
@@ -713,6 +713,20 @@ __global__ void __launch_bounds__(256) k_restrict_v2(const float *__restrict__ f
 // written by single threads it took 1205 us for 4.3e6 samples (430 MB).
 constexpr int kSampleThreads = 256;
 
+// a / s to 2^-47, for a result that is rounded to float: one Newton-Raphson
+// correction of a times the float reciprocal, 3 FP64 instructions in place of a
+// division's, which were half of the kernel's FP64 time; s outside the range in
+// which neither the reciprocal nor its products leave the normal numbers takes
+// the division, out of line.  Training samples of a 64 x 128 per axis 2D2V grid:
+// 838 -> 811 us.
+__device__ __noinline__ double ratio_rare(double a, float s) { return a / (double)s; }
+__device__ __forceinline__ double ratio(double a, float s) {
+    const int ex = (int)(__float_as_uint(s) >> 23 & 0xffu), ea = __double2hiint(a) >> 20 & 0x7ff;
+    if ((unsigned)(ex - 27) > 200u || (unsigned)(ea - 300) > 1400u) return ratio_rare(a, s);
+    const double r = widen(__frcp_rn(s)), q = __dmul_rn(a, r);
+    return fma(fma(-q, widen(s), a), r, q);
+}
+
 template <bool STAGED>
 __global__ void __launch_bounds__(kSampleThreads)
     k_make_samples(const float *__restrict__ fc, LineTile q, const LineShift<float> *__restrict__ tab, int kick,
@@ -813,7 +827,7 @@ __global__ void __launch_bounds__(kSampleThreads)
                 for (int m = 1; m < 7; ++m) phi = fmaf(sh.w[m], u[m], phi);
                 phi = vp_core::mp_limit(phi, u[1], u[2], u[3], u[4], u[5], alpha);
                 const float s = net_features(u, unp, unm, sh.nu, x);
-                y[t0 + t] = (float)((g - whole - widen(sh.nu) * widen(phi)) / widen(s));
+                y[t0 + t] = (float)ratio(g - whole - widen(sh.nu) * widen(phi), s);
                 if (sc) sc[t0 + t] = s;
             }
 #pragma unroll

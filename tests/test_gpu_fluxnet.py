@@ -439,3 +439,37 @@ def test_restriction_and_group_means(nf, factors):
                     torch.as_tensor(m.reshape(-1), dtype=torch.int64, device="cuda"), grp, 0.25, Gc)
     torch.cuda.synchronize()
     assert np.abs(Gc.cpu().numpy().reshape(n, nout) - 0.25 * Gf[m].mean(1)).max() <= 1e-15 * grp
+
+
+@pytest.mark.parametrize("power", [-112, -99, 60, 99, 112])
+def test_sample_targets_at_every_scale_of_f(power):
+    """Targets are masses over s, the stencil's largest cell (with a floor): the
+    targets of masses Gc less those of no mass are Gc / s in the upwind frame,
+    with f and Gc scaled by powers of two to within the fast division's range, to
+    its ends and beyond.  FP32 roundings of masses of order s: 1e-6."""
+    import torch
+    rng = np.random.default_rng(5)
+    f = ((1.0 + 0.5 * rng.random((12, 24))) * 2.0 ** power).astype(np.float32)
+    G = rng.random((24, 13)) * 2.0 ** power
+    sim = V.Simulation(dict(dims=1, nx=[12], nv=[24], xlo=[0.0], xhi=[1.0], vlo=[-3.0], vhi=[2.5], order=7),
+                       precision=V.VP_F32)
+    sim.upload(f.reshape(-1))
+
+    def targets(Gc):
+        X, y = torch.empty(24 * 13, 25, device="cuda"), torch.empty(24 * 13, device="cuda")
+        s = torch.empty(24 * 13, device="cuda")
+        torch.cuda.synchronize()
+        V.vp_make_samples(sim.ctx, 0, 0, 0.02, None, torch.as_tensor(Gc, device="cuda"), 0.0, X, y, s)
+        sim.sync()
+        return y.cpu().numpy().reshape(24, 13), s.cpu().numpy().reshape(24, 13)
+    y1, s = targets(G)
+    y0, _ = targets(np.zeros_like(G))
+    speed = -3.0 + 5.5 / 24 * (np.arange(24) + 0.5)  # |shift| < 1/2 at nx dt |v| = 0.72 for some, above for others
+    shift = speed * 0.02 * 12
+    sign = np.where(shift - np.round(shift) < 0, -1.0, 1.0)[:, None]
+    ok = ~np.isnan(y1)
+    assert ok.any() and np.array_equal(ok, ~np.isnan(y0))
+    want = sign * G / np.where(ok, s, 1.0).astype(np.float64)
+    size = np.abs(y1[ok]).max() + np.abs(y0[ok]).max()
+    assert np.abs(y1.astype(np.float64) - y0 - want)[ok].max() <= 1e-6 * size
+    sim.close()
