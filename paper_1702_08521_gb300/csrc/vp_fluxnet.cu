@@ -80,14 +80,16 @@ __device__ __forceinline__ float net_features(const float *u, const float *up, c
 // weight gradients, whose contraction runs over the samples.  (tcgen05 needs
 // 128-row operands in shared memory and a barrier round trip per layer; three
 // chained 32 x 32 layers of 16 rows are all latency there.)
-//   forward   Z = W A + b: bfloat16 operands as defined, FP32 sums;
+//   forward   Z = W A + b: bfloat16 operands as defined, FP32 sums, and those
+//             whose last bits could decide the bfloat16 activation once more,
+//             exactly (activate);
 //   backward  the FP32 deltas are split into three bfloat16 terms (24 bits), so
 //             that no bit of them is lost: dA = W^T delta, dW += delta A^T.
 // Weight gradients stay in registers over all of a warp's tiles, are summed over
 // the CTA in shared memory and added to global memory once per CTA.
-// 32 768 samples: 62 -> 13.7 us; with one thread per sample and both operands of
-// every FMA read from shared memory the LSU pipe set the time (67% busy, 256
-// CTAs of 75 KB, 10% of the warps).
+// A training step of 32 768 samples: 65 -> 27.3 us; with one thread per sample and
+// both operands of every FMA read from shared memory the LSU pipe set the time
+// (67% busy, 256 CTAs of 75 KB, 10% of the warps).
 // Samples come in consecutive groups of `group` (1 or 2; a pair = the two
 // interfaces of one cell) whose residual is r = sum_k a_k (g_k - y_k) (a_k =
 // coef[k], 1 without coef); the loss is the mean of r^2 over groups.
@@ -110,6 +112,12 @@ __device__ __forceinline__ uint32_t transpose8x8(uint32_t a) {
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t *>(&v);
+}
+// bf16(max(lo, 0)) in the low half, bf16(max(hi, 0)) in the high half
+__device__ __forceinline__ uint32_t pack_relu_bf16(float lo, float hi) {
+    uint32_t d;
+    asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+    return d;
 }
 __device__ __forceinline__ float low_half(uint32_t p) { return __uint_as_float(p << 16); }
 __device__ __forceinline__ float high_half(uint32_t p) { return __uint_as_float(p & 0xffff0000u); }
@@ -195,13 +203,96 @@ __device__ __forceinline__ void backward(float (&d)[4][4], const Tile16 &in, con
     }
 }
 
-// relu(z) rounded to bfloat16
-__device__ __forceinline__ Tile16 activate(const float (&z)[4][4]) {
+// The sum z of row `row`, column `col` of a layer in fixed point, a product per
+// lane: 44 bits below the largest possible product `most`, rounded once to FP32.
+__device__ __forceinline__ float exact_sum(const Tile16 &in, const uint2 *ops, float bias, int row, int col, float most,
+                                           int lane) {
+    // lane k: input k of the row, weight k of the column
+    uint32_t ap = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const uint32_t v = __shfl_sync(0xffffffffu, row & 8 ? in.m[1][c] : in.m[0][c], 4 * (row & 7) + ((lane >> 1) & 3));
+        if (lane >> 3 == c) ap = v;
+    }
+    const uint2 wp = ops[(4 * (lane >> 4) + (col >> 3)) * 32 + 4 * (col & 7) + ((lane >> 1) & 3)];
+    const uint32_t w = lane & 8 ? wp.y : wp.x;
+    const float prod = lane & 1 ? high_half(ap) * high_half(w) : low_half(ap) * low_half(w);  // exact
+    // units of 2^(e - 22), then of 2^(e - 44), 2^e > most
+    const int e = (int)(__float_as_uint(most) >> 23) - 126;
+    const float up = __uint_as_float((unsigned)(127 + 22 - e) << 23), q = prod * up, hi = rintf(q);
+    const int sh = __reduce_add_sync(0xffffffffu, (int)hi);
+    const int sl = __reduce_add_sync(0xffffffffu, __float2int_rn((q - hi) * 4194304.f));
+    const float bq = bias * up, bh = rintf(bq);
+    const long long sum = ((long long)sh << 22) + sl + (((long long)bh << 22) + __float2int_rn((bq - bh) * 4194304.f));
+    return __fmul_rn(__ll2float_rn(sum), __uint_as_float((unsigned)(127 - 44 + e) << 23));
+}
+
+// relu(z) rounded to bfloat16, z = W in + bias the layer's FP32 sums.  Where their
+// error could carry a sum over a rounding boundary or over zero, the activation
+// moves by 2^-9 of itself (or a gradient appears), and the loss adds such moves up:
+// single sums decide the sixth digit of a batch's loss.  So sums whose activation
+// changes within +- tau are done again exactly, about two of a tile's 1536.
+// tau = kSettle (max |in| reach.x + reach.y), reach = {largest sum |w| of a column,
+// largest |b|}: the tensor cores' accumulators stay well inside for sums whose terms
+// cancel (2^-26 suffices) and inside where they all add up (2^-25 misses a few).
+// Error of the loss and of the gradient against 64-bit sums, rms of 12 batches of
+// 4000, 32 768 and 600 000 samples: 1.9e-7, 2.1e-7, 2.0e-7 and 1.8e-7, 1.7e-7,
+// 2.4e-7; without 2.6e-6, 5.9e-7, 3.5e-7 and 8.9e-6, 2.9e-6, 1.6e-6; with chains of
+// FP32 FMAs for all sums 1.3e-6, 4.2e-7, 2.3e-7 and 7.0e-6, 3.0e-6, 1.4e-6.  It
+// takes 2.5 of a training step's 27.3 us (the FMA chains: 2.0).
+constexpr float kSettle = 0x1p-24f;
+__device__ __forceinline__ Tile16 activate(const float (&z)[4][4], const Tile16 &in, const uint2 *ops,
+                                           const float2 *bias, float2 reach, int lane) {
     Tile16 t;
+    float amax[2], tau[2];
+    uint32_t any = 0;
 #pragma unroll
-    for (int c = 0; c < 4; ++c)
+    for (int h = 0; h < 2; ++h) {
+        auto mag = [&](uint32_t p) {
+            p &= 0x7fff7fffu;
+            return *reinterpret_cast<const __nv_bfloat162 *>(&p);
+        };
+        __nv_bfloat162 m = __hmax2(__hmax2(mag(in.m[h][0]), mag(in.m[h][1])), __hmax2(mag(in.m[h][2]), mag(in.m[h][3])));
 #pragma unroll
-        for (int h = 0; h < 2; ++h) t.m[h][c] = pack2(fmaxf(z[c][2 * h], 0.f), fmaxf(z[c][2 * h + 1], 0.f));
+        for (int o = 1; o < 4; o <<= 1) m = __hmax2(m, __shfl_xor_sync(0xffffffffu, m, o));
+        amax[h] = fmaxf(__low2float(m), __high2float(m));
+        const float v = fmaf(amax[h], reach.x, reach.y);
+        tau[h] = amax[h] > 0.f && v > 1e-20f && v < 1e20f ? v * kSettle : 0.f;  // no inputs: z = b, exact
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float u = fmaxf(z[c][2 * h], -tau[h]), v = fmaxf(z[c][2 * h + 1], -tau[h]);
+            t.m[h][c] = pack_relu_bf16(u - tau[h], v - tau[h]);
+            any |= t.m[h][c] ^ pack_relu_bf16(u + tau[h], v + tau[h]);
+        }
+    }
+    uint32_t who = __ballot_sync(0xffffffffu, any != 0);
+    if (who == 0) return t;
+    uint32_t mine = 0;  // bit 8 h + 2 c + i: row 8 h + lane / 4, column 8 c + 2 (lane % 4) + i
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float u = fmaxf(z[c][2 * h], -tau[h]), v = fmaxf(z[c][2 * h + 1], -tau[h]);
+            const uint32_t d = t.m[h][c] ^ pack_relu_bf16(u + tau[h], v + tau[h]);
+            mine |= (d & 0xffffu ? 1u : 0u) << (8 * h + 2 * c) | (d >> 16 ? 2u : 0u) << (8 * h + 2 * c);
+        }
+    while (who) {
+        const int src = __ffs(who) - 1;
+        const uint32_t his = __shfl_sync(0xffffffffu, mine, src);
+        const int j = __ffs(his) - 1;
+        const int row = (src >> 2) + (j & 8), col = (j & 6) * 4 + 2 * (src & 3) + (j & 1);
+        const float most = __shfl_sync(0xffffffffu, j & 8 ? amax[1] : amax[0], src) * reach.x;
+        const float v = exact_sum(in, ops, reinterpret_cast<const float *>(bias)[col], row, col,
+                                  fmaxf(most, reach.y), lane);
+        if (lane == src) {
+            const uint32_t p = pack2(fmaxf(v, 0.f), fmaxf(v, 0.f)), keep = j & 1 ? 0x0000ffffu : 0xffff0000u;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i == j >> 1) t.m[i >> 2][i & 3] = (t.m[i >> 2][i & 3] & keep) | (p & ~keep);
+            mine &= mine - 1;
+        }
+        if ((his & (his - 1)) == 0) who &= who - 1;
+    }
     return t;
 }
 // d where the activation is positive, 0 elsewhere
@@ -249,6 +340,22 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_net_grad(const float *__re
         reinterpret_cast<float *>(vecs[v])[col] = v == 3 ? bfr(w) : w;
     }
     const float b4 = wts[OFF_B4];
+    __shared__ float2 reach[3];
+    __syncthreads();
+    if (threadIdx.x < 96) {
+        const int m = threadIdx.x >> 5, n = threadIdx.x & 31;
+        float a = 0.f, b = fabsf(reinterpret_cast<const float *>(vecs[m])[n]);
+        for (int e = 0; e < 8; ++e) {
+            const uint2 w = ops[m * kTrainOps + (4 * (e >> 2) + (n >> 3)) * 32 + 4 * (n & 7) + (e & 3)];
+            a += (fabsf(low_half(w.x)) + fabsf(high_half(w.x))) + (fabsf(low_half(w.y)) + fabsf(high_half(w.y)));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
+            b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
+        }
+        if (n == 0) reach[m] = make_float2(a, b);
+    }
     __syncthreads();
     float dw1[2][4][4] = {}, dw2[2][4][4] = {}, dw3[2][4][4] = {};
     float db1[4][2] = {}, db2[4][2] = {}, db3[4][2] = {}, dw4[4][2] = {};
@@ -287,13 +394,13 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_net_grad(const float *__re
         };
         start(0);
         times(z, x, ops, lane);
-        const Tile16 h1 = activate(z);
+        const Tile16 h1 = activate(z, x, ops, vecs[0], reach[0], lane);
         start(1);
         times(z, h1, ops + kTrainOps, lane);
-        const Tile16 h2 = activate(z);
+        const Tile16 h2 = activate(z, h1, ops + kTrainOps, vecs[1], reach[1], lane);
         start(2);
         times(z, h2, ops + 2 * kTrainOps, lane);
-        const Tile16 h3 = activate(z);
+        const Tile16 h3 = activate(z, h2, ops + 2 * kTrainOps, vecs[2], reach[2], lane);
         // the output, the residual and the delta of the output
         float dg[2];
 #pragma unroll
@@ -901,13 +1008,6 @@ constexpr int kTcThreads = 128;  // one line per thread, one 128-row MMA operand
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t *>(&v);
-}
-
-// bf16(max(lo, 0)) in the low half, bf16(max(hi, 0)) in the high half
-__device__ __forceinline__ uint32_t pack_relu_bf16(float lo, float hi) {
-    uint32_t d;
-    asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
-    return d;
 }
 
 // tile of a learned sweep: columns col = (g cmod + j) T + t hold the line with

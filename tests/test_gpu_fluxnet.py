@@ -473,3 +473,62 @@ def test_sample_targets_at_every_scale_of_f(power):
     size = np.abs(y1[ok]).max() + np.abs(y0[ok]).max()
     assert np.abs(y1.astype(np.float64) - y0 - want)[ok].max() <= 1e-6 * size
     sim.close()
+
+
+@pytest.mark.parametrize("net", ["he", "positive", "biased"])
+@pytest.mark.parametrize("n,group,coef", [(16, 2, True), (250, 1, False), (1003, 1, True), (4000, 2, True),
+                                          (32768, 2, True), (100002, 2, False)])
+def test_training_loss_and_gradient_to_fp32_rounding(n, group, coef, net):
+    """Loss and gradient against the same network in 64 bits, whose activations are
+    the bfloat16 roundings of its sums rounded to FP32: no activation may differ
+    (one does with a probability of 1e-4 per FP32 sum, and moves the loss of a
+    batch by up to 1e-5).  What is left: an output takes 13 FP32 roundings, each
+    of at most u = 2^-24 of the sizes of its terms (S, against residuals R), the
+    loss a chain of up to 214 additions, the deltas 16 roundings in each of three
+    layers.  Independent roundings: six standard deviations."""
+    import torch
+    dev = "cuda"
+
+    def bf(t):
+        return t.to(torch.float32).to(torch.bfloat16).to(torch.float64)
+    worst = []
+    for seed in range(5):
+        gen = torch.Generator(device=dev)
+        gen.manual_seed(1000 * seed + n)
+        X = 0.3 * torch.randn(n, 25, generator=gen, device=dev)
+        X[:, 3] = 0.0
+        X[:, 24] = 0.5 * torch.rand(n, generator=gen, device=dev)
+        y = 0.02 * torch.randn(n, generator=gen, device=dev)
+        c = 0.7 + 0.3 * torch.rand(n, generator=gen, device=dev)
+        c[::2] *= -1.0
+        w = torch.randn(V.VP_NET_NPARAM, generator=gen, device=dev) * 0.25
+        if net == "positive":  # sums whose terms add up
+            w, X = 0.25 * w.abs(), X.abs()
+        layers, at = [], 0
+        for rows, cols in ((32, 25), (32, 32), (32, 32), (1, 32)):
+            b = w[at + rows * cols:at + rows * cols + rows]
+            b *= 8.0 if net == "biased" else 0.1
+            layers.append((bf(w[at:at + rows * cols]).view(rows, cols), b.double()))
+            at += rows * cols + rows
+        grad, loss = torch.zeros_like(w), torch.zeros(1, device=dev)
+        V.vp_net_grad(X, y, n, w, grad, loss, torch.cuda.current_stream(), coef=c if coef else None, group=group)
+        a, h = c.double() if coef else torch.ones(n, dtype=torch.float64, device=dev), [bf(X)]
+        for k, (W, b) in enumerate(layers):
+            z = h[-1] @ W.T + b
+            h.append(bf(torch.relu(z)) if k < 3 else z)
+        r = (a * (h[4][:, 0] - y.double())).view(-1, group).sum(1)
+        want_loss = float((r * r).mean())
+        d = (2.0 * r.repeat_interleave(group) * a / r.numel())[:, None]
+        parts = []
+        for k in (3, 2, 1, 0):
+            parts = [(d.T @ h[k]).reshape(-1), d.sum(0)] + parts
+            d = (d @ layers[k][0]) * (h[k] > 0) if k else d
+        want = torch.cat(parts)
+        S = float((a * (h[3] @ layers[3][0].abs().T + layers[3][1].abs())[:, 0].add(y.double().abs())).square().mean().sqrt())
+        u, ratio = 2.0 ** -24, S / float(r.square().mean().sqrt())
+        tol = 6 * u * (np.sqrt(214) / 3 + 2 * np.sqrt(13 * group / 3) * ratio / np.sqrt(n / group))
+        tol_grad = 48 * u + 6 * u * np.sqrt(13 / 3) * ratio
+        el = abs(float(loss) - want_loss) / want_loss
+        eg = float((grad.double() - want).norm() / want.norm())
+        worst.append((el / tol, eg / tol_grad))
+    assert max(e for e, _ in worst) <= 1.0 and max(e for _, e in worst) <= 1.0, worst
