@@ -38,6 +38,7 @@
 #include <vector>
 
 #include "vp_internal.cuh"
+#include "vp_sum.cuh"
 #include "vp_sweep_core.cuh"
 #include "vp_tma.cuh"
 
@@ -375,22 +376,8 @@ __device__ __forceinline__ void tile_rows(float *pool, const RunDesc &r, const S
     }
 }
 
-__device__ double warp_sum_d(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // density of spatial points [x0, x1): one warp per point, compensated float
 // sums per lane (two, of alternate 16-byte pieces) combined in double
-struct PairSum {
-    float s = 0.f, e = 0.f;
-    __device__ __forceinline__ void add(float y) {
-        const float t = s + y, bp = t - s;
-        e += (s - (t - bp)) + (y - bp);
-        s = t;
-    }
-};
 __device__ void density_points(const float *pool, const RunDesc &r, long long x0, long long x1,
                                double *rho_pool) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -400,7 +387,7 @@ __device__ void density_points(const float *pool, const RunDesc &r, long long x0
     for (long long x = x0 + warp; x < x1; x += nw) {
         const float *p = pool + r.f_off + x * r.NV;
         const float4 *q = reinterpret_cast<const float4 *>(p);
-        PairSum a, b;
+        vp_sum::PairSum a, b;
         int i = lane;
         for (; i + 96 < nq; i += 128) {
             float4 v[4];
@@ -422,7 +409,7 @@ __device__ void density_points(const float *pool, const RunDesc &r, long long x0
             b.add(v.w);
         }
         for (int v = 4 * nq + lane; v < NV; v += 32) a.add(ldcg(p + v));
-        const double tot = warp_sum_d(((double)a.s + (double)a.e) + ((double)b.s + (double)b.e));
+        const double tot = vp_sum::warp_sum(((double)a.s + (double)a.e) + ((double)b.s + (double)b.e));
         if (lane == 0) rho_pool[r.rho_off + x] = tot * dV;
     }
 }

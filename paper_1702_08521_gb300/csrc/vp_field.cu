@@ -3,24 +3,23 @@
 // diagnostics reductions and analytic initial conditions, all on the device.
 //
 // Precision: f is read as float or double; every sum over velocity space is
-// carried in double precision (for float input, a compensated float sum per
-// thread -- Knuth's two-sum -- whose value and error term are combined in
-// double, then double across threads).  Fourier transforms, Green functions
+// carried in double precision (for float input, short compensated float sums per
+// thread -- Knuth's two-sum -- whose values are added in double, then double
+// across threads).  Fourier transforms, Green functions
 // and forces are double precision throughout.
 #include <cmath>
 #include <mutex>
 
 #include "vp_internal.cuh"
+#include "vp_sum.cuh"
 
 namespace {
 
 constexpr int kBlock = 256;
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
+using vp_sum::PairSum;
+using vp_sum::warp_sum;
+using vp_sum::widen;
 
 // ---- sums over velocity space --------------------------------------------------
 //
@@ -80,26 +79,58 @@ __device__ __forceinline__ double block_sums(const double (&v)[K], double (*sh)[
 
 // ---- density moment ----------------------------------------------------------
 
+// the same sum, for all lanes (or threads) of a point where the value of a pair
+// left the float range or a cell is not finite: NaN then, also for an infinite cell
+__device__ __noinline__ double part_sum_rare(const float *p, long long n, int t, int nt) {
+    double a = 0.0;
+    for (long long i = t; i < n; i += nt) {
+        const float x = p[i];
+        a += (double)x + (double)(x - x);
+    }
+    return a;
+}
+__device__ __forceinline__ double part_sum_rare(const double *, long long, int, int) { return 0.0; }
+
 // the lane's (or thread's) part of sum p[0..n): 16-byte loads between the
-// unaligned ends, two independent sums
-__device__ __forceinline__ CSum part_sum(const float *p, long long n, int t, int nt) {
-    CSum a{0.f, 0.f}, b{0.f, 0.f};
+// unaligned ends, two independent pair sums whose values go to a double every 8
+// cells (the error of a pair sum of K cells is up to K 2^-51; its error term stays)
+__device__ __forceinline__ double part_sum(const float *p, long long n, int t, int nt) {
+    PairSum a, b;
+    double d = 0.0;
+    auto flush = [&]() {
+        a.add(b.s);
+        d += widen(a.s);
+        a.s = b.s = 0.f;
+    };
+    auto quad = [&](const float4 &v) {
+        a.add(v.x);
+        b.add(v.y);
+        a.add(v.z);
+        b.add(v.w);
+    };
     long long head = (long long)((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15) / 4;
     head = head < n ? head : n;
     for (long long i = t; i < head; i += nt) a.add(p[i]);
     const float4 *q = reinterpret_cast<const float4 *>(p + head);
     const long long nq = (n - head) / 4;
-#pragma unroll 4
-    for (long long i = t; i < nq; i += nt) {
-        const float4 v = q[i];
-        a.add(v.x);
-        b.add(v.y);
-        a.add(v.z);
-        b.add(v.w);
+    long long i = t;
+    for (; i + 3 * nt < nq; i += 4 * nt) {
+        float4 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = q[i + k * nt];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            quad(v[k]);
+            if (k & 1) flush();
+        }
     }
-    for (long long i = head + 4 * nq + t; i < n; i += nt) b.add(p[i]);
-    a.add(b);
-    return a;
+    for (; i < nq; i += nt) {
+        quad(q[i]);
+        flush();
+    }
+    for (i = head + 4 * nq + t; i < n; i += nt) b.add(p[i]);
+    flush();
+    return d + (widen(a.e) + widen(b.e));
 }
 
 __device__ __forceinline__ double part_sum(const double *p, long long n, int t, int nt) {
@@ -125,12 +156,26 @@ __global__ void __launch_bounds__(kBlock) k_moment(const T *f, long long NX, lon
     if (WARP) {
         const long long x = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
         if (x >= NX) return;
-        const double s = warp_total(part_sum(f + x * NV, NV, threadIdx.x & 31, 32));
+        double s = part_sum(f + x * NV, NV, threadIdx.x & 31, 32);
+        if (sizeof(T) == 4 && __any_sync(0xffffffffu, !isfinite(s))) s = part_sum_rare(f + x * NV, NV, threadIdx.x & 31, 32);
+        s = warp_sum(s);
         if ((threadIdx.x & 31) == 0) rho[x] = s * dV;
     } else {
-        __shared__ double sh[1][32];
-        const double v[1] = {warp_total(part_sum(f + (long long)blockIdx.x * NV, NV, threadIdx.x, blockDim.x))};
-        const double s = block_sums<1>(v, sh);
+        // one warp adds the threads' parts: a shuffle tree in every warp would keep
+        // the FP64 pipe busy three times as long
+        __shared__ double sh[kBlock];
+        const T *p = f + (long long)blockIdx.x * NV;
+        double s = part_sum(p, NV, threadIdx.x, blockDim.x);
+        sh[threadIdx.x] = s;
+        if (__syncthreads_or(sizeof(T) == 4 && !isfinite(s))) {
+            sh[threadIdx.x] = part_sum_rare(p, NV, threadIdx.x, blockDim.x);
+            __syncthreads();
+        }
+        if (threadIdx.x >= 32) return;
+        s = 0.0;
+#pragma unroll
+        for (int i = 0; i < kBlock / 32; ++i) s += sh[32 * i + threadIdx.x];
+        s = warp_sum(s);
         if (threadIdx.x == 0) rho[blockIdx.x] = s * dV;
     }
 }

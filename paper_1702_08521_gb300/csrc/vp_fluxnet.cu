@@ -29,10 +29,14 @@
 #include <cmath>
 
 #include "vp_internal.cuh"
+#include "vp_sum.cuh"
 #include "vp_sweep_core.cuh"
 #include "vp_umma.cuh"
 
 namespace {
+
+using vp_sum::PairSum;
+using vp_sum::widen;
 
 constexpr int H = VP_NET_HIDDEN;
 constexpr int NF = VP_NET_FEATURES;
@@ -511,28 +515,8 @@ __global__ void k_adam(float *__restrict__ wts, float *__restrict__ m, float *__
 
 // FP64 instructions take 16 cycles each here, conversions included, and the
 // outputs are tens of millions of doubles: sums of a few floats are kept as a
-// value and its error term (two-sum), and a normal float becomes a double on
-// its bits; other numbers take the conversion, out of line (as a
-// predicated instruction it occupies the FP64 pipe for every number).
-__device__ __noinline__ double widen_rare(float x) { return (double)x; }
-__device__ __forceinline__ double widen(float x) {
-    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-    const unsigned hi = (b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
-    double d = __hiloint2double((int)hi, (int)(b << 29));
-    if (m != 0u && m - 0x00800000u >= 0x7f000000u) d = widen_rare(x);
-    return d;
-}
-
-struct PairSum {
-    float s, e;
-    __device__ __forceinline__ void add(float x) {
-        const float t = s + x;
-        const float bp = t - s;
-        e += (s - (t - bp)) + (x - bp);
-        s = t;
-    }
-    __device__ __forceinline__ double value() const { return widen(s) + widen(e); }
-};
+// value and its error term (vp_sum.cuh).
+__device__ __forceinline__ double pair_value(const PairSum &p) { return widen(p.s) + widen(p.e); }
 
 // geometry of the line kernels below: lines of L cells at stride inner, W (a
 // power of two, at most kTileLines) consecutive lines per CTA
@@ -699,14 +683,14 @@ __global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, 
                     Gs[i * NP + j] = widen(sg > 0 ? M : -M);
                     return;
                 }
-                PairSum p{0.f, 0.f};
+                PairSum p;
                 const float *v = ui + (sg > 0 ? (n >= 0 ? c - n : c) : (n >= 0 ? c : c + n)) * WP;
                 const float one = n >= 0 ? 1.f : -1.f;
                 for (int m = n >= 0 ? n : -n; m > 0; --m, v += WP) p.add(one * *v);
                 p.add(M);
                 p.s = sg > 0 ? p.s : -p.s;
                 p.e = sg > 0 ? p.e : -p.e;
-                g = p.value();
+                g = pair_value(p);
             }
             Gs[i * NP + j] = g;
         };
@@ -791,7 +775,7 @@ __global__ void __launch_bounds__(256) k_restrict_v2(const float *__restrict__ f
     }
     const unsigned J1 = fdiv(J, nc2), J2 = J - J1 * nc2.d;
     const float *p = ff + x * nf12 + (long long)J1 * factor1 * nf2 + (long long)J2 * factor2;
-    PairSum a{0.f, 0.f};
+    PairSum a;
     if (quad) {
 #pragma unroll 4
         for (int k = 0; k < factor1; ++k) {
@@ -805,7 +789,7 @@ __global__ void __launch_bounds__(256) k_restrict_v2(const float *__restrict__ f
         for (int k = 0; k < factor1; ++k)
             for (int b = 0; b < factor2; ++b) a.add(p[(long long)k * nf2 + b]);
     }
-    fc[t] = (float)(inv != 0.0 ? a.value() * inv : a.value() / (factor1 * factor2));
+    fc[t] = (float)(inv != 0.0 ? pair_value(a) * inv : pair_value(a) / (factor1 * factor2));
 }
 
 // Samples on coarse lines: for every coarse interface with |zeta| >= zmin,

@@ -214,3 +214,38 @@ def test_overlapped_launches_on_every_kind_of_stream(spec):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(phi, want[0]) and torch.equal(acc, want[1])
+
+
+@pytest.mark.parametrize("nv", [[7], [128], [999], [2048], [2049], [33, 70], [128, 128]])
+@pytest.mark.parametrize("scale", [1.0, 2.9e38, 1e-40])
+def test_density_of_fp32_cells_of_any_size(nv, scale):
+    """Densities of FP32 grids at scales whose sums leave the float range (and of
+    subnormal cells), against exact sums.  A thread's float-pair sums of up to 16
+    cells are off by at most 16 roundings of their error term, 16 2^-51 of the sum,
+    its error terms of n cells by n / 16 such; doubles beyond that."""
+    import math
+    D, NX = len(nv), [3] * len(nv)
+    g = dict(dims=D, nx=NX, nv=nv, xlo=[0.0] * D, xhi=[1.0] * D, vlo=[0.0] * D, vhi=[float(n) for n in nv])
+    sim, og = both(g, V.VP_F32)
+    rng = np.random.default_rng(nv[0])
+    v = np.arange(og.NV) / og.NV - 0.5
+    f = ((rng.random((og.NX, 1)) + 0.1) * np.exp(-20 * v * v) * (0.9 + 0.1 * rng.random((og.NX, og.NV))) / 1.1 * scale)
+    f = f.astype(np.float32)
+    to_gpu(sim, f)
+    V.vp_density_moment(sim.ctx, sim.rho)
+    sim.sync()
+    rho = sim.rho.cpu().numpy()
+    want = np.array([math.fsum(r) for r in f.astype(np.float64)])
+    assert np.isfinite(rho).all()
+    tol = max(16, og.NV // 32 / 16) * 2.0 ** -51 + 2.0 ** -50
+    assert (np.abs(rho - want) <= tol * want).all(), np.abs(rho / want - 1).max()
+    # independent roundings of every pair sum: 6 standard deviations of the mean square
+    rms = np.sqrt(np.mean((rho / want - 1) ** 2))
+    assert rms <= 6 * (2.0 ** -51 * 16 / np.sqrt(12 * max(1, min(og.NV, 32))) + 2.0 ** -53), rms
+    f[1, 0] = np.inf
+    to_gpu(sim, f)
+    V.vp_density_moment(sim.ctx, sim.rho)
+    sim.sync()
+    bad = np.isnan(sim.rho.cpu().numpy())
+    assert bad[1] and bad.sum() == 1
+    sim.close()
