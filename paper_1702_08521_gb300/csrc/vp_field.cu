@@ -17,9 +17,8 @@ namespace {
 
 constexpr int kBlock = 256;
 
-using vp_sum::PairSum;
 using vp_sum::warp_sum;
-using vp_sum::widen;
+using vp_sum::widen_any;
 
 // ---- sums over velocity space --------------------------------------------------
 //
@@ -92,21 +91,21 @@ __device__ __noinline__ double part_sum_rare(const float *p, long long n, int t,
 __device__ __forceinline__ double part_sum_rare(const double *, long long, int, int) { return 0.0; }
 
 // the lane's (or thread's) part of sum p[0..n): 16-byte loads between the
-// unaligned ends, two independent pair sums whose values go to a double every 8
-// cells (the error of a pair sum of K cells is up to K 2^-51; its error term stays)
+// unaligned ends, a pair sum whose value goes to a double every 8 cells and whose
+// error term is folded then (an error term of n cells rounds by up to n 2^-51)
 __device__ __forceinline__ double part_sum(const float *p, long long n, int t, int nt) {
-    PairSum a, b;
+    vp_sum::LongSum a;
     double d = 0.0;
     auto flush = [&]() {
-        a.add(b.s);
-        d += widen(a.s);
-        a.s = b.s = 0.f;
+        d += widen_any(a.s);
+        a.s = 0.f;
+        a.fold();
     };
     auto quad = [&](const float4 &v) {
         a.add(v.x);
-        b.add(v.y);
+        a.add(v.y);
         a.add(v.z);
-        b.add(v.w);
+        a.add(v.w);
     };
     long long head = (long long)((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15) / 4;
     head = head < n ? head : n;
@@ -128,9 +127,9 @@ __device__ __forceinline__ double part_sum(const float *p, long long n, int t, i
         quad(q[i]);
         flush();
     }
-    for (i = head + 4 * nq + t; i < n; i += nt) b.add(p[i]);
+    for (i = head + 4 * nq + t; i < n; i += nt) a.add(p[i]);
     flush();
-    return d + (widen(a.e) + widen(b.e));
+    return d + widen_any(a.error());
 }
 
 __device__ __forceinline__ double part_sum(const double *p, long long n, int t, int nt) {

@@ -18,22 +18,44 @@ __device__ __forceinline__ double widen(float x) {
     return d;
 }
 
-// value and error term of a sum of floats (Knuth's two-sum)
+// the error of t = a + b (Knuth's two-sum)
+__device__ __forceinline__ float two_sum_error(float a, float b, float t) {
+    const float bp = t - a;
+    return (a - (t - bp)) + (b - bp);
+}
+
+// value and error term of a sum of floats
 struct PairSum {
     float s = 0.f, e = 0.f;
     __device__ __forceinline__ void add(float x) {
         const float t = s + x;
-        const float bp = t - s;
-        e += (s - (t - bp)) + (x - bp);
+        e += two_sum_error(s, x, t);
         s = t;
     }
-    // a b, both rounding errors kept
-    __device__ __forceinline__ void add_product(float a, float b) {
-        const float p = a * b;
-        add(p);
-        e += fmaf(a, b, -p);
-    }
 };
+
+// the same for sums of many: every few terms fold() adds the error term of those
+// to the others', with an error term of its own (a plain error term of hundreds of
+// cells rounds, often always the same way, by 2^-50 of the sum)
+struct LongSum : PairSum {
+    float far = 0.f, rest = 0.f;
+    __device__ __forceinline__ void fold() {
+        const float t = far + e;
+        rest += two_sum_error(far, e, t);
+        far = t;
+        e = 0.f;
+    }
+    __device__ __forceinline__ float error() const { return (e + rest) + far; }
+};
+
+// the same for every number on the integer pipe, where subnormal ones are common
+// (sums over the empty tails of a distribution)
+__device__ __forceinline__ double widen_any(float x) {
+    const bool small = fabsf(x) < 0x1p-126f;
+    const unsigned b = __float_as_uint(small ? x * 0x1p64f : x), m = b & 0x7fffffffu;
+    const unsigned bias = small ? 0x34000000u : (m < 0x7f800000u ? 0x38000000u : 0x70000000u);
+    return __hiloint2double((int)((b & 0x80000000u) | (m ? (m >> 3) + bias : 0u)), (int)(b << 29));
+}
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
