@@ -17,6 +17,7 @@ namespace {
 
 constexpr int kBlock = 256;
 
+using vp_sum::PairSum;
 using vp_sum::warp_sum;
 using vp_sum::widen_any;
 
@@ -26,55 +27,12 @@ using vp_sum::widen_any;
 // per SM and clock): tree sums of doubles over 256 threads took 20 us for 4096
 // points of 1024 cells (67 MB, 10 us of HBM), and the diagnostics' per-cell
 // double arithmetic and 64-bit remainders 12.3 ms for 3.1e8 cells (0.18 ms).
-// So float sums stay float pairs -- value and error term of Knuth's two-sum,
-// products with their exact error from an FMA -- through the warp's shuffles,
-// and one double per warp and sum is left: 7.1 us and 1.7 ms.
-
-struct CSum {
-    float s, e;
-    __device__ __forceinline__ void add(float x) {
-        const float t = s + x;
-        const float bp = t - s;
-        e += (s - (t - bp)) + (x - bp);
-        s = t;
-    }
-    __device__ __forceinline__ void add(const CSum &o) {
-        add(o.s);
-        e += o.e;
-    }
-    // a b, both rounding errors kept
-    __device__ __forceinline__ void add_product(float a, float b) {
-        const float p = a * b;
-        add(p);
-        e += fmaf(a, b, -p);
-    }
-    __device__ __forceinline__ double value() const { return (double)s + (double)e; }
-};
-
-__device__ __forceinline__ double warp_total(CSum c) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const CSum u{__shfl_xor_sync(0xffffffffu, c.s, o), __shfl_xor_sync(0xffffffffu, c.e, o)};
-        c.add(u);
-    }
-    return c.value();
-}
-__device__ __forceinline__ double warp_total(double v) { return warp_sum(v); }
-
-// sums of K doubles over the block, in thread 0 .. K - 1 (thread k: sum k);
-// sh: K x 32 doubles.  v: the thread's warp totals (already summed over the warp).
-template <int K>
-__device__ __forceinline__ double block_sums(const double (&v)[K], double (*sh)[32]) {
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-    if (l == 0)
-#pragma unroll
-        for (int k = 0; k < K; ++k) sh[k][w] = v[k];
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x < K)
-        for (int i = 0; i < nw; ++i) t += sh[threadIdx.x][i];
-    return t;
-}
+// So runs of a few cells are summed as float pairs -- value and error term of
+// Knuth's two-sum, products with their exact error from an FMA --, their values
+// added in double, and one warp adds the threads' doubles: the density of 3.1e8
+// cells 180 us, the diagnostics 0.72 ms (0.92 ms where most cells are subnormal or
+// nearly), with the errors of sums in double: 1e-16 of the mass, energy and
+// squares.  Whole threads' sums as pairs took 0.80 ms and were off by up to 7e-15.
 
 // ---- density moment ----------------------------------------------------------
 
@@ -561,52 +519,110 @@ struct DiagSum;
 template <>
 struct DiagSum<float> {
     using W = WPair;
-    // regular cells, and cells below 2^-50 multiplied by 2^100 (exactly): no
-    // product of either class, nor its error term, leaves the float range.
-    // Fallen tails of a distribution are full of such cells; sending them
-    // through FP64 instead took 5.9 ms for 3.1e8 cells.
-    CSum m0{0.f, 0.f}, m2{0.f, 0.f}, l2{0.f, 0.f}, m2t{0.f, 0.f}, l2t{0.f, 0.f}, neg{0.f, 0.f};
-    float mn = INFINITY, mx = -INFINITY;
+    // A thread's sums of its cells times `scale`, 2^100 until it meets one of 2^-40,
+    // then 1 (with the sums so far): no product of scaled cells, nor its error term,
+    // leaves the float range, and what underflows in those of small cells beside a
+    // larger one is below 2^-69 of the sums.  Fallen tails of a distribution are full
+    // of such cells; sending them through FP64 took 5.9 ms for 3.1e8 cells.
+    vp_sum::LongSum m0;
+    vp_sum::ProductSum m2;
+    vp_sum::SquareSum l2;
+    PairSum neg;
+    // the values of the pairs so far: cells, weighted cells, negative cells, squares
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    float mn = INFINITY, mx = -INFINITY, scale = kUp;
     bool huge = false, bad = false;  // a cell above 2^60: the point is summed again in double
-    static constexpr float kTiny = 8.8817842e-16f, kHuge = 1.1529215e18f, kUp = 1.2676506e30f;
-    static __device__ __forceinline__ void weigh(CSum &c, float x, const W &w) {
-        c.add_product(x, w.hi);
-        c.e = fmaf(x, w.lo, c.e);
+    static constexpr float kUp = 0x1p100f, kPlain = 0x1p-40f, kHuge = 0x1p60f;
+    static constexpr double kDown = 0x1p-100;
+    __device__ __forceinline__ void any(float x, const W &w) {
+        m2.add_product(x, w.hi);
+        m2.q = fmaf(x, w.lo, m2.q);
+    }
+    // to the scale 1
+    __device__ __forceinline__ void unscale() {
+        flush();
+        flush_errors();
+        v[0] *= kDown;
+        v[1] *= kDown;
+        v[2] *= kDown;
+        v[3] *= kDown * kDown;
+        m0 = vp_sum::LongSum();
+        m2 = vp_sum::ProductSum();
+        l2 = vp_sum::SquareSum();
+        neg = PairSum();
+        scale = 1.f;
     }
     __device__ __forceinline__ void cell(float x, const W &w, const W *w2) {
         mn = fminf(mn, x);
         mx = fmaxf(mx, x);
-        const float ax = fabsf(x);
-        if (!(ax <= kHuge)) huge = true;
-        m0.add(x);
-        if (x < 0.f) neg.add(x);
-        if (ax < kTiny) {
-            const float y = x * kUp;
-            weigh(m2t, y, w);
-            if (w2) weigh(m2t, y, *w2);
-            l2t.add_product(y, y);
-        } else {
-            weigh(m2, x, w);
-            if (w2) weigh(m2, x, *w2);
-            l2.add_product(x, x);
+        if (!(fabsf(x) <= kHuge)) huge = true;
+        if (fabsf(x) >= kPlain && scale != 1.f) unscale();
+        const float y = x * scale;
+        m0.add(y);
+        any(y, w);
+        if (w2) any(y, *w2);
+        l2.add_square(y);
+        if (x < 0.f) neg.add(y);
+    }
+    // four cells of one index of the last axis
+    __device__ __forceinline__ void cells(const float (&x)[4], const W (&w)[4]) {
+        const float lo = fminf(fminf(x[0], x[1]), fminf(x[2], x[3])), hi = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
+        mn = fminf(mn, lo);
+        mx = fmaxf(mx, hi);
+        const float size = fmaxf(hi, -lo);
+        // (x - x: not a number for cells that are not finite, which the extrema skip)
+        const float z = ((x[0] - x[0]) + (x[1] - x[1])) + ((x[2] - x[2]) + (x[3] - x[3]));
+        if (!(size + z <= kHuge)) huge = true;
+        if (size == 0.f) return;
+        if (size >= kPlain && scale != 1.f) unscale();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float y = x[k] * scale;
+            m0.add(y);
+            any(y, w[k]);
+            l2.add_square(y);
+            if (k == 1) l2.fold();
+        }
+        if (lo < 0.f)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (x[k] < 0.f) neg.add(x[k] * scale);
+        fold();
+    }
+    // every four cells: the error terms
+    __device__ __forceinline__ void fold() {
+        m0.fold();
+        m2.fold();
+        l2.fold();
+    }
+    // the pairs' values to the doubles, every 16 cells (the errors of a pair sum
+    // grow with its value)
+    __device__ __forceinline__ void flush() {
+        v[0] += widen_any(m0.s);
+        v[1] += widen_any(m2.s);
+        v[3] += widen_any(l2.s);
+        m0.s = m2.s = l2.s = 0.f;
+        if (neg.s != 0.f) {
+            v[2] += widen_any(neg.s);
+            neg.s = 0.f;
         }
     }
-    // the part of a thread whose cells share the weight w of the last axis:
-    // m2 += w (sum of the cells)
-    __device__ __forceinline__ void common(const W &w) {
-        const bool tiny = fabsf(m0.s) < kTiny;
-        const float u = tiny ? kUp : 1.f, y = m0.s * u;
-        CSum &c = tiny ? m2t : m2;
-        weigh(c, y, w);
-        c.e = fmaf(m0.e * u, w.hi, c.e);
+    __device__ __forceinline__ void flush_errors() {
+        v[0] += widen_any(m0.error());
+        v[1] += widen_any(m2.error());
+        v[3] += widen_any(l2.error()) + widen_any(l2.product_error());
+        if (neg.e != 0.f) v[2] += widen_any(neg.e);
     }
-    // {sum, weighted sum, sum of negatives, sum of squares} of the warp
-    __device__ __forceinline__ void totals(double (&v)[4]) {
-        constexpr double kDown = 7.888609052210118e-31;  // 2^-100
-        v[0] = warp_total(m0);
-        v[1] = fma(warp_total(m2t), kDown, warp_total(m2));
-        v[2] = __any_sync(0xffffffffu, mn < 0.f) ? warp_total(neg) : 0.0;
-        v[3] = fma(warp_total(l2t), kDown * kDown, warp_total(l2));
+    // the end of a thread's sums, its cells of one index of the last axis with its
+    // weight (NULL: weighed already)
+    __device__ __forceinline__ void finish(const W *w) {
+        if (scale != 1.f) {
+            unscale();
+        } else {
+            flush();
+            flush_errors();
+        }
+        if (w) v[1] = fma(widen_any(w->hi) + widen_any(w->lo), v[0], v[1]);
     }
 };
 
@@ -625,7 +641,6 @@ __device__ __noinline__ void diag_in_double(const float *p, long long NV, int nl
         if (x < 0.0) v[2] += x;
         v[3] = fma(x, x, v[3]);
     }
-    for (int k = 0; k < 4; ++k) v[k] = warp_sum(v[k]);
 }
 __device__ __forceinline__ void diag_in_double(const double *, long long, int, const double *, const double *,
                                                double (&)[4], bool &) {}
@@ -633,7 +648,7 @@ __device__ __forceinline__ void diag_in_double(const double *, long long, int, c
 template <>
 struct DiagSum<double> {
     using W = double;
-    double m0 = 0.0, m2 = 0.0, l2 = 0.0, neg = 0.0;
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
     double mn = INFINITY, mx = -INFINITY;
     bool bad = false;
     static constexpr bool huge = false;
@@ -641,17 +656,19 @@ struct DiagSum<double> {
         mn = fmin(mn, x);
         mx = fmax(mx, x);
         if (!isfinite(x)) bad = true;
-        m0 += x;
-        m2 = fma(x, w2 ? w + *w2 : w, m2);
-        l2 = fma(x, x, l2);
-        if (x < 0.0) neg += x;
+        v[0] += x;
+        v[1] = fma(x, w2 ? w + *w2 : w, v[1]);
+        v[3] = fma(x, x, v[3]);
+        if (x < 0.0) v[2] += x;
     }
-    __device__ __forceinline__ void common(const W &w) { m2 = fma(m0, w, m2); }
-    __device__ __forceinline__ void totals(double (&v)[4]) {
-        v[0] = warp_sum(m0);
-        v[1] = warp_sum(m2);
-        v[2] = warp_sum(neg);
-        v[3] = warp_sum(l2);
+    __device__ __forceinline__ void cells(const double (&x)[4], const W (&w)[4]) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) cell(x[k], w[k], nullptr);
+    }
+    __device__ __forceinline__ void fold() {}
+    __device__ __forceinline__ void flush() {}
+    __device__ __forceinline__ void finish(const W *w) {
+        if (w) v[1] = fma(v[0], *w, v[1]);
     }
 };
 
@@ -670,7 +687,7 @@ __global__ void __launch_bounds__(kBlock) k_diag_part(const T *f, long long NV, 
                                                       const typename DiagSum<T>::W *wlast, double unit,
                                                       double dV, double *part,
                                                       double *rho, int *bad) {
-    __shared__ double sh[4][32];
+    __shared__ double sh[4][kBlock];
     __shared__ T smin[32], smax[32];
     dep_wait();
     dep_launch();
@@ -685,7 +702,7 @@ __global__ void __launch_bounds__(kBlock) k_diag_part(const T *f, long long NV, 
             const int step = nr * nlast;
             // four cells and weights in flight
             long long r = r0;
-            for (; r + 3 * nr < rows; r += 4 * nr) {
+            for (int it = 1; r + 3 * nr < rows; r += 4 * nr, ++it) {
                 T x[4];
                 typename DiagSum<T>::W w[4];
 #pragma unroll
@@ -694,25 +711,30 @@ __global__ void __launch_bounds__(kBlock) k_diag_part(const T *f, long long NV, 
                     w[k] = wrow[r + k * nr];
                     c += step;
                 }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) q.cell(x[k], w[k], nullptr);
+                q.cells(x, w);
+                if ((it & 3) == 0) q.flush();
             }
             for (; r < rows; r += nr) {
                 q.cell(*c, wrow[r], nullptr);
                 c += step;
             }
-            q.common(wlast[j]);
+            q.finish(wlast + j);
         }
     } else {
-        for (long long v = threadIdx.x; v < NV; v += blockDim.x) {
+        int it = 1;
+        for (long long v = threadIdx.x; v < NV; v += blockDim.x, ++it) {
             const long long r = v / nlast;
             q.cell(p[v], wrow[r], wlast + (v - r * nlast));
+            if ((it & 3) == 0) q.fold();
+            if ((it & 15) == 0) q.flush();
         }
+        q.finish(nullptr);
     }
-    double v[4];
-    q.totals(v);
-    if (sizeof(T) == 4 && __syncthreads_or(q.huge)) diag_in_double(p, NV, nlast, wrow, wlast, v, q.bad);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    if (sizeof(T) == 4 && __syncthreads_or(q.huge)) diag_in_double(p, NV, nlast, wrow, wlast, q.v, q.bad);
     if (q.bad) atomicExch(bad, 1);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) sh[k][threadIdx.x] = q.v[k];
     T mn = q.mn, mx = q.mx;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -723,23 +745,26 @@ __global__ void __launch_bounds__(kBlock) k_diag_part(const T *f, long long NV, 
         smin[threadIdx.x >> 5] = mn;
         smax[threadIdx.x >> 5] = mx;
     }
-    const double t = block_sums<4>(v, sh);
+    __syncthreads();
+    // one warp per sum (a shuffle tree per sum in every warp keeps the FP64 pipe
+    // busy three times as long)
+    if (warp >= 4) return;
+    double t = 0.0;
+    for (int i = 0; i < nw; ++i) t += sh[warp][32 * i + lane];
+    t = warp_sum(t);
+    if (lane) return;
     double *o = part + (long long)blockIdx.x * 6;
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
         o[0] = t;
         rho[blockIdx.x] = t * dV;
-        for (int k = 1; k < (int)blockDim.x / 32; ++k) {
+        for (int k = 1; k < nw; ++k) {
             mn = vmin(mn, smin[k]);
             mx = vmax(mx, smax[k]);
         }
         o[4] = (double)mn;
         o[5] = (double)mx;
-    } else if (threadIdx.x == 1) {
-        o[1] = 0.5 * unit * t;
-    } else if (threadIdx.x == 2) {
-        o[2] = t;
-    } else if (threadIdx.x == 3) {
-        o[3] = t;
+    } else {
+        o[warp] = warp == 1 ? 0.5 * unit * t : t;
     }
 }
 

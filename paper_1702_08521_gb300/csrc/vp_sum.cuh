@@ -48,6 +48,32 @@ struct LongSum : PairSum {
     __device__ __forceinline__ float error() const { return (e + rest) + far; }
 };
 
+// A sum of products with the products' own errors.  Those are kept apart from
+// the sum's: the latter are few bits and mostly add up exactly, in one term they
+// would make each other round.
+struct ProductSum : LongSum {
+    float q = 0.f;
+    __device__ __forceinline__ void add_product(float a, float b) {
+        const float p = __fmul_rn(a, b);  // (never part of an FMA: the sum is of the rounded product)
+        add(p);
+        q += fmaf(a, b, -p);
+    }
+    __device__ __forceinline__ float error() const { return LongSum::error() + q; }
+};
+
+// A sum of squares: the errors of squares are not even in sign, so that their sum
+// grows with the number of cells and rounds always the same way; it gets an error
+// term of its own.
+struct SquareSum : LongSum {
+    PairSum q;
+    __device__ __forceinline__ void add_square(float a) {
+        const float p = __fmul_rn(a, a);
+        add(p);
+        q.add(fmaf(a, a, -p));
+    }
+    __device__ __forceinline__ float product_error() const { return q.e + q.s; }
+};
+
 // the same for every number on the integer pipe, where subnormal ones are common
 // (sums over the empty tails of a distribution)
 __device__ __forceinline__ double widen_any(float x) {

@@ -249,3 +249,46 @@ def test_density_of_fp32_cells_of_any_size(nv, scale):
     bad = np.isnan(sim.rho.cpu().numpy())
     assert bad[1] and bad.sum() == 1
     sim.close()
+
+
+@pytest.mark.parametrize("nx,nv", [([5], [128]), ([3], [5000]), ([2, 3], [64, 64]), ([4], [4099]), ([2, 2, 2], [32, 32, 32]), ([2, 1, 2], [9, 20, 33])])
+@pytest.mark.parametrize("kind", ["large", "order one", "tiny", "straddling", "mixed points"])
+def test_fp32_diagnostic_sums_as_float_pairs(nx, nv, kind):
+    """Sums of FP32 cells that stay below the size at which a point is summed in
+    double: all near that size (their squares leave the float range in sums of a few
+    hundred), of order one, all tiny, on both sides of the scaled class's limit, and
+    some points above it beside others below.  Pair sums of up to 19 cells: 19
+    roundings of their error term, 2^-51 each, and weights of 48 bits; independent
+    over the grid's runs of 16 cells where every term is positive: six standard
+    deviations, and two roundings of the double result."""
+    import math
+    D = len(nx)
+    g = dict(dims=D, nx=nx, nv=nv, xlo=[0.0] * D, xhi=[1.0] * D, vlo=[-2.0] * D, vhi=[3.0] * D)
+    sim, og = both(g, V.VP_F32)
+    rng = np.random.default_rng(sum(nv) + len(kind))
+    shape = (og.NX, og.NV)
+    f = rng.random(shape) + 0.1
+    if kind == "large":
+        f = 1e18 * f
+    elif kind == "tiny":
+        f = f * 10.0 ** rng.uniform(-40, -20, size=shape)
+    elif kind == "straddling":
+        f = np.where(rng.random(shape) < 0.2, -f, f) * 2.0 ** rng.uniform(-60, -40, size=shape)
+    elif kind == "mixed points":
+        f[::2] *= 10.0 ** rng.uniform(16, 25, size=(f[::2].shape[0], 1))
+    f = f.astype(np.float32)
+    to_gpu(sim, f)
+    d = V.vp_diagnostics(sim.ctx, 1)
+    dX, dV = float(np.prod([1.0 / n for n in nx])), float(np.prod([5.0 / n for n in nv]))
+    fx = f.astype(np.float64).reshape([og.NX] + list(nv))
+    v2 = sum((np.asarray(og.v_centres(k)) ** 2).reshape([-1 if j == k else 1 for j in range(D)]) for k in range(D))
+    terms = dict(mass=fx, ke=0.5 * fx * v2, l1=np.abs(fx), l2=fx ** 2)
+    for k, t in terms.items():
+        size = math.fsum(np.abs(t).reshape(-1)) * dX * dV
+        off = abs(d[k] - math.fsum(t.reshape(-1)) * dX * dV) / size
+        assert off <= 19 * 2.0 ** -51 + 2.0 ** -47, (k, off)
+        if kind == "order one":
+            weights = 2.0 ** -48 if k == "ke" else 0.0
+            assert off <= 6 * (16 * 2.0 ** -51 + weights) / np.sqrt(12 * max(1, fx.size / 16)) + 2.0 ** -51, (k, off)
+    assert d["min_f"] == f.min() and d["max_f"] == f.max()
+    sim.close()
