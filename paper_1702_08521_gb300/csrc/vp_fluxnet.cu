@@ -1557,7 +1557,8 @@ int vp_fine_flux(vp_ctx *c, int kick, int dim, double dt, const double *accel_de
 
 int vp_restrict_velocity(const float *f_fine, float *f_coarse, long long NX, int nf1, int nf2, int factor1,
                          int factor2, void *stream) {
-    if (!f_fine || !f_coarse || factor1 < 1 || factor2 < 1 || nf1 % factor1 || nf2 % factor2) return VP_EINVAL;
+    if (!f_fine || !f_coarse || factor1 < 1 || factor2 < 1 || nf1 < 1 || nf2 < 1 || nf1 % factor1 || nf2 % factor2)
+        return VP_EINVAL;
     const int nc1 = nf1 / factor1, nc2 = nf2 / factor2;
     const long long n = NX * nc1 * nc2;
     const int quad = factor2 == 4 && (reinterpret_cast<uintptr_t>(f_fine) & 15) == 0, ff = factor1 * factor2;

@@ -22,7 +22,7 @@ struct __align__(16) LineShift {
 };
 
 // Geometry of one sweep: f viewed as [outer][L][inner].
-// Division of 32-bit unsigned values by a divisor fixed before the launch
+// Division of 32-bit unsigned values by a divisor (not 0) fixed before the launch
 // (Granlund & Montgomery 1994, Fig. 4.1): with l = ceil(log2 d) and
 // m = floor(2^32 (2^l - d) / d) + 1, n / d = (t + ((n - t) >> s1)) >> s2
 // where t = high word of m n, s1 = min(l, 1), s2 = max(l - 1, 0).

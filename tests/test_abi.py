@@ -110,3 +110,12 @@ def test_host_buffer_and_ensemble_calls_check_their_arguments_without_gpu_work(l
     assert L.vp_ensemble_set_flat_vote(None, 1) == vlasov.VP_EINVAL
     assert L.vp_ensemble_get_flat_vote(None, ctypes.byref(on)) == vlasov.VP_EINVAL
     assert on.value == 7
+
+
+@pytest.mark.parametrize("nf1,nf2", [(0, 4), (4, 0), (0, 0), (-4, 4), (4, -4), (-4, -4)])
+def test_restriction_refuses_empty_velocity_axes_without_gpu_work(lib, nf1, nf2):
+    """No velocity cells (or a negative number) is a bad argument, found before any
+    CUDA call."""
+    L = vlasov.load()
+    p = ctypes.c_void_p(4096)
+    assert L.vp_restrict_velocity(p, p, 3, nf1, nf2, 1, 1, None) == vlasov.VP_EINVAL
