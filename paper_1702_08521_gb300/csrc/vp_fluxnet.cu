@@ -759,6 +759,13 @@ __global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, 
 // velocity grid [nf1][nf2] (nf2 = factor2 = 1 for one velocity dimension).
 // The sum as a float pair (a conversion and an addition in double per fine
 // cell took 328 us for 6.7e7 cells); quad: factor2 = 4 on 16-byte rows.
+// the same sum in double, where it leaves the float range (or a cell is not finite)
+__device__ __noinline__ double restrict_rare(const float *p, int nf2, int factor1, int factor2) {
+    double sum = 0.0;
+    for (int k = 0; k < factor1; ++k)
+        for (int b = 0; b < factor2; ++b) sum += (double)p[(long long)k * nf2 + b];
+    return sum;
+}
 __global__ void __launch_bounds__(256) k_restrict_v2(const float *__restrict__ ff, float *__restrict__ fc,
                                                      long long total, FastDiv nc12, FastDiv nc2, int nf2, long long nf12,
                                                      int factor1, int factor2, int quad, double inv) {
@@ -789,7 +796,9 @@ __global__ void __launch_bounds__(256) k_restrict_v2(const float *__restrict__ f
         for (int k = 0; k < factor1; ++k)
             for (int b = 0; b < factor2; ++b) a.add(p[(long long)k * nf2 + b]);
     }
-    fc[t] = (float)(inv != 0.0 ? pair_value(a) * inv : pair_value(a) / (factor1 * factor2));
+    double sum = pair_value(a);
+    if (!isfinite(a.s)) sum = restrict_rare(p, nf2, factor1, factor2);
+    fc[t] = (float)(inv != 0.0 ? sum * inv : sum / (factor1 * factor2));
 }
 
 // Samples on coarse lines: for every coarse interface with |zeta| >= zmin,

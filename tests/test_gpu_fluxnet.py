@@ -532,3 +532,22 @@ def test_training_loss_and_gradient_to_fp32_rounding(n, group, coef, net):
         eg = float((grad.double() - want).norm() / want.norm())
         worst.append((el / tol, eg / tol_grad))
     assert max(e for e, _ in worst) <= 1.0 and max(e for _, e in worst) <= 1.0, worst
+
+
+@pytest.mark.parametrize("factors", [(4, 4), (3, 5), (8, 1)])
+def test_restriction_of_cells_whose_sum_leaves_the_float_range(factors):
+    """Means of cells up to FLT_MAX are finite: one FP32 rounding of sums in double.
+    Cells that are not finite stay so."""
+    import torch
+    a, b = factors
+    rng = np.random.default_rng(a)
+    f = (rng.random((5, 2 * a, 3 * b)) * 3.4e38).astype(np.float32)
+    f[3, 0, 0], f[4, 0, 0] = np.inf, np.nan
+    out = torch.empty(5 * 6, device="cuda")
+    V.vp_restrict_velocity(torch.as_tensor(f.reshape(-1), device="cuda"), out, 5, 2 * a, 3 * b, a, b)
+    torch.cuda.synchronize()
+    want = f.astype(np.float64).reshape(5, 2, a, 3, b).mean((2, 4)).reshape(-1)
+    out = out.cpu().numpy().astype(np.float64)
+    fine = np.isfinite(want)
+    assert (~fine).sum() == 2 and np.isinf(out[18]) and np.isnan(out[24])
+    assert (np.abs(out - want)[fine] <= 2.0 ** -23 * want[fine]).all()
