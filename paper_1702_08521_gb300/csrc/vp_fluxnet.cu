@@ -656,6 +656,7 @@ __global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, 
         // the shift of the stencil: modulo the line, or just off its ends
         const int ns = q.periodic ? n % L : (n < -2 * L - 8 ? -2 * L - 8 : (n > 2 * L + 8 ? 2 * L + 8 : n));
         const float *ui = u + i;
+        bool over = false;  // a pair sum left the float range (or a cell is not finite)
         // the mass through interface j, M the fractional one in the upwind frame
         auto emit = [&](int j, float M) {
             const int c = j * every;
@@ -688,6 +689,7 @@ __global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, 
                 const float one = n >= 0 ? 1.f : -1.f;
                 for (int m = n >= 0 ? n : -n; m > 0; --m, v += WP) p.add(one * *v);
                 p.add(M);
+                over |= !isfinite(p.s);
                 p.s = sg > 0 ? p.s : -p.s;
                 p.e = sg > 0 ? p.e : -p.e;
                 g = pair_value(p);
@@ -743,6 +745,25 @@ __global__ void __launch_bounds__(256) k_fine_flux(const float *__restrict__ f, 
                 ++k;
             }
         }
+        // the thread's interfaces again, the sums in double
+        if (!PREFIX && over)
+            for (int j = j0; j < j1; ++j) {
+                const int c = j * every, d = n >= 0 ? 1 : -1;
+                int a = sg > 0 ? c - ns - 4 : c + ns - 3;
+                if (q.periodic) {
+                    while (a < -kEdge) a += L;
+                    while (a > L + 1) a -= L;
+                } else {
+                    a = a < -7 ? -7 : (a > L ? L : a);
+                }
+                const float *v = ui + (sg > 0 ? a : a + 6) * WP;
+                const int s = sg * WP;
+                double g = (double)vp_core::flux<float, 7, true>(sh, v[0], v[s], v[2 * s], v[3 * s], v[4 * s], v[5 * s],
+                                                                 v[6 * s], alpha, 1, 1);
+                v = ui + (sg > 0 ? (n >= 0 ? c - n : c) : (n >= 0 ? c : c + n)) * WP;
+                for (int m = 0; m < d * n; ++m) g += (double)(d * v[m * WP]);
+                Gs[i * NP + j] = sg > 0 ? g : -g;
+            }
     }
     __syncthreads();
     double *out = G + l0 * nout;

@@ -551,3 +551,37 @@ def test_restriction_of_cells_whose_sum_leaves_the_float_range(factors):
     fine = np.isfinite(want)
     assert (~fine).sum() == 2 and np.isinf(out[18]) and np.isnan(out[24])
     assert (np.abs(out - want)[fine] <= 2.0 ** -23 * want[fine]).all()
+
+
+@pytest.mark.parametrize("dt", [1.875, -1.875, 5.0])
+def test_fine_flux_of_cells_whose_sum_leaves_the_float_range(dt):
+    """Masses of several whole cells of 6e37 are finite doubles, as direct sums of a
+    few cells and (longer shifts) as differences of prefix sums of a line: where a
+    shift is a whole number of cells, the sum of the swept cells, to 40 roundings of
+    the sum of a line in double and the rounding of the shift."""
+    import torch
+    nx, nv = 40, 17
+    g = dict(dims=1, nx=[nx], nv=[nv], xlo=[0.0], xhi=[float(nx)], vlo=[-3.4], vhi=[3.4], order=7)
+    sim = V.Simulation(g, precision=V.VP_F32)
+    rng = np.random.default_rng(3)
+    f = ((0.9 + 0.1 * rng.random((nx, nv))) * 6.5e37).astype(np.float32)
+    sim.upload(f.reshape(-1))
+    G = torch.empty(nv * (nx + 1), dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    V.vp_fine_flux(sim.ctx, 0, 0, dt, None, 1, G)
+    sim.sync()
+    G = G.cpu().numpy().reshape(nv, nx + 1)
+    assert np.isfinite(G).all()
+    f = f.astype(np.float64)
+    seen = 0.0
+    for k in range(nv):
+        s = (-3.4 + 0.4 * (k + 0.5)) * dt
+        n = int(round(s))
+        if abs(s - n) > 1e-9:
+            continue
+        whole = np.array([sum(f[(j - 1 - m) % nx, k] for m in range(n)) - sum(f[(j + m) % nx, k] for m in range(-n))
+                          for j in range(nx + 1)])
+        assert np.abs(G[k] - whole).max() <= 40 * 40 * 2.0 ** -53 * 6.5e37 + 1e-13 * 6.5e37
+        seen = max(seen, np.abs(whole).max())
+    assert seen > 3.5e38
+    sim.close()
