@@ -522,11 +522,8 @@ __device__ __forceinline__ double pair_value(const PairSum &p) { return widen(p.
 // power of two, at most kTileLines) consecutive lines per CTA
 constexpr int kTileLines = 64;
 
-struct LineTile {
-    long long lines, inner;
-    int L, W, logW, periodic, from_inner;
-    unsigned cdiv, cmod;
-    FastDiv fd_inner, fd_cdiv, fd_cmod;
+struct LineTile : LineShape {
+    int W, logW;
 };
 // element of a line's first cell, and its class
 struct LinePos {
@@ -534,13 +531,7 @@ struct LinePos {
     unsigned cls[kTileLines];
 };
 __device__ __forceinline__ void place_lines(const LineTile &q, long long l0, int nl, LinePos &p) {
-    for (int i = threadIdx.x; i < nl; i += blockDim.x) {
-        const long long line = l0 + i;
-        const long long o = q.lines < (1LL << 32) ? (long long)fdiv((unsigned)line, q.fd_inner) : line / q.inner;
-        const long long c = line - o * q.inner;
-        p.base[i] = o * q.L * q.inner + c;
-        p.cls[i] = q.from_inner ? fmod_u(fdiv((unsigned)c, q.fd_cdiv), q.fd_cmod) : fdiv((unsigned)o, q.fd_cdiv);
-    }
+    for (int i = threadIdx.x; i < nl; i += blockDim.x) p.cls[i] = q.place(l0 + i, p.base[i]);
 }
 
 // rows beyond the line that the 7- and 8-cell stencils reach (zero, or the
@@ -788,21 +779,21 @@ __device__ __noinline__ double restrict_rare(const float *p, int nf2, int factor
     return sum;
 }
 __global__ void __launch_bounds__(256) k_restrict_v2(const float *__restrict__ ff, float *__restrict__ fc,
-                                                     long long total, FastDiv nc12, FastDiv nc2, int nf2, long long nf12,
+                                                     long long total, long long ncell, FastDiv nc12, FastDiv nc2,
+                                                     int nf2, long long nf12,
                                                      int factor1, int factor2, int quad, double inv) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total) return;
-    long long x;
-    unsigned J;
+    long long x, J1;
     if (total < (1LL << 32)) {
         x = fdiv((unsigned)t, nc12);
-        J = (unsigned)t - (unsigned)x * nc12.d;
+        J1 = fdiv((unsigned)t - (unsigned)x * nc12.d, nc2);
     } else {
-        x = t / nc12.d;
-        J = (unsigned)(t - x * nc12.d);
+        x = t / ncell;
+        J1 = (t - x * ncell) / nc2.d;
     }
-    const unsigned J1 = fdiv(J, nc2), J2 = J - J1 * nc2.d;
-    const float *p = ff + x * nf12 + (long long)J1 * factor1 * nf2 + (long long)J2 * factor2;
+    const long long J2 = t - x * ncell - J1 * nc2.d;
+    const float *p = ff + x * nf12 + J1 * factor1 * nf2 + J2 * factor2;
     PairSum a;
     if (quad) {
 #pragma unroll 4
@@ -876,7 +867,7 @@ __global__ void __launch_bounds__(kSampleThreads)
     if (STAGED) {
         for (int k = 0; k < 3; ++k) {  // the lines, then class + 1 and class - 1
             float *d = tile + (size_t)k * W * P + kEdge;
-            stage_lines(fc, q, pos, nl, k == 0 ? 0 : (k == 1 ? 1 : -1) * (long long)q.cdiv,
+            stage_lines(fc, q, pos, nl, k == 0 ? 0 : (k == 1 ? 1 : -1) * q.cdiv,
                         [&](int i) { return k == 0 || (nbr[i] & (k == 1 ? 2 : 4)); },
                         [&](int i, int row) { return d + i * P + row; });
         }
@@ -913,7 +904,7 @@ __global__ void __launch_bounds__(kSampleThreads)
                     if (nb && !(nbr[i] & (nb > 0 ? 2 : 4))) return 0.f;
                     if (q.periodic) r = wrap_row(r, L);
                     else if (r < 0 || r >= L) return 0.f;
-                    return base[(long long)r * q.inner + nb * (long long)q.cdiv];
+                    return base[(long long)r * q.inner + nb * q.cdiv];
                 };
                 // stencil cells: rows a .. a + 7, in upwind order by sg
                 const int nsh = q.periodic ? n % L : (n < -2 * L - 8 ? -2 * L - 8 : (n > 2 * L + 8 ? 2 * L + 8 : n));
@@ -1435,11 +1426,9 @@ LineTile line_tile(const LineGeo &q) {
     t.L = q.L;
     t.periodic = q.periodic;
     t.from_inner = q.from_inner;
-    t.cdiv = (unsigned)q.cdiv;
+    t.cdiv = q.cdiv;
     t.cmod = (unsigned)q.cmod;
-    t.fd_inner = make_fastdiv((unsigned)q.inner);
-    t.fd_cdiv = make_fastdiv(t.cdiv);
-    t.fd_cmod = make_fastdiv(t.cmod);
+    t.prepare();
     return t;
 }
 void set_width(LineTile &t, int W) {
@@ -1590,11 +1579,11 @@ int vp_restrict_velocity(const float *f_fine, float *f_coarse, long long NX, int
     if (!f_fine || !f_coarse || factor1 < 1 || factor2 < 1 || nf1 < 1 || nf2 < 1 || nf1 % factor1 || nf2 % factor2)
         return VP_EINVAL;
     const int nc1 = nf1 / factor1, nc2 = nf2 / factor2;
-    const long long n = NX * nc1 * nc2;
+    const long long ncell = (long long)nc1 * nc2, n = NX * ncell;
     const int quad = factor2 == 4 && (reinterpret_cast<uintptr_t>(f_fine) & 15) == 0, ff = factor1 * factor2;
     const double inv = (ff & (ff - 1)) == 0 ? 1.0 / ff : 0.0;  // exact
     k_restrict_v2<<<(unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        f_fine, f_coarse, n, make_fastdiv((unsigned)(nc1 * nc2)), make_fastdiv((unsigned)nc2), nf2,
+        f_fine, f_coarse, n, ncell, make_fastdiv(n < (1LL << 32) ? (unsigned)ncell : 1u), make_fastdiv((unsigned)nc2), nf2,
         (long long)nf1 * nf2, factor1, factor2, quad, inv);
     return cudaGetLastError() == cudaSuccess ? VP_OK : VP_ECUDA;
 }

@@ -43,11 +43,44 @@ inline FastDiv make_fastdiv(unsigned d) {
 }
 
 #ifdef __CUDACC__
-__device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv &f) {
+__host__ __device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv &f) {
+#ifdef __CUDA_ARCH__
     const unsigned t = __umulhi(n, f.m);
+#else
+    const unsigned t = (unsigned)(((unsigned long long)n * f.m) >> 32);
+#endif
     return (t + ((n - t) >> f.s1)) >> f.s2;
 }
-__device__ __forceinline__ unsigned fmod_u(unsigned n, const FastDiv &f) { return n - fdiv(n, f) * f.d; }
+__host__ __device__ __forceinline__ unsigned fmod_u(unsigned n, const FastDiv &f) { return n - fdiv(n, f) * f.d; }
+
+// The lines along one axis of f viewed as [outer][L][inner], `lines` = outer inner
+// of them, and their classes: of the inner index (from_inner) or the outer one,
+// divided by cdiv, modulo cmod.  Multiplications in place of divisions for fewer
+// than 2^32 lines (the indices and cdiv are then below 2^32 too), 64-bit ones beyond.
+struct LineShape {
+    long long lines, inner, cdiv;
+    int L, periodic, from_inner;
+    unsigned cmod;
+    FastDiv fd_inner, fd_cdiv, fd_cmod;
+
+    void prepare() {
+        const bool narrow = lines < (1LL << 32);
+        fd_inner = make_fastdiv(narrow ? (unsigned)inner : 1u);
+        fd_cdiv = make_fastdiv(narrow ? (unsigned)cdiv : 1u);
+        fd_cmod = make_fastdiv(cmod);
+    }
+    // the line's class; base: element of its first cell
+    __host__ __device__ __forceinline__ unsigned place(long long line, long long &base) const {
+        if (lines < (1LL << 32)) {
+            const unsigned o = fdiv((unsigned)line, fd_inner), c = (unsigned)line - o * (unsigned)inner;
+            base = (long long)o * L * inner + c;
+            return from_inner ? fmod_u(fdiv(c, fd_cdiv), fd_cmod) : fdiv(o, fd_cdiv);
+        }
+        const long long o = line / inner, c = line - o * inner;
+        base = o * L * inner + c;
+        return (unsigned)(from_inner ? c / cdiv % cmod : o / cdiv);
+    }
+};
 #endif
 
 // Programmatic dependent launch: a kernel launched by vp_launch_dep may start
