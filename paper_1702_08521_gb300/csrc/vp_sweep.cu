@@ -748,6 +748,9 @@ int launch_cols(vp_ctx *c, SweepGeo geo, const SweepTune &tu, const SweepShift &
         const int wt = (int)geo.inner;
         const bool tma = tu.impl == 2 && tma_eligible<T>(c, geo, wt);
         long long k = tma ? 1 : W / wt;
+        // (of lines so long that W columns do not fit, as many as do)
+        const long long fit = 200 * 1024 / ((long long)(L + 2 * ghost_rows(geo)) * wt * (int)sizeof(T));
+        k = k > fit && fit > 0 ? fit : k;
         k = k > geo.outer ? geo.outer : k;
         geo.kblk = (int)k;
         W = wt * geo.kblk;

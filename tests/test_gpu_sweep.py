@@ -376,3 +376,33 @@ def test_blocks_side_by_side_and_rows_of_every_width(precision, nx, nv):
             else:
                 O.drift_sweep(og, f_o, d, 0.29)
             assert rel_l1(out[0], f_o) <= (2e-6 if precision == V.VP_F32 else 1e-12)
+
+
+@pytest.mark.parametrize("precision,n", [(V.VP_F32, 12000), (V.VP_F32, 20000), (V.VP_F64, 5000), (V.VP_F64, 9000)])
+@pytest.mark.parametrize("tune", [0, 1])
+def test_long_lines_in_blocks_of_two_columns(precision, n, tune):
+    """Strided lines whose tile of two columns fits shared memory but one of four does
+    not (and ones where four just fit): the same cells as contiguous lines of a grid of
+    one velocity dimension, kicked by the same accelerations."""
+    import torch
+    rng = np.random.default_rng(n)
+    f = inputs.random_f(6 * n * 2, seed=n).reshape(6, n, 2)
+    f = f.astype(np.float32 if precision == V.VP_F32 else np.float64)
+    acc = rng.uniform(-3.0, 3.0, size=6)
+    g2 = dict(dims=2, nx=[3, 2], nv=[n, 2], xlo=[0.0] * 2, xhi=[1.0] * 2, vlo=[-2.0] * 2, vhi=[3.0] * 2, order=7)
+    sim = V.Simulation(g2, precision=precision)
+    V.vp_set_option(sim.ctx, 2, tune)
+    sim.upload(f.reshape(-1))
+    V.vp_kick_sweep(sim.ctx, 0, 0.0021, torch.as_tensor(acc, device="cuda"))
+    sim.sync()
+    got = sim.f.cpu().numpy().reshape(6, n, 2)
+    sim.close()
+    g1 = dict(dims=1, nx=[12], nv=[n], xlo=[0.0], xhi=[1.0], vlo=[-2.0], vhi=[3.0], order=7)
+    sim = V.Simulation(g1, precision=precision)
+    V.vp_set_option(sim.ctx, 2, 0)
+    sim.upload(np.ascontiguousarray(f.transpose(0, 2, 1)).reshape(-1))
+    V.vp_kick_sweep(sim.ctx, 0, 0.0021, torch.as_tensor(np.repeat(acc, 2), device="cuda"))
+    sim.sync()
+    want = sim.f.cpu().numpy().reshape(6, 2, n).transpose(0, 2, 1)
+    sim.close()
+    assert not np.array_equal(want, f) and np.array_equal(got, want)
