@@ -284,9 +284,6 @@ __global__ void __launch_bounds__(64) k_rk_lines(float *__restrict__ f, const Li
     edges();
 #pragma unroll 1
     for (int stage = 0; stage < 3; ++stage) {
-        // the walk reads its line as restricted, and a stage reads what the one
-        // before it wrote: no access moves across this point
-        asm volatile("" ::: "memory");
         const float ca = stage == 0 ? 0.f : (stage == 1 ? 0.75f : 1.f / 3.f);
         const float cv = stage == 0 ? 1.f : (stage == 1 ? 0.25f : 2.f / 3.f);
         // cells in walk order from row i0 on; the last stage writes f
@@ -302,16 +299,15 @@ __global__ void __launch_bounds__(64) k_rk_lines(float *__restrict__ f, const Li
         };
         if (both) {
             const vp_core::LineShiftP2 sh = vp_core::pair_shift(sa, sb);
-            vp_core::walk<P2, 5, false, FULL, E>(reinterpret_cast<const P2 *>(A + cc), W >> 1, L, sh, 0, L,
+            vp_core::walk_in_place<P2, 5, false, FULL, E>(reinterpret_cast<const P2 *>(A + cc), W >> 1, L, sh, 0, L,
                                                  P2((float)lp.alpha), lp.mp, lp.pp, store(P2(), cc, sh.sigma));
         } else {
             for (int k = (PAIR && cc + 1 < wc ? 1 : 0); k >= 0; --k) {
                 const LineShift<float> &sl = k ? sb : sa;
-                vp_core::walk<float, 5, false, FULL, E>(A + cc + k, W, L, sl, 0, L, (float)lp.alpha, lp.mp, lp.pp,
+                vp_core::walk_in_place<float, 5, false, FULL, E>(A + cc + k, W, L, sl, 0, L, (float)lp.alpha, lp.mp, lp.pp,
                                                         store(0.f, cc + k, sl.sigma));
             }
         }
-        asm volatile("" ::: "memory");
         if (geo.periodic && stage < 2) edges();
     }
 }
@@ -381,7 +377,6 @@ __global__ void __launch_bounds__(32) k_rk_line_rows(float *__restrict__ f, cons
         const bool both = two && sa.sigma == sb.sigma;
 #pragma unroll 1
         for (int stage = 0; stage < 3; ++stage) {
-            asm volatile("" ::: "memory");  // as in k_rk_lines
             const float ca = stage == 0 ? 0.f : (stage == 1 ? 0.75f : 1.f / 3.f);
             const float cv = stage == 0 ? 1.f : (stage == 1 ? 0.25f : 2.f / 3.f);
             auto store = [&](auto t, int line, int sigma) {
@@ -394,16 +389,15 @@ __global__ void __launch_bounds__(32) k_rk_line_rows(float *__restrict__ f, cons
             };
             if (both) {
                 const vp_core::LineShiftP2 sh = vp_core::pair_shift(sa, sb);
-                vp_core::walk<P2, 5, false, FULL, E>(reinterpret_cast<const P2 *>(A + ia(l, 0)), 1, L, sh, 0, L,
+                vp_core::walk_in_place<P2, 5, false, FULL, E>(reinterpret_cast<const P2 *>(A + ia(l, 0)), 1, L, sh, 0, L,
                                                      P2((float)lp.alpha), lp.mp, lp.pp, store(P2(), l, sh.sigma));
             } else {
                 for (int k = two ? 1 : 0; k >= 0; --k) {
                     const LineShift<float> &sl = k ? sb : sa;
-                    vp_core::walk<float, 5, false, FULL, E>(A + ia(l + k, 0), 2, L, sl, 0, L, (float)lp.alpha, lp.mp,
+                    vp_core::walk_in_place<float, 5, false, FULL, E>(A + ia(l + k, 0), 2, L, sl, 0, L, (float)lp.alpha, lp.mp,
                                                             lp.pp, store(0.f, l + k, sl.sigma));
                 }
             }
-            asm volatile("" ::: "memory");
         }
     }
     __syncwarp();

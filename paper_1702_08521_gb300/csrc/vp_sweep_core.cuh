@@ -359,11 +359,14 @@ __device__ __forceinline__ T flux_walk(const SH &sh, T um3, T um2, T um1, T u0, 
 // negative cell take the PP limiter's theta form (pp_theta_mass) instead of
 // the clamp (scalar T only).  FLAT = false leaves the flat-stencil vote out
 // (the same results; for data that is nowhere flat the vote only costs).
+// walk_in_place: the store may write the line's own rows (a whole zero-inflow
+// line with ghost rows: a row is read before the cell four before it is stored,
+// and not again).  walk: what the store writes is not read.
 
 template <typename T, int ORDER, bool PERIODIC, bool FULL, int GP, bool NEG = false, bool FLAT = true,
           typename Store, typename SH>
-__device__ __forceinline__ bool walk(const T *__restrict__ sm0, int ss, int L, const SH &sh,
-                                     int r0, int r1, T alpha, int mp, int pp, Store store) {
+__device__ __forceinline__ bool walk_in_place(const T *sm0, int ss, int L, const SH &sh,
+                                              int r0, int r1, T alpha, int mp, int pp, Store store) {
     if (r0 >= r1) return false;
     // FD: the largest |u| of the segment (high words), for the caller's repeat
     int big = 0;
@@ -574,6 +577,13 @@ __device__ __forceinline__ bool walk(const T *__restrict__ sm0, int ss, int L, c
 #undef VP_WALK_STEPS
 #undef VP_WALK_BLOCK
     return big >= FD::kBig;
+}
+
+template <typename T, int ORDER, bool PERIODIC, bool FULL, int GP, bool NEG = false, bool FLAT = true,
+          typename Store, typename SH>
+__device__ __forceinline__ bool walk(const T *__restrict__ sm0, int ss, int L, const SH &sh, int r0, int r1, T alpha,
+                                     int mp, int pp, Store store) {
+    return walk_in_place<T, ORDER, PERIODIC, FULL, GP, NEG, FLAT>(sm0, ss, L, sh, r0, r1, alpha, mp, pp, store);
 }
 
 // The walk of one line in the arithmetic of its type: FP64 lines with integer
