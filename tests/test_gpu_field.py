@@ -292,3 +292,37 @@ def test_fp32_diagnostic_sums_as_float_pairs(nx, nv, kind):
             assert off <= 6 * (16 * 2.0 ** -51 + weights) / np.sqrt(12 * max(1, fx.size / 16)) + 2.0 ** -51, (k, off)
     assert d["min_f"] == f.min() and d["max_f"] == f.max()
     sim.close()
+
+
+@pytest.mark.parametrize("n", [7, 64, 300])
+@pytest.mark.parametrize("order", [2, 6])
+def test_field_of_a_density_on_a_large_background(n, order):
+    """One dimension: a uniform density has no field at all, and a variation on a
+    background 1e6 times as large has its own field to 1e-12 of the sizes of its
+    convolution's terms (the kernels' own 2 n roundings of sums of n terms)."""
+    ld = np.longdouble
+    pi = ld("3.14159265358979323846264338327950288")
+    L, S = 4.0, -1.5
+    g = dict(dims=1, nx=[n], nv=[8], xlo=[0.0], xhi=[L], vlo=[-1.0], vhi=[1.0], pois_order=order, coupling=S, rho_bg=1.0)
+    th, h = 2 * pi * np.arange(n).astype(ld) / n, ld(L) / n
+    b, den = {2: ([1], 1), 6: ([270, -27, 2], 180)}[order]
+    c, fden = {2: ([1], 2), 6: ([45, -9, 1], 60)}[order]
+    lam = sum(-4 * ld(x) * np.sin((m + 1) * th / 2) ** 2 for m, x in enumerate(b)) / den / h ** 2
+    green = np.concatenate([[ld(0)], ld(S) / lam[1:] / n])
+    sym = sum(2 * ld(x) * np.sin((m + 1) * th) for m, x in enumerate(c)) / (fden * h)
+    j = np.arange(n)
+    ang = 2 * pi * ((j[:, None] * j) % n).astype(ld) / n
+    shift = (j[:, None] - j) % n
+    kernels = [(green * np.cos(ang)).sum(1)[shift], (green * sym * np.sin(ang)).sum(1)[shift]]
+    rng = np.random.default_rng(n)
+    sim, _ = both(g, V.VP_F64)
+    for rho in (np.full(n, 1e6 + 0.1), 1e6 + np.cos(2 * np.pi * j / n) + 0.1 * rng.standard_normal(n)):
+        sim.rho.copy_(sim.torch.as_tensor(rho))
+        sim.torch.cuda.synchronize()
+        V.vp_poisson_solve(sim.ctx, sim.rho, sim.phi, sim.accel)
+        sim.sync()
+        r = rho.astype(ld) - np.median(rho[[0, n // 3, 2 * (n // 3)]])
+        for out, K in zip((sim.phi, sim.accel), kernels):
+            off = np.abs(out.cpu().numpy() - K @ r)
+            assert (off <= 1e-12 * (np.abs(K) @ np.abs(r))).all(), off.max()
+    sim.close()
