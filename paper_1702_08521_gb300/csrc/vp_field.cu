@@ -30,7 +30,7 @@ using vp_sum::widen_any;
 // So runs of a few cells are summed as float pairs -- value and error term of
 // Knuth's two-sum, products with their exact error from an FMA --, their values
 // added in double, and one warp adds the threads' doubles: the density of 3.1e8
-// cells 180 us, the diagnostics 0.72 ms (0.92 ms where most cells are subnormal or
+// cells 180 us, the diagnostics 0.74 ms (0.93 ms where most cells are subnormal or
 // nearly), with the errors of sums in double: 1e-16 of the mass, energy and
 // squares.  Whole threads' sums as pairs took 0.80 ms and were off by up to 7e-15.
 
@@ -540,14 +540,17 @@ struct DiagSum<float> {
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     float mn = INFINITY, mx = -INFINITY, scale = kUp;
     bool huge = false, bad = false;  // a cell above 2^60: the point is summed again in double
+    bool held = false;               // the doubles hold sums
     static constexpr float kUp = 0x1p100f, kPlain = 0x1p-40f, kHuge = 0x1p60f;
     static constexpr double kDown = 0x1p-100;
     __device__ __forceinline__ void any(float x, const W &w) {
         m2.add_product(x, w.hi);
         m2.q = fmaf(x, w.lo, m2.q);
     }
-    // to the scale 1
+    // to the scale 1 (mostly before any cell that is not empty)
     __device__ __forceinline__ void unscale() {
+        scale = 1.f;
+        if (l2.s == 0.f && !held) return;
         flush();
         flush_errors();
         v[0] *= kDown;
@@ -558,7 +561,6 @@ struct DiagSum<float> {
         m2 = vp_sum::ProductSum();
         l2 = vp_sum::SquareSum();
         neg = PairSum();
-        scale = 1.f;
     }
     __device__ __forceinline__ void cell(float x, const W &w, const W *w2) {
         mn = fminf(mn, x);
@@ -606,6 +608,7 @@ struct DiagSum<float> {
     // the pairs' values to the doubles, every 16 cells (the errors of a pair sum
     // grow with its value)
     __device__ __forceinline__ void flush() {
+        held = true;
         v[0] += widen_any(m0.s);
         v[1] += widen_any(m2.s);
         v[3] += widen_any(l2.s);
@@ -624,11 +627,15 @@ struct DiagSum<float> {
     // the end of a thread's sums, its cells of one index of the last axis with its
     // weight (NULL: weighed already)
     __device__ __forceinline__ void finish(const W *w) {
-        if (scale != 1.f) {
-            unscale();
-        } else {
+        if (scale != 1.f) unscale();
+        if (held) {
             flush();
             flush_errors();
+        } else {
+            v[0] = widen_any(m0.s) + widen_any(m0.error());
+            v[1] = widen_any(m2.s) + widen_any(m2.error());
+            v[3] = widen_any(l2.s) + (widen_any(l2.error()) + widen_any(l2.product_error()));
+            if (neg.s != 0.f) v[2] = widen_any(neg.s) + widen_any(neg.e);
         }
         if (w) v[1] = fma(widen_any(w->hi) + widen_any(w->lo), v[0], v[1]);
     }
@@ -690,7 +697,7 @@ __device__ __forceinline__ double vmax(double a, double b) { return fmax(a, b); 
 // once, to the thread's sum) and walks the rows; longer last axes are walked
 // cell by cell with both weights.
 template <typename T>
-__global__ void __launch_bounds__(kBlock) k_diag_part(const T *f, long long NV, int nlast, FastDiv fd_last,
+__global__ void __launch_bounds__(kBlock, 4) k_diag_part(const T *f, long long NV, int nlast, FastDiv fd_last,
                                                       const typename DiagSum<T>::W *wrow,
                                                       const typename DiagSum<T>::W *wlast, double unit,
                                                       double dV, double *part,
@@ -729,12 +736,24 @@ __global__ void __launch_bounds__(kBlock) k_diag_part(const T *f, long long NV, 
             q.finish(wlast + j);
         }
     } else {
-        int it = 1;
-        for (long long v = threadIdx.x; v < NV; v += blockDim.x, ++it) {
-            const long long r = v / nlast;
-            q.cell(p[v], wrow[r], wlast + (v - r * nlast));
-            if ((it & 3) == 0) q.fold();
-            if ((it & 15) == 0) q.flush();
+        for (long long v = threadIdx.x, it = 1; v < NV; v += 4 * (int)blockDim.x, ++it) {
+            T x[4];
+            typename DiagSum<T>::W w[4], w2[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const long long i = v + k * (int)blockDim.x;
+                if (i < NV) {
+                    const long long r = NV < (1LL << 32) ? (long long)fdiv((unsigned)i, fd_last) : i / nlast;
+                    x[k] = p[i];
+                    w[k] = wrow[r];
+                    w2[k] = wlast[i - r * nlast];
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (v + k * (int)blockDim.x < NV) q.cell(x[k], w[k], &w2[k]);
+            q.fold();
+            if ((it & 3) == 0) q.flush();
         }
         q.finish(nullptr);
     }
