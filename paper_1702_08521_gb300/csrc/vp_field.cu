@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kBlock) k_moment(const T *f, long long NX, lon
 // FP64 is the scarce unit here (two FMA lanes per SM and clock) and a launch
 // costs 2.5-4 us, so the solve is few launches that spread the FP64 work:
 //   * k_fft_lines transforms B lines of one axis in shared memory (Stockham,
-//     radices 4, 2, 3, 5 and direct sums for larger primes) with a table of
+//     radices 4 and 2, odd prime factors as direct sums) with a table of
 //     the n roots of unity, read from the context or, for callers without
 //     one, computed once per CTA.  The first axis reads rho itself, and the
 //     last forward axis multiplies by the Green function and transforms back
@@ -1020,7 +1020,7 @@ struct FftLaunch {
     size_t smem;
 };
 
-FftLaunch fft_axis(const int *m, int dims, int axis, int mode, const double2 *tw) {
+FftLaunch fft_axis(const int *m, int dims, int axis, int mode, const double2 *tw, int sms) {
     FftLaunch l{};
     FftArgs &f = l.f;
     f.p = fft_plan(m[axis]);
@@ -1033,9 +1033,9 @@ FftLaunch fft_axis(const int *m, int dims, int axis, int mode, const double2 *tw
     const int n = m[axis];
     f.lines = total / n;
     f.inner = (unsigned)inner;
-    // one line per CTA until the chip holds two CTAs per SM, then up to four
-    // neighbouring lines (64-byte rows on a strided axis)
-    int B = f.lines >= 1216 ? 4 : (f.lines >= 608 ? 2 : 1);
+    // up to four neighbouring lines per CTA (64-byte rows on a strided axis), as many
+    // as leave two CTAs per SM
+    int B = f.lines >= 8LL * sms ? 4 : (f.lines >= 4LL * sms ? 2 : 1);
     while (B > 1 && (size_t)(1 + 2 * B) * n * sizeof(double2) > 96 * 1024) B /= 2;
     f.B = B;
     l.blocks = inner == 1 ? (unsigned)((f.lines + B - 1) / B)
@@ -1242,7 +1242,7 @@ int vp_field_setup(vp_ctx *c) {
     free(h_k);
     VP_CUDA_TRY(c, cudaStreamSynchronize(cudaStreamLegacy));
     for (int d = 2; d >= 0; --d)
-        c->launches += fft_launch(c->stream, c->d_ghat, fft_axis(c->m, 3, d, FFT_FWD, c->roots[d]));
+        c->launches += fft_launch(c->stream, c->d_ghat, fft_axis(c->m, 3, d, FFT_FWD, c->roots[d], c->sm_count));
     VP_CUDA_TRY(c, cudaGetLastError());
     VP_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     return VP_OK;
@@ -1297,7 +1297,7 @@ int vp_launch_poisson(vp_ctx *c, const double *rho, double *phi, double *acc) {
     // forward along the last axis (reading rho) .. the second, then the first
     // axis forward, times the Green function, and back; the others back
     for (int d = D - 1; d >= 0; --d) {
-        FftLaunch l = fft_axis(c->m, D, d, d ? FFT_FWD : FFT_CONV, c->roots[d]);
+        FftLaunch l = fft_axis(c->m, D, d, d ? FFT_FWD : FFT_CONV, c->roots[d], c->sm_count);
         if (d == D - 1) {
             l.f.rho = rho;
             l.f.bg = g.rho_bg;
@@ -1314,7 +1314,7 @@ int vp_launch_poisson(vp_ctx *c, const double *rho, double *phi, double *acc) {
         c->launches += fft_launch(c->stream, c->d_fft, l);
     }
     for (int d = 1; d < D; ++d)
-        c->launches += fft_launch(c->stream, c->d_fft, fft_axis(c->m, D, d, FFT_INV, c->roots[d]));
+        c->launches += fft_launch(c->stream, c->d_fft, fft_axis(c->m, D, d, FFT_INV, c->roots[d], c->sm_count));
     vp_launch_dep(k_force, nblk(c->NX, kBlock), kBlock, 0, c->stream, c->d_fft, phi, acc, force_args(g, c->m,
                   c->NX));
     c->launches++;
@@ -1431,6 +1431,7 @@ namespace {
 constexpr int kNoallocMaxDevices = 64;
 std::mutex g_noalloc_mu;
 double2 *g_noalloc_dev_ptr[kNoallocMaxDevices];
+int g_noalloc_sms[kNoallocMaxDevices];
 
 __device__ double noalloc_stencil_eig(int order, double theta) {
     // eigenvalue of the symmetric discrete Laplacian stencil (b_0..b_3)/den
@@ -1494,6 +1495,7 @@ extern "C" int vp_poisson_periodic_noalloc(const vp_grid *g, void *cuda_stream, 
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kNoallocMaxDevices) return VP_ECUDA;
     double2 *buf = nullptr;
+    int sms = 0;
     {
         // once per device, with that device current: the device address of the
         // static array (its name in host code is only a host-side stand-in)
@@ -1502,18 +1504,20 @@ extern "C" int vp_poisson_periodic_noalloc(const vp_grid *g, void *cuda_stream, 
             void *p = nullptr;
             if (cudaGetSymbolAddress(&p, g_noalloc_fft) != cudaSuccess || !p) return VP_ECUDA;
             if (cudaFuncSetAttribute(k_fft_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, kFftSmem) !=
-                cudaSuccess)
+                    cudaSuccess ||
+                cudaDeviceGetAttribute(&g_noalloc_sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
                 return VP_ECUDA;
             g_noalloc_dev_ptr[dev] = static_cast<double2 *>(p);
         }
         buf = g_noalloc_dev_ptr[dev];
+        sms = g_noalloc_sms[dev];
     }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const int3 nb = make_int3(g->nx[0], D > 1 ? g->nx[1] : 1, D > 2 ? g->nx[2] : 1);
     const int m[3] = {nb.x, nb.y, nb.z};
     // every element of the work array that is read is written first: no clearing needed
     for (int d = D - 1; d >= 0; --d) {
-        FftLaunch l = fft_axis(m, D, d, FFT_FWD, nullptr);
+        FftLaunch l = fft_axis(m, D, d, FFT_FWD, nullptr, sms);
         if (d == D - 1) {
             l.f.rho = rho_dev;
             l.f.bg = g->rho_bg;
@@ -1525,7 +1529,7 @@ extern "C" int vp_poisson_periodic_noalloc(const vp_grid *g, void *cuda_stream, 
                                    D > 1 ? (g->xhi[1] - g->xlo[1]) / g->nx[1] : 1.0,
                                    D > 2 ? (g->xhi[2] - g->xlo[2]) / g->nx[2] : 1.0);
     k_green_onfly<<<nblk(NX, kBlock), kBlock, 0, st>>>(buf, NX, D, nb, h, g->pois_order, g->coupling);
-    for (int d = 0; d < D; ++d) fft_launch(st, buf, fft_axis(m, D, d, FFT_INV, nullptr));
+    for (int d = 0; d < D; ++d) fft_launch(st, buf, fft_axis(m, D, d, FFT_INV, nullptr, sms));
     vp_launch_dep(k_force, nblk(NX, kBlock), kBlock, 0, st, buf, phi_dev, accel_dev, force_args(*g, m, NX));
     return cudaGetLastError() == cudaSuccess ? VP_OK : VP_ECUDA;
 }
