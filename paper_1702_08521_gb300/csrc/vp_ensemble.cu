@@ -66,7 +66,6 @@ struct StageDesc {
     int kind;
     int kick;        // 1: velocity axis (speed = acceleration), 0: spatial axis
     int axis;        // axis index within x or v
-    int half;        // 1: dt/2
     long long outer, inner;
     int L;
     int periodic;
@@ -731,13 +730,12 @@ static int ens_fail(vp_ens *e, int code, const char *msg) {
 // stage lists of one run
 static int build_stages(RunDesc &r, int W, int R, int xpt, int &slot) {
     const int D = r.dims;
-    auto cols = [&](int kick, int axis, int half, long long outer, int L, long long inner, int per,
+    auto cols = [&](int kick, int axis, long long outer, int L, long long inner, int per,
                     long long cdiv, long long cmod) {
         StageDesc s{};
         s.kind = ST_COLS;
         s.kick = kick;
         s.axis = axis;
-        s.half = half;
         s.outer = outer;
         s.L = L;
         s.inner = inner;
@@ -761,7 +759,6 @@ static int build_stages(RunDesc &r, int W, int R, int xpt, int &slot) {
         s.kind = ST_ROWS;
         s.kick = 1;
         s.axis = axis;
-        s.half = 1;
         s.outer = outer;
         s.L = L;
         s.inner = 1;
@@ -779,7 +776,7 @@ static int build_stages(RunDesc &r, int W, int R, int xpt, int &slot) {
     int k = 0;
     if (D == 1) {
         r.st[k++] = rows(0, r.NX, r.nv[0], 1);
-        r.st[k++] = cols(0, 0, 0, 1, r.nx[0], r.NV, 1, 1, r.nv[0]);
+        r.st[k++] = cols(0, 0, 1, r.nx[0], r.NV, 1, 1, r.nv[0]);
         StageDesc p{};
         p.kind = ST_POISSON;
         p.tiles = 1;
@@ -787,11 +784,11 @@ static int build_stages(RunDesc &r, int W, int R, int xpt, int &slot) {
         r.st[k++] = rows(0, r.NX, r.nv[0], 1);
     } else {
         // kick v1 (strided over v2), kick v2 (contiguous)
-        r.st[k++] = cols(1, 0, 1, r.NX, r.nv[0], r.nv[1], 0, 1, 1);
+        r.st[k++] = cols(1, 0, r.NX, r.nv[0], r.nv[1], 0, 1, 1);
         r.st[k++] = rows(1, r.NX * r.nv[0], r.nv[1], r.nv[0]);
         // drift x2 then x1 (Eq. 55 order)
-        r.st[k++] = cols(0, 1, 0, r.nx[0], r.nx[1], r.NV, 1, 1, r.nv[1]);
-        r.st[k++] = cols(0, 0, 0, 1, r.nx[0], (long long)r.nx[1] * r.NV, 1, r.nv[1], r.nv[0]);
+        r.st[k++] = cols(0, 1, r.nx[0], r.nx[1], r.NV, 1, 1, r.nv[1]);
+        r.st[k++] = cols(0, 0, 1, r.nx[0], (long long)r.nx[1] * r.NV, 1, r.nv[1], r.nv[0]);
         StageDesc m{};
         m.kind = ST_MOMENT;
         m.tiles = (int)((r.NX + xpt - 1) / xpt);
@@ -813,7 +810,7 @@ static int build_stages(RunDesc &r, int W, int R, int xpt, int &slot) {
             solve(ST_FFT_BACK, wr, n0 / wr);
             solve(ST_FORCE, kFftTile, (int)(r.NX / kFftTile));
         }
-        r.st[k++] = cols(1, 0, 1, r.NX, r.nv[0], r.nv[1], 0, 1, 1);
+        r.st[k++] = cols(1, 0, r.NX, r.nv[0], r.nv[1], 0, 1, 1);
         r.st[k++] = rows(1, r.NX * r.nv[0], r.nv[1], r.nv[0]);
     }
     r.nstage = k;

@@ -1053,12 +1053,6 @@ int fft_launch(cudaStream_t st, double2 *buf, const FftLaunch &l) {
 
 constexpr int kFftSmem = 3 * 4096 * (int)sizeof(double2);  // table and two buffers of the longest axis
 
-// largest periodic 1D axis solved as a convolution (its densities are staged
-// in 32 KB of shared memory)
-constexpr int kConvMax = 4096;
-
-ForceArgs force_args(const vp_grid &g, const int *m, long long NX);
-
 Fda fda_coeffs(int order) {
     // central differences of Eqs. (C9)-(C11): sum_k c_k (phi_{i+k} - phi_{i-k}) / (den h)
     Fda f{};

@@ -20,9 +20,10 @@
 // the fine-grid mass through every coarse interface (mean over the fine
 // lines a coarse line aggregates), minus the coarse integer-shift part and
 // the coarse MP-limited fractional mass, over s, is the target of g.
-// Training: per-sample forward/backward (FP32, bfloat16-rounded weights and
-// activations, straight-through backward), per-CTA weight-gradient
-// reductions, Adam.
+// Training: forward and backward on the tensor cores, a tile of 16 samples per
+// warp (bfloat16-rounded weights, inputs and activations, FP32 sums, deltas in
+// three bfloat16 terms, straight-through backward), weight gradients summed per
+// CTA, Adam.
 #include <cuda_bf16.h>
 
 #include <atomic>
@@ -1010,11 +1011,6 @@ __global__ void __launch_bounds__(256) k_group_mean(const double *__restrict__ G
 
 constexpr int kTcThreads = 128;  // one line per thread, one 128-row MMA operand per interface step
 
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t *>(&v);
-}
-
 // tile of a learned sweep: columns col = (g cmod + j) T + t hold the line with
 // inner index c = c_tile + g cmod cdiv + j cdiv + t (class j); tiles per outer
 // index: (inner / (G cmod cdiv)) (cdiv / T)
@@ -1170,7 +1166,7 @@ __global__ void __launch_bounds__(kTcThreads) k_learned_walk(const float *__rest
 #pragma unroll
         for (int kk = 4; kk < vp_umma::kK / 8; ++kk)
             *reinterpret_cast<uint4 *>(A + b * kABytes + vp_umma::kmajor_offset(threadIdx.x, 8 * kk)) =
-                kk == 4 ? make_uint4(pack_bf16(1.f, 1.f), 0u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+                kk == 4 ? make_uint4(pack2(1.f, 1.f), 0u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x < 32) vp_umma::tmem_alloc(&tslot, tmem_cols(LC));
     if (threadIdx.x == 0) {
         vp_tma::mbar_init(&bar, 1);
@@ -1281,13 +1277,13 @@ __global__ void __launch_bounds__(kTcThreads) k_learned_walk(const float *__rest
             const float hinv = 0.5f * inv;
             uint32_t w[16];
 #pragma unroll
-            for (int m = 0; m < 4; ++m) w[m] = pack_bf16((u[2 * m] - u[3]) * inv, (u[2 * m + 1] - u[3]) * inv);
-            w[1] = pack_bf16((u[2] - u[3]) * inv, 0.f);
+            for (int m = 0; m < 4; ++m) w[m] = pack2((u[2 * m] - u[3]) * inv, (u[2 * m + 1] - u[3]) * inv);
+            w[1] = pack2((u[2] - u[3]) * inv, 0.f);
 #pragma unroll
-            for (int m = 0; m < 4; ++m) w[4 + m] = pack_bf16(dv[2 * m] * hinv, dv[2 * m + 1] * hinv);
+            for (int m = 0; m < 4; ++m) w[4 + m] = pack2(dv[2 * m] * hinv, dv[2 * m + 1] * hinv);
 #pragma unroll
-            for (int m = 0; m < 4; ++m) w[8 + m] = pack_bf16(cv[2 * m] * inv, cv[2 * m + 1] * inv);
-            w[12] = pack_bf16(nu, 0.f);
+            for (int m = 0; m < 4; ++m) w[8 + m] = pack2(cv[2 * m] * inv, cv[2 * m + 1] * inv);
+            w[12] = pack2(nu, 0.f);
             w[13] = w[14] = w[15] = 0u;
             store_row(A + b * kABytes, threadIdx.x, w);
             // advance the window and the MP carries

@@ -203,7 +203,7 @@ struct vp_ctx {
     double *d_diag;                     // VP_NDIAG doubles
     void *d_vw;                         // kinetic-energy weights: velocity rows, then the last axis
     double vw_unit;                     // the power of two they are divided by
-    double *d_diagblk;                  // diagnostics: per-block results, then the counter of finished blocks
+    double *d_diagblk;                  // diagnostics: per-block results (d_diagctr: finished blocks)
     unsigned *d_diagctr;
     int *d_flag;                        // non-finite flag
     long long launches;
@@ -302,7 +302,7 @@ FieldSizes vp_field_sizes(const vp_ctx *c);
 int vp_field_setup(vp_ctx *c);          // fills those tables, the isolated Green function (at create)
 // CSL weight polynomials of the given order (5 or 7), from the definition of the SL flux
 WPoly vp_csl_weight_polys(int order);
-// learned flux correction network: 9 features, 3 hidden layers of 32
+// learned flux correction network: 25 features, 3 hidden layers of 32
 #define VP_NET_FEATURES 25
 #define VP_NET_HIDDEN 32
 // analytic initial condition into any f array of grid g (precision from g)

@@ -624,15 +624,6 @@ __device__ __forceinline__ double csl_weight(const WPoly &wp, int k, double nu) 
     for (int j = wp.nterm - 1; j >= 0; --j) acc = fma(acc, nu, wp.c[j][k]);
     return acc;
 }
-template <typename T>
-__device__ __forceinline__ LineShift<T> make_shift(double speed, double dt, double h, const WPoly &wp) {
-    LineShift<T> sh;
-    const double nu = split_shift(speed, dt, h, sh);
-#pragma unroll
-    for (int k = 0; k < 7; ++k) sh.w[k] = (T)csl_weight(wp, k, nu);
-    return sh;
-}
-
 // velocity of cell j of an axis: lo + (j + 1/2) dv, rounded step by step
 __device__ __forceinline__ double cell_centre(double lo, double dvel, int j) {
     return __dadd_rn(lo, __dmul_rn((double)j + 0.5, dvel));
