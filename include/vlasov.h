@@ -427,7 +427,8 @@ int vp_group_mean(const double *G_fine, long long n_coarse_lines, int nout, cons
 
 /* coarse f = mean over factor1 x factor2 fine velocity cells ([NX][nf1][nf2]
  * -> [NX][nf1/factor1][nf2/factor2]; nf2 = factor2 = 1 for one velocity
- * dimension); device arrays */
+ * dimension); device arrays.  VP_EINVAL for NULL arrays, empty axes or factors
+ * that do not divide them */
 int vp_restrict_velocity(const float *f_fine, float *f_coarse, long long NX, int nf1, int nf2, int factor1,
                          int factor2, void *cuda_stream);
 
